@@ -805,7 +805,7 @@ int build_handle(const std::vector<Spec> &specs, void *stream, bd_handle **out) 
     BD_TRY(dalloc(h, &d.pos, nv));
     BD_TRY(dalloc(h, &d.prev, nv));
     BD_TRY(dalloc(h, &d.pos0, nv));
-    BD_TRY(dalloc(h, &d.work, (size_t)np));
+    BD_TRY(dalloc(h, &d.work, nv));
     BD_TRY(dalloc(h, &d.theta, (size_t)np));
     BD_TRY(dalloc(h, &d.theta0, (size_t)np));
     BD_TRY(dalloc(h, &d.species, (size_t)np));
@@ -1033,6 +1033,15 @@ int build_handle(const std::vector<Spec> &specs, void *stream, bd_handle **out) 
     // chosen by timing (or fixed by BD_FORCE_VARIANT / BD_FORCE_TILES)
     {
       BD_TRY(bd_launch_work_copy(d, c, st));
+      // the ghost points' FP32 pairs (they never move)
+      std::vector<float4> gw(ng_total);
+      for (int k = 0; k < ng_total; ++k) {
+        const double gx = X[np + k], gy = Y[np + k];
+        const float xh = (float)gx, yh = (float)gy;
+        gw[k] = make_float4(xh, yh, (float)(gx - (double)xh), (float)(gy - (double)yh));
+      }
+      if (ng_total)
+        BD_TRY(cudaMemcpyAsync(d.work + np, gw.data(), gw.size() * sizeof(float4), cudaMemcpyHostToDevice, st));
       BD_TRY(cudaStreamSynchronize(st));
       const char *fv = getenv("BD_FORCE_VARIANT"), *ft = getenv("BD_FORCE_TILES");
       long long nmax = 0;

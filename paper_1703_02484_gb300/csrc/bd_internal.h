@@ -121,7 +121,7 @@ struct BdRep {
 struct BdDev {
   // disks (internal order, np slots), then the ghost points of every replica
   double2 *pos, *prev, *pos0;
-  float4 *work;            // (x_hi, y_hi, x_lo, y_lo) FP32 pair of each coordinate
+  float4 *work;            // (x_hi, y_hi, x_lo, y_lo) FP32 pair of each coordinate (disks and ghosts)
   float *theta, *theta0;
   uint8_t *species;        // 255 = empty slot
   int *ext_id;             // index within its replica (-1 = empty slot): the Philox counter

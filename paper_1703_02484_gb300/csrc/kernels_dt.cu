@@ -92,7 +92,11 @@ struct Ctx {
 // exact inputs (3e-16 / 1.1e-15 relative in FP64, i.e. about 4 and 11 units
 // of the working precision) plus one unit per input factor, times a safety
 // factor of about four.  Outside the bound the FP32 sign is the exact sign;
-// inside it, or for ghost points (no FP32 copy), the integer path decides.
+// inside it the integer path decides.  Ghost points hold the same pairs (rows
+// beside the walls: a test with one used to take the integer path, and the
+// threads that did set the length of the whole pass), and a corner with an
+// image shift takes its differences from the integer grid instead, one
+// rounding each.
 __device__ __forceinline__ float fdiff(float bh, float bl, float ah, float al) {
   return __fadd_rn(__fsub_rn(bh, ah), __fsub_rn(bl, al));
 }
@@ -165,60 +169,63 @@ __device__ __forceinline__ void count_exact(const Ctx &x) {
   atomicAdd((unsigned long long *)&x.d.ctl->st_exact, 1ull);
 }
 
-// the filters on preloaded FP32 pairs (filt: all corners are disks, whose
-// pairs are loaded; ghost points have none)
-__device__ __forceinline__ int orient_pre(const Ctx &x, bool filt, const float4 &wa, const float4 &wb,
+// the filters themselves, on coordinate differences that each carry about one
+// FP32 rounding of themselves: the sign, or 0 when the bound does not decide
+__device__ __forceinline__ int orient_f(float bax, float bay, float cax, float cay) {
+  const float l = __fmul_rn(bax, cay), r = __fmul_rn(bay, cax);
+  const float det = __fsub_rn(l, r);
+  const float bound = 1.5e-6f * __fadd_rn(fabsf(l), fabsf(r));
+  return det > bound ? 1 : (-det > bound ? -1 : 0);
+}
+
+__device__ __forceinline__ int incircle_f(float adx, float ady, float bdx, float bdy, float cdx, float cdy) {
+  const float bcl = __fmul_rn(bdx, cdy), bcr = __fmul_rn(bdy, cdx);
+  const float cal = __fmul_rn(cdx, ady), car = __fmul_rn(cdy, adx);
+  const float abl = __fmul_rn(adx, bdy), abr = __fmul_rn(ady, bdx);
+  const float al = __fadd_rn(__fmul_rn(adx, adx), __fmul_rn(ady, ady));
+  const float bl = __fadd_rn(__fmul_rn(bdx, bdx), __fmul_rn(bdy, bdy));
+  const float cl = __fadd_rn(__fmul_rn(cdx, cdx), __fmul_rn(cdy, cdy));
+  const float det = __fadd_rn(__fadd_rn(__fmul_rn(al, __fsub_rn(bcl, bcr)), __fmul_rn(bl, __fsub_rn(cal, car))),
+                              __fmul_rn(cl, __fsub_rn(abl, abr)));
+  const float perm =
+      __fadd_rn(__fadd_rn(__fmul_rn(al, __fadd_rn(fabsf(bcl), fabsf(bcr))), __fmul_rn(bl, __fadd_rn(fabsf(cal), fabsf(car)))),
+                __fmul_rn(cl, __fadd_rn(fabsf(abl), fabsf(abr))));
+  const float bound = 4e-6f * perm;
+  return det > bound ? 1 : (-det > bound ? -1 : 0);
+}
+
+// the filters on preloaded FP32 pairs (disks: all corners are disks, whose
+// undecided tests are counted; ghost points hold the same FP32 pairs)
+__device__ __forceinline__ int orient_pre(const Ctx &x, bool disks, const float4 &wa, const float4 &wb,
                                           const float4 &wc, int a, int b, int c) {
-  if (filt) {
-    const float bax = fdiff(wb.x, wb.z, wa.x, wa.z), bay = fdiff(wb.y, wb.w, wa.y, wa.w);
-    const float cax = fdiff(wc.x, wc.z, wa.x, wa.z), cay = fdiff(wc.y, wc.w, wa.y, wa.w);
-    const float l = __fmul_rn(bax, cay), r = __fmul_rn(bay, cax);
-    const float det = __fsub_rn(l, r);
-    const float bound = 1.5e-6f * __fadd_rn(fabsf(l), fabsf(r));
-    if (det > bound) return 1;
-    if (-det > bound) return -1;
-    count_exact(x);
-  }
+  const int o = orient_f(fdiff(wb.x, wb.z, wa.x, wa.z), fdiff(wb.y, wb.w, wa.y, wa.w),
+                         fdiff(wc.x, wc.z, wa.x, wa.z), fdiff(wc.y, wc.w, wa.y, wa.w));
+  if (o) return o;
+  if (disks) count_exact(x);
   return orient_exact(x.d.pos, x.g, a, b, c);
 }
 
-__device__ __forceinline__ int incircle_pre(const Ctx &x, bool filt, const float4 &wa, const float4 &wb,
+__device__ __forceinline__ int incircle_pre(const Ctx &x, bool disks, const float4 &wa, const float4 &wb,
                                             const float4 &wc, const float4 &wp, int a, int b, int c, int p) {
-  if (filt) {
-    const float adx = fdiff(wa.x, wa.z, wp.x, wp.z), ady = fdiff(wa.y, wa.w, wp.y, wp.w);
-    const float bdx = fdiff(wb.x, wb.z, wp.x, wp.z), bdy = fdiff(wb.y, wb.w, wp.y, wp.w);
-    const float cdx = fdiff(wc.x, wc.z, wp.x, wp.z), cdy = fdiff(wc.y, wc.w, wp.y, wp.w);
-    const float bcl = __fmul_rn(bdx, cdy), bcr = __fmul_rn(bdy, cdx);
-    const float cal = __fmul_rn(cdx, ady), car = __fmul_rn(cdy, adx);
-    const float abl = __fmul_rn(adx, bdy), abr = __fmul_rn(ady, bdx);
-    const float al = __fadd_rn(__fmul_rn(adx, adx), __fmul_rn(ady, ady));
-    const float bl = __fadd_rn(__fmul_rn(bdx, bdx), __fmul_rn(bdy, bdy));
-    const float cl = __fadd_rn(__fmul_rn(cdx, cdx), __fmul_rn(cdy, cdy));
-    const float det = __fadd_rn(__fadd_rn(__fmul_rn(al, __fsub_rn(bcl, bcr)), __fmul_rn(bl, __fsub_rn(cal, car))),
-                                __fmul_rn(cl, __fsub_rn(abl, abr)));
-    const float perm =
-        __fadd_rn(__fadd_rn(__fmul_rn(al, __fadd_rn(fabsf(bcl), fabsf(bcr))), __fmul_rn(bl, __fadd_rn(fabsf(cal), fabsf(car)))),
-                  __fmul_rn(cl, __fadd_rn(fabsf(abl), fabsf(abr))));
-    const float bound = 4e-6f * perm;
-    if (det > bound) return 1;
-    if (-det > bound) return -1;
-    count_exact(x);
-  }
+  const int o = incircle_f(fdiff(wa.x, wa.z, wp.x, wp.z), fdiff(wa.y, wa.w, wp.y, wp.w),
+                           fdiff(wb.x, wb.z, wp.x, wp.z), fdiff(wb.y, wb.w, wp.y, wp.w),
+                           fdiff(wc.x, wc.z, wp.x, wp.z), fdiff(wc.y, wc.w, wp.y, wp.w));
+  if (o) return o;
+  if (disks) count_exact(x);
   return incircle_exact(x.d.pos, x.g, a, b, c, p);
 }
 
-__device__ __forceinline__ float4 work_of(const Ctx &x, int v) {
-  return v < x.np ? x.d.work[v] : make_float4(0.f, 0.f, 0.f, 0.f);
-}
+// FP32 (hi, lo) pair of a disk or ghost point
+__device__ __forceinline__ float4 work_of(const Ctx &x, int v) { return x.d.work[v]; }
 
 __device__ __forceinline__ int orient_v(const Ctx &x, int a, int b, int c) {
-  const bool filt = a < x.np && b < x.np && c < x.np;
-  return orient_pre(x, filt, work_of(x, a), work_of(x, b), work_of(x, c), a, b, c);
+  const bool disks = a < x.np && b < x.np && c < x.np;
+  return orient_pre(x, disks, work_of(x, a), work_of(x, b), work_of(x, c), a, b, c);
 }
 
 __device__ __forceinline__ int incircle_v(const Ctx &x, int a, int b, int c, int p) {
-  const bool filt = a < x.np && b < x.np && c < x.np && p < x.np;
-  return incircle_pre(x, filt, work_of(x, a), work_of(x, b), work_of(x, c), work_of(x, p), a, b, c, p);
+  const bool disks = a < x.np && b < x.np && c < x.np && p < x.np;
+  return incircle_pre(x, disks, work_of(x, a), work_of(x, b), work_of(x, c), work_of(x, p), a, b, c, p);
 }
 
 // Sec. 4.3 reversal test r0 . r1 < 0 of the edge u -> w, exact on the grid:
@@ -275,6 +282,11 @@ __device__ __forceinline__ Lift lift(const Ctx &x, int v, int sx, int sy, long l
   return {bdpred::to_int(p.x, x.g) + sx * LQ, bdpred::to_int(p.y, x.g) + sy * LQ};
 }
 
+// difference of two lifted coordinates, exact in grid units, rounded once to FP32
+__device__ __forceinline__ float lift_diff(const Ctx &x, long long b, long long a) {
+  return bdem::grid_to_float(b - a, x.g.s);
+}
+
 __device__ __forceinline__ long long rep_LQ(const Ctx &x, int v) { return x.d.rep[x.d.rep_of[v]].LQ; }
 
 // orientation of corners (a, b, c) with shifts (sa, sb, sc)
@@ -283,6 +295,9 @@ __device__ __forceinline__ int orient_s(const Ctx &x, int a, int sax, int say, i
   if ((sax | say | sbx | sby | scx | scy) == 0) return orient_v(x, a, b, c);
   const long long LQ = rep_LQ(x, a);
   const Lift A = lift(x, a, sax, say, LQ), B = lift(x, b, sbx, sby, LQ), C = lift(x, c, scx, scy, LQ);
+  const int o = orient_f(lift_diff(x, B.x, A.x), lift_diff(x, B.y, A.y), lift_diff(x, C.x, A.x),
+                         lift_diff(x, C.y, A.y));
+  if (o) return o;
   return orient_lifted(A.x, A.y, B.x, B.y, C.x, C.y);
 }
 
@@ -294,6 +309,9 @@ __device__ __forceinline__ int incircle_s(const Ctx &x, const int4 &v, int p, in
   const long long LQ = rep_LQ(x, v.x);
   const Lift A = lift(x, v.x, shx(w, 0), shy(w, 0), LQ), B = lift(x, v.y, shx(w, 1), shy(w, 1), LQ);
   const Lift C = lift(x, v.z, shx(w, 2), shy(w, 2), LQ), P = lift(x, p, spx, spy, LQ);
+  const int o = incircle_f(lift_diff(x, A.x, P.x), lift_diff(x, A.y, P.y), lift_diff(x, B.x, P.x),
+                           lift_diff(x, B.y, P.y), lift_diff(x, C.x, P.x), lift_diff(x, C.y, P.y));
+  if (o) return o;
   return incircle_lifted(A.x, A.y, B.x, B.y, C.x, C.y, P.x, P.y);
 }
 
@@ -829,17 +847,24 @@ __global__ void __launch_bounds__(BD_DT_THREADS, 3) k_triangulation(BdDev d, BdC
             long long LQ = 0;
             if (rsx | rsy) LQ = rep_LQ(x, u);
             const bool plain = (rsx | rsy) == 0;   // the edge carries no image shift
-            // r1 = r_w - r_u from the FP32 pairs (unshifted edges)
-            const float r1x = plain ? fdiff(W[kw].x, W[kw].z, W[ku].x, W[ku].z) : 0.f;
-            const float r1y = plain ? fdiff(W[kw].y, W[kw].w, W[ku].y, W[ku].w) : 0.f;
+            // r1 = r_w - r_u from the FP32 pairs, or for a shifted edge from the grid
+            float r1x, r1y;
+            if (plain) {
+              r1x = fdiff(W[kw].x, W[kw].z, W[ku].x, W[ku].z);
+              r1y = fdiff(W[kw].y, W[kw].w, W[ku].y, W[ku].w);
+            } else {
+              const Lift U = lift(x, u, 0, 0, LQ), V = lift(x, w, rsx, rsy, LQ);
+              r1x = lift_diff(x, V.x, U.x);
+              r1y = lift_diff(x, V.y, U.y);
+            }
             if (disks && mv) {
-              // Sec. 4.3 first criterion: r0 . r1 < 0.  An unshifted edge whose
-              // ends did not re-enter is screened in FP32 from r1 and the moves,
-              // as with walls; otherwise, and near zero, exact on the grid (the
-              // edge's shift before the move is the present one less the
-              // re-entries of its end points)
+              // Sec. 4.3 first criterion: r0 . r1 < 0.  An edge whose ends did
+              // not re-enter is screened in FP32 from r1 and the moves, as with
+              // walls; otherwise, and near zero, exact on the grid (the edge's
+              // shift before the move is the present one less the re-entries
+              // of its end points)
               int dec = 0;   // 1 reversed, -1 not, 0 undecided
-              if (plain && (wr[ku] | wr[kw]) == 0) {
+              if ((wr[ku] | wr[kw]) == 0) {
                 const float2 mu = mvd[ku] ? d.dmove[u] : make_float2(0.f, 0.f);
                 const float2 mw = mvd[kw] ? d.dmove[w] : make_float2(0.f, 0.f);
                 const float r0x = __fsub_rn(r1x, __fsub_rn(mw.x, mu.x)), r0y = __fsub_rn(r1y, __fsub_rn(mw.y, mu.y));
@@ -850,7 +875,7 @@ __global__ void __launch_bounds__(BD_DT_THREADS, 3) k_triangulation(BdDev d, BdC
                                                     __fadd_rn(__fmul_rn(mw.x, mw.x), __fmul_rn(mw.y, mw.y))));
                 const float bound = 4e-6f * S;
                 dec = dot > bound ? -1 : (-dot > bound ? 1 : 0);
-                if (dec == 0) count_exact(x);
+                if (dec == 0 && plain) count_exact(x);
               }
               int ox = rsx, oy = rsy;
               if (dec == 0) {
@@ -888,9 +913,8 @@ __global__ void __launch_bounds__(BD_DT_THREADS, 3) k_triangulation(BdDev d, BdC
             }
             if (disks && scan) {
               // FP32 screen: a pair whose FP32 squared distance exceeds
-              // sigma^2 (1 + 1e-5) is farther than sigma (FP32 error ~3e-7);
-              // edges across a periodic box edge skip it
-              if (plain && __fadd_rn(__fmul_rn(r1x, r1x), __fmul_rn(r1y, r1y)) > x.sig2f) continue;
+              // sigma^2 (1 + 1e-5) is farther than sigma (FP32 error ~3e-7)
+              if (__fadd_rn(__fmul_rn(r1x, r1x), __fmul_rn(r1y, r1y)) > x.sig2f) continue;
               double2 v;
               double del;
               if (edge_overlap(x, u, w, rsx, rsy, LQ, v, del)) {
