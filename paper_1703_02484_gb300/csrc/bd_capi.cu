@@ -915,7 +915,7 @@ int build_handle(const std::vector<Spec> &specs, void *stream, bd_handle **out) 
       BD_TRY(dalloc(h, &d.cell_cursor, nc2));
       BD_TRY(dalloc(h, &d.cell_idx, (size_t)np));
       BD_TRY(dalloc(h, &d.cell_of, (size_t)np));
-      BD_TRY(dalloc(h, &d.scan_sums, (nc2 + 511) / 512 + 1));
+      BD_TRY(dalloc(h, &d.scan_sums, BD_VL_MAXGRID));
     }
     if (c.overlap_verlet) {
       BD_TRY(dalloc(h, &d.vc_hit, (size_t)np));
@@ -1062,6 +1062,7 @@ int build_handle(const std::vector<Spec> &specs, void *stream, bd_handle **out) 
       }
     }
     if (bd_dt_grid_for(std::max(nt, np), &h->dt_grid, &h->dt_block) != 0 ||
+        (c.any_short && bd_vl_grid_for(np, &c.vl_grid) != 0) ||
         (c.overlap_verlet && bd_vcorr_grid_for(np, &h->vc_grid, &h->vc_block) != 0)) {
       bd_free(h);
       return BD_ERR_CUDA;
@@ -1113,6 +1114,7 @@ int finish_status(bd_handle *h, int status) {
     cudaMemsetAsync(h->d.ctl, 0, offsetof(BdCtl, epoch), st);
   }
   cudaMemsetAsync(&h->d.ctl->cnt[0][0], 0, sizeof(h->d.ctl->cnt), st);
+  cudaMemsetAsync(&h->d.ctl->in_move, 0, sizeof(int), st);
   cudaMemsetAsync(&h->d.ctl->status, 0, sizeof(int), st);
   cudaStreamSynchronize(st);
   return status;

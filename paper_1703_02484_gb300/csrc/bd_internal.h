@@ -21,6 +21,11 @@
 // neighbours within 5.6a even at close packing)
 #define BD_VL_MAX 64
 
+// threads per block of the Verlet-list kernels, and the largest grid of the
+// rebuild launch (BdDev::scan_sums holds a word of each block)
+#define BD_VL_THREADS 256
+#define BD_VL_MAXGRID 1024
+
 // threads (and i disks) per block of the all-pairs force adjoint
 #define BD_ADJ_T 128
 
@@ -81,6 +86,8 @@ struct BdCtl {
   long long step_dev;              // index of the next step (advanced by the triangulation kernel)
   int n_wrapped;                   // periodic box: disks that re-entered in the last move (consumed
                                    // by the triangulation kernel's shift pass; not a statistic)
+  int in_move;                     // positions have moved and their correction has not finished: what a
+                                   // timed-out barrier has to undo (set by the mover, cleared by the corrector)
   int act_n[3];                    // lengths of the rotating triangle lists (zeroed at kernel exit)
   int cl_n[3];                     // lengths of the candidate lists (zeroed at kernel exit)
   unsigned act_gen;                // next list generation (grows across launches)
@@ -221,6 +228,7 @@ struct BdConst {
   int tri_fuse;            // 1: a Lawson round tests the outer edges of its flips and keeps the
                            // overlap sums (no check pass between rounds); 0: a check pass after
                            // every round (environment variable BD_TRI_FUSE at init)
+  int vl_grid;             // blocks of the Verlet-list rebuild launch
   double vl_reach2;        // squared displacement since the list build below which the lists
                            // still hold every pair closer than sigma
   int log_pairs_cap, log_pass_cap;   // rollout log capacities
@@ -250,6 +258,7 @@ cudaError_t bd_launch_state_out(const BdDev &d, const BdConst &c, cudaStream_t s
 cudaError_t bd_launch_periodic_wraps(const BdDev &d, const BdConst &c, cudaStream_t s);
 cudaError_t bd_launch_force_short(const BdDev &d, const BdConst &c, cudaStream_t s);
 int bd_short_launches();
+int bd_vl_grid_for(int np, int *grid);
 cudaError_t bd_launch_force_sum(const BdDev &d, const BdConst &c, double2 *out, cudaStream_t s);
 cudaError_t bd_launch_force_sym(const BdDev &d, const BdConst &c, int variant, cudaStream_t s);
 // advance = 0: a piece of a halved step (the step counter does not advance);
@@ -259,7 +268,8 @@ cudaError_t bd_launch_overlap_verlet(const BdDev &d, const BdConst &c, cudaStrea
                                      int advance = 1);
 // a halved step completed: advance the device step counter and the step count
 cudaError_t bd_launch_advance_step(const BdDev &d, cudaStream_t s);
-// after a timed-out grid barrier: undo the step (or the new positions of
+// after a timed-out grid barrier: make the next step rebuild Verlet lists whose
+// rebuild it cut off and, if positions had moved, undo the step (or the new positions of
 // bd_set_state) from the step-start copies and the undo journal, as their own
 // failure path does, and clear the flip claims and list marks the abandoned
 // launch may have left

@@ -45,7 +45,9 @@ enum { BC_CNT = 0, BC_ACT = 8, BC_CL = 11, BC_N = 14 };
 // bounded grid barrier; returns false if the grid must stop.  With bc (block
 // shared, BC_N ints): bc[BC_CNT + k] = the counters of the phase that just
 // ended, bc[BC_ACT + l] = the lengths of the triangle lists, bc[BC_CL + l]
-// those of the candidate lists.
+// those of the candidate lists.  HOLD: the barrier obeys the host's test hold
+// (the kernels of a move do; the Verlet-list rebuild does not).
+template <bool HOLD = true>
 static __device__ bool grid_sync(BdCtl *ctl, Bar &b, int *bc = nullptr) {
   __shared__ int s_ok;
   __syncthreads();
@@ -58,7 +60,7 @@ static __device__ bool grid_sync(BdCtl *ctl, Bar &b, int *bc = nullptr) {
       // host-set limit and test hold (read once per barrier by one thread)
       const unsigned long long lim_set = *(volatile const unsigned long long *)&ctl->bar_limit_ns;
       const unsigned long long limit = lim_set ? lim_set : BD_BARRIER_TIMEOUT_NS;
-      const unsigned hold = *(volatile const unsigned *)&ctl->bar_hold;
+      const unsigned hold = HOLD ? *(volatile const unsigned *)&ctl->bar_hold : 0u;
       const unsigned last = gridDim.x - 1u + (hold != 0u && hold == target ? 1u : 0u);
       __threadfence();
       unsigned arrived = atomicAdd(&ctl->bar_count, 1u);

@@ -699,6 +699,7 @@ __global__ void __launch_bounds__(BD_DT_THREADS, 3) k_triangulation(BdDev d, BdC
   BdCtl *ctl = d.ctl;
   if (ld_status(&ctl->status) != 0 || (mode == 1 && *(volatile const int *)&ctl->n_set_moved == 0)) {
     // (bd_set_state that moved no disk: the triangulation stands as it was)
+    if (blockIdx.x == 0 && threadIdx.x == 0 && ld_status(&ctl->status) == 0) ctl->in_move = 0;
     block_exit(ctl);
     return;
   }
@@ -1406,6 +1407,7 @@ __global__ void __launch_bounds__(BD_DT_THREADS, 3) k_triangulation(BdDev d, BdC
       d.log_step_pass[log_step + 1] = log_npass;
     }
     ctl->epoch = epoch + 1;
+    ctl->in_move = 0;
     ctl->act_gen = g0 + (unsigned)kp + 3u;
     ctl->st_tri_visits += tri_visits;
     ctl->st_corr_iters += corr_iter;
@@ -1433,6 +1435,11 @@ __global__ void __launch_bounds__(BD_DT_THREADS, 3) k_triangulation(BdDev d, BdC
 __global__ void k_restore_step(BdDev d, BdConst c) {
   const int tid = blockIdx.x * blockDim.x + threadIdx.x;
   const int nth = gridDim.x * blockDim.x;
+  // a rebuild of the Verlet lists was cut off (the force that follows it takes
+  // the request back): references parked far away make the next step rebuild
+  if (c.any_short && *(volatile const int *)&d.ctl->vl_need)
+    for (int i = tid; i < c.np; i += nth) d.vl_ref[i] = make_double2(1e30, 1e30);
+  if (!*(volatile const int *)&d.ctl->in_move) return;   // nothing had moved yet
   for (int i = tid; i < c.np; i += nth) {
     if (d.ext_id[i] < 0) continue;
     const double2 p0 = d.pos0[i];

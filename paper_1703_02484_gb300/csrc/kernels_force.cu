@@ -539,6 +539,7 @@ __global__ void k_integrate(BdDev d, BdConst c, long long step, int log_step, in
   if (ctl_failed(d.ctl)) return;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= c.np) return;
+  if (i == 0) d.ctl->in_move = 1;
   if (step < 0) step = *(volatile const long long *)&d.ctl->step_dev;
   const int e = d.ext_id[i];
   if (e < 0) return;

@@ -61,6 +61,7 @@ __global__ void k_state_in(BdDev d, BdConst c, int with_theta) {
   if (*(volatile const int *)&d.ctl->status) return;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= c.np) return;
+  if (i == 0) d.ctl->in_move = 1;
   const int e = d.ext_glob[i];
   if (e < 0) return;
   const BdRep &R = d.rep[d.rep_of[i]];

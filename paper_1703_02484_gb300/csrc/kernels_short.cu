@@ -25,8 +25,8 @@
 
 #include "bd_internal.h"
 #include "em.cuh"
+#include "gridsync.cuh"
 
-#define BD_SCAN_B 512
 
 namespace {
 
@@ -94,27 +94,21 @@ __device__ __forceinline__ const BdRep *short_rep(const BdDev &d, int i) {
   return R->law == BD_LAW_SHORT ? R : nullptr;
 }
 
-// block-uniform early exit: one thread reads the flags
-__device__ __forceinline__ bool skip_block(const BdCtl *ctl, bool need_rebuild) {
-  __shared__ int s_skip;
-  if (threadIdx.x == 0) s_skip = failed(ctl) || (need_rebuild && !need(ctl));
-  __syncthreads();
-  return s_skip != 0;
-}
-
 }  // namespace
 
-// 1. displacement trigger: some disk moved more than skin/2 since the build
-__global__ void k_vl_check(BdDev d, BdConst c) {
-  if (skip_block(d.ctl, false)) return;
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
+// Displacement trigger: some disk moved more than skin/2 since the build.
+// Bound by memory (36 bytes a disk); every load of a thread is issued before
+// the status is looked at.
+__global__ void __launch_bounds__(BD_VL_THREADS) k_vl_check(BdDev d, BdConst c) {
+  const int i = blockIdx.x * BD_VL_THREADS + threadIdx.x;
+  const int bad = failed(d.ctl);
   bool hit = false;
   if (i < c.np) {
+    const double2 p = d.pos[i], r = d.vl_ref[i];
     const BdRep *R = short_rep(d, i);
-    if (R) {
+    if (R && !bad) {
       // displacement since the build in grid units (exact), screened in FP32;
       // only a displacement within 1e-5 of skin/2 is decided in FP64
-      const double2 p = d.pos[i], r = d.vl_ref[i];
       const bdpred::Grid g{c.q, c.inv_q, c.qshift};
       if (r.x > 1e29) {
         hit = true;   // never built (reference parked far away)
@@ -143,170 +137,167 @@ __global__ void k_vl_check(BdDev d, BdConst c) {
   if (__any_sync(0xffffffffu, hit) && (threadIdx.x & 31) == 0) atomicExch(&d.ctl->vl_need, 1);
 }
 
-// 2. clear cell counts (grid-stride)
-__global__ void k_vl_clear(BdDev d, BdConst c) {
-  if (skip_block(d.ctl, true)) return;
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < c.ncell_total; k += gridDim.x * blockDim.x)
-    d.cell_count[k] = 0;
+// neighbour list of disk i from the cell grid (sorted), and its reference position
+__device__ __forceinline__ void vl_build_one(const BdDev &d, const BdConst &c, int i) {
+  const BdRep *Rp = short_rep(d, i);
+  if (!Rp || d.ext_id[i] < 0) {
+    d.vl_cnt[i] = 0;
+    return;
+  }
+  const BdRep &R = *Rp;
+  const double2 p = d.pos[i];
+  d.vl_ref[i] = p;
+  const float4 wi = d.work[i];
+  const float rl2f = (float)R.rl2;
+  const int k = d.cell_of[i] - R.cell_base;
+  const int cx = k % R.ncell, cy = k / R.ncell;
+  int buf[BD_VL_MAX];
+  int m = 0;
+  bool over = false;
+  for (int gy0 = cy - 1; gy0 <= cy + 1; ++gy0) {
+    // periodic box: the cells wrap around (at least three per side)
+    const int gy = R.periodic ? (gy0 + R.ncell) % R.ncell : gy0;
+    if (gy < 0 || gy >= R.ncell) continue;
+    for (int gx0 = cx - 1; gx0 <= cx + 1; ++gx0) {
+      const int gx = R.periodic ? (gx0 + R.ncell) % R.ncell : gx0;
+      if (gx < 0 || gx >= R.ncell) continue;
+      const int cc = R.cell_base + gy * R.ncell + gx;
+      const int b = d.cell_start[cc], e = b + d.cell_count[cc];
+      for (int s = b; s < e; ++s) {
+        const int j = d.cell_idx[s];
+        if (j == i) continue;
+        // FP32 screen from the (hi, lo) pairs: the hi difference is exact
+        // (Sterbenz) or off by at most half an ulp of a coordinate below 12
+        // (4.8e-7), so the computed r^2 is within 1e-6 of the exact one
+        // relative to the reach; only pairs within 1e-5 of the reach (and
+        // pairs across a periodic edge) take the FP64 decision
+        const float4 wj = d.work[j];
+        const float hx = __fsub_rn(wi.x, wj.x), hy = __fsub_rn(wi.y, wj.y);
+        bool in;
+        bool exact = R.periodic && (fabsf(hx) > R.hLf || fabsf(hy) > R.hLf);
+        if (!exact) {
+          const float fx = __fadd_rn(hx, __fsub_rn(wi.z, wj.z)), fy = __fadd_rn(hy, __fsub_rn(wi.w, wj.w));
+          const float f2 = __fadd_rn(__fmul_rn(fx, fx), __fmul_rn(fy, fy));
+          if (f2 < rl2f * 0.99999f) in = true;
+          else if (f2 > rl2f * 1.00001f) in = false;
+          else exact = true;
+        }
+        if (exact) {
+          const double2 q = d.pos[j];
+          const double dx = dmin_image(__dsub_rn(p.x, q.x), R), dy = dmin_image(__dsub_rn(p.y, q.y), R);
+          in = __dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)) < R.rl2;
+        }
+        if (in) {
+          if (m < BD_VL_MAX) {
+            // insertion in sorted position
+            int t = m++;
+            while (t > 0 && buf[t - 1] > j) {
+              buf[t] = buf[t - 1];
+              --t;
+            }
+            buf[t] = j;
+          } else {
+            over = true;
+          }
+        }
+      }
+    }
+  }
+  for (int t = 0; t < m; ++t) d.vl_idx[(size_t)t * c.np + i] = buf[t];
+  d.vl_cnt[i] = m;
+  if (over) atomicCAS(&d.ctl->status, 0, BD_ERR_UNSUPPORTED);
 }
 
-// 3. count disks per cell (grid-stride)
-__global__ void k_vl_count(BdDev d, BdConst c) {
-  if (skip_block(d.ctl, true)) return;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < c.np; i += gridDim.x * blockDim.x) {
+// exclusive prefix sum over the block of one value per thread; *total = the sum
+__device__ __forceinline__ int block_scan(int v, int *total) {
+  __shared__ int ws[BD_VL_THREADS / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int s = v;
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, s, o);
+    if (lane >= o) s += t;
+  }
+  if (lane == 31) ws[warp] = s;
+  __syncthreads();
+  int base = 0, all = 0;
+#pragma unroll
+  for (int w = 0; w < BD_VL_THREADS / 32; ++w) {
+    if (w < warp) base += ws[w];
+    all += ws[w];
+  }
+  __syncthreads();   // ws is reused by the next call
+  *total = all;
+  return base + s - v;
+}
+
+// Rebuild of the cell grid and the lists when the trigger fired, one
+// cooperative launch (a step that needs none leaves at once).  As seven
+// launches (clear, count, three of the scan, scatter, build) the seven of every
+// step without a rebuild took about 20 us of the device's time under ncu; now a
+// step at 2^20 disks takes 540 us instead of 549, at 20000 polydisperse disks 109
+// instead of 113.  Phases, each ended by
+// a bounded grid barrier: clear the cell counts; count; sum each block's share
+// of the cells; scan it from the sums before it, setting the scatter cursors;
+// scatter; build, which needs no barrier after it (its reads of the grid go
+// through L1, which the barrier's acquire has emptied; past L1 ten steps at
+// 2^20 disks with one rebuild took 6.06 instead of 5.40 ms).
+__global__ void __launch_bounds__(BD_VL_THREADS, 4) k_vl_rebuild(BdDev d, BdConst c) {
+  if (failed(d.ctl) || !need(d.ctl)) return;   // the same for every block: both words are set by earlier kernels
+  bdgs::Bar b;
+  b.gen = 0;
+  b.ph = 0;
+  const int tid = blockIdx.x * BD_VL_THREADS + threadIdx.x, nth = gridDim.x * BD_VL_THREADS;
+  const int nc = c.ncell_total;
+  for (int k = tid; k < nc; k += nth) d.cell_count[k] = 0;
+  if (!bdgs::grid_sync<false>(d.ctl, b)) { bdgs::block_exit(d.ctl); return; }
+  for (int i = tid; i < c.np; i += nth) {
     const BdRep *R = short_rep(d, i);
     if (!R || d.ext_id[i] < 0) {
       d.cell_of[i] = -1;
       continue;
     }
-    int k = cell_of(d.pos[i], *R);
+    const int k = cell_of(d.pos[i], *R);
     d.cell_of[i] = k;
     atomicAdd(&d.cell_count[k], 1);
   }
-}
-
-// 4a. exclusive scan within blocks of BD_SCAN_B cells
-__global__ void __launch_bounds__(BD_SCAN_B) k_scan_blocks(BdDev d, BdConst c) {
-  if (skip_block(d.ctl, true)) return;
-  __shared__ int s[BD_SCAN_B];
-  const int nc2 = c.ncell_total;
-  int k = blockIdx.x * BD_SCAN_B + threadIdx.x;
-  int v = k < nc2 ? d.cell_count[k] : 0;
-  s[threadIdx.x] = v;
-  __syncthreads();
-  for (int off = 1; off < BD_SCAN_B; off <<= 1) {
-    int t = threadIdx.x >= off ? s[threadIdx.x - off] : 0;
-    __syncthreads();
-    s[threadIdx.x] += t;
-    __syncthreads();
+  if (!bdgs::grid_sync<false>(d.ctl, b)) { bdgs::block_exit(d.ctl); return; }
+  const int per = (nc + (int)gridDim.x - 1) / (int)gridDim.x;
+  const int k0 = min(nc, (int)blockIdx.x * per), k1 = min(nc, k0 + per);
+  int total = 0;
+  {
+    int v = 0;
+    for (int k = k0 + (int)threadIdx.x; k < k1; k += BD_VL_THREADS) v += d.cell_count[k];
+    block_scan(v, &total);
+    if (threadIdx.x == 0) d.scan_sums[blockIdx.x] = total;
   }
-  if (k < nc2) d.cell_start[k] = s[threadIdx.x] - v;
-  if (threadIdx.x == BD_SCAN_B - 1) d.scan_sums[blockIdx.x] = s[threadIdx.x];
-}
-
-// 4b. exclusive scan of the block sums (one block, sequential chunks)
-__global__ void __launch_bounds__(BD_SCAN_B) k_scan_top(BdDev d, BdConst c, int nblocks) {
-  if (skip_block(d.ctl, true)) return;
-  __shared__ int s[BD_SCAN_B];
-  __shared__ int carry;
-  if (threadIdx.x == 0) carry = 0;
-  __syncthreads();
-  for (int base = 0; base < nblocks; base += BD_SCAN_B) {
-    int k = base + threadIdx.x;
-    int v = k < nblocks ? d.scan_sums[k] : 0;
-    s[threadIdx.x] = v;
-    __syncthreads();
-    for (int off = 1; off < BD_SCAN_B; off <<= 1) {
-      int t = threadIdx.x >= off ? s[threadIdx.x - off] : 0;
-      __syncthreads();
-      s[threadIdx.x] += t;
-      __syncthreads();
-    }
-    if (k < nblocks) d.scan_sums[k] = carry + s[threadIdx.x] - v;
-    __syncthreads();
-    if (threadIdx.x == BD_SCAN_B - 1) carry += s[threadIdx.x];
-    __syncthreads();
-  }
-}
-
-// 4c. add block offsets; reset the scatter cursors
-__global__ void __launch_bounds__(BD_SCAN_B) k_scan_add(BdDev d, BdConst c) {
-  if (skip_block(d.ctl, true)) return;
-  const int nc2 = c.ncell_total;
-  int k = blockIdx.x * BD_SCAN_B + threadIdx.x;
-  if (k < nc2) {
-    int v = d.cell_start[k] + d.scan_sums[blockIdx.x];
-    d.cell_start[k] = v;
-    d.cell_cursor[k] = v;
-  }
-}
-
-// 5. scatter disk ids into cell order (grid-stride)
-__global__ void k_vl_scatter(BdDev d, BdConst c) {
-  if (skip_block(d.ctl, true)) return;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < c.np; i += gridDim.x * blockDim.x) {
-    int k = d.cell_of[i];
-    if (k < 0) continue;
-    int slot = atomicAdd(&d.cell_cursor[k], 1);
-    d.cell_idx[slot] = i;
-  }
-}
-
-// 6. per-disk neighbour lists (sorted), reference positions (grid-stride)
-__global__ void k_vl_build(BdDev d, BdConst c) {
-  if (skip_block(d.ctl, true)) return;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < c.np; i += gridDim.x * blockDim.x) {
-    const BdRep *Rp = short_rep(d, i);
-    if (!Rp || d.ext_id[i] < 0) {
-      d.vl_cnt[i] = 0;
-      continue;
-    }
-    const BdRep &R = *Rp;
-    const double2 p = d.pos[i];
-    d.vl_ref[i] = p;
-    const float4 wi = d.work[i];
-    const float rl2f = (float)R.rl2;
-    const int k = d.cell_of[i] - R.cell_base;
-    const int cx = k % R.ncell, cy = k / R.ncell;
-    int buf[BD_VL_MAX];
-    int m = 0;
-    bool over = false;
-    for (int gy0 = cy - 1; gy0 <= cy + 1; ++gy0) {
-      // periodic box: the cells wrap around (at least three per side)
-      const int gy = R.periodic ? (gy0 + R.ncell) % R.ncell : gy0;
-      if (gy < 0 || gy >= R.ncell) continue;
-      for (int gx0 = cx - 1; gx0 <= cx + 1; ++gx0) {
-        const int gx = R.periodic ? (gx0 + R.ncell) % R.ncell : gx0;
-        if (gx < 0 || gx >= R.ncell) continue;
-        int cc = R.cell_base + gy * R.ncell + gx;
-        int b = d.cell_start[cc], e = b + d.cell_count[cc];
-        for (int s = b; s < e; ++s) {
-          int j = d.cell_idx[s];
-          if (j == i) continue;
-          // FP32 screen from the (hi, lo) pairs: the hi difference is exact
-          // (Sterbenz) or off by at most half an ulp of a coordinate below 12
-          // (4.8e-7), so the computed r^2 is within 1e-6 of the exact one
-          // relative to the reach; only pairs within 1e-5 of the reach (and
-          // pairs across a periodic edge) take the FP64 decision
-          const float4 wj = d.work[j];
-          const float hx = __fsub_rn(wi.x, wj.x), hy = __fsub_rn(wi.y, wj.y);
-          bool in;
-          bool exact = R.periodic && (fabsf(hx) > R.hLf || fabsf(hy) > R.hLf);
-          if (!exact) {
-            const float fx = __fadd_rn(hx, __fsub_rn(wi.z, wj.z)), fy = __fadd_rn(hy, __fsub_rn(wi.w, wj.w));
-            const float f2 = __fadd_rn(__fmul_rn(fx, fx), __fmul_rn(fy, fy));
-            if (f2 < rl2f * 0.99999f) in = true;
-            else if (f2 > rl2f * 1.00001f) in = false;
-            else exact = true;
-          }
-          if (exact) {
-            const double2 q = d.pos[j];
-            const double dx = dmin_image(__dsub_rn(p.x, q.x), R), dy = dmin_image(__dsub_rn(p.y, q.y), R);
-            in = __dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)) < R.rl2;
-          }
-          if (in) {
-            if (m < BD_VL_MAX) {
-              // insertion in sorted position
-              int t = m++;
-              while (t > 0 && buf[t - 1] > j) {
-                buf[t] = buf[t - 1];
-                --t;
-              }
-              buf[t] = j;
-            } else {
-              over = true;
-            }
-          }
-        }
+  if (!bdgs::grid_sync<false>(d.ctl, b)) { bdgs::block_exit(d.ctl); return; }
+  {
+    int v = 0;
+    for (int k = threadIdx.x; k < (int)blockIdx.x; k += BD_VL_THREADS) v += d.scan_sums[k];
+    int base = 0;
+    block_scan(v, &base);
+    for (int kk = k0; kk < k1; kk += BD_VL_THREADS) {
+      const int k = kk + (int)threadIdx.x;
+      const int n = k < k1 ? d.cell_count[k] : 0;
+      const int e = base + block_scan(n, &total);
+      if (k < k1) {
+        d.cell_start[k] = e;
+        d.cell_cursor[k] = e;
       }
+      base += total;
     }
-    for (int t = 0; t < m; ++t) d.vl_idx[(size_t)t * c.np + i] = buf[t];
-    d.vl_cnt[i] = m;
-    if (over) atomicCAS(&d.ctl->status, 0, BD_ERR_UNSUPPORTED);
   }
+  if (!bdgs::grid_sync<false>(d.ctl, b)) { bdgs::block_exit(d.ctl); return; }
+  for (int i = tid; i < c.np; i += nth) {
+    const int k = d.cell_of[i];   // this thread's own store
+    if (k >= 0) d.cell_idx[atomicAdd(&d.cell_cursor[k], 1)] = i;
+  }
+  if (!bdgs::grid_sync<false>(d.ctl, b)) { bdgs::block_exit(d.ctl); return; }
+  for (int i = tid; i < c.np; i += nth) vl_build_one(d, c, i);
+  bdgs::block_exit(d.ctl);
 }
 
-// 7. short-range force over the lists; clears the rebuild flag
+// short-range force over the lists; clears the rebuild flag
 // three resident blocks of 256 per SM (at most 80 registers): the gathers are
 // latency-bound, and the polydisperse branch must not cost the equal-disk
 // case its occupancy (86 registers, 2 blocks: 0.118 -> 0.174 ms at 2^20 disks)
@@ -429,25 +420,30 @@ __global__ void __launch_bounds__(256, 3) k_force_verlet(BdDev d, BdConst c) {
   d.fpart[i] = make_double2((double)tx.hi, (double)ty.hi);
 }
 
+int bd_vl_grid_for(int np, int *grid) {
+  int dev = 0, sms = 0, per = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return -1;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return -1;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_vl_rebuild, BD_VL_THREADS, 0) != cudaSuccess) return -1;
+  if (per < 1) return -1;
+  const int want = (np + BD_VL_THREADS - 1) / BD_VL_THREADS;   // at most one disk per thread
+  int g = sms * per;
+  if (g > BD_VL_MAXGRID) g = BD_VL_MAXGRID;
+  *grid = want < 1 ? 1 : (want < g ? want : g);
+  return 0;
+}
+
 cudaError_t bd_launch_force_short(const BdDev &d, const BdConst &c, cudaStream_t s) {
   if (!c.any_short) return cudaSuccess;
-  const int b = 256;
-  const int gn = (c.np + b - 1) / b;
-  const int nsb = (c.ncell_total + BD_SCAN_B - 1) / BD_SCAN_B;
-  int dev = 0, sms = 148;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int gs = 4 * sms;   // grid-stride launches: cheap when no rebuild is due
-  k_vl_check<<<gn, b, 0, s>>>(d, c);
-  k_vl_clear<<<gs, b, 0, s>>>(d, c);
-  k_vl_count<<<gs, b, 0, s>>>(d, c);
-  k_scan_blocks<<<nsb, BD_SCAN_B, 0, s>>>(d, c);
-  k_scan_top<<<1, BD_SCAN_B, 0, s>>>(d, c, nsb);
-  k_scan_add<<<nsb, BD_SCAN_B, 0, s>>>(d, c);
-  k_vl_scatter<<<gs, b, 0, s>>>(d, c);
-  k_vl_build<<<gs, 128, 0, s>>>(d, c);
-  k_force_verlet<<<gn, b, 0, s>>>(d, c);
+  const int gn = (c.np + BD_VL_THREADS - 1) / BD_VL_THREADS;
+  k_vl_check<<<gn, BD_VL_THREADS, 0, s>>>(d, c);
+  BdDev dd = d;
+  BdConst cc = c;
+  void *args[] = {&dd, &cc};
+  cudaError_t e = cudaLaunchCooperativeKernel((const void *)k_vl_rebuild, dim3(c.vl_grid), dim3(BD_VL_THREADS), args, 0, s);
+  if (e != cudaSuccess) return e;
+  k_force_verlet<<<gn, 256, 0, s>>>(d, c);
   return cudaGetLastError();
 }
 
-int bd_short_launches() { return 9; }
+int bd_short_launches() { return 3; }

@@ -225,6 +225,7 @@ __global__ void __launch_bounds__(BD_VC_THREADS) k_overlap_verlet(BdDev d, BdCon
   }
   if (lead) {
     ctl->epoch = lbase + 1;
+    ctl->in_move = 0;
     ctl->st_corr_iters += corr_iter;
     ctl->st_overlap_pairs += st_overlap;
     ctl->st_barriers += b.gen;
