@@ -178,8 +178,11 @@ struct SymPlan {
 // (512 disks x 8 B), so long chunks cut the partial traffic; the last part of
 // the work is cut into 2-tile items, placed at the end of the launch order, so
 // the final waves of resident blocks stay full.
+// (FP64: blocks of BD_F64_SB disks and groups of BD_F64_TJ in their place.)
 void make_sym(const bd_handle *h, int tiles, int variant, SymPlan &S) {
-  const int nblocks = h->np / BD_SB, ntiles = h->np / BD_TJ;
+  const bool f64 = h->c.precision == 1;
+  const int SB = f64 ? BD_F64_SB : BD_SB, TJ = f64 ? BD_F64_TJ : BD_TJ;
+  const int nblocks = h->np / SB, ntiles = h->np / TJ, tpb = SB / TJ;
   std::vector<std::vector<int>> bl(nblocks), tl(ntiles);
   S.items.clear();
   S.n_jtiles = 0;
@@ -189,11 +192,11 @@ void make_sym(const bd_handle *h, int tiles, int variant, SymPlan &S) {
   std::vector<Chunk> ch;
   for (const RepHost &R : h->reps) {
     if (R.p.law != BD_LAW_LONG) continue;
-    const int tb = R.tile_begin, te = R.tile_end;
-    for (int P = tb / 2; P < te / 2; ++P)
-      for (int c0 = 2 * P; c0 < te; c0 += tiles) ch.push_back({P, c0, std::min(te, c0 + tiles)});
+    const int tb = R.slot_begin / TJ, te = R.slot_end / TJ;
+    for (int P = tb / tpb; P < te / tpb; ++P)
+      for (int c0 = tpb * P; c0 < te; c0 += tiles) ch.push_back({P, c0, std::min(te, c0 + tiles)});
   }
-  if (tiles > 2) {
+  if (tiles > 2 && !f64) {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -211,7 +214,7 @@ void make_sym(const bd_handle *h, int tiles, int variant, SymPlan &S) {
     ch.insert(ch.end(), small.begin(), small.end());
   }
   for (const Chunk &c : ch) {
-    const int jt0 = std::max(c.c0, 2 * c.P + 2);
+    const int jt0 = std::max(c.c0, tpb * (c.P + 1));
     const int it = (int)S.items.size();
     S.items.push_back(make_int4(c.P, c.c0, c.c1, S.n_jtiles));
     bl[c.P].push_back(it);
@@ -256,8 +259,13 @@ cudaError_t upload_sym(bd_handle *h, const SymPlan &S) {
   if (e == cudaSuccess) e = upload_vec(h, &d.red_iidx, S.iidx);
   if (e == cudaSuccess) e = upload_vec(h, &d.red_jptr, S.jptr);
   if (e == cudaSuccess) e = upload_vec(h, &d.red_jidx, S.jidx);
-  if (e == cudaSuccess) e = realloc_dev(h, &d.ipart, S.items.size() * BD_SB);
-  if (e == cudaSuccess) e = realloc_dev(h, &d.jpart, (size_t)S.n_jtiles * BD_TJ);
+  if (h->c.precision == 1) {
+    if (e == cudaSuccess) e = realloc_dev(h, &d.ipart64, S.items.size() * BD_F64_SB);
+    if (e == cudaSuccess) e = realloc_dev(h, &d.jpart64, (size_t)S.n_jtiles * BD_F64_TJ);
+  } else {
+    if (e == cudaSuccess) e = realloc_dev(h, &d.ipart, S.items.size() * BD_SB);
+    if (e == cudaSuccess) e = realloc_dev(h, &d.jpart, (size_t)S.n_jtiles * BD_TJ);
+  }
   if (e != cudaSuccess) return e;
   h->c.n_sitems = (int)S.items.size();
   h->c.max_nchunk = 1;
@@ -326,7 +334,7 @@ cudaError_t upload_items(bd_handle *h, const std::vector<int4> &items, int max_c
 cudaError_t use_variant(bd_handle *h, int variant, int tiles) {
   h->c.force_variant = variant;
   h->tune_tiles = tiles;
-  if (variant >= 2) {
+  if (variant >= 2 || h->c.f64_sym) {
     SymPlan S;
     make_sym(h, tiles, variant, S);
     return upload_sym(h, S);
@@ -335,6 +343,25 @@ cudaError_t use_variant(bd_handle *h, int variant, int tiles) {
   int mc = 1;
   make_items(h, tiles, items, mc);
   return upload_items(h, items, mc);
+}
+
+// FP64: the symmetric sweep's j-partial storage, and its groups of j per work
+// item: one while the items are few (a block then fills an SM for the length
+// of one group), about sixteen items per SM beyond
+unsigned long long f64_sym_units(const bd_handle *h) {
+  unsigned long long u = 0;
+  for (const RepHost &R : h->reps) {
+    if (R.p.law != BD_LAW_LONG) continue;
+    const unsigned long long s = (unsigned long long)(R.slot_end - R.slot_begin);
+    u += (s / BD_F64_SB + 1) * (s / BD_F64_TJ) / 2;
+  }
+  return u;
+}
+int f64_sym_tiles(const bd_handle *h) {
+  int dev = 0, sms = 148;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return (int)std::max(1ull, f64_sym_units(h) / (16ull * sms));
 }
 
 // Autotuner of the all-pairs sweep: time the force launch for each candidate
@@ -789,6 +816,7 @@ int build_handle(const std::vector<Spec> &specs, void *stream, bd_handle **out) 
     c.n_species = std::max(c.n_species, p.n_species);
   }
   c.ncell_total = cell_base;
+  c.f64_sym = c.precision == 1 && c.any_long && f64_sym_units(h) * BD_F64_TJ * sizeof(double2) <= BD_F64_BYTES ? 1 : 0;
   h->step = p0.step0;
   h->graph_off = getenv("BD_NO_GRAPH") != nullptr;
 
@@ -897,7 +925,7 @@ int build_handle(const std::vector<Spec> &specs, void *stream, bd_handle **out) 
       h->fpart_cap.assign(R, 1);
       for (int r = 0; r < R; ++r) {
         const int nt_r = h->reps[r].tile_end - h->reps[r].tile_begin;
-        const int want = c.precision == 1 ? std::max(nt_r, f64_want) : nt_r;
+        const int want = c.f64_sym ? 1 : (c.precision == 1 ? std::max(nt_r, f64_want) : nt_r);
         const int cap = h->reps[r].p.law == BD_LAW_LONG ? std::min(64, std::max(1, want)) : 1;
         h->fpart_cap[r] = cap;
         slots = std::max(slots, cap);
@@ -1048,7 +1076,8 @@ int build_handle(const std::vector<Spec> &specs, void *stream, bd_handle **out) 
       for (const RepHost &RH : h->reps)
         if (RH.p.law == BD_LAW_LONG) nmax = std::max<long long>(nmax, RH.n);
       if (c.precision == 1 || !c.any_long) {
-        BD_TRY(use_variant(h, c.precision == 1 ? 1 : c.force_variant, R == 1 ? single_system_tiles(h) : 16));
+        BD_TRY(use_variant(h, c.precision == 1 ? 1 : c.force_variant,
+                           c.f64_sym ? f64_sym_tiles(h) : (R == 1 ? single_system_tiles(h) : 16)));
       } else if (fv) {
         int v = std::min(3, std::max(0, atoi(fv)));
         if (c.any_periodic && v == 1) v = 0;   // the packed one-sided sweep has no periodic form
@@ -1206,7 +1235,7 @@ cudaError_t capture_step_graph(bd_handle *h) {
     if (tm) el = cudaEventRecordWithFlags(h->graph_ev[0], cs, cudaEventRecordExternal);
     if (el == cudaSuccess) el = bd_launch_force_long(h->d, h->c, cs);
     if (el == cudaSuccess && tm) el = cudaEventRecordWithFlags(h->graph_ev[1], cs, cudaEventRecordExternal);
-    launches += h->c.precision == 0 ? bd_force_launches(h->c.force_variant) : 1;
+    launches += bd_force_launches(h->c);
   }
   if (el == cudaSuccess && h->c.any_short) {
     el = bd_launch_force_short(h->d, h->c, cs);
@@ -1286,7 +1315,7 @@ int queue_steps(bd_handle *h, int32_t nsteps, int64_t *launches_out) {
         cudaEventRecord(h->ev_pool[2 * s + 1], st);
         ++timed;
       }
-      launches += h->c.precision == 0 ? bd_force_launches(h->c.force_variant) : 1;
+      launches += bd_force_launches(h->c);
     }
     if (h->c.any_short) {
       e = bd_launch_force_short(h->d, h->c, st);
@@ -1356,7 +1385,7 @@ cudaError_t launch_piece(bd_handle *h, int node, int64_t *launches) {
   cudaError_t e = cudaSuccess;
   if (h->c.any_long) {
     e = bd_launch_force_long(h->d, h->c, st);
-    *launches += h->c.precision == 0 ? bd_force_launches(h->c.force_variant) : 1;
+    *launches += bd_force_launches(h->c);
   }
   if (e == cudaSuccess && h->c.any_short) {
     e = bd_launch_force_short(h->d, h->c, st);
@@ -1869,7 +1898,7 @@ int bd_get_tuning(bd_handle *h, int32_t *tiles_per_item, int32_t *variant, int32
   if (!h) return BD_ERR_ARG;
   if (tiles_per_item) *tiles_per_item = h->tune_tiles;
   if (variant) *variant = h->c.force_variant;
-  if (n_items) *n_items = h->c.force_variant >= 2 ? h->c.n_sitems : h->c.n_items;
+  if (n_items) *n_items = h->c.force_variant >= 2 || h->c.f64_sym ? h->c.n_sitems : h->c.n_items;
   return BD_OK;
 }
 

@@ -14,6 +14,12 @@
 // segments are padded to whole blocks so a block holds one species
 #define BD_SB 512
 
+// FP64 symmetric sweep: blocks of 128 disks i, groups of 32 disks j
+#define BD_F64_SB 128
+#define BD_F64_TJ 32
+// the largest j-partial storage it may take; beyond it the one-sided FP64 sweep runs
+#define BD_F64_BYTES (512ull << 20)
+
 // species per system (the long-range table is stored BD_MAX_SPECIES wide)
 #define BD_MAX_SPECIES 4
 
@@ -182,6 +188,7 @@ struct BdDev {
   float2 *sorigin;         // per block: integer origin for re-centring
   float2 *ipart;           // [item][BD_SB] i-side partial forces
   float2 *jpart;           // [j-partial tile][BD_TJ] j-side partial forces
+  double2 *ipart64, *jpart64;  // the same for the FP64 sweep: [item][BD_F64_SB], [j-partial group][BD_F64_TJ]
   int *red_iptr, *red_iidx;  // per block: the items whose i side it is
   int *red_jptr, *red_jidx;  // per tile: the j-partial tiles that hold it
   // short range: Verlet lists (column-major ELL) and the cell grids
@@ -221,6 +228,7 @@ struct BdConst {
   int max_corr_iters, max_flip_rounds;
   int force_variant;       // 0: scalar FP32 sweep, 1: packed f32x2 sweep, 2, 3: symmetric packed sweeps
   int n_sitems;            // symmetric sweep work items
+  int f64_sym;             // precision 1: the symmetric FP64 sweep (its items in the symmetric tables)
   int overlap_verlet;      // 1: Algorithm 2 over the Verlet lists, no triangulation kept
   int tri_lists;           // check passes after the first of a move: 0 lists when a full pass
                            // is throughput-bound (many triangles per thread), 1 always lists,
@@ -260,6 +268,7 @@ cudaError_t bd_launch_force_short(const BdDev &d, const BdConst &c, cudaStream_t
 int bd_short_launches();
 int bd_vl_grid_for(int np, int *grid);
 cudaError_t bd_launch_force_sum(const BdDev &d, const BdConst &c, double2 *out, cudaStream_t s);
+cudaError_t bd_launch_force_f64s(const BdDev &d, const BdConst &c, cudaStream_t s);
 cudaError_t bd_launch_force_sym(const BdDev &d, const BdConst &c, int variant, cudaStream_t s);
 // advance = 0: a piece of a halved step (the step counter does not advance);
 // advance = -1: positions set from outside, a pair closer than sigma rejects them
@@ -275,7 +284,7 @@ cudaError_t bd_launch_advance_step(const BdDev &d, cudaStream_t s);
 // launch may have left
 cudaError_t bd_launch_restore_step(const BdDev &d, const BdConst &c, cudaStream_t s);
 int bd_vcorr_grid_for(int work_items, int *grid, int *block);
-int bd_force_launches(int variant);   // kernel launches of one long-range force evaluation
+int bd_force_launches(const BdConst &c);   // kernel launches of one long-range force evaluation
 int bd_force_sym_blocks_per_sm(int variant, int periodic);   // resident blocks of the symmetric sweep
 // Philox words and clamped normals (FP32 and FP64 forms) for n counters (uint4 each)
 cudaError_t bd_launch_noise_sample(unsigned long long seed, unsigned replica, int n, const void *ctr, void *words,

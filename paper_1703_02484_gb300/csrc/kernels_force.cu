@@ -453,7 +453,8 @@ __global__ void __launch_bounds__(BD_FT) k_force_long_f32x2(BdDev d, BdConst c) 
   }
 }
 
-// FP64 variant (precision = 1): one disk per thread, FP64 master positions;
+// One-sided FP64 sweep (precision = 1, systems whose partial sums would not fit
+// the symmetric one's storage): one disk per thread, FP64 master positions;
 // grid (disk blocks, j chunks), chunk k of a replica covers a k-th of its slots
 __global__ void __launch_bounds__(128) k_force_long_f64(BdDev d, BdConst c) {
   if (ctl_failed(d.ctl)) return;
@@ -498,14 +499,10 @@ __global__ void __launch_bounds__(128) k_force_long_f64(BdDev d, BdConst c) {
         double rx = pi.x - sp[k].x, ry = pi.y - sp[k].y;
         if (R.periodic) {
           // minimum image (Sec. 2.1)
-          rx -= R.L * rint(rx / R.L);
-          ry -= R.L * rint(ry / R.L);
+          if (abs_above(rx, 0.5 * R.L)) rx -= copysign(R.L, rx);
+          if (abs_above(ry, 0.5 * R.L)) ry -= copysign(R.L, ry);
         }
-        double r2 = rx * rx + ry * ry;
-        // |r|^-3 from the library's reciprocal square root (within an ulp):
-        // three multiplies instead of a square root and a division
-        const double rs = rsqrt(r2);
-        double cf = R.alpha_d[BD_MAX_SPECIES * si + sk] * (rs * rs * rs);
+        const double cf = R.alpha_d[BD_MAX_SPECIES * si + sk] * inv_r3(rx * rx + ry * ry);
         fx += cf * rx;
         fy += cf * ry;
       }
@@ -620,6 +617,8 @@ cudaError_t bd_launch_force_long_variant(const BdDev &d, const BdConst &c, int v
       k_force_long_f32x2<BD_IPT><<<c.n_items, BD_FT, 0, s>>>(d, c);
     else
       k_force_long_f32<<<c.n_items, BD_FT, 0, s>>>(d, c);
+  } else if (c.f64_sym) {
+    return bd_launch_force_f64s(d, c, s);
   } else {
     k_force_long_f64<<<dim3((c.np + 127) / 128, c.max_nchunk), 128, 0, s>>>(d, c);
   }
@@ -632,7 +631,10 @@ cudaError_t bd_launch_force_long(const BdDev &d, const BdConst &c, cudaStream_t 
 
 cudaError_t bd_launch_integrate(const BdDev &d, const BdConst &c, int64_t step, int log_step,
                                 cudaStream_t s, int node) {
-  k_integrate<<<(c.np + 255) / 256, 256, 0, s>>>(d, c, (long long)step, log_step, node);
+  // the FP64 move is some 300 instructions of the FP64 pipe (two lanes per
+  // SM): one warp per block spreads a small system over the SMs
+  const int b = c.precision == 1 ? 32 : 256;
+  k_integrate<<<(c.np + b - 1) / b, b, 0, s>>>(d, c, (long long)step, log_step, node);
   return cudaGetLastError();
 }
 

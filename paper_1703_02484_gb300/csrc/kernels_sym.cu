@@ -620,7 +620,7 @@ __global__ void __launch_bounds__(4 * BD_RED_D) k_force_sym_reduce(BdDev d, BdCo
   d.fpart[i] = make_double2(fx, fy);
 }
 
-int bd_force_launches(int variant) { return variant >= 2 ? 2 : 1; }
+int bd_force_launches(const BdConst &c) { return (c.precision == 0 ? c.force_variant >= 2 : c.f64_sym) ? 2 : 1; }
 
 int bd_force_sym_blocks_per_sm(int variant, int periodic) {
   int per = 0;
