@@ -335,7 +335,8 @@ int bd_batch_step(bd_handle *h, int32_t nsteps, bd_step_stats *per_replica);
 int bd_get_replica(bd_handle *h, int32_t r, double *xy, float *theta, int32_t *tri, int32_t *n_tri,
                    int32_t *n, double *L);
 
-/* The all-pairs sweep's tuning: j tiles (256 disks each) per work item, the
+/* The all-pairs sweep's tuning: j tiles (256 disks each; a part of one counts
+ * as one) per work item, the
  * kernel variant (0 scalar FP32 one-sided, 1 packed f32x2 one-sided, 2 and 3
  * symmetric packed f32x2 -- each unordered pair once -- with 4 warps x 4 or
  * 2 warps x 8 disks per lane) and the number of work items.  Periodic boxes

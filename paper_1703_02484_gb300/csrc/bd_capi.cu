@@ -164,49 +164,65 @@ void make_items(bd_handle *h, int tiles, std::vector<int4> &items, int &max_chun
 }
 
 // Work items of the symmetric sweep: block P of a long-range replica against
-// its own two tiles (i side only) and every later tile of the replica, in
-// chunks of at most `tiles` tiles, plus the reduction lists (per block its
-// items, per tile its j-partial tiles, both in item order).
+// its own groups of 32 disks j (i side only) and every later group of the
+// replica, in chunks of at most `groups`, plus the reduction lists (per block
+// its items, per group its j partials, both in item order).
 struct SymPlan {
   std::vector<int4> items;
   std::vector<int> iptr, iidx, jptr, jidx;
-  int n_jtiles = 0;
+  int n_jgroups = 0;
 };
 
-// Work items of the symmetric sweep: each row of block P (its tiles from 2P
-// on) in chunks of `tiles`.  The i side of an item is written as one partial
-// (512 disks x 8 B), so long chunks cut the partial traffic; the last part of
-// the work is cut into 2-tile items, placed at the end of the launch order, so
-// the final waves of resident blocks stay full.
-// (FP64: blocks of BD_F64_SB disks and groups of BD_F64_TJ in their place.)
-void make_sym(const bd_handle *h, int tiles, int variant, SymPlan &S) {
+// groups of all rows (block P's row: the groups from its own first to the
+// replica's end) of blocks of SB disks
+long long sym_units(const bd_handle *h, int SB) {
+  long long u = 0;
+  for (const RepHost &R : h->reps) {
+    if (R.p.law != BD_LAW_LONG) continue;
+    const long long nb = (R.slot_end - R.slot_begin) / SB;
+    u += nb * (nb + 1) / 2 * (SB / BD_SG);
+  }
+  return u;
+}
+
+// co-resident blocks of the FP32 symmetric sweep
+long sym_slots(const bd_handle *h, int variant) {
+  int dev = 0, sms = 148;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return (long)sms * std::max(1, bd_force_sym_blocks_per_sm(variant, h->c.any_periodic));
+}
+
+// Work items of the symmetric sweep: each row of block P in chunks of
+// `groups`.  The i side of an item is written as one partial (512 disks x 8 B),
+// so long chunks cut the partial traffic; with chunks of more than two tiles
+// (16 groups) the last part of the work is cut into items of two tiles, placed at
+// the end of the launch order, so the final waves of resident blocks stay full.
+// (FP64: blocks of BD_F64_SB disks.)
+void make_sym(const bd_handle *h, int groups, int variant, SymPlan &S) {
   const bool f64 = h->c.precision == 1;
-  const int SB = f64 ? BD_F64_SB : BD_SB, TJ = f64 ? BD_F64_TJ : BD_TJ;
-  const int nblocks = h->np / SB, ntiles = h->np / TJ, tpb = SB / TJ;
-  std::vector<std::vector<int>> bl(nblocks), tl(ntiles);
+  const int SB = f64 ? BD_F64_SB : BD_SB;
+  const int nblocks = h->np / SB, ngroups = h->np / BD_SG, gpb = SB / BD_SG;
+  std::vector<std::vector<int>> bl(nblocks), gl(ngroups);
   S.items.clear();
-  S.n_jtiles = 0;
+  S.n_jgroups = 0;
   struct Chunk {
     int P, c0, c1;
   };
   std::vector<Chunk> ch;
   for (const RepHost &R : h->reps) {
     if (R.p.law != BD_LAW_LONG) continue;
-    const int tb = R.slot_begin / TJ, te = R.slot_end / TJ;
-    for (int P = tb / tpb; P < te / tpb; ++P)
-      for (int c0 = tpb * P; c0 < te; c0 += tiles) ch.push_back({P, c0, std::min(te, c0 + tiles)});
+    const int gb = R.slot_begin / BD_SG, ge = R.slot_end / BD_SG;
+    for (int P = gb / gpb; P < ge / gpb; ++P)
+      for (int c0 = gpb * P; c0 < ge; c0 += groups) ch.push_back({P, c0, std::min(ge, c0 + groups)});
   }
-  if (tiles > 2 && !f64) {
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const long slots = (long)sms * std::max(1, bd_force_sym_blocks_per_sm(variant, h->c.any_periodic));
-    long tail = 4 * slots;   // tile units: two waves of 2-tile items
+  if (groups > 16 && !f64) {
+    long tail = 32 * sym_slots(h, variant);   // groups: two waves of two-tile items
     std::vector<Chunk> small;
     while (!ch.empty() && tail > 0) {
       const Chunk c = ch.back();
       ch.pop_back();
-      for (int s = c.c0; s < c.c1; s += 2) small.push_back({c.P, s, std::min(c.c1, s + 2)});
+      for (int s = c.c0; s < c.c1; s += 16) small.push_back({c.P, s, std::min(c.c1, s + 16)});
       tail -= c.c1 - c.c0;
     }
     std::stable_sort(small.begin(), small.end(),
@@ -214,12 +230,12 @@ void make_sym(const bd_handle *h, int tiles, int variant, SymPlan &S) {
     ch.insert(ch.end(), small.begin(), small.end());
   }
   for (const Chunk &c : ch) {
-    const int jt0 = std::max(c.c0, tpb * (c.P + 1));
+    const int jg0 = std::max(c.c0, gpb * (c.P + 1));
     const int it = (int)S.items.size();
-    S.items.push_back(make_int4(c.P, c.c0, c.c1, S.n_jtiles));
+    S.items.push_back(make_int4(c.P, c.c0, c.c1, S.n_jgroups));
     bl[c.P].push_back(it);
-    for (int t = jt0; t < c.c1; ++t) tl[t].push_back(S.n_jtiles + (t - jt0));
-    S.n_jtiles += std::max(0, c.c1 - jt0);
+    for (int g = jg0; g < c.c1; ++g) gl[g].push_back(S.n_jgroups + (g - jg0));
+    S.n_jgroups += std::max(0, c.c1 - jg0);
   }
   auto flatten = [](const std::vector<std::vector<int>> &v, std::vector<int> &ptr, std::vector<int> &idx) {
     ptr.assign(v.size() + 1, 0);
@@ -230,7 +246,7 @@ void make_sym(const bd_handle *h, int tiles, int variant, SymPlan &S) {
     }
   };
   flatten(bl, S.iptr, S.iidx);
-  flatten(tl, S.jptr, S.jidx);
+  flatten(gl, S.jptr, S.jidx);
 }
 
 // replace a device array owned by the handle
@@ -261,10 +277,10 @@ cudaError_t upload_sym(bd_handle *h, const SymPlan &S) {
   if (e == cudaSuccess) e = upload_vec(h, &d.red_jidx, S.jidx);
   if (h->c.precision == 1) {
     if (e == cudaSuccess) e = realloc_dev(h, &d.ipart64, S.items.size() * BD_F64_SB);
-    if (e == cudaSuccess) e = realloc_dev(h, &d.jpart64, (size_t)S.n_jtiles * BD_F64_TJ);
+    if (e == cudaSuccess) e = realloc_dev(h, &d.jpart64, (size_t)S.n_jgroups * BD_SG);
   } else {
     if (e == cudaSuccess) e = realloc_dev(h, &d.ipart, S.items.size() * BD_SB);
-    if (e == cudaSuccess) e = realloc_dev(h, &d.jpart, (size_t)S.n_jtiles * BD_TJ);
+    if (e == cudaSuccess) e = realloc_dev(h, &d.jpart, (size_t)S.n_jgroups * BD_SG);
   }
   if (e != cudaSuccess) return e;
   h->c.n_sitems = (int)S.items.size();
@@ -330,44 +346,38 @@ cudaError_t upload_items(bd_handle *h, const std::vector<int4> &items, int max_c
                     cudaMemcpyHostToDevice);
 }
 
-// set up the work list of a sweep variant with `tiles` j tiles per item
-cudaError_t use_variant(bd_handle *h, int variant, int tiles) {
+// set up the work list of a sweep variant with `chunk` j tiles (one-sided
+// sweeps) or groups of 32 disks j (symmetric ones) per item
+cudaError_t use_variant(bd_handle *h, int variant, int chunk) {
   h->c.force_variant = variant;
-  h->tune_tiles = tiles;
+  h->tune_chunk = chunk;
   if (variant >= 2 || h->c.f64_sym) {
     SymPlan S;
-    make_sym(h, tiles, variant, S);
+    make_sym(h, chunk, variant, S);
     return upload_sym(h, S);
   }
   std::vector<int4> items;
   int mc = 1;
-  make_items(h, tiles, items, mc);
+  make_items(h, chunk, items, mc);
   return upload_items(h, items, mc);
 }
 
-// FP64: the symmetric sweep's j-partial storage, and its groups of j per work
-// item: one while the items are few (a block then fills an SM for the length
-// of one group), about sixteen items per SM beyond
-unsigned long long f64_sym_units(const bd_handle *h) {
-  unsigned long long u = 0;
-  for (const RepHost &R : h->reps) {
-    if (R.p.law != BD_LAW_LONG) continue;
-    const unsigned long long s = (unsigned long long)(R.slot_end - R.slot_begin);
-    u += (s / BD_F64_SB + 1) * (s / BD_F64_TJ) / 2;
-  }
-  return u;
-}
-int f64_sym_tiles(const bd_handle *h) {
+// FP64: groups of j per work item: one while the items are few (a block then
+// fills an SM for the length of one group), about sixteen items per SM beyond
+int f64_sym_groups(const bd_handle *h) {
   int dev = 0, sms = 148;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  return (int)std::max(1ull, f64_sym_units(h) / (16ull * sms));
+  return (int)std::max(1ll, sym_units(h, BD_F64_SB) / (16ll * sms));
 }
 
 // Autotuner of the all-pairs sweep: time the force launch for each candidate
-// (kernel variant, j tiles per work item) and keep the fastest.  Candidates:
-// the one-sided sweeps (scalar, packed) and the symmetric sweep over several
-// chunk sizes; a single system also tries the wave-filling chunk size.
+// (kernel variant, chunk size) and keep the fastest.  Candidates: the one-sided
+// sweeps (scalar, packed) of a batch, and of a single system with its
+// wave-filling chunk size; the symmetric sweep with chunks of 2 groups (64
+// disks j) to 32 tiles, as long as they leave between one item for every two
+// co-resident blocks and 24 items for each (outside that range the SMs
+// idle, or the partial sums' traffic grows past any gain).
 cudaError_t autotune(bd_handle *h) {
   std::vector<int2> cand;
   if (h->c.any_periodic) {
@@ -381,8 +391,12 @@ cudaError_t autotune(bd_handle *h) {
     for (int t : {2, 4, 8, 16, 32, 64}) cand.push_back(make_int2(0, t));
     for (int t : {2, 4, 8, 16, 32, 64}) cand.push_back(make_int2(1, t));
   }
-  for (int v : {2, 3})
-    for (int t : {2, 4, 8, 16, 32}) cand.push_back(make_int2(v, t));
+  const long long units = sym_units(h, BD_SB);
+  for (int v : {2, 3}) {
+    const long long slots = sym_slots(h, v);
+    for (int g : {2, 4, 8, 16, 32, 64, 128, 256})
+      if (units / g <= 24 * slots && (g == 2 || units / g >= slots / 2)) cand.push_back(make_int2(v, g));
+  }
   float best_ms = 1e30f;
   int2 best = cand[0];
   cudaEvent_t a, b;
@@ -816,7 +830,7 @@ int build_handle(const std::vector<Spec> &specs, void *stream, bd_handle **out) 
     c.n_species = std::max(c.n_species, p.n_species);
   }
   c.ncell_total = cell_base;
-  c.f64_sym = c.precision == 1 && c.any_long && f64_sym_units(h) * BD_F64_TJ * sizeof(double2) <= BD_F64_BYTES ? 1 : 0;
+  c.f64_sym = c.precision == 1 && c.any_long && sym_units(h, BD_F64_SB) * BD_SG * (long long)sizeof(double2) <= BD_F64_BYTES ? 1 : 0;
   h->step = p0.step0;
   h->graph_off = getenv("BD_NO_GRAPH") != nullptr;
 
@@ -1077,15 +1091,15 @@ int build_handle(const std::vector<Spec> &specs, void *stream, bd_handle **out) 
         if (RH.p.law == BD_LAW_LONG) nmax = std::max<long long>(nmax, RH.n);
       if (c.precision == 1 || !c.any_long) {
         BD_TRY(use_variant(h, c.precision == 1 ? 1 : c.force_variant,
-                           c.f64_sym ? f64_sym_tiles(h) : (R == 1 ? single_system_tiles(h) : 16)));
+                           c.f64_sym ? f64_sym_groups(h) : (R == 1 ? single_system_tiles(h) : 16)));
       } else if (fv) {
         int v = std::min(3, std::max(0, atoi(fv)));
         if (c.any_periodic && v == 1) v = 0;   // the packed one-sided sweep has no periodic form
         const int t = ft && atoi(ft) > 0 ? atoi(ft) : (v >= 2 ? 8 : (R == 1 ? single_system_tiles(h) : 16));
-        BD_TRY(use_variant(h, v, t));
+        BD_TRY(use_variant(h, v, v >= 2 ? t * (BD_TJ / BD_SG) : t));
       } else if (nmax * nmax > 180000000000LL) {
         // a launch takes more than ~50 ms: no timing at init
-        BD_TRY(use_variant(h, 2, 16));
+        BD_TRY(use_variant(h, 2, 128));
       } else {
         BD_TRY(autotune(h));
       }
@@ -1744,12 +1758,12 @@ int bd_set_force_shard(bd_handle *h, int32_t rank, int32_t world) {
   if (h->reps.size() != 1 || !h->c.any_long || h->c.precision != 0 || h->max_halvings > 0)
     return BD_ERR_UNSUPPORTED;
   cudaError_t e = cudaSuccess;
-  if (h->c.force_variant < 2) e = use_variant(h, 3, 8);   // shards cut the symmetric sweep's plan
+  if (h->c.force_variant < 2) e = use_variant(h, 3, 64);   // shards cut the symmetric sweep's plan
   if (e != cudaSuccess) return cuda_fail(e);
   // the plan as uploaded (make_sym is deterministic); an item's cost is its
-  // number of j tiles (pairs of a 512-disk block with a 256-disk tile)
+  // number of j groups (pairs of a 512-disk block with 32 disks)
   SymPlan S;
-  make_sym(h, h->tune_tiles, h->c.force_variant, S);
+  make_sym(h, h->tune_chunk, h->c.force_variant, S);
   const int ni = (int)S.items.size();
   std::vector<double> cum(ni + 1, 0.0);
   for (int k = 0; k < ni; ++k) cum[k + 1] = cum[k] + (S.items[k].z - S.items[k].y);
@@ -1761,7 +1775,7 @@ int bd_set_force_shard(bd_handle *h, int32_t rank, int32_t world) {
   const int b0 = rank == 0 ? 0 : first(rank), b1 = rank + 1 == world ? ni : first(rank + 1);
   // partials of items that are not this rank's stay zero in the reduction
   e = cudaMemsetAsync(h->d.ipart, 0, (size_t)ni * BD_SB * sizeof(float2), h->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(h->d.jpart, 0, (size_t)S.n_jtiles * BD_TJ * sizeof(float2), h->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(h->d.jpart, 0, (size_t)S.n_jgroups * BD_SG * sizeof(float2), h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return cuda_fail(e);
   h->c.sitem0 = b0;
@@ -1896,9 +1910,11 @@ int bd_get_geometry(bd_handle *h, double *q, double *L) {
 
 int bd_get_tuning(bd_handle *h, int32_t *tiles_per_item, int32_t *variant, int32_t *n_items) {
   if (!h) return BD_ERR_ARG;
-  if (tiles_per_item) *tiles_per_item = h->tune_tiles;
+  const bool sym = h->c.force_variant >= 2 || h->c.f64_sym;   // chunks in groups, not tiles
+  const int per = BD_TJ / BD_SG;
+  if (tiles_per_item) *tiles_per_item = sym ? (h->tune_chunk + per - 1) / per : h->tune_chunk;
   if (variant) *variant = h->c.force_variant;
-  if (n_items) *n_items = h->c.force_variant >= 2 || h->c.f64_sym ? h->c.n_sitems : h->c.n_items;
+  if (n_items) *n_items = sym ? h->c.n_sitems : h->c.n_items;
   return BD_OK;
 }
 

@@ -44,7 +44,7 @@ struct bd_handle {
   double force_ms = 0.0;
   int64_t force_launches = 0;
   int64_t last_launches = 0;
-  int tune_tiles = 0;              // j tiles per work item chosen for the sweep
+  int tune_chunk = 0;              // j tiles (one-sided sweeps) or groups (symmetric) per work item
   int fpart_slots = 0;             // partial-force slots allocated
   std::vector<int> fpart_cap;      // per replica: chunks that fit
   BdRollout *ro = nullptr;         // differentiated rollout state (lazily created)

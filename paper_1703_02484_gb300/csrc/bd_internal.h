@@ -13,12 +13,12 @@
 // symmetric sweep: blocks of BD_SB consecutive slots (two j tiles); species
 // segments are padded to whole blocks so a block holds one species
 #define BD_SB 512
+#define BD_SG 32             // and their work items and j partials count groups of 32 disks j
 
-// FP64 symmetric sweep: blocks of 128 disks i, groups of 32 disks j
+// FP64 symmetric sweep: blocks of 128 disks i (and groups of BD_SG disks j)
 #define BD_F64_SB 128
-#define BD_F64_TJ 32
 // the largest j-partial storage it may take; beyond it the one-sided FP64 sweep runs
-#define BD_F64_BYTES (512ull << 20)
+#define BD_F64_BYTES (512ll << 20)
 
 // species per system (the long-range table is stored BD_MAX_SPECIES wide)
 #define BD_MAX_SPECIES 4
@@ -183,14 +183,14 @@ struct BdDev {
   int4 *items;             // work items (i block, first tile, end tile, partial slot)
   double2 *fpart;          // [max_nchunk][np] partial forces
   // symmetric sweep (each unordered pair once, both disks updated)
-  int4 *sitems;            // (block, first tile, end tile, first j-partial tile)
+  int4 *sitems;            // (block, first group, end group, first j-partial group)
   int2 *sblock;            // per block: (replica, species)
   float2 *sorigin;         // per block: integer origin for re-centring
   float2 *ipart;           // [item][BD_SB] i-side partial forces
-  float2 *jpart;           // [j-partial tile][BD_TJ] j-side partial forces
-  double2 *ipart64, *jpart64;  // the same for the FP64 sweep: [item][BD_F64_SB], [j-partial group][BD_F64_TJ]
+  float2 *jpart;           // [j-partial group][BD_SG] j-side partial forces
+  double2 *ipart64, *jpart64;  // the same for the FP64 sweep: [item][BD_F64_SB], [j-partial group][BD_SG]
   int *red_iptr, *red_iidx;  // per block: the items whose i side it is
-  int *red_jptr, *red_jidx;  // per tile: the j-partial tiles that hold it
+  int *red_jptr, *red_jidx;  // per group: the j-partial groups that hold it
   // short range: Verlet lists (column-major ELL) and the cell grids
   int *vl_idx, *vl_cnt;
   double2 *vl_ref;

@@ -37,10 +37,10 @@ template <bool PER>
 __global__ void __launch_bounds__(BD_F64_SB) k_force_long_f64s(BdDev d, BdConst c) {
   if (ctl_failed(d.ctl)) return;
   constexpr int NW = BD_F64_SB / 32;
-  __shared__ double2 shj[NW][BD_F64_TJ];
+  __shared__ double2 shj[NW][BD_SG];
   const int4 item = d.sitems[blockIdx.x];
   const int P = item.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int gsym = (P + 1) * (BD_F64_SB / BD_F64_TJ);   // first group met from both sides
+  const int gsym = (P + 1) * (BD_F64_SB / BD_SG);   // first group met from both sides
   const int2 binfo = d.sblock[P / (BD_SB / BD_F64_SB)];
   const BdRep &R = d.rep[binfo.x];
   const int a = binfo.y;
@@ -53,10 +53,10 @@ __global__ void __launch_bounds__(BD_F64_SB) k_force_long_f64s(BdDev d, BdConst 
   for (int g = item.y; g < item.z; ++g) {
     const int own = g - P * NW;                         // the warp whose disks i are this group's j
     const bool both = g >= gsym;
-    const int j0 = g * BD_F64_TJ + lane;
+    const int j0 = g * BD_SG + lane;
     double2 pj = d.pos[j0];
     int jl = d.ext_id[j0] >= 0 ? 1 : 0;
-    const int b = d.tile_species[g * BD_F64_TJ / BD_TJ];
+    const int b = d.tile_species[g * BD_SG / BD_TJ];
     double ax = 0.0, ay = 0.0, hx = 0.0, hy = 0.0;
     const int src = (lane + 1) & 31;
     auto pair = [&](bool skip) {
@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(BD_F64_SB) k_force_long_f64s(BdDev d, BdConst 
     if (both) {
       shj[warp][lane] = make_double2(hx, hy);
       __syncthreads();
-      if (tid < BD_F64_TJ) {
+      if (tid < BD_SG) {
         const double alj = R.alpha_d[BD_MAX_SPECIES * b + a];
         double sx = 0.0, sy = 0.0;
 #pragma unroll
@@ -107,7 +107,7 @@ __global__ void __launch_bounds__(BD_F64_SB) k_force_long_f64s(BdDev d, BdConst 
           sx += shj[w][tid].x;
           sy += shj[w][tid].y;
         }
-        d.jpart64[(size_t)njp * BD_F64_TJ + tid] = make_double2(alj * sx, alj * sy);
+        d.jpart64[(size_t)njp * BD_SG + tid] = make_double2(alj * sx, alj * sy);
       }
       __syncthreads();
       ++njp;
@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(256) k_force_f64_reduce(BdDev d, BdConst c) {
   if (ctl_failed(d.ctl)) return;
   __shared__ double2 sh[8][32];
   const int g = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int i = g * BD_F64_TJ + lane, P = i / BD_F64_SB;
+  const int i = g * BD_SG + lane, P = i / BD_F64_SB;
   double fx = 0.0, fy = 0.0;
   for (int k = d.red_iptr[P] + w; k < d.red_iptr[P + 1]; k += 8) {
     const double2 v = d.ipart64[(size_t)d.red_iidx[k] * BD_F64_SB + (i - P * BD_F64_SB)];
@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(256) k_force_f64_reduce(BdDev d, BdConst c) {
     fy += v.y;
   }
   for (int k = d.red_jptr[g] + w; k < d.red_jptr[g + 1]; k += 8) {
-    const double2 v = d.jpart64[(size_t)d.red_jidx[k] * BD_F64_TJ + lane];
+    const double2 v = d.jpart64[(size_t)d.red_jidx[k] * BD_SG + lane];
     fx += v.x;
     fy += v.y;
   }
@@ -154,6 +154,6 @@ cudaError_t bd_launch_force_f64s(const BdDev &d, const BdConst &c, cudaStream_t 
   if (c.n_sitems == 0) return cudaSuccess;
   if (c.any_periodic) k_force_long_f64s<true><<<c.n_sitems, BD_F64_SB, 0, s>>>(d, c);
   else k_force_long_f64s<false><<<c.n_sitems, BD_F64_SB, 0, s>>>(d, c);
-  k_force_f64_reduce<<<c.np / BD_F64_TJ, 256, 0, s>>>(d, c);
+  k_force_f64_reduce<<<c.np / BD_SG, 256, 0, s>>>(d, c);
   return cudaGetLastError();
 }

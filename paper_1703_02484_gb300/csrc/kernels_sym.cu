@@ -5,10 +5,12 @@
 // -A[s_j][s_i] g_ij to j; the table need not be symmetric).
 //
 // Disks sit in blocks of BD_SB = 512 consecutive slots (two j tiles), each of
-// one species.  A work item pairs block P with a range of tiles:
-//  - tiles of P itself: the i side only, all ordered pairs inside P;
-//  - later tiles (index >= 2P + 2): every pair once, both sides.
-// Pairs with an earlier tile are done by that tile's block.
+// one species.  A work item pairs block P with a range of groups of 32 disks j:
+//  - groups of P itself: the i side only, all ordered pairs inside P;
+//  - groups of later blocks: every pair once, both sides.
+// Pairs with an earlier group are done by that group's block.  Items are cut in
+// groups, not in whole tiles of 256, so that a small system still has several
+// items for every resident block.
 //
 // Inside an item each warp holds a share of the disks i of P in registers
 // (four or eight per lane, as packed f32x2 pairs).  A tile of 256 disks j is staged
@@ -21,8 +23,8 @@
 // the one-sided sweep.
 //
 // Partial forces are written, not added: the i side of each item to ipart,
-// the j side of each (item, tile) to jpart.  k_force_sym_reduce then sums, for
-// every disk, its block's i partials and its tile's j partials in a fixed
+// the j side of each (item, group) to jpart.  k_force_sym_reduce then sums, for
+// every disk, its block's i partials and its group's j partials in a fixed
 // order, so the force is deterministic.  Coordinates are re-centred on the
 // block's integer origin from the (hi, lo) FP32 pair of each FP64 coordinate,
 // as in the one-sided sweep; per-tile FP32 sums are added in (hi, lo) pairs
@@ -39,6 +41,10 @@
 #include "f32x2.cuh"
 
 using namespace bdf;
+
+// below this many slots the reduction takes sixteen shares per disk, not four:
+// about the slots whose four shares fill the SMs' threads
+#define BD_RED_SMALL 65536
 
 namespace {
 
@@ -154,7 +160,8 @@ __device__ __forceinline__ void force_long_sym_body(const BdDev &d, const BdCons
   constexpr int T = NW * 32;         // threads
   constexpr int NQ = 2 * NP;         // disks i per thread
   constexpr int NS = BD_TJ / T;      // j disks each thread stages per tile
-  constexpr int NG = BD_TJ / 32;     // groups of 32 disks j per tile
+  constexpr int NG = BD_TJ / BD_SG;  // groups of 32 disks j per tile
+  static_assert(NJ == 1, "a ring carries one group of 32 disks j");
   static_assert(BD_SB == T * NQ, "a block is BD_SB disks");
   __shared__ float2 sjp[2][STAGE ? 1 : BD_TJ];   // j positions, re-centred
   __shared__ __align__(16) float4 sraw[2][STAGE ? BD_TJ : 1];   // STAGE 1: j as stored (x_hi, y_hi, x_lo, y_lo);
@@ -168,7 +175,7 @@ __device__ __forceinline__ void force_long_sym_body(const BdDev &d, const BdCons
   const int4 item = d.sitems[item_id];
   const int P = item.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int base = P * BD_SB;
-  const int tsym = 2 * P + 2;        // first tile met from both sides
+  const int gsym = (P + 1) * (BD_SB / BD_SG);   // first group met from both sides
   const int2 binfo = d.sblock[P];
   const BdRep &R = d.rep[binfo.x];
   const int a = binfo.y;
@@ -223,8 +230,9 @@ __device__ __forceinline__ void force_long_sym_body(const BdDev &d, const BdCons
   }
   const float e0 = 1e-20f * (float)(c.a * c.a);   // makes the self pair exactly 0
   const u64 eps2 = pk2(e0, e0);
-  const int t_begin = item.y, t_end = item.z;
-  const int jt0 = max(t_begin, tsym);
+  const int t_begin = item.y / NG, t_end = (item.z + NG - 1) / NG;   // tiles staged
+  // j sums: group G of the item at slot item.w + G - max(item.y, gsym)
+  float2 *const jout = d.jpart + ((ptrdiff_t)item.w - max(item.y, gsym)) * BD_SG;
   float4 st[STAGE ? 1 : NS];
   int buf = 0;
   auto fetch = [&](int tile) {
@@ -504,17 +512,18 @@ __device__ __forceinline__ void force_long_sym_body(const BdDev &d, const BdCons
   for (int t = t_begin; t < t_end; ++t) {
     if (t + 1 < t_end) fetch(t + 1);
     const int b = d.tile_species[t];
-    if (t < tsym) {
-      for (int g = 0; g < NG; ++g)
+    const int ga = max(item.y - t * NG, 0), gz = min(item.z - t * NG, NG);   // the item's groups of the tile
+    if (t * NG < gsym) {
+      for (int g = ga; g < gz; ++g)
         dispatch(pair_mode(g, 1), [&](auto M) { own_group(M, g); });
     } else {
-      for (int g = 0; g < BD_TJ / (32 * NJ); ++g)
-        dispatch(pair_mode(g * NJ, NJ), [&](auto M) { ring_group(M, g); });
+      for (int g = ga; g < gz; ++g)
+        dispatch(pair_mode(g, 1), [&](auto M) { ring_group(M, g); });
       __syncthreads();
       // j side of this tile: F_j += A[s_j][s_i] sum_i (r_j - r_i)/r^3
       const float alj = R.alpha[BD_MAX_SPECIES * b + a];
-      float2 *out = d.jpart + (size_t)(item.w + (t - jt0)) * BD_TJ;
-      for (int jj = tid; jj < BD_TJ; jj += T) {
+      float2 *out = jout + (ptrdiff_t)t * BD_TJ;
+      for (int jj = ga * BD_SG + tid; jj < gz * BD_SG; jj += T) {
         float hx = 0.f, hy = 0.f;
 #pragma unroll
         for (int w = 0; w < NW; ++w) {
@@ -556,40 +565,35 @@ __device__ __forceinline__ void force_long_sym_body(const BdDev &d, const BdCons
   }
 }
 
-template <int NW, int NP, int NJ, bool COMB, int UR, bool PER>
-__global__ void __launch_bounds__(NW * 32) k_force_long_sym(BdDev d, BdConst c) {
-  force_long_sym_body<NW, NP, NJ, COMB, UR, PER>(d, c);
-}
-
-// the same with a register budget for MINB resident blocks per SM
+// with a register budget for MINB resident blocks per SM
 template <int NW, int NP, int NJ, bool COMB, int UR, bool PER, int MINB, int STAGE, int ACC>
 __global__ void __launch_bounds__(NW * 32, MINB) k_force_long_sym_mb(BdDev d, BdConst c) {
   force_long_sym_body<NW, NP, NJ, COMB, UR, PER, STAGE, ACC>(d, c);
 }
 
-// F_i = sum of its block's i partials + sum of its tile's j partials, in the
+// F_i = sum of its block's i partials + sum of its group's j partials, in the
 // order the host listed them (item order), into partial-force slot 0.
-// A block of 256 threads serves 64 consecutive disks: thread group g (of 4)
-// takes every fourth partial (entries g, g + 4, ...) of the 64 disks, so the
-// loads stay coalesced and four times as many warps hide their latency; the
-// four group sums are added in a fixed order.  Sums are float-float (TwoSum
-// into a (hi, lo) FP32 pair, about 48 bits): FP64 adds run at 1/64 of the FP32
-// rate on this part and would bound the kernel.
-#define BD_RED_D 64   // disks per reduction block
-__global__ void __launch_bounds__(4 * BD_RED_D) k_force_sym_reduce(BdDev d, BdConst c) {
-  __shared__ float4 part[4][BD_RED_D];
+// Bound by the partials' reads.  ND disks per block, NS shares: thread share g
+// takes every NS-th partial (entries g, g + NS, ...) of the ND disks, so the
+// loads stay coalesced and NS times as many warps hide their latency; the
+// shares' sums are added in a fixed order.  Sums are float-float (TwoSum into
+// a (hi, lo) FP32 pair, about 48 bits): FP64 adds run at 1/64 of the FP32 rate
+// on this part and would bound the kernel.
+template <int ND, int NS>
+__global__ void __launch_bounds__(ND * NS) k_force_sym_reduce(BdDev d, BdConst c) {
+  __shared__ float4 part[NS][ND];
   if (ctl_failed(d.ctl)) return;
-  const int g = threadIdx.x / BD_RED_D, dl = threadIdx.x % BD_RED_D;
-  const int i = blockIdx.x * BD_RED_D + dl;        // np is a multiple of 512: i < np
-  const int P = i / BD_SB, t = i / BD_TJ;           // the same for the whole block
+  const int g = threadIdx.x / ND, dl = threadIdx.x % ND;
+  const int i = blockIdx.x * ND + dl;               // np is a multiple of 512: i < np
+  const int P = i / BD_SB, t = i / BD_SG;            // the same for the whole warp
   const float2 *ib = d.ipart + (i - P * BD_SB);
-  const float2 *jb = d.jpart + (i - t * BD_TJ);
+  const float2 *jb = d.jpart + (i - t * BD_SG);
   float xh[2] = {0.f, 0.f}, xl[2] = {0.f, 0.f}, yh[2] = {0.f, 0.f}, yl[2] = {0.f, 0.f};
   auto run = [&](const int *idx, int k0, int k1, const float2 *b, int stride) {
     int k = k0 + g;
-    for (; k + 4 < k1; k += 8) {
+    for (; k + NS < k1; k += 2 * NS) {
       const float2 v0 = b[(size_t)__ldg(idx + k) * stride];
-      const float2 v1 = b[(size_t)__ldg(idx + k + 4) * stride];
+      const float2 v1 = b[(size_t)__ldg(idx + k + NS) * stride];
       two_sum(xh[0], xl[0], v0.x);
       two_sum(yh[0], yl[0], v0.y);
       two_sum(xh[1], xl[1], v1.x);
@@ -602,7 +606,7 @@ __global__ void __launch_bounds__(4 * BD_RED_D) k_force_sym_reduce(BdDev d, BdCo
     }
   };
   run(d.red_iidx, d.red_iptr[P], d.red_iptr[P + 1], ib, BD_SB);
-  run(d.red_jidx, d.red_jptr[t], d.red_jptr[t + 1], jb, BD_TJ);
+  run(d.red_jidx, d.red_jptr[t], d.red_jptr[t + 1], jb, BD_SG);
   two_sum(xh[0], xl[0], xh[1]);
   two_sum(yh[0], yl[0], yh[1]);
   part[g][dl] = make_float4(xh[0], __fadd_rn(xl[0], xl[1]), yh[0], __fadd_rn(yl[0], yl[1]));
@@ -610,14 +614,16 @@ __global__ void __launch_bounds__(4 * BD_RED_D) k_force_sym_reduce(BdDev d, BdCo
   if (g != 0) return;
   const int r = d.rep_of[i];
   if (r < 0 || d.rep[r].law != BD_LAW_LONG) return;
-  double fx = 0.0, fy = 0.0;
+  float sx = 0.f, ex = 0.f, sy = 0.f, ey = 0.f;
 #pragma unroll
-  for (int m = 0; m < 4; ++m) {
+  for (int m = 0; m < NS; ++m) {
     const float4 q = part[m][dl];
-    fx += (double)q.x + (double)q.y;
-    fy += (double)q.z + (double)q.w;
+    two_sum(sx, ex, q.x);
+    two_sum(sy, ey, q.z);
+    ex = __fadd_rn(ex, q.y);
+    ey = __fadd_rn(ey, q.w);
   }
-  d.fpart[i] = make_double2(fx, fy);
+  d.fpart[i] = make_double2((double)sx + (double)ex, (double)sy + (double)ey);
 }
 
 int bd_force_launches(const BdConst &c) { return (c.precision == 0 ? c.force_variant >= 2 : c.f64_sym) ? 2 : 1; }
@@ -632,7 +638,7 @@ int bd_force_sym_blocks_per_sm(int variant, int periodic) {
                            &per, k_force_long_sym_mb<2, 4, 1, false, 2, true, 12, 1, 2>, 64, 0);
   else
     e = variant == 2 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                           &per, k_force_long_sym<4, 2, 1, false, 2, false>, 128, 0)
+                           &per, k_force_long_sym_mb<4, 2, 1, false, 2, false, 8, 1, 2>, 128, 0)
                      : cudaOccupancyMaxActiveBlocksPerMultiprocessor(
                            &per, k_force_long_sym_mb<2, 4, 1, false, 2, false, 16, 1, 2>, 64, 0);
   return e == cudaSuccess ? per : 0;
@@ -654,7 +660,7 @@ cudaError_t bd_launch_force_sym(const BdDev &d, const BdConst &c, int variant, c
       k_force_long_sym_mb<2, 4, 1, false, 2, true, 12, 1, 2><<<c.n_sitems, 64, 0, s>>>(d, c);
   } else {
     if (variant == 2)
-      k_force_long_sym<4, 2, 1, false, 2, false><<<c.n_sitems, 128, 0, s>>>(d, c);
+      k_force_long_sym_mb<4, 2, 1, false, 2, false, 8, 1, 2><<<c.n_sitems, 128, 0, s>>>(d, c);
     else
       // 16 resident blocks (32 warps) per SM in 64 registers, j tiles staged by
       // cp.async: measured 1.776 -> 1.668 ms at N = 1e5 against the
@@ -665,6 +671,7 @@ cudaError_t bd_launch_force_sym(const BdDev &d, const BdConst &c, int variant, c
       // lane (+2.7 %)
       k_force_long_sym_mb<2, 4, 1, false, 2, false, 16, 1, 2><<<c.n_sitems, 64, 0, s>>>(d, c);
   }
-  k_force_sym_reduce<<<c.np / BD_RED_D, 4 * BD_RED_D, 0, s>>>(d, c);
+  if (c.np < BD_RED_SMALL) k_force_sym_reduce<32, 16><<<c.np / 32, 512, 0, s>>>(d, c);
+  else k_force_sym_reduce<64, 4><<<c.np / 64, 256, 0, s>>>(d, c);
   return cudaGetLastError();
 }
