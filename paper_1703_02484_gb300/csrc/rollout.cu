@@ -58,10 +58,11 @@ struct BdRollout {
   double2 *seg_x = nullptr;
   float *seg_th = nullptr;
   int seg_steps_cap = 0;
-  double2 *seg_z = nullptr;
+  double2 *seg_z = nullptr, *seg_zd = nullptr;   // positions before each pass, its displacement sums
   int seg_pass_cap = 0;
   double2 *lam = nullptr, *mud = nullptr, *rpos = nullptr, *rdisp = nullptr, *jpart = nullptr;
-  float4 *rwork = nullptr;
+  float4 *rwork = nullptr, *vx = nullptr;
+  float2 *vm = nullptr;
   float *rth = nullptr;
   double *gpart = nullptr;
   int jpart_chunks = 0, gpart_cap = 0;
@@ -192,7 +193,9 @@ cudaError_t ensure_scratch(bd_handle *h, BdRollout *r) {
     if (e == cudaSuccess) e = regrow(&r->rth, 0, np, s);
     int jchunk = 0;
     const int nch = bd_adj_force_chunks(h->c, &jchunk);
-    const int nbi = (h->np + BD_ADJ_T - 1) / BD_ADJ_T;
+    const int nbi = h->np / (2 * BD_ADJ_T);
+    if (e == cudaSuccess) e = regrow(&r->vx, 0, np, s);
+    if (e == cudaSuccess) e = regrow(&r->vm, 0, np, s);
     if (e == cudaSuccess) e = regrow(&r->jpart, 0, (size_t)nch * np, s);
     if (e == cudaSuccess) e = regrow(&r->gpart, 0, (size_t)nch * nbi * 5, s);
     if (e != cudaSuccess) return e;
@@ -212,6 +215,7 @@ cudaError_t ensure_scratch(bd_handle *h, BdRollout *r) {
   }
   if (maxp > r->seg_pass_cap) {
     e = regrow(&r->seg_z, 0, (size_t)maxp * np, s);
+    if (e == cudaSuccess) e = regrow(&r->seg_zd, 0, (size_t)maxp * np, s);
     if (e != cudaSuccess) return e;
     r->seg_pass_cap = maxp;
   }
@@ -241,21 +245,14 @@ cudaError_t replay(bd_handle *h, BdRollout *r, const BdDev &dr, int t0, int t1, 
   const int pb0 = r->step_pass[t0];
   cudaError_t e = cudaSuccess;
   for (int t = t0; t < t1 && e == cudaSuccess; ++t) {
-    if (store) {
-      e = cudaMemcpyAsync(r->seg_x + (size_t)(t - t0) * np, dr.pos, np * sizeof(double2),
-                          cudaMemcpyDeviceToDevice, s);
-      if (e == cudaSuccess)
-        e = cudaMemcpyAsync(r->seg_th + (size_t)(t - t0) * np, dr.theta, np * sizeof(float),
-                            cudaMemcpyDeviceToDevice, s);
-    }
-    if (e == cudaSuccess) e = bd_launch_force_long(dr, h->c, s);
-    if (e == cudaSuccess) e = bd_adj_rp_em(dr, h->c, (long long)(r->step0 + t), t, s);
-    for (int p = r->step_pass[t]; p < r->step_pass[t + 1] && e == cudaSuccess; ++p) {
-      if (store)
-        e = cudaMemcpyAsync(r->seg_z + (size_t)(p - pb0) * np, dr.pos, np * sizeof(double2),
-                            cudaMemcpyDeviceToDevice, s);
-      if (e == cudaSuccess) e = bd_adj_rp_pass(dr, h->c, p, r->pass_begin[p], r->pass_begin[p + 1], s);
-    }
+    e = bd_launch_force_long(dr, h->c, s);
+    if (e == cudaSuccess)
+      e = bd_adj_rp_em(dr, h->c, (long long)(r->step0 + t), t, store ? r->seg_x + (size_t)(t - t0) * np : nullptr,
+                       store ? r->seg_th + (size_t)(t - t0) * np : nullptr, s);
+    for (int p = r->step_pass[t]; p < r->step_pass[t + 1] && e == cudaSuccess; ++p)
+      e = bd_adj_rp_pass(dr, h->c, p, r->pass_begin[p], r->pass_begin[p + 1],
+                         store ? r->seg_z + (size_t)(p - pb0) * np : nullptr,
+                         store ? r->seg_zd + (size_t)(p - pb0) * np : nullptr, s);
   }
   return e;
 }
@@ -294,6 +291,9 @@ void rollout_release(bd_handle *h) {
   release(&r->seg_x);
   release(&r->seg_th);
   release(&r->seg_z);
+  release(&r->seg_zd);
+  release(&r->vx);
+  release(&r->vm);
   release(&r->lam);
   release(&r->mud);
   release(&r->rpos);
@@ -532,13 +532,13 @@ int bd_rollout_vjp(bd_handle *h, double *grad) {
     for (int t = t1 - 1; t >= t0 && e == cudaSuccess; --t) {
       for (int p = r->step_pass[t + 1] - 1; p >= r->step_pass[t] && e == cudaSuccess; --p) {
         e = bd_adj_vjp_pass(dr, h->c, p, r->pass_begin[p], r->pass_begin[p + 1], r->seg_z + (size_t)(p - pb0) * np,
-                            r->lam, r->mud, s);
-        launches += 3;
+                            r->seg_zd + (size_t)(p - pb0) * np, r->lam, r->mud, s);
+        launches += 2;
       }
       if (e == cudaSuccess)
         e = bd_adj_vjp_em(dr, h->c, t, r->seg_x + (size_t)(t - t0) * np, r->seg_th + (size_t)(t - t0) * np,
-                          r->lam, r->jpart, r->gpart, r->acc + 8, s);
-      launches += 4;
+                          r->lam, r->vx, r->vm, r->jpart, r->gpart, r->acc + 8, s);
+      launches += 3;
     }
   }
   double gh[5] = {0, 0, 0, 0, 0};
