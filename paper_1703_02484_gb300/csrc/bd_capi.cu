@@ -1104,6 +1104,7 @@ int build_handle(const std::vector<Spec> &specs, void *stream, bd_handle **out) 
         BD_TRY(autotune(h));
       }
     }
+    c.tri_cluster = c.overlap_verlet ? 0 : bd_dt_cluster_for(nt);
     if (bd_dt_grid_for(std::max(nt, np), &h->dt_grid, &h->dt_block) != 0 ||
         (c.any_short && bd_vl_grid_for(np, &c.vl_grid) != 0) ||
         (c.overlap_verlet && bd_vcorr_grid_for(np, &h->vc_grid, &h->vc_block) != 0)) {

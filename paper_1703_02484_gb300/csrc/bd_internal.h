@@ -53,8 +53,8 @@ struct BdCtl {
   int status;
   unsigned int exit_count;         // blocks that have left the triangulation kernel
   unsigned int pad0[29];
-  unsigned int bar_gen;            // on a 128-byte line of its own: the blocks waiting at a
-  unsigned int pad1[31];           // barrier poll it, and only it
+  uint4 bar_pub[8];                // on a 128-byte line of its own, which the blocks waiting at a
+                                   // barrier poll: (generation, three words of its counters) chunks
   unsigned long long epoch;        // flip-round counter, grows across launches
   int cnt[4][8];                   // per-phase counters, rotated every barrier
   // statistics accumulated over a bd_step call
@@ -236,6 +236,7 @@ struct BdConst {
   int tri_fuse;            // 1: a Lawson round tests the outer edges of its flips and keeps the
                            // overlap sums (no check pass between rounds); 0: a check pass after
                            // every round (environment variable BD_TRI_FUSE at init)
+  int tri_cluster;         // > 0: the triangulation kernel runs as one cluster of so many blocks
   int vl_grid;             // blocks of the Verlet-list rebuild launch
   double vl_reach2;        // squared displacement since the list build below which the lists
                            // still hold every pair closer than sigma
@@ -254,6 +255,8 @@ cudaError_t bd_launch_dt(const BdDev &d, const BdConst &c, int mode, cudaStream_
                          int log_step = -1);
 int bd_dt_grid(int *grid, int *block);
 int bd_dt_grid_for(int work_items, int *grid, int *block);
+// blocks of the one cluster that serves a triangulation of nt triangles (0: the grid does)
+int bd_dt_cluster_for(int nt);
 int bd_force_blocks_per_sm(int variant);
 cudaError_t bd_launch_work_copy(const BdDev &d, const BdConst &c, cudaStream_t s);
 // caller-order positions (and directions) in xfer_* -> checked, grid-rounded slots; a

@@ -43,8 +43,10 @@
 // On any failure the step is undone from the launch's undo journal: the first
 // change a launch makes to a triangle (a flip, its back-pointers, a periodic
 // shift) records the triangle's corners and neighbours as they were.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <stdlib.h>
 
 #include "bd_internal.h"
 #include "em.cuh"
@@ -52,6 +54,7 @@
 #include "predicates.cuh"
 
 #define BD_DT_THREADS 256
+#define BD_DTC_THREADS 512   // threads per block of the cluster form
 
 using namespace bdgs;
 
@@ -80,6 +83,7 @@ struct Ctx {
   int np;
   float sig2f;   // sigma^2 (1 + 1e-5): FP32 screen of the overlap scan
   unsigned jstamp;   // this launch's undo-journal mark (odd)
+  int *cl_n;         // lengths of the candidate lists
 };
 
 // FP32 filters in front of the exact integer predicates.  Every disk's
@@ -480,7 +484,7 @@ __device__ __forceinline__ int key_corner(unsigned long long key) {
 __device__ __forceinline__ void push_owner(const Ctx &x, unsigned long long e, int t) {
   if (atomicExch(&x.d.clmark[t], (unsigned)e) == (unsigned)e) return;
   const int l = (int)(e % 3);
-  x.d.clist[(size_t)l * x.T + atomicAdd(&x.d.ctl->cl_n[l], 1)] = t;
+  x.d.clist[(size_t)l * x.T + atomicAdd(&x.cl_n[l], 1)] = t;
 }
 
 // Stamp triangle t for the check pass of generation byte s.  The word is
@@ -684,9 +688,11 @@ __device__ __forceinline__ int tri_rep(const BdDev &d, int np, const int4 &v) {
 // the exact-predicate fallbacks (measured: 3 blocks 20 % faster than 2 on
 // 2^20 disks; 4 blocks (64 registers) 1.5 % faster on 2^20 disks but 16 %
 // slower in the check passes at 1e5; 5 blocks slower on both).
-template <bool PER>
-__global__ void __launch_bounds__(BD_DT_THREADS, 3) k_triangulation(BdDev d, BdConst c, int mode,
-                                                                 int log_step) {
+//
+// CL: the launch is one thread-block cluster (a small system): hardware
+// barriers, the phase words in the first block's shared memory, 128 registers.
+template <bool PER, bool CL>
+__device__ __forceinline__ void triangulation_body(const BdDev &d, const BdConst &c, int mode, int log_step) {
   Ctx x;
   x.d = d;
   x.c = c;
@@ -700,13 +706,36 @@ __global__ void __launch_bounds__(BD_DT_THREADS, 3) k_triangulation(BdDev d, BdC
   if (ld_status(&ctl->status) != 0 || (mode == 1 && *(volatile const int *)&ctl->n_set_moved == 0)) {
     // (bd_set_state that moved no disk: the triangulation stands as it was)
     if (blockIdx.x == 0 && threadIdx.x == 0 && ld_status(&ctl->status) == 0) ctl->in_move = 0;
-    block_exit(ctl);
+    if (!CL) block_exit(ctl);
     return;
   }
   Bar b;
   b.gen = 0;
   b.ph = 0;
   __shared__ int bc[BC_N];                // phase counters and list lengths, per barrier
+  // the phase words: in the control block, or in the cluster's first block
+  __shared__ int s_words[CL ? BW_N : 1];
+  int *words = nullptr, *wcnt = &ctl->cnt[0][0], *wact = ctl->act_n;
+  x.cl_n = ctl->cl_n;
+  unsigned hold = 0;
+  if (CL) {
+    hold = *(volatile const unsigned *)&ctl->bar_hold;
+    if (threadIdx.x < BW_N) s_words[threadIdx.x] = 0;
+    words = cooperative_groups::this_cluster().map_shared_rank(s_words, 0);
+    wcnt = words + BW_CNT;
+    wact = words + BW_ACT;
+    x.cl_n = words + BW_CL;
+    cluster_barrier();
+  }
+  auto sync = [&]() -> bool { return CL ? cluster_sync(ctl, words, hold, b, bc) : grid_sync(ctl, b, bc); };
+  auto leave = [&]() {
+    if (CL) cluster_barrier();   // the first block's words are read until the last one is here
+    else block_exit(ctl);
+  };
+  auto pcnt = [&](int slot) -> int * { return wcnt + 8 * (b.ph & 3) + slot; };
+  auto phase_start = [&]() {   // clear the counters two phases ahead
+    if (blockIdx.x == 0 && threadIdx.x < 8) wcnt[8 * ((b.ph + 2) & 3) + threadIdx.x] = 0;
+  };
   unsigned long long t_mark = gtimer();   // stage timing (lead thread)
   const int tid = blockIdx.x * blockDim.x + threadIdx.x;
   const int nth = gridDim.x * blockDim.x;
@@ -754,8 +783,8 @@ __global__ void __launch_bounds__(BD_DT_THREADS, 3) k_triangulation(BdDev d, BdC
   for (;;) {
     ++epoch;
     if (lead) {
-      ctl->cl_n[(epoch + 2) % 3] = 0;   // the candidate list two rounds ahead
-      ctl->act_n[(kp + 2) % 3] = 0;     // the triangle list two passes ahead
+      x.cl_n[(epoch + 2) % 3] = 0;   // the candidate list two rounds ahead
+      wact[(kp + 2) % 3] = 0;     // the triangle list two passes ahead
     }
     const int slot = kp % 3, nslot = (kp + 1) % 3;
     const unsigned gen = g0 + (unsigned)kp, ngen = gen + 1u;
@@ -764,10 +793,10 @@ __global__ void __launch_bounds__(BD_DT_THREADS, 3) k_triangulation(BdDev d, BdC
     const unsigned *cmark = d.act_mark + (size_t)slot * x.T;
     int *nlist = d.act + (size_t)nslot * x.T;
     unsigned *nmark = d.act_mark + (size_t)nslot * x.T;
-    int *ncount = &ctl->act_n[nslot];
+    int *ncount = &wact[nslot];
     // ---------------- W: shifts of triangles whose corners re-entered (periodic box) ----------------
     if (PER && fresh && *(volatile int *)&ctl->n_wrapped != 0) {
-      phase_begin(ctl, b);
+      phase_start();
       for (int t = tid; t < x.T; t += nth) {
         const int4 v = d.tv[t];
         const uint8_t w0 = d.wrap[v.x], w1 = d.wrap[v.y], w2 = d.wrap[v.z];
@@ -784,7 +813,7 @@ __global__ void __launch_bounds__(BD_DT_THREADS, 3) k_triangulation(BdDev d, BdC
         for (int k = 0; k < 3; ++k) nw |= put_shift(k, sx[k] - sx[0], sy[k] - sy[0]);
         d.tv[t].w = nw;
       }
-      if (!grid_sync(ctl, b, bc)) { block_exit(ctl); return; }
+      if (!sync()) { leave(); return; }
       if (lead) ctl->n_wrapped = 0;
     }
     // ---------------- P: check, mark, scan ----------------
@@ -795,7 +824,7 @@ __global__ void __launch_bounds__(BD_DT_THREADS, 3) k_triangulation(BdDev d, BdC
     const int dom_n = full ? x.T : bc[BC_ACT + slot];
     if (need_p) {
       if (lead) tri_visits += dom_n;
-      phase_begin(ctl, b);
+      phase_start();
       {
         int inv = 0, rej = 0, cand = 0, nov = 0;
         double mx = 0.0;
@@ -922,7 +951,7 @@ __global__ void __launch_bounds__(BD_DT_THREADS, 3) k_triangulation(BdDev d, BdC
                 disp_add(x, u, -v.x, -v.y);
                 disp_add(x, w, v.x, v.y);
                 if (use_lists) push_tri(nlist, nmark, ncount, ngen, t);   // checked again in the next pass
-                const int k_ov = atomicAdd(cnt(ctl, b.ph, C_OVERLAP), 1);
+                const int k_ov = atomicAdd(pcnt(C_OVERLAP), 1);
                 if (logging) {
                   if (log_head + k_ov < c.log_pairs_cap) d.log_pairs[log_head + k_ov] = make_int2(u, w);
                   else atomicExch(&ctl->log_overflow, 1);
@@ -1034,7 +1063,7 @@ __global__ void __launch_bounds__(BD_DT_THREADS, 3) k_triangulation(BdDev d, BdC
                 disp_add(x, u, -v.x, -v.y);
                 disp_add(x, w, v.x, v.y);
                 if (use_lists) push_tri(nlist, nmark, ncount, ngen, t);   // checked again in the next pass
-                const int k_ov = atomicAdd(cnt(ctl, b.ph, C_OVERLAP), 1);
+                const int k_ov = atomicAdd(pcnt(C_OVERLAP), 1);
                 if (logging) {
                   if (log_head + k_ov < c.log_pairs_cap) d.log_pairs[log_head + k_ov] = make_int2(u, w);
                   else atomicExch(&ctl->log_overflow, 1);
@@ -1044,13 +1073,15 @@ __global__ void __launch_bounds__(BD_DT_THREADS, 3) k_triangulation(BdDev d, BdC
             }
           }
         }
-        block_add(cnt(ctl, b.ph, C_INV), inv);
-        block_add(cnt(ctl, b.ph, C_REJECT), rej);
-        block_add(cnt(ctl, b.ph, C_CAND), cand);
+        {
+          int *const to[3] = {pcnt(C_INV), pcnt(C_REJECT), pcnt(C_CAND)};
+          const int v[3] = {inv, rej, cand};
+          block_add(to, v);
+        }
         (void)nov;
         if (mx > 0.0) atomicMax(&ctl->st_max_overlap_bits, (unsigned long long)__double_as_longlong(mx));
       }
-      if (!grid_sync(ctl, b, bc)) { block_exit(ctl); return; }
+      if (!sync()) { leave(); return; }
       if (lead) stage_tick(ctl, full ? STAGE_P : STAGE_PL, t_mark);
       const int n_inv = bc[BC_CNT + C_INV];
       const int n_rej = bc[BC_CNT + C_REJECT];
@@ -1068,8 +1099,8 @@ __global__ void __launch_bounds__(BD_DT_THREADS, 3) k_triangulation(BdDev d, BdC
         bool first_round = true;
         for (;;) {
           ++epoch;
-          if (lead) ctl->cl_n[(epoch + 2) % 3] = 0;   // the candidate list two rounds ahead
-          phase_begin(ctl, b);
+          if (lead) x.cl_n[(epoch + 2) % 3] = 0;   // the candidate list two rounds ahead
+          phase_start();
           {
             if (first_round) {
               for (int i = tid; i < x.np; i += nth) d.disp[i] = make_double2(0.0, 0.0);
@@ -1110,10 +1141,10 @@ __global__ void __launch_bounds__(BD_DT_THREADS, 3) k_triangulation(BdDev d, BdC
                 }
               }
             }
-            block_add(cnt(ctl, b.ph, C_INV), inv);
-            block_add(cnt(ctl, b.ph, C_CAND), ncand);
+            block_add(pcnt(C_INV), inv);
+            block_add(pcnt(C_CAND), ncand);
           }
-          if (!grid_sync(ctl, b, bc)) { block_exit(ctl); return; }
+          if (!sync()) { leave(); return; }
           if (lead) stage_tick(ctl, STAGE_R, t_mark);
           first_round = false;
           const int ni = bc[BC_CNT + C_INV];
@@ -1124,7 +1155,7 @@ __global__ void __launch_bounds__(BD_DT_THREADS, 3) k_triangulation(BdDev d, BdC
             if (lead) { ctl->st_fail_phase = nc == 0 ? 2 : 3; ctl->st_fail_count = ni; }
             break;
           }
-          phase_begin(ctl, b);
+          phase_start();
           {
             int nf = 0;
             for (int t = tid; t < x.T; t += nth) {
@@ -1138,9 +1169,9 @@ __global__ void __launch_bounds__(BD_DT_THREADS, 3) k_triangulation(BdDev d, BdC
               flip_owned<PER>(x, cm, o, ngen8);   // both new triangles are counter-clockwise by the rule
               ++nf;
             }
-            block_add(cnt(ctl, b.ph, C_FLIPS), nf);
+            block_add(pcnt(C_FLIPS), nf);
           }
-          if (!grid_sync(ctl, b, bc)) { block_exit(ctl); return; }
+          if (!sync()) { leave(); return; }
           if (lead) stage_tick(ctl, STAGE_R, t_mark);
           st_rflips += bc[BC_CNT + C_FLIPS];
         }
@@ -1163,7 +1194,7 @@ __global__ void __launch_bounds__(BD_DT_THREADS, 3) k_triangulation(BdDev d, BdC
         if (lead) ctl->st_fail_phase = 4;
         break;
       }
-      phase_begin(ctl, b);
+      phase_start();
       {
         const bool voided = !fuse && n_ov;   // unfused: the marking pass's scan is void
         if (voided || fresh)
@@ -1233,14 +1264,16 @@ __global__ void __launch_bounds__(BD_DT_THREADS, 3) k_triangulation(BdDev d, BdC
             if (use_lists) push_tri(nlist, nmark, ncount, ngen, t);
           }
         }
-        block_add(cnt(ctl, b.ph, C_FLIPS), nf);
+        {
+          int *const to[3] = {pcnt(C_FLIPS), pcnt(C_LOSE), pcnt(C_OVADJ)};
+          const int v[3] = {nf, fuse ? nlose : 0, adj};
+          block_add(to, v);
+        }
         if (fuse) {
-          block_add(cnt(ctl, b.ph, C_LOSE), nlose);
-          block_add(cnt(ctl, b.ph, C_OVADJ), adj);
           if (fmx > 0.0) atomicMax(&ctl->st_max_overlap_bits, (unsigned long long)__double_as_longlong(fmx));
         }
       }
-      if (!grid_sync(ctl, b, bc)) { block_exit(ctl); return; }
+      if (!sync()) { leave(); return; }
       if (lead) stage_tick(ctl, STAGE_F, t_mark);
       st_flips += bc[BC_CNT + C_FLIPS];
       st_rounds += 1;
@@ -1301,7 +1334,7 @@ __global__ void __launch_bounds__(BD_DT_THREADS, 3) k_triangulation(BdDev d, BdC
       ++log_npass;
     }
     // ---------------- A: apply (capped at sigma/4) ----------------
-    phase_begin(ctl, b);
+    phase_start();
     {
       int nwrap = 0;
       for (int i = tid; i < x.np; i += nth) {
@@ -1368,7 +1401,7 @@ __global__ void __launch_bounds__(BD_DT_THREADS, 3) k_triangulation(BdDev d, BdC
       }
       if (PER) block_add(&ctl->n_wrapped, nwrap);
     }
-    if (!grid_sync(ctl, b, bc)) { block_exit(ctl); return; }
+    if (!sync()) { leave(); return; }
     if (lead) stage_tick(ctl, STAGE_A, t_mark);
     fresh = true;
     full = !use_lists;
@@ -1379,7 +1412,7 @@ __global__ void __launch_bounds__(BD_DT_THREADS, 3) k_triangulation(BdDev d, BdC
   if (status) {
     // undo the step: positions and directions from the step start, the
     // triangulation from the undo journal
-    phase_begin(ctl, b);
+    phase_start();
     for (int i = tid; i < x.np; i += nth) {
       if (d.ext_id[i] < 0) continue;
       const double2 p0 = d.pos0[i];
@@ -1422,7 +1455,16 @@ __global__ void __launch_bounds__(BD_DT_THREADS, 3) k_triangulation(BdDev d, BdC
     else if (!status) ctl->st_steps += 1;
     if (!status && mode == 0) ctl->step_dev += 1;
   }
-  block_exit(ctl);
+  leave();
+}
+
+template <bool PER>
+__global__ void __launch_bounds__(BD_DT_THREADS, 3) k_triangulation(BdDev d, BdConst c, int mode, int log_step) {
+  triangulation_body<PER, false>(d, c, mode, log_step);
+}
+template <bool PER>
+__global__ void __launch_bounds__(BD_DTC_THREADS, 1) k_triangulation_cl(BdDev d, BdConst c, int mode, int log_step) {
+  triangulation_body<PER, true>(d, c, mode, log_step);
 }
 
 // Undo a step whose persistent kernel left at a timed-out barrier (the
@@ -1506,6 +1548,36 @@ int bd_dt_grid(int *grid, int *block) {
   return 0;
 }
 
+// One cluster serves triangulations of up to BD_DTC_TRIS triangles: its barriers
+// cost a fraction of the grid's, its threads (8192 in sixteen blocks) are fewer.
+#define BD_DTC_TRIS 16384
+int bd_dt_cluster_for(int nt) {
+  const char *env = getenv("BD_TRI_CLUSTER");   // 0: never, n: up to n triangles
+  const int most = env ? atoi(env) : BD_DTC_TRIS;
+  if (nt > most) return 0;
+  for (int n = 16; n >= 8; n /= 2) {
+    int ok = 1;
+    for (int per = 0; per < 2 && ok; ++per) {
+      const void *fn = per ? (const void *)k_triangulation_cl<true> : (const void *)k_triangulation_cl<false>;
+      if (n > 8 && cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) ok = 0;
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(n);
+      cfg.blockDim = dim3(BD_DTC_THREADS);
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = n;
+      at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+      cfg.attrs = at;
+      cfg.numAttrs = 1;
+      int can = 0;
+      if (!ok || cudaOccupancyMaxActiveClusters(&can, fn, &cfg) != cudaSuccess || can < 1) ok = 0;
+    }
+    if (ok) return n;
+    cudaGetLastError();
+  }
+  return 0;
+}
+
 cudaError_t bd_launch_dt(const BdDev &d, const BdConst &c, int mode, cudaStream_t s, int grid,
                          int block, int log_step) {
   // the barrier words and phase counters were reset by the previous
@@ -1514,6 +1586,20 @@ cudaError_t bd_launch_dt(const BdDev &d, const BdConst &c, int mode, cudaStream_
   BdConst cc = c;
   int m = mode, ls = log_step;
   void *args[] = {&dd, &cc, &m, &ls};
+  if (c.tri_cluster) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(c.tri_cluster);
+    cfg.blockDim = dim3(BD_DTC_THREADS);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = c.tri_cluster;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelExC(
+        &cfg, c.any_periodic ? (const void *)k_triangulation_cl<true> : (const void *)k_triangulation_cl<false>, args);
+  }
   const void *fn = c.any_periodic ? (const void *)k_triangulation<true> : (const void *)k_triangulation<false>;
   return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(block), args, 0, s);
 }
