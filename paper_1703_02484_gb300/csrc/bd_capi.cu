@@ -125,6 +125,19 @@ int validate(const bd_params *p) {
   return BD_OK;
 }
 
+// Screens of a displacement against d > 0 in FP32 without 64-bit conversions:
+// grid units are taken in steps of 2^shift, d about 2^28 of them (an int holds
+// eight times d), and d^2 in those steps
+int screen_shift(double d, double inv_q) {
+  int e = 0;
+  frexp(d * inv_q, &e);   // d / q < 2^e
+  return std::min(62, std::max(0, e - 28));
+}
+float screen_square(double d, double inv_q, int shift) {
+  const double v = ldexp(d * inv_q, -shift);
+  return (float)(v * v);
+}
+
 double snap_host(double v, double q, double inv_q) { return nearbyint(v * inv_q) * q; }
 
 // a periodic coordinate in [0, L) on the grid (L is a multiple of q)
@@ -741,6 +754,10 @@ int build_handle(const std::vector<Spec> &specs, void *stream, bd_handle **out) 
   c.precision = p0.precision;
   c.a = a;
   c.sigma = 2.0 * a;
+  c.sigf = (float)c.sigma;
+  c.rwca2f = (float)(1.2599210498948732 * c.sigma * c.sigma);
+  c.s2h = (float)(c.sigma * c.sigma);
+  c.s2l = (float)(c.sigma * c.sigma - (double)c.s2h);
   c.q = q;
   c.inv_q = inv_q;
   c.qshift = s_shift;
@@ -809,6 +826,11 @@ int build_handle(const std::vector<Spec> &specs, void *stream, bd_handle **out) 
     B.r_cut = p.r_cut;
     B.skin = p.skin;
     B.rl2 = (p.r_cut + p.skin) * (p.r_cut + p.skin);
+    B.rc2f = (float)(p.r_cut * p.r_cut);
+    B.epsf = (float)p.eps;
+    B.kapf = (float)p.kappa;
+    B.vl_shift = screen_shift(0.5 * p.skin, inv_q);
+    B.vl_thr = screen_square(0.5 * p.skin, inv_q, B.vl_shift);
     rep_set_alpha(B, p.alpha, p.n_species);
     B.seed = p.seed;
     B.replica = (unsigned)p.replica;

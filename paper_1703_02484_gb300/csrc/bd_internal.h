@@ -120,6 +120,9 @@ struct BdRep {
   long long LQ;
   double dt, amp, amp_r, v0;
   double eps, kappa, r_cut, skin, rl2, cell_size;
+  float rc2f, epsf, kapf;         // r_cut^2, eps, kappa rounded to FP32
+  int vl_shift;                   // Verlet trigger: displacements in steps of 2^vl_shift of the grid,
+  float vl_thr;                   //   and (skin / 2)^2 in those
   double alpha_d[BD_MAX_SPECIES * BD_MAX_SPECIES];   // A[s_i][s_j] at [BD_MAX_SPECIES s_i + s_j]
   float alpha[BD_MAX_SPECIES * BD_MAX_SPECIES];
   unsigned long long seed;
@@ -215,6 +218,7 @@ struct BdConst {
   int any_periodic;        // some replica has a periodic box
   int precision, n_species;
   double a, sigma;
+  float sigf, rwca2f, s2h, s2l;   // sigma, (2^(1/6) sigma)^2, sigma^2 as a float-float pair
   double q, inv_q;
   int qshift;              // q = 2^-qshift
   // Algorithm 2's displacement sums over the triangulation edges are added as

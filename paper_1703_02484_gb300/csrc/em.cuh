@@ -46,6 +46,14 @@ __device__ __forceinline__ double2 force_sum(const BdDev &d, const BdConst &c, c
 // pattern).  The conversions used here run on the conversion pipe, whereas FP64
 // arithmetic issues at 1/64 of the FP32 rate on this part.
 
+// a float as a double, by its bits: conversions between FP32 and FP64 run on the
+// FP64 pipe (two lanes per SM)
+__device__ __forceinline__ double f64_of(float f) {
+  const unsigned u = __float_as_uint(f);
+  if ((u >> 23 & 255u) - 1u > 253u) return (double)f;   // zero, subnormal, infinity, NaN
+  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7FFFFFFFu) >> 3) + (896u << 20))), (int)(u << 29));
+}
+
 // X q as a double: exact int64 -> FP64 conversion, then 2^-s on the exponent
 __device__ __forceinline__ double grid_to_double(long long X, int s) {
   if (X == 0) return 0.0;

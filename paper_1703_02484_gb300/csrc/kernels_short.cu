@@ -107,8 +107,9 @@ __global__ void __launch_bounds__(BD_VL_THREADS) k_vl_check(BdDev d, BdConst c) 
     const double2 p = d.pos[i], r = d.vl_ref[i];
     const BdRep *R = short_rep(d, i);
     if (R && !bad) {
-      // displacement since the build in grid units (exact), screened in FP32;
-      // only a displacement within 1e-5 of skin/2 is decided in FP64
+      // displacement since the build in grid units (exact), screened in FP32
+      // in steps of 2^vl_shift of them (2^-27 of skin/2 or finer); only a
+      // displacement within 1e-5 of skin/2 is decided in FP64
       const bdpred::Grid g{c.q, c.inv_q, c.qshift};
       if (r.x > 1e29) {
         hit = true;   // never built (reference parked far away)
@@ -121,11 +122,11 @@ __global__ void __launch_bounds__(BD_VL_THREADS) k_vl_check(BdDev d, BdConst c) 
           ex = ex > h ? ex - R->LQ : (ex < -h ? ex + R->LQ : ex);
           ey = ey > h ? ey - R->LQ : (ey < -h ? ey + R->LQ : ey);
         }
-        const float fx = bdem::grid_to_float(ex, c.qshift);
-        const float fy = bdem::grid_to_float(ey, c.qshift);
+        const long long sx = ex >> R->vl_shift, sy = ey >> R->vl_shift;
+        const float fx = (float)(int)sx, fy = (float)(int)sy;
         const float d2 = __fadd_rn(__fmul_rn(fx, fx), __fmul_rn(fy, fy));
-        const float thr = (float)(0.25 * R->skin * R->skin);
-        if (d2 > thr * 1.00001f) {
+        const float thr = R->vl_thr;
+        if (sx != (int)sx || sy != (int)sy || d2 > thr * 1.00001f) {
           hit = true;
         } else if (d2 >= thr * 0.99999f) {
           double dx = dmin_image(p.x - r.x, *R), dy = dmin_image(p.y - r.y, *R);
@@ -297,11 +298,44 @@ __global__ void __launch_bounds__(BD_VL_THREADS, 4) k_vl_rebuild(BdDev d, BdCons
   bdgs::block_exit(d.ctl);
 }
 
-// short-range force over the lists; clears the rebuild flag
-// three resident blocks of 256 per SM (at most 80 registers): the gathers are
-// latency-bound, and the polydisperse branch must not cost the equal-disk
-// case its occupancy (86 registers, 2 blocks: 0.118 -> 0.174 ms at 2^20 disks)
-__global__ void __launch_bounds__(256, 3) k_force_verlet(BdDev d, BdConst c) {
+// r_i - r_j as FP32 (hi, lo) pairs: from the disks' own pairs, exact for near
+// pairs; a pair across a periodic box edge is formed exactly in grid units from
+// the FP64 masters instead (its hi parts differ by ~L)
+__device__ __forceinline__ void pair_diff(const BdDev &d, const BdConst &c, const BdRep &R, int i, int j,
+                                          const float4 &wi, const float4 &wj, float &hx, float &lx, float &hy,
+                                          float &ly) {
+  hx = __fsub_rn(wi.x, wj.x);
+  hy = __fsub_rn(wi.y, wj.y);
+  lx = __fsub_rn(wi.z, wj.z);
+  ly = __fsub_rn(wi.w, wj.w);
+  if (R.periodic && (fabsf(hx) > R.hLf || fabsf(hy) > R.hLf)) {
+    const bdpred::Grid g{c.q, c.inv_q, c.qshift};
+    const double2 pi = d.pos[i], pj = d.pos[j];
+    long long X = bdpred::to_int(pi.x, g) - bdpred::to_int(pj.x, g);
+    long long Y = bdpred::to_int(pi.y, g) - bdpred::to_int(pj.y, g);
+    const long long h = R.LQ / 2;
+    X = X > h ? X - R.LQ : (X < -h ? X + R.LQ : X);
+    Y = Y > h ? Y - R.LQ : (Y < -h ? Y + R.LQ : Y);
+    const float2 sx = bdem::grid_split(X, c.qshift), sy = bdem::grid_split(Y, c.qshift);
+    hx = sx.x; lx = sx.y;
+    hy = sy.x; ly = sy.y;
+  }
+}
+
+// short-range force over the lists; clears the rebuild flag.
+// Two passes over a disk's list.  The first adds the Yukawa tail of every entry
+// within the cut-off and marks those inside the WCA core in a bit mask (a list
+// holds at most 64); the second walks the mask and adds the float-float core,
+// some 150 instructions for the two or three contacts of a disk.  In one pass a
+// warp ran the core for nearly every list position, since at each one some lane
+// of the 32 had a contact there.  The sums take the same terms in the same
+// order.  Four resident blocks of 256 per SM (64 registers, without spills now): the
+// gathers want the warps, and the polydisperse branch must not cost the
+// equal-disk case its occupancy.  The law's constants come rounded from the
+// host and the result is widened by its bits: formed here, their dozen FP64
+// products and conversions a disk kept the FP64 pipe (two lanes per SM) busy for
+// 59 % of the kernel's time.
+__global__ void __launch_bounds__(256, 4) k_force_verlet(BdDev d, BdConst c) {
   if (failed(d.ctl)) return;
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i == 0) {
@@ -316,22 +350,19 @@ __global__ void __launch_bounds__(256, 3) k_force_verlet(BdDev d, BdConst c) {
   const BdRep &R = *Rp;
   const float4 wi = d.work[i];
   const int m = d.vl_cnt[i];
-  const float rc2 = (float)(R.r_cut * R.r_cut);
-  const float eps = (float)R.eps, kap = (float)R.kappa;
+  const float rc2 = R.rc2f;
+  const float eps = R.epsf, kap = R.kapf;
   // the law's length scale s: 2a, or a_i + a_j for polydisperse disks (then
   // formed per pair from the radii's FP32 (hi, lo) pairs, exact to ~2^-48)
   const bool poly = d.radf != nullptr;
   const float2 ai = poly ? d.radf[i] : make_float2(0.f, 0.f);
-  const float sg0 = (float)c.sigma;
-  const float rwca20 = (float)(1.2599210498948732 * c.sigma * c.sigma);  // (2^(1/6) s)^2
-  const float s2h0 = (float)(c.sigma * c.sigma);
-  const float s2l0 = (float)(c.sigma * c.sigma - (double)s2h0);
+  const float sg0 = c.sigf;
+  const float rwca20 = c.rwca2f;   // (2^(1/6) s)^2
   float fx = 0.f, fy = 0.f;      // Yukawa tail, FP32
-  ff gx = {0.f, 0.f}, gy = {0.f, 0.f};   // WCA core, float-float sums
+  unsigned long long core = 0ull;
   // four list entries at a time: their position gathers are issued before
   // any of them is used, and the next four indices are loaded while these
-  // are evaluated (the loop is bound by the latency of these dependent loads,
-  // not by arithmetic)
+  // are evaluated
   int jn[4];
 #pragma unroll
   for (int u = 0; u < 4; ++u) jn[u] = u < m ? d.vl_idx[(size_t)u * c.np + i] : i;
@@ -348,36 +379,17 @@ __global__ void __launch_bounds__(256, 3) k_force_verlet(BdDev d, BdConst c) {
     for (int u = 0; u < 4; ++u) {
       if (t0 + u >= m) break;
       const int j = jj[u];
-      const float4 wj = wv[u];
-      // r_i - r_j as an FP32 (hi, lo) pair: from the disks' own pairs, exact
-      // for near pairs; a pair across a periodic box edge is formed exactly in
-      // grid units from the FP64 masters instead (its hi parts differ by ~L)
-      float hx = __fsub_rn(wi.x, wj.x), hy = __fsub_rn(wi.y, wj.y);
-      float lx = __fsub_rn(wi.z, wj.z), ly = __fsub_rn(wi.w, wj.w);
-      if (R.periodic && (fabsf(hx) > R.hLf || fabsf(hy) > R.hLf)) {
-        const bdpred::Grid g{c.q, c.inv_q, c.qshift};
-        const double2 pi = d.pos[i], pj = d.pos[j];
-        long long X = bdpred::to_int(pi.x, g) - bdpred::to_int(pj.x, g);
-        long long Y = bdpred::to_int(pi.y, g) - bdpred::to_int(pj.y, g);
-        const long long h = R.LQ / 2;
-        X = X > h ? X - R.LQ : (X < -h ? X + R.LQ : X);
-        Y = Y > h ? Y - R.LQ : (Y < -h ? Y + R.LQ : Y);
-        const float2 sx = bdem::grid_split(X, c.qshift), sy = bdem::grid_split(Y, c.qshift);
-        hx = sx.x; lx = sx.y;
-        hy = sy.x; ly = sy.y;
-      }
+      float hx, lx, hy, ly;
+      pair_diff(d, c, R, i, j, wi, wv[u], hx, lx, hy, ly);
       const float dx = __fadd_rn(hx, lx);
       const float dy = __fadd_rn(hy, ly);
       const float r2 = __fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy));
-      float sg = sg0, rwca2 = rwca20, s2h = s2h0, s2l = s2l0;
+      float sg = sg0, rwca2 = rwca20;
       if (poly) {
         const float2 aj = d.radf[j];
         const ff sp = ff_add(ff_make(ai.x, ai.y), ff_make(aj.x, aj.y));
-        const ff sq = ff_mul(sp, sp);
         sg = sp.hi;
-        rwca2 = 1.2599210498948732f * sq.hi;
-        s2h = sq.hi;
-        s2l = sq.lo;
+        rwca2 = 1.2599210498948732f * ff_mul(sp, sp).hi;
       }
       if (fabsf(r2 - rc2) < 1e-5f * rc2) {
         // at the cut-off the force jumps: decide as the FP64 reference does
@@ -394,30 +406,44 @@ __global__ void __launch_bounds__(256, 3) k_force_verlet(BdDev d, BdConst c) {
       const float my = -eps * sg * __expf(-kap * (r - sg)) * (ir * ir + kap * ir) * ir;
       fx = fmaf(my, dx, fx);
       fy = fmaf(my, dy, fy);
-      if (r2 < rwca2) {
-        // WCA core near contact: -U'(r) ~ r^-13 turns FP32 rounding into
-        // errors above 1e-5 of the net force, so the core is evaluated in
-        // float-float arithmetic (FP32 instructions, ~48-bit significands) from
-        // the exact coordinate differences
-        ff ex = ff_make(hx, lx);
-        ff ey = ff_make(hy, ly);
-        ff q2 = ff_add(ff_mul(ex, ex), ff_mul(ey, ey));
-        // 1 / r^2 once (one fast reciprocal, one residual step), then products
-        const ff iq2 = ff_div_r({1.0f, 0.f}, q2, __fdividef(1.0f, q2.hi));
-        ff s2 = ff_mul({s2h, s2l}, iq2);   // (s / r)^2 as a float-float pair
-        ff s6 = ff_mul(ff_mul(s2, s2), s2);
-        ff s12 = ff_mul(s6, s6);
-        ff t = ff_add({2.0f * s12.hi, 2.0f * s12.lo}, {-s6.hi, -s6.lo});   // exact doubling
-        ff cw = ff_mul(ff_scale(t, 24.0f * eps), iq2);
-        gx = ff_add(gx, ff_mul(cw, ex));
-        gy = ff_add(gy, ff_mul(cw, ey));
-      }
+      if (r2 < rwca2) core |= 1ull << (t0 + u);
     }
+  }
+  // WCA core near contact: -U'(r) ~ r^-13 turns FP32 rounding into errors above
+  // 1e-5 of the net force, so the core is evaluated in float-float arithmetic
+  // (FP32 instructions, ~48-bit significands) from the exact coordinate differences
+  ff gx = {0.f, 0.f}, gy = {0.f, 0.f};
+  float s2h = c.s2h, s2l = c.s2l;   // s^2 as a float-float pair
+  while (core) {
+    const int t = __ffsll((long long)core) - 1;
+    core &= core - 1ull;
+    const int j = d.vl_idx[(size_t)t * c.np + i];
+    float hx, lx, hy, ly;
+    pair_diff(d, c, R, i, j, wi, d.work[j], hx, lx, hy, ly);
+    if (poly) {
+      const float2 aj = d.radf[j];
+      const ff sp = ff_add(ff_make(ai.x, ai.y), ff_make(aj.x, aj.y));
+      const ff sq = ff_mul(sp, sp);
+      s2h = sq.hi;
+      s2l = sq.lo;
+    }
+    ff ex = ff_make(hx, lx);
+    ff ey = ff_make(hy, ly);
+    ff q2 = ff_add(ff_mul(ex, ex), ff_mul(ey, ey));
+    // 1 / r^2 once (one fast reciprocal, one residual step), then products
+    const ff iq2 = ff_div_r({1.0f, 0.f}, q2, __fdividef(1.0f, q2.hi));
+    ff s2 = ff_mul({s2h, s2l}, iq2);   // (s / r)^2 as a float-float pair
+    ff s6 = ff_mul(ff_mul(s2, s2), s2);
+    ff s12 = ff_mul(s6, s6);
+    ff t2 = ff_add({2.0f * s12.hi, 2.0f * s12.lo}, {-s6.hi, -s6.lo});   // exact doubling
+    ff cw = ff_mul(ff_scale(t2, 24.0f * eps), iq2);
+    gx = ff_add(gx, ff_mul(cw, ex));
+    gy = ff_add(gy, ff_mul(cw, ey));
   }
   // the float-float total, rounded once to FP32 (the move reads the force in
   // FP32), stored as a double without FP64 arithmetic
   const ff tx = ff_add(gx, {fx, 0.f}), ty = ff_add(gy, {fy, 0.f});
-  d.fpart[i] = make_double2((double)tx.hi, (double)ty.hi);
+  d.fpart[i] = make_double2(bdem::f64_of(tx.hi), bdem::f64_of(ty.hi));
 }
 
 int bd_vl_grid_for(int np, int *grid) {
