@@ -798,6 +798,10 @@ int build_handle(const std::vector<Spec> &specs, void *stream, bd_handle **out) 
     double reach = 1e300;
     for (const Spec &sp : specs) reach = std::min(reach, 0.5 * (sp.p.r_cut + sp.p.skin - 2.0 * sp.p.a));
     c.vl_reach2 = c.overlap_verlet ? reach * reach * (1.0 - 1e-9) : 0.0;
+    if (c.overlap_verlet) {
+      c.vl_rshift = screen_shift(reach, inv_q);
+      c.vl_reach2f = screen_square(reach, inv_q, c.vl_rshift);
+    }
   }
   c.max_flip_rounds = p0.max_flip_rounds;
   c.force_variant = 1;
@@ -984,6 +988,8 @@ int build_handle(const std::vector<Spec> &specs, void *stream, bd_handle **out) 
     if (c.overlap_verlet) {
       BD_TRY(dalloc(h, &d.vc_hit, (size_t)np));
       BD_TRY(cudaMemsetAsync(d.vc_hit, 0, (size_t)np, h->stream));
+      BD_TRY(dalloc(h, &d.vc_near, (size_t)np));
+      BD_TRY(cudaMemsetAsync(d.vc_near, 0, (size_t)np, h->stream));
     }
     h->max_halvings = specs[0].p.max_dt_halvings;
     if (h->max_halvings > 0) {

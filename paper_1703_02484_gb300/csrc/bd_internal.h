@@ -198,7 +198,8 @@ struct BdDev {
   int *vl_idx, *vl_cnt;
   double2 *vl_ref;
   int *cell_count, *cell_start, *cell_cursor, *cell_idx, *cell_of, *scan_sums;
-  uint8_t *vc_hit;         // Verlet-list overlap correction: the disk overlapped in the last pass
+  uint8_t *vc_hit;         // Verlet-list overlap correction: the disk overlapped in the last scan
+  uint8_t *vc_near;        //   the last correction pass in which a disk of its list moved (near_stamp)
   // rollout log for the adjoint (null when not recording)
   uint8_t *log_refl;       // [step][np] wall-reflection flags of the Euler-Maruyama move
   uint8_t *log_pflags;     // [pass][np] bit 16: capped; bits 1,2,4,8: reflections of the pass
@@ -244,6 +245,8 @@ struct BdConst {
   int vl_grid;             // blocks of the Verlet-list rebuild launch
   double vl_reach2;        // squared displacement since the list build below which the lists
                            // still hold every pair closer than sigma
+  int vl_rshift;           // the same in steps of 2^vl_rshift of the grid, FP32 (the screen)
+  float vl_reach2f;
   int log_pairs_cap, log_pass_cap;   // rollout log capacities
 };
 

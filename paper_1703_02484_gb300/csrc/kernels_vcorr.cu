@@ -12,7 +12,8 @@
 // previous pass keeps its distance, and was not overlapping then (every disk of
 // an overlapping pair is flagged as moved, even when its displacements
 // cancel).  So after the first pass (every disk moved by the integrator) only
-// entries with a moved end are examined.  An FP32 screen of the squared
+// entries with a moved end are examined, and only by the disks that moved or
+// that a moved disk marked from its own list.  An FP32 screen of the squared
 // distance (from the FP32 (hi, lo) position pairs, margin 1e-5) discards clearly
 // separated pairs; the decision r < sigma itself is FP64, as in the oracle.
 //
@@ -54,6 +55,10 @@ __device__ __forceinline__ long long imin_image(long long d, const BdRep &R) {
   return d > h ? d - R.LQ : (d < -h ? d + R.LQ : d);
 }
 
+// mark of the disks near one that moved in correction pass k (a stale mark of
+// another pass that happens to match only adds work)
+__device__ __forceinline__ uint8_t near_stamp(int k) { return (uint8_t)(1 + (k & 127)); }
+
 // lead thread only: charge the time since the last mark to a stage
 __device__ __forceinline__ void stage_tick(BdCtl *ctl, int stage, unsigned long long &mark) {
   const unsigned long long now = gtimer();
@@ -92,17 +97,30 @@ __global__ void __launch_bounds__(BD_VC_THREADS) k_overlap_verlet(BdDev d, BdCon
     {
       int nov = 0, stale = 0;
       double mx = 0.0;
+      const uint8_t near = near_stamp(corr_iter);   // the pass before marked with it
       for (int i = tid; i < c.np; i += nth) {
-        if (d.ext_id[i] < 0) continue;
         const bool mi = d.moved[i] != 0;
+        // after the first scan only moved disks and those with a moved disk in
+        // their list have anything to do (the others' sums are 0 already)
+        if (corr_iter > 0 && !mi && d.vc_near[i] != near) continue;
+        if (d.ext_id[i] < 0) continue;
         const double2 pi = d.pos[i];
         const BdRep &R = d.rep[d.rep_of[i]];
         const bdpred::Grid g{c.q, c.inv_q, c.qshift};
         if (mi) {
           const double2 r0 = d.vl_ref[i];
-          const double ex = bdem::grid_to_double(imin_image(bdpred::to_int(pi.x, g) - bdpred::to_int(r0.x, g), R), c.qshift);
-          const double ey = bdem::grid_to_double(imin_image(bdpred::to_int(pi.y, g) - bdpred::to_int(r0.y, g), R), c.qshift);
-          if (__dadd_rn(__dmul_rn(ex, ex), __dmul_rn(ey, ey)) > c.vl_reach2) {
+          const long long ix = imin_image(bdpred::to_int(pi.x, g) - bdpred::to_int(r0.x, g), R);
+          const long long iy = imin_image(bdpred::to_int(pi.y, g) - bdpred::to_int(r0.y, g), R);
+          // screened in FP32 as the rebuild trigger is, decided in FP64 near the reach
+          const long long sx2 = ix >> c.vl_rshift, sy2 = iy >> c.vl_rshift;
+          const float hx = (float)(int)sx2, hy = (float)(int)sy2;
+          const float h2 = __fadd_rn(__fmul_rn(hx, hx), __fmul_rn(hy, hy));
+          bool beyond = sx2 != (int)sx2 || sy2 != (int)sy2 || h2 > c.vl_reach2f * 1.00001f;
+          if (!beyond && h2 >= c.vl_reach2f * 0.99999f) {
+            const double ex = bdem::grid_to_double(ix, c.qshift), ey = bdem::grid_to_double(iy, c.qshift);
+            beyond = __dadd_rn(__dmul_rn(ex, ex), __dmul_rn(ey, ey)) > c.vl_reach2;
+          }
+          if (beyond) {
             ++stale;
             atomicExch(&ctl->st_fail_item, i);
           }
@@ -111,25 +129,45 @@ __global__ void __launch_bounds__(BD_VC_THREADS) k_overlap_verlet(BdDev d, BdCon
         const int m = d.vl_cnt[i];
         double sx = 0.0, sy = 0.0;
         uint8_t hit = 0;
-        for (int t = 0; t < m; ++t) {
-          const int j = d.vl_idx[(size_t)t * c.np + i];
-          if (!mi && !d.moved[j]) continue;   // neither end moved since the last pass
-          const float4 wj = d.work[j];
-          const float fx = fdiff_p(wj.x, wj.z, wi.x, wi.z, R), fy = fdiff_p(wj.y, wj.w, wi.y, wi.w, R);
-          if (__fadd_rn(__fmul_rn(fx, fx), __fmul_rn(fy, fy)) > sig2f) continue;
-          const double2 pj = d.pos[j];
-          // the exact difference (grid units), its minimum image in a periodic box
-          const double dx = bdem::grid_to_double(imin_image(bdpred::to_int(pj.x, g) - bdpred::to_int(pi.x, g), R), c.qshift);
-          const double dy = bdem::grid_to_double(imin_image(bdpred::to_int(pj.y, g) - bdpred::to_int(pi.y, g), R), c.qshift);
-          const double r = sqrt(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)));
-          const double sg = d.rad ? d.rad[i] + d.rad[j] : sigma;   // polydisperse: a_i + a_j
-          if (r < sg) {
-            const double del = sg - r;
-            sx -= del * (dx / r);
-            sy -= del * (dy / r);
-            hit = 1;
-            if (j > i) ++nov;      // each pair counted once
-            mx = fmax(mx, del);
+        // four entries at a time: their positions (and moved flags) are loaded
+        // together, and the next four indices while they are tested
+        int jn[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) jn[u] = u < m ? d.vl_idx[(size_t)u * c.np + i] : i;
+        for (int t0 = 0; t0 < m; t0 += 4) {
+          int jj[4];
+          float4 wv[4];
+          bool mv[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) jj[u] = jn[u];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            wv[u] = d.work[jj[u]];
+            mv[u] = mi || d.moved[jj[u]] != 0;
+          }
+#pragma unroll
+          for (int u = 0; u < 4; ++u) jn[u] = t0 + 4 + u < m ? d.vl_idx[(size_t)(t0 + 4 + u) * c.np + i] : i;
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            if (t0 + u >= m) break;
+            if (!mv[u]) continue;   // neither end moved since the last pass
+            const int j = jj[u];
+            const float fx = fdiff_p(wv[u].x, wv[u].z, wi.x, wi.z, R), fy = fdiff_p(wv[u].y, wv[u].w, wi.y, wi.w, R);
+            if (__fadd_rn(__fmul_rn(fx, fx), __fmul_rn(fy, fy)) > sig2f) continue;
+            const double2 pj = d.pos[j];
+            // the exact difference (grid units), its minimum image in a periodic box
+            const double dx = bdem::grid_to_double(imin_image(bdpred::to_int(pj.x, g) - bdpred::to_int(pi.x, g), R), c.qshift);
+            const double dy = bdem::grid_to_double(imin_image(bdpred::to_int(pj.y, g) - bdpred::to_int(pi.y, g), R), c.qshift);
+            const double r = sqrt(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)));
+            const double sg = d.rad ? d.rad[i] + d.rad[j] : sigma;   // polydisperse: a_i + a_j
+            if (r < sg) {
+              const double del = sg - r;
+              sx -= del * (dx / r);
+              sy -= del * (dy / r);
+              hit = 1;
+              if (j > i) ++nov;      // each pair counted once
+              mx = fmax(mx, del);
+            }
           }
         }
         d.disp[i] = make_double2(sx, sy);
@@ -169,9 +207,19 @@ __global__ void __launch_bounds__(BD_VC_THREADS) k_overlap_verlet(BdDev d, BdCon
     {
       const double cap_eq = 0.25 * sigma;
       for (int i = tid; i < c.np; i += nth) {
-        if (d.ext_id[i] < 0) continue;
+        const uint8_t hit = d.vc_hit[i];   // 0 for empty slots
+        d.moved[i] = hit;
+        if (!hit) continue;   // (its sum is 0)
         const double2 dd = d.disp[i];
-        d.moved[i] = d.vc_hit[i];
+        // a disk the next scan skips keeps a sum of 0 and no hit
+        d.disp[i] = make_double2(0.0, 0.0);
+        d.vc_hit[i] = 0;
+        {
+          // the disks whose lists hold this one (the lists are symmetric)
+          const uint8_t near = near_stamp(corr_iter);
+          const int m = d.vl_cnt[i];
+          for (int t = 0; t < m; ++t) d.vc_near[d.vl_idx[(size_t)t * c.np + i]] = near;
+        }
         if (dd.x == 0.0 && dd.y == 0.0) continue;
         if (d.rep_stats) {
           // the first disk of a replica moved by this pass counts the pass
@@ -182,7 +230,6 @@ __global__ void __launch_bounds__(BD_VC_THREADS) k_overlap_verlet(BdDev d, BdCon
             atomicAdd((unsigned long long *)&d.rep_stats[3 * rr], 1ull);
         }
         const double2 p = d.pos[i];
-        d.prev[i] = p;
         const double mag = sqrt(__dadd_rn(__dmul_rn(dd.x, dd.x), __dmul_rn(dd.y, dd.y)));
         const double cap = d.rad ? 0.5 * d.rad[i] : cap_eq;   // half the disk's own radius
         const double sc = mag > cap ? cap / mag : 1.0;
@@ -215,7 +262,6 @@ __global__ void __launch_bounds__(BD_VC_THREADS) k_overlap_verlet(BdDev d, BdCon
       if (d.ext_id[i] < 0) continue;
       const double2 p0 = d.pos0[i];
       d.pos[i] = p0;
-      d.prev[i] = p0;
       d.work[i] = bdem::split(p0);
       d.theta[i] = d.theta0[i];
       d.disp[i] = make_double2(0.0, 0.0);
