@@ -49,12 +49,11 @@
 
 // device control block of the triangulation kernel
 struct BdCtl {
-  unsigned int bar_count;
+  unsigned int bar_count;          // on a 128-byte line of its own: the blocks at a barrier arrive at it
+  unsigned int pad0[31];           // and poll it
   int status;
   unsigned int exit_count;         // blocks that have left the triangulation kernel
-  unsigned int pad0[29];
-  uint4 bar_pub[8];                // on a 128-byte line of its own, which the blocks waiting at a
-                                   // barrier poll: (generation, three words of its counters) chunks
+  unsigned int pad1[30];
   unsigned long long epoch;        // flip-round counter, grows across launches
   int cnt[4][8];                   // per-phase counters, rotated every barrier
   // statistics accumulated over a bd_step call
