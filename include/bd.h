@@ -344,10 +344,9 @@ int bd_get_replica(bd_handle *h, int32_t r, double *xy, float *theta, int32_t *t
  * bd_init picks the FP32 variant and chunk size by timing the candidates on
  * the device; the environment variables BD_FORCE_VARIANT (0-3) and
  * BD_FORCE_TILES fix them (BD_NCHUNK = k: a single system's one-sided
- * sweeps split each row of tiles into k chunks).  BD_TRI_LISTS selects the
- * triangulation's check passes: 0 (default) the triangles of a list once a
- * full pass has more than four triangles per thread, 1 always lists, 2
- * always full passes. */
+ * sweeps split each row of tiles into k chunks).  BD_TRI_LISTS = 2 makes
+ * every check pass of the triangulation test every triangle (by default only
+ * the first of a move does; later ones test those near moved disks and flips). */
 int bd_get_tuning(bd_handle *h, int32_t *tiles_per_item, int32_t *variant, int32_t *n_items);
 
 /* Copy the current state to host memory ("Ensure P updated to current
@@ -428,8 +427,8 @@ int64_t bd_last_launch_count(bd_handle *h);
  * its stages (Sec. 6): ms[0] the validity check / Lawson marks / overlap scan
  * passes (Sec. 4.3-4.4), ms[1] inversion repair (Sec. 4.3), ms[2] Lawson flip
  * rounds, ms[3] applying the capped corrections (Algorithm 2), ms[4] the part
- * of ms[0] spent in check passes that visit only a list of triangles; each
- * stage's work plus its closing grid barrier, measured on the device clock.
+ * of ms[0] spent in check passes that test only the triangles near moved disks
+ * and flips; each stage's work plus its closing grid barrier, measured on the device clock.
  * phases[k] counts the stage's passes.  ms and phases hold 5 entries; either
  * may be NULL; reset = 1 clears the totals after reading.  The force and
  * integration kernels are separate launches (bd_force_timing covers the

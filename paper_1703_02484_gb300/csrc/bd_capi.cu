@@ -754,6 +754,7 @@ int build_handle(const std::vector<Spec> &specs, void *stream, bd_handle **out) 
   c.precision = p0.precision;
   c.a = a;
   c.sigma = 2.0 * a;
+  c.sig2f = (float)(c.sigma * c.sigma * (1.0 + 1e-5));
   c.sigf = (float)c.sigma;
   c.rwca2f = (float)(1.2599210498948732 * c.sigma * c.sigma);
   c.s2h = (float)(c.sigma * c.sigma);
@@ -788,7 +789,7 @@ int build_handle(const std::vector<Spec> &specs, void *stream, bd_handle **out) 
   c.overlap_verlet = p0.overlap_mode == BD_OVERLAP_VERLET ? 1 : 0;
   {
     const char *tl = getenv("BD_TRI_LISTS");
-    c.tri_lists = tl ? std::min(2, std::max(0, atoi(tl))) : 0;
+    c.tri_all = tl && atoi(tl) == 2 ? 1 : 0;
     const char *tf = getenv("BD_TRI_FUSE");
     c.tri_fuse = tf ? (atoi(tf) != 0 ? 1 : 0) : 1;
   }
@@ -900,6 +901,8 @@ int build_handle(const std::vector<Spec> &specs, void *stream, bd_handle **out) 
       BD_TRY(cudaMemsetAsync(d.wrap, 0, (size_t)np, h->stream));
     }
     BD_TRY(dalloc(h, &d.disp, (size_t)np));
+    BD_TRY(dalloc(h, &d.hit, (size_t)np));
+    BD_TRY(cudaMemsetAsync(d.hit, 0, (size_t)np, h->stream));
     d.rad = nullptr;
     d.radf = nullptr;
     d.wall = nullptr;
@@ -945,9 +948,6 @@ int build_handle(const std::vector<Spec> &specs, void *stream, bd_handle **out) 
     BD_TRY(cudaMemsetAsync(d.clmark, 0, (size_t)nt * sizeof(unsigned), h->stream));
     BD_TRY(cudaMemsetAsync(d.tinv, 0, (size_t)nt, h->stream));
     BD_TRY(dalloc(h, &d.vt, nv));
-    BD_TRY(dalloc(h, &d.act, 3 * (size_t)nt));
-    BD_TRY(dalloc(h, &d.act_mark, 3 * (size_t)nt));
-    BD_TRY(cudaMemsetAsync(d.act_mark, 0, 3 * (size_t)nt * sizeof(unsigned), h->stream));
     BD_TRY(dalloc(h, &d.iperm, (size_t)std::max(1, h->np_i)));
     BD_TRY(dalloc(h, &d.iorigin, (size_t)std::max(1, iblock)));
     BD_TRY(dalloc(h, &d.tile_species, std::max<size_t>(1, tile_sp.size())));
@@ -1133,7 +1133,7 @@ int build_handle(const std::vector<Spec> &specs, void *stream, bd_handle **out) 
       }
     }
     c.tri_cluster = c.overlap_verlet ? 0 : bd_dt_cluster_for(nt);
-    if (bd_dt_grid_for(std::max(nt, np), &h->dt_grid, &h->dt_block) != 0 ||
+    if (bd_dt_grid_for(std::max(3 * (long long)nt, (long long)np), &h->dt_grid, &h->dt_block) != 0 ||
         (c.any_short && bd_vl_grid_for(np, &c.vl_grid) != 0) ||
         (c.overlap_verlet && bd_vcorr_grid_for(np, &h->vc_grid, &h->vc_block) != 0)) {
       bd_free(h);

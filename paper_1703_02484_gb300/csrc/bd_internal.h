@@ -93,9 +93,8 @@ struct BdCtl {
                                    // by the triangulation kernel's shift pass; not a statistic)
   int in_move;                     // positions have moved and their correction has not finished: what a
                                    // timed-out barrier has to undo (set by the mover, cleared by the corrector)
-  int act_n[3];                    // lengths of the rotating triangle lists (zeroed at kernel exit)
   int cl_n[3];                     // lengths of the candidate lists (zeroed at kernel exit)
-  unsigned act_gen;                // next list generation (grows across launches)
+  unsigned act_gen;                // next check-pass generation (grows across launches)
   // set by the host (bd_set_wait_limit), kept across calls: the time limit of a
   // grid barrier wait (0 = BD_BARRIER_TIMEOUT_NS) and, for tests of the
   // timeout path, the generation of the barrier (1 = the first of a launch) that
@@ -106,7 +105,7 @@ struct BdCtl {
 };
 
 // counter slots within BdCtl::cnt[phase % 4]
-enum { C_INV = 0, C_REJECT = 1, C_FLIPS = 2, C_OVERLAP = 3, C_CAND = 4, C_LOSE = 5, C_OVADJ = 6 };
+enum { C_INV = 0, C_REJECT = 1, C_FLIPS = 2, C_OVERLAP = 3, C_CAND = 4, C_LOSE = 5, C_OVADJ = 6, C_VISIT = 7 };
 
 // Per-replica parameters (a handle advances R >= 1 independent systems; a
 // single system is R = 1).  Device-resident table read by the kernels.
@@ -153,6 +152,7 @@ struct BdDev {
                                   // unique to the pass: never repeats within a handle's life)
   uint8_t *wrap;           // periodic box: re-entries of the last move (bits 0-1 x, 2-3 y; 1 = -L, 3 = +L)
   double2 *disp;
+  uint8_t *hit;            // the disk may have a displacement sum that is not 0
   // polydisperse disks (null when every disk has radius a): per slot its
   // radius and its wall bounds (lo, hi) on the position grid
   double *rad;
@@ -176,8 +176,6 @@ struct BdDev {
   uint8_t *tinv;
   int *clist;
   unsigned *clmark;        // per triangle: the epoch of the candidate list it last joined
-  int *act;                // 3 x nt: rotating lists of the triangles a check pass visits
-  unsigned *act_mark;      // 3 x nt: generation at which a triangle joined each list
   // force sweep
   int *iperm;              // spatial order of i per block (np_i slots, -1 = none)
   float2 *iorigin;         // per i-block origin (integers)
@@ -218,6 +216,7 @@ struct BdConst {
   int any_periodic;        // some replica has a periodic box
   int precision, n_species;
   double a, sigma;
+  float sig2f;                    // sigma^2 (1 + 1e-5): FP32 screen of the overlap scans
   float sigf, rwca2f, s2h, s2l;   // sigma, (2^(1/6) sigma)^2, sigma^2 as a float-float pair
   double q, inv_q;
   int qshift;              // q = 2^-qshift
@@ -234,9 +233,8 @@ struct BdConst {
   int n_sitems;            // symmetric sweep work items
   int f64_sym;             // precision 1: the symmetric FP64 sweep (its items in the symmetric tables)
   int overlap_verlet;      // 1: Algorithm 2 over the Verlet lists, no triangulation kept
-  int tri_lists;           // check passes after the first of a move: 0 lists when a full pass
-                           // is throughput-bound (many triangles per thread), 1 always lists,
-                           // 2 always full (environment variable BD_TRI_LISTS at init)
+  int tri_all;             // 1: every check pass tests every triangle, not only the first of a move
+                           // (environment variable BD_TRI_LISTS=2 at init)
   int tri_fuse;            // 1: a Lawson round tests the outer edges of its flips and keeps the
                            // overlap sums (no check pass between rounds); 0: a check pass after
                            // every round (environment variable BD_TRI_FUSE at init)
@@ -260,7 +258,9 @@ cudaError_t bd_launch_integrate(const BdDev &d, const BdConst &c, int64_t step, 
 cudaError_t bd_launch_dt(const BdDev &d, const BdConst &c, int mode, cudaStream_t s, int grid, int block,
                          int log_step = -1);
 int bd_dt_grid(int *grid, int *block);
-int bd_dt_grid_for(int work_items, int *grid, int *block);
+int bd_dt_grid_for(long long work_items, int *grid, int *block);
+// whether the check passes of nt triangles run through the warps' queues
+int bd_dt_queue_for(int nt, int grid, int block);
 // blocks of the one cluster that serves a triangulation of nt triangles (0: the grid does)
 int bd_dt_cluster_for(int nt);
 int bd_force_blocks_per_sm(int variant);

@@ -34,12 +34,11 @@ __device__ __forceinline__ int ld_status(const int *p) {
 // Words every thread needs after a barrier, read once per block by thread 0
 // and handed to the block through shared memory (116k threads reading one
 // global line would queue ~18k requests on one L2 slice per barrier).
-enum { BC_CNT = 0, BC_ACT = 8, BC_CL = 11, BC_N = 14 };
+enum { BC_CNT = 0, BC_CL = 8, BC_N = 11 };
 
 // Bounded grid barrier; returns false if the grid must stop.  With bc (block
 // shared, BC_N ints): bc[BC_CNT + k] = the counters of the phase that just
-// ended, bc[BC_ACT + l] = the lengths of the triangle lists, bc[BC_CL + l]
-// those of the candidate lists.  HOLD: the barrier obeys the host's test hold
+// ended, bc[BC_CL + l] = the lengths of the candidate lists.  HOLD: the barrier obeys the host's test hold
 // (the kernels of a move do; the Verlet-list rebuild does not).
 //
 // A barrier is its chain of L2 round trips, kept to three: the arrival, the
@@ -89,9 +88,8 @@ static __device__ bool grid_sync(BdCtl *ctl, Bar &b, int *bc = nullptr) {
     }
     __syncwarp();
     if (bc && lane < BC_N)
-      bc[lane] = lane < BC_ACT ? ((const volatile int *)ctl->cnt[b.ph & 3])[lane]
-                               : (lane < BC_CL ? ((const volatile int *)ctl->act_n)[lane - BC_ACT]
-                                               : ((const volatile int *)ctl->cl_n)[lane - BC_CL]);
+      bc[lane] = lane < BC_CL ? ((const volatile int *)ctl->cnt[b.ph & 3])[lane]
+                              : ((const volatile int *)ctl->cl_n)[lane - BC_CL];
   }
   __syncthreads();
   b.gen++;
@@ -111,7 +109,7 @@ static __device__ void block_exit(BdCtl *ctl) {
     unsigned k = atomicAdd(&ctl->exit_count, 1u);
     if (k == gridDim.x - 1) {
       ctl->bar_count = 0;
-      for (int l = 0; l < 3; ++l) ctl->act_n[l] = ctl->cl_n[l] = 0;
+      for (int l = 0; l < 3; ++l) ctl->cl_n[l] = 0;
       for (int a = 0; a < 4; ++a)
         for (int b = 0; b < 8; ++b) ctl->cnt[a][b] = 0;
       __threadfence();
@@ -125,7 +123,7 @@ static __device__ void block_exit(BdCtl *ctl) {
 // hardware's, and the phase counters and list lengths sit in the first block's
 // shared memory (words: BW_N ints there, reached by every block of the
 // cluster), so that a phase ends without a round trip through L2.
-enum { BW_CNT = 0, BW_ACT = 32, BW_CL = 35, BW_N = 38 };
+enum { BW_CNT = 0, BW_CL = 32, BW_N = 35 };
 
 __device__ __forceinline__ void cluster_barrier() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -147,7 +145,7 @@ static __device__ bool cluster_sync(BdCtl *ctl, const int *words, unsigned hold,
   }
   if (threadIdx.x < BC_N) {
     const int k = threadIdx.x;
-    const int at = k < BC_ACT ? BW_CNT + 8 * (b.ph & 3) + k : (k < BC_CL ? BW_ACT + k - BC_ACT : BW_CL + k - BC_CL);
+    const int at = k < BC_CL ? BW_CNT + 8 * (b.ph & 3) + k : BW_CL + k - BC_CL;
     bc[k] = ((const volatile int *)words)[at];
   }
   __syncthreads();

@@ -54,6 +54,7 @@
 #include "predicates.cuh"
 
 #define BD_DT_THREADS 256
+#define BD_DT_LIST 2048       // triangles a block looks over at a time for the dirty ones
 #define BD_DTC_THREADS 512   // threads per block of the cluster form
 
 using namespace bdgs;
@@ -76,8 +77,8 @@ __device__ __forceinline__ void set_vk(int4 &v, int k, int val) {
 }
 
 struct Ctx {
-  BdDev d;
-  BdConst c;
+  const BdDev &d;     // the kernel's parameters, where they lie
+  const BdConst &c;
   bdpred::Grid g;
   int T;
   int np;
@@ -109,7 +110,11 @@ __device__ __forceinline__ float fdiff(float bh, float bl, float ah, float al) {
 // long; they are kept out of line, one copy each, so that a thread that needs
 // one fetches a single shared instruction stream rather than a cold inlined
 // copy at every call site (a miss in the instruction cache costs about an L2
-// round trip per line, and the slowest thread of a pass sets its length).
+// round trip per line, and the slowest thread of a pass sets its length).  For
+// the same reason the overlap of a pair and the registration of a candidate are
+// out of line, and the loops over a triangle's edges and a flip's outer edges
+// are not unrolled: in a small system a launch runs each phase's code once or
+// twice, and waiting for instructions was the largest stall after the barriers.
 __device__ __noinline__ int orient_exact(const double2 *__restrict__ pos, bdpred::Grid g, int a, int b, int c) {
   const double2 pa = pos[a], pb = pos[b], pc = pos[c];
   return bdpred::orient(pa.x, pa.y, pb.x, pb.y, pc.x, pc.y, g);
@@ -136,10 +141,12 @@ __device__ __noinline__ int incircle_lifted(long long ax, long long ay, long lon
 // after the pass) does not depend on the order the edges arrive in.  A
 // contribution is rounded to disp_unscale (a small fraction of the position
 // grid) once; zero is the same bit pattern in both readings of the words.
-__device__ __forceinline__ void disp_add(const Ctx &x, int i, double vx, double vy) {
-  long long *w = (long long *)&x.d.disp[i];
-  atomicAdd((unsigned long long *)&w[0], (unsigned long long)__double2ll_rn(__dmul_rn(vx, x.c.disp_scale)));
-  atomicAdd((unsigned long long *)&w[1], (unsigned long long)__double2ll_rn(__dmul_rn(vy, x.c.disp_scale)));
+// (A pass applies the sums of the disks marked in hit; a disk whose contributions
+// were withdrawn again keeps its mark and a sum of 0.)
+__device__ __forceinline__ void disp_add(const BdDev &d, const BdConst &c, int i, double vx, double vy) {
+  long long *w = (long long *)&d.disp[i];
+  atomicAdd((unsigned long long *)&w[0], (unsigned long long)__double2ll_rn(__dmul_rn(vx, c.disp_scale)));
+  atomicAdd((unsigned long long *)&w[1], (unsigned long long)__double2ll_rn(__dmul_rn(vy, c.disp_scale)));
 }
 __device__ __forceinline__ double2 disp_get(const Ctx &x, int i) {
   const longlong2 w = *(const longlong2 *)&x.d.disp[i];
@@ -149,23 +156,30 @@ __device__ __forceinline__ double2 disp_get(const Ctx &x, int i) {
 // Algorithm 2's overlap test of the disk pair (u, w), w's image shifted by
 // (rsx, rsy) L: an exact pre-test in grid units, |r_w - r_u|^2 <= (sigma/q)^2
 // (1 + 1e-9), then the decision r < a_u + a_w in FP64 as the reference makes
-// it (the difference of two grid values is exact in FP64).  On overlap, v is
-// the push of w, (a_u + a_w - r) (r_w - r_u) / r; u's is -v.
-__device__ __forceinline__ bool edge_overlap(const Ctx &x, int u, int w, int rsx, int rsy, long long LQ, double2 &v,
-                                             double &del) {
-  const double2 pu = x.d.pos[u], pw = x.d.pos[w];
-  const int64_t ix = bdpred::to_int(pw.x, x.g) - bdpred::to_int(pu.x, x.g) + rsx * LQ;
-  const int64_t iy = bdpred::to_int(pw.y, x.g) - bdpred::to_int(pu.y, x.g) + rsy * LQ;
+// it (the difference of two grid values is exact in FP64).  On overlap the push
+// of w, (a_u + a_w - r) (r_w - r_u) / r, and u's, the negative, are added to the
+// sums (sgn = -1: withdrawn), the disks are marked, and the depth
+// a_u + a_w - r is returned (0: no overlap).
+__device__ __noinline__ double overlap_push(const BdDev &d, const BdConst &c, int u, int w, int rsx, int rsy,
+                                            long long LQ, int sgn) {
+  const bdpred::Grid g{c.q, c.inv_q, c.qshift};
+  const double2 pu = d.pos[u], pw = d.pos[w];
+  const int64_t ix = bdpred::to_int(pw.x, g) - bdpred::to_int(pu.x, g) + rsx * LQ;
+  const int64_t iy = bdpred::to_int(pw.y, g) - bdpred::to_int(pu.y, g) + rsy * LQ;
   const bdpred::i128 ir2 = bdpred::add128(bdpred::smul64(ix, ix), bdpred::smul64(iy, iy));
-  const bool near = ir2.hi < x.c.sig2q_hi || (ir2.hi == x.c.sig2q_hi && ir2.lo <= x.c.sig2q_lo);
-  if (!near) return false;
-  const double dx = bdem::grid_to_double(ix, x.g.s), dy = bdem::grid_to_double(iy, x.g.s);
+  const bool near = ir2.hi < c.sig2q_hi || (ir2.hi == c.sig2q_hi && ir2.lo <= c.sig2q_lo);
+  if (!near) return 0.0;
+  const double dx = bdem::grid_to_double(ix, g.s), dy = bdem::grid_to_double(iy, g.s);
   const double r = sqrt(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)));
-  const double sg = x.d.rad ? x.d.rad[u] + x.d.rad[w] : x.c.sigma;   // polydisperse: a_u + a_w
-  if (!(r < sg)) return false;
-  del = sg - r;
-  v = make_double2(del * (dx / r), del * (dy / r));
-  return true;
+  const double sg = d.rad ? d.rad[u] + d.rad[w] : c.sigma;   // polydisperse: a_u + a_w
+  if (!(r < sg)) return 0.0;
+  const double del = sg - r;
+  const double vx = sgn * (del * (dx / r)), vy = sgn * (del * (dy / r));
+  disp_add(d, c, u, -vx, -vy);
+  disp_add(d, c, w, vx, vy);
+  d.hit[u] = 1;
+  d.hit[w] = 1;
+  return del;
 }
 
 // a test the FP32 filter could not decide (rare: near-degenerate inputs)
@@ -234,21 +248,19 @@ __device__ __forceinline__ int incircle_v(const Ctx &x, int a, int b, int c, int
 
 // Sec. 4.3 reversal test r0 . r1 < 0 of the edge u -> w, exact on the grid:
 // r1 from the present positions, r0 from those before the move (ox, oy: the
-// edge's image shift before the move, in units of LQ)
+// edge's image shift before the move, in units of LQ); only a disk that moved
+// (mu, mw) has its position before the move in prev (for the launch's first
+// pass, pos0)
 __device__ __noinline__ bool reversed_grid(const double2 *__restrict__ prev, const double2 *__restrict__ pos,
-                                           bdpred::Grid g, int u, int w, int ox, int oy, int rsx, int rsy,
-                                           long long LQ) {
-  const double2 a0 = prev[u], b0 = prev[w], a1 = pos[u], b1 = pos[w];
+                                           bdpred::Grid g, int u, int w, bool mu, bool mw, int ox, int oy, int rsx,
+                                           int rsy, long long LQ) {
+  const double2 a1 = pos[u], b1 = pos[w];
+  const double2 a0 = mu ? prev[u] : a1, b0 = mw ? prev[w] : b1;
   const int64_t ux = bdpred::to_int(b0.x, g) - bdpred::to_int(a0.x, g) + ox * LQ;
   const int64_t uy = bdpred::to_int(b0.y, g) - bdpred::to_int(a0.y, g) + oy * LQ;
   const int64_t vx = bdpred::to_int(b1.x, g) - bdpred::to_int(a1.x, g) + rsx * LQ;
   const int64_t vy = bdpred::to_int(b1.y, g) - bdpred::to_int(a1.y, g) + rsy * LQ;
   return bdpred::sign128(bdpred::add128(bdpred::smul64(ux, vx), bdpred::smul64(uy, vy))) < 0;
-}
-
-__device__ __forceinline__ bool reversed_exact(const Ctx &x, int u, int w, int ox, int oy, int rsx, int rsy,
-                                               long long LQ) {
-  return reversed_grid(x.d.prev, x.d.pos, x.g, u, w, ox, oy, rsx, rsy, LQ);
 }
 
 // ---- periodic box: image shifts of triangle corners (Sec. 2.1, 4.1) ----
@@ -351,10 +363,10 @@ __device__ __forceinline__ unsigned long long *claims(const Ctx &x, unsigned lon
   return x.d.claim + (size_t)(e & 1ull) * x.T;
 }
 
-__device__ __forceinline__ void claim6(const Ctx &x, unsigned long long *cb, int t, int k, const int4 &nn, int o,
+__device__ __forceinline__ void claim6(const int4 *tn, unsigned long long *cb, int t, int k, const int4 &nn, int o,
                                        unsigned long long key) {
   const int t1 = o / 3, k1 = o % 3;
-  const int4 nn1 = x.d.tn[t1];
+  const int4 nn1 = tn[t1];
   atomicMax(&cb[t], key);
   atomicMax(&cb[t1], key);
   int e[4] = {vk(nn, (k + 1) % 3), vk(nn, (k + 2) % 3), vk(nn1, (k1 + 1) % 3), vk(nn1, (k1 + 2) % 3)};
@@ -478,13 +490,21 @@ __device__ __forceinline__ int key_corner(unsigned long long key) {
   return (int)(0xFFFFFFFFu - (unsigned)(key & 0xFFFFFFFFull));
 }
 
-// Register triangle t as a candidate owner for the round of epoch e, once:
-// the marking pass and the previous fused round both register owners for a
-// round, and an owner listed twice would be flipped by two threads at once.
-__device__ __forceinline__ void push_owner(const Ctx &x, unsigned long long e, int t) {
-  if (atomicExch(&x.d.clmark[t], (unsigned)e) == (unsigned)e) return;
+// Register the edge facing corner cc (o: the corner across it) as a flip
+// candidate of the round of epoch e: its six claims (cb), and its triangle in
+// the round's list of owners -- once: the marking pass and the previous fused
+// round both register owners for a round, and an owner listed twice would be
+// flipped by two threads at once.
+__device__ __noinline__ void register_edge(const int4 *tn, unsigned long long *cb, unsigned *clmark, int *list, int *n,
+                                           unsigned long long e, int cc, int o) {
+  const int t = cc / 3;
+  claim6(tn, cb, t, cc % 3, tn[t], o, claim_key(e, cc));
+  if (atomicExch(&clmark[t], (unsigned)e) == (unsigned)e) return;
+  list[atomicAdd(n, 1)] = t;
+}
+__device__ __forceinline__ void register_edge(const Ctx &x, unsigned long long *cb, unsigned long long e, int cc, int o) {
   const int l = (int)(e % 3);
-  x.d.clist[(size_t)l * x.T + atomicAdd(&x.cl_n[l], 1)] = t;
+  register_edge(x.d.tn, cb, x.d.clmark, x.d.clist + (size_t)l * x.T, &x.cl_n[l], e, cc, o);
 }
 
 // Stamp triangle t for the check pass of generation byte s.  The word is
@@ -499,34 +519,56 @@ __device__ __forceinline__ void stamp_tri(const Ctx &x, int t, uint8_t s) {
   } while (old != seen);
 }
 
-// A fused Lawson round's flip of the edge facing corner c0 (pair and outer
-// neighbours owned).  Its loads are issued by level -- the pair and the
-// journal marks; the four outer neighbours' corner tables and the quad's
-// FP32 pairs; the opposite vertices' FP32 pairs -- before any store.  It
-// withdraws the overlap of diagonal bc, adds that of ad, flips, and tests the
-// four outer edges, registering the illegal ones (claims in nb, keys of
-// epoch ne, owners listed once).  Returns the change in overlapping edges
-// and the depth of an added overlap (0 if none).
+// A fused Lawson round's flip of the candidate that triangle t0 registered for
+// the round of epoch ce, if it holds its six claims (cb).  Its loads are issued
+// by level, before any store and before the claims have decided -- t0's claim,
+// tables and journal mark; the other triangle's, with t0's corners' FP32 pairs;
+// the four outer neighbours' claims and corner tables; the opposite vertices'
+// FP32 pairs -- since a round is as long as this chain (what a candidate that
+// lost has read of triangles others are flipping is dropped).  It withdraws the
+// overlap of diagonal bc, adds that of ad, flips, and tests the four outer
+// edges, registering the illegal ones (claims in nb, keys of epoch ce + 1, owners
+// listed once).  Returns the other triangle (-1: claims lost), the change in
+// overlapping edges and the depth of an added overlap (0 if none).
 struct FusedOut {
+  int t1;
   int adj;
   double mx;
 };
 template <bool PER>
-__device__ __forceinline__ FusedOut fused_flip(const Ctx &x, int c0, int o0, unsigned long long *nb,
-                                             unsigned long long ne) {
+__device__ __forceinline__ FusedOut fused_flip(const Ctx &x, int t0, unsigned long long ce, const unsigned long long *cb,
+                                               unsigned long long *nb) {
   const BdDev &d = x.d;
-  const int t0 = c0 / 3, k0 = c0 % 3, t1 = o0 / 3, k1 = o0 % 3;
-  const unsigned m0 = d.jmark[t0], m1 = d.jmark[t1];
-  const int4 oV0 = d.tv[t0], oV1 = d.tv[t1], oN0 = d.tn[t0], oN1 = d.tn[t1];
-  const int a = vk(oV0, k0), b = vk(oV0, (k0 + 1) % 3), c = vk(oV0, (k0 + 2) % 3), dd = vk(oV1, k1);
+  FusedOut r = {-1, 0, 0.0};
+  const unsigned long long ne = ce + 1;
+  const unsigned long long key = cb[t0];
+  const unsigned m0 = d.jmark[t0];
+  const int4 oV0 = d.tv[t0], oN0 = d.tn[t0];
+  const int c0 = key_corner(key);
+  if ((key >> 32) != ce || c0 / 3 != t0) return r;
+  const int k0 = c0 % 3, o0 = vk(oN0, k0), t1 = o0 / 3, k1 = o0 % 3;
+  const int a = vk(oV0, k0), b = vk(oV0, (k0 + 1) % 3), c = vk(oV0, (k0 + 2) % 3);
+  bool own = cb[t1] == key;
+  const unsigned m1 = d.jmark[t1];
+  const int4 oV1 = d.tv[t1], oN1 = d.tn[t1];
+  const float4 Pa = work_of(x, a), Pb = work_of(x, b), Pc = work_of(x, c);
+  const int dd = vk(oV1, k1);
   const int n_ca = vk(oN0, (k0 + 1) % 3), n_ab = vk(oN0, (k0 + 2) % 3);
   const int n_bd = vk(oN1, (k1 + 1) % 3), n_dc = vk(oN1, (k1 + 2) % 3);
   // outer edges in the order (t0, facing k0+1), (t0, k0+2), (t1, k1+1), (t1, k1+2)
   const int nbr[4] = {n_ab, n_bd, n_dc, n_ca};
   int4 Wn[4];
+  unsigned long long cn[4];
 #pragma unroll
-  for (int m = 0; m < 4; ++m) Wn[m] = nbr[m] >= 0 ? d.tv[nbr[m] / 3] : make_int4(0, 0, 0, 0);
-  const float4 Pa = work_of(x, a), Pb = work_of(x, b), Pc = work_of(x, c), Pd = work_of(x, dd);
+  for (int m = 0; m < 4; ++m) {
+    cn[m] = nbr[m] >= 0 ? cb[nbr[m] / 3] : key;
+    Wn[m] = nbr[m] >= 0 ? d.tv[nbr[m] / 3] : make_int4(0, 0, 0, 0);
+  }
+  const float4 Pd = work_of(x, dd);
+#pragma unroll
+  for (int m = 0; m < 4; ++m) own = own && cn[m] == key;
+  if (!own) return r;
+  r.t1 = t1;
   int q[4];
   float4 Pq[4];
 #pragma unroll
@@ -572,7 +614,6 @@ __device__ __forceinline__ FusedOut fused_flip(const Ctx &x, int c0, int o0, uns
   V1.w = with_stamp(nw1, tstamp(w1));
   // overlaps of the old and the new diagonal (a shifted edge takes the exact
   // test directly; a plain one is screened in FP32 first, as in a check pass)
-  FusedOut r = {0, 0.0};
   auto diag = [&](int u, int w, const float4 &Pu, const float4 &Pw, int sx, int sy, int sgn) {
     if (u >= x.np || w >= x.np) return;
     if ((sx | sy) == 0) {
@@ -580,11 +621,8 @@ __device__ __forceinline__ FusedOut fused_flip(const Ctx &x, int c0, int o0, uns
       if (__fadd_rn(__fmul_rn(fx, fx), __fmul_rn(fy, fy)) > x.sig2f) return;
     }
     const long long LQ = (sx | sy) ? rep_LQ(x, u) : 0;
-    double2 v;
-    double del;
-    if (!edge_overlap(x, u, w, sx, sy, LQ, v, del)) return;
-    disp_add(x, u, -sgn * v.x, -sgn * v.y);
-    disp_add(x, w, sgn * v.x, sgn * v.y);
+    const double del = overlap_push(d, x.c, u, w, sx, sy, LQ, sgn);
+    if (del == 0.0) return;
     r.adj += sgn;
     if (sgn > 0) r.mx = fmax(r.mx, del);
   };
@@ -609,50 +647,24 @@ __device__ __forceinline__ FusedOut fused_flip(const Ctx &x, int c0, int o0, uns
   journal(x, t1, oV1, oN1, m1);
   // the four outer edges: the opposite vertex inside the new triangle's
   // circumcircle makes the edge illegal (a candidate of the next round)
-  float4 W0[3], W1[3];
-  W0[k0] = Pb; W0[(k0 + 1) % 3] = Pd; W0[(k0 + 2) % 3] = Pa;
-  W1[k1] = Pc; W1[(k1 + 1) % 3] = Pa; W1[(k1 + 2) % 3] = Pd;
-  bool reg0 = false, reg1 = false;
-#pragma unroll
+#pragma unroll 1
   for (int m = 0; m < 4; ++m) {
     if (nbr[m] < 0) continue;
+    // t0 = (b, d, a), t1 = (c, a, d)
     const bool first = m < 2;
-    const int tt = first ? t0 : t1, kt = first ? k0 : k1;
-    const int k = (kt + 1 + (m & 1)) % 3;
-    const int4 &V = first ? V0 : V1;
-    const float4 *Wt = first ? W0 : W1;
+    const int tt = first ? t0 : t1, k = ((first ? k0 : k1) + 1 + (m & 1)) % 3;
+    const int i0 = first ? b : c, i1 = first ? dd : a, i2 = first ? a : dd;
+    const float4 P0 = first ? Pb : Pc, P1 = first ? Pd : Pa, P2 = first ? Pa : Pd;
+    const int w = first ? V0.w : V1.w;
     int sqx, sqy;
-    opp_shift<PER>(V.w, k, Wn[m].w, nbr[m] % 3, sqx, sqy);
-    const bool flat = (V.w & BD_TRI_SHIFT_BITS) == 0 && (sqx | sqy) == 0;
-    const int ic = flat ? incircle_pre(x, V.x < x.np && V.y < x.np && V.z < x.np && q[m] < x.np, Wt[0], Wt[1],
-                                       Wt[2], Pq[m], V.x, V.y, V.z, q[m])
-                        : incircle_s<PER>(x, V, q[m], sqx, sqy);
-    if (ic > 0) {
-      claim6(x, nb, tt, k, first ? N0 : N1, nbr[m], claim_key(ne, 3 * tt + k));
-      bool &reg = first ? reg0 : reg1;
-      if (!reg) {
-        reg = true;
-        push_owner(x, ne, tt);
-      }
-    }
+    opp_shift<PER>(w, k, Wn[m].w, nbr[m] % 3, sqx, sqy);
+    const bool flat = (w & BD_TRI_SHIFT_BITS) == 0 && (sqx | sqy) == 0;
+    const int ic = flat ? incircle_pre(x, i0 < x.np && i1 < x.np && i2 < x.np && q[m] < x.np, P0, P1, P2, Pq[m], i0, i1,
+                                       i2, q[m])
+                        : incircle_s<PER>(x, first ? V0 : V1, q[m], sqx, sqy);
+    if (ic > 0) register_edge(x, nb, ne, 3 * tt + k, nbr[m]);
   }
   return r;
-}
-
-// Append triangle t to a list once per generation (a list is visited by one
-// check pass; its generation tags the members).  The lanes of a warp that
-// append together reserve their slots with one atomic on the list length.
-__device__ __forceinline__ void push_tri(int *list, unsigned *mark, int *n, unsigned gen, int t) {
-  const bool add = atomicExch(&mark[t], gen) != gen;
-  const unsigned act = __activemask();
-  const unsigned want = __ballot_sync(act, add);
-  if (!want) return;
-  const int lane = threadIdx.x & 31;
-  const int leader = __ffs(want) - 1;
-  int base = 0;
-  if (lane == leader) base = atomicAdd(n, __popc(want));
-  base = __shfl_sync(act, base, leader);
-  if (add) list[base + __popc(want & ((1u << lane) - 1u))] = t;
 }
 
 // the replica of a triangle (its first disk corner; -1 if it has none)
@@ -693,15 +705,7 @@ __device__ __forceinline__ int tri_rep(const BdDev &d, int np, const int4 &v) {
 // barriers, the phase words in the first block's shared memory, 128 registers.
 template <bool PER, bool CL>
 __device__ __forceinline__ void triangulation_body(const BdDev &d, const BdConst &c, int mode, int log_step) {
-  Ctx x;
-  x.d = d;
-  x.c = c;
-  x.g.q = c.q;
-  x.g.inv_q = c.inv_q;
-  x.g.s = c.qshift;
-  x.T = c.nt;
-  x.np = c.np;
-  x.sig2f = (float)(c.sigma * c.sigma * (1.0 + 1e-5));
+  Ctx x = {d, c, {c.q, c.inv_q, c.qshift}, c.nt, c.np, c.sig2f, 0u, d.ctl->cl_n};
   BdCtl *ctl = d.ctl;
   if (ld_status(&ctl->status) != 0 || (mode == 1 && *(volatile const int *)&ctl->n_set_moved == 0)) {
     // (bd_set_state that moved no disk: the triangulation stands as it was)
@@ -715,15 +719,13 @@ __device__ __forceinline__ void triangulation_body(const BdDev &d, const BdConst
   __shared__ int bc[BC_N];                // phase counters and list lengths, per barrier
   // the phase words: in the control block, or in the cluster's first block
   __shared__ int s_words[CL ? BW_N : 1];
-  int *words = nullptr, *wcnt = &ctl->cnt[0][0], *wact = ctl->act_n;
-  x.cl_n = ctl->cl_n;
+  int *words = nullptr, *wcnt = &ctl->cnt[0][0];
   unsigned hold = 0;
   if (CL) {
     hold = *(volatile const unsigned *)&ctl->bar_hold;
     if (threadIdx.x < BW_N) s_words[threadIdx.x] = 0;
     words = cooperative_groups::this_cluster().map_shared_rank(s_words, 0);
     wcnt = words + BW_CNT;
-    wact = words + BW_ACT;
     x.cl_n = words + BW_CL;
     cluster_barrier();
   }
@@ -737,7 +739,10 @@ __device__ __forceinline__ void triangulation_body(const BdDev &d, const BdConst
     if (blockIdx.x == 0 && threadIdx.x < 8) wcnt[8 * ((b.ph + 2) & 3) + threadIdx.x] = 0;
   };
   unsigned long long t_mark = gtimer();   // stage timing (lead thread)
-  const int tid = blockIdx.x * blockDim.x + threadIdx.x;
+  // CL: a few thousand items are spread over the blocks warp by warp, so that
+  // every scheduler of the cluster's SMs has its share of them
+  const int tid = CL ? (int)(((threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31))
+                     : (int)(blockIdx.x * blockDim.x + threadIdx.x);
   const int nth = gridDim.x * blockDim.x;
   const bool lead = (blockIdx.x == 0 && threadIdx.x == 0);
   unsigned long long epoch = ctl->epoch;   // written only at kernel end by the lead thread
@@ -753,30 +758,27 @@ __device__ __forceinline__ void triangulation_body(const BdDev &d, const BdConst
   int log_head = logging ? ctl->log_npairs : 0;
   int log_npass = logging ? ctl->log_npass : 0;
   int log_pidx = -1;
-  // Check-pass domains.  The first pass of a move (and the pass after an
-  // inversion repair) visits every triangle; a later pass visits only a list:
-  // the triangles a flip touched or left dirty, those with an overlapping
-  // edge, and after a correction move the stars of the moved disks.  Every
-  // other edge kept its end points and its place in the triangulation since it
-  // was last checked, so its earlier verdicts (legal, not overlapping) stand.
-  // Lists rotate over three slots: pass kp visits slot kp % 3 (generation
-  // g0 + kp) and fills slot (kp + 1) % 3; the lead empties slot (kp + 2) % 3.
+  // Check passes.  The first pass of a move (and the pass after an inversion
+  // repair) tests every triangle; a later pass only the dirty ones: those with a
+  // corner that the last correction moved, and those stamped with the pass's
+  // generation byte (flips, flip candidates left unresolved).  Every other edge
+  // kept its end points and its place in the triangulation since it was last
+  // checked, so its earlier verdicts (legal, not overlapping) stand.  A clean
+  // triangle costs its corner table and three flags.  (Lists of the triangles
+  // to visit, kept by the flips and by walks round the moved disks, measured
+  // slower at every size: 513 against 492 us per step in a batch of 350000 disks,
+  // 378 against 373 at 2^20.)
   const unsigned g0 = *(volatile unsigned *)&ctl->act_gen;
   int kp = 0;
-  bool full = true;
-  // Lists pay off when a full pass is bound by the number of triangles per
-  // thread; with a few triangles per thread a full pass is as short as one
-  // thread's chain of dependent loads, which a list pass (an extra
-  // indirection and membership reads) only lengthens (measured: 2^20 disks,
-  // 18 triangles per thread, check stage 0.37 -> 0.30 ms per step; 10^5
-  // disks, 1.8 per thread, 0.13 -> 0.17 ms).
-  const bool use_lists = c.tri_lists == 1 || (c.tri_lists == 0 && x.T > 4 * nth);
   long long tri_visits = 0;
   // the next iteration opens with a check pass (need_p) that scans the
   // overlaps (scan); the overlapping edges of the current triangulation
   // (ov_now); Lawson rounds fused with their re-tests (not while a rollout
   // logs its pairs, which wants every pair of a pass from one scan)
   bool need_p = true, scan = true;
+  // the next pass tests every edge: the first pass of a launch, and a pass whose
+  // overlap sums start from nothing
+  bool sweep_all = true;
   int ov_now = 0;
   const bool fuse = c.tri_fuse && !logging;
 
@@ -784,16 +786,9 @@ __device__ __forceinline__ void triangulation_body(const BdDev &d, const BdConst
     ++epoch;
     if (lead) {
       x.cl_n[(epoch + 2) % 3] = 0;   // the candidate list two rounds ahead
-      wact[(kp + 2) % 3] = 0;     // the triangle list two passes ahead
     }
-    const int slot = kp % 3, nslot = (kp + 1) % 3;
     const unsigned gen = g0 + (unsigned)kp, ngen = gen + 1u;
     const uint8_t gen8 = (uint8_t)gen, ngen8 = (uint8_t)ngen;   // check-pass stamps of this pass and the next
-    const int *dom = d.act + (size_t)slot * x.T;
-    const unsigned *cmark = d.act_mark + (size_t)slot * x.T;
-    int *nlist = d.act + (size_t)nslot * x.T;
-    unsigned *nmark = d.act_mark + (size_t)nslot * x.T;
-    int *ncount = &wact[nslot];
     // ---------------- W: shifts of triangles whose corners re-entered (periodic box) ----------------
     if (PER && fresh && *(volatile int *)&ctl->n_wrapped != 0) {
       phase_start();
@@ -821,196 +816,114 @@ __device__ __forceinline__ void triangulation_body(const BdDev &d, const BdConst
     // change; a pass that follows such rounds only marks, scan = false, since
     // the rounds keep the overlap sums of the triangulation they leave)
     int n_ov = 0;
-    const int dom_n = full ? x.T : bc[BC_ACT + slot];
     if (need_p) {
-      if (lead) tri_visits += dom_n;
       phase_start();
       {
-        int inv = 0, rej = 0, cand = 0, nov = 0;
+        int inv = 0, rej = 0, cand = 0, vis = 0;
         double mx = 0.0;
-        if constexpr (PER)
-        for (int it = tid; it < dom_n; it += nth) {
-          const int t = full ? it : dom[it];
-          const int4 v = d.tv[t];
-          const int4 nn = d.tn[t];
-          // corners loaded once: FP32 pairs, moved flags and re-entries serve the
-          // filters of triangles and edges that carry no image shift
-          const int vv[3] = {v.x, v.y, v.z};
-          const bool isd[3] = {v.x < x.np, v.y < x.np, v.z < x.np};
-          const bool flat = (v.w & BD_TRI_SHIFT_BITS) == 0;
-          float4 W[3];
-          uint8_t mvd[3], wr[3];
-  #pragma unroll
-          for (int k = 0; k < 3; ++k) {
-            W[k] = work_of(x, vv[k]);
-            mvd[k] = fresh ? d.moved[vv[k]] : (uint8_t)0;
-            wr[k] = isd[k] ? d.wrap[vv[k]] : (uint8_t)0;
+        const bool skip = !sweep_all && !c.tri_all;
+        __shared__ int s_list[BD_DT_LIST], s_nd;
+        auto clean = [&](const int4 &v) -> bool {
+          if (tstamp(v.w) == gen8) return false;
+          return !(fresh && (d.moved[v.x] | d.moved[v.y] | d.moved[v.z]));
+        };
+        // One corner of a triangle per item, testing the edge that faces it (and
+        // for the first corner the triangle's orientation): the chain of loads and
+        // tests behind an item, which sets the length of a pass in all but the
+        // largest systems, is a third of a whole triangle's.
+        // The first pass takes the corners of all triangles in turn; a later pass
+        // those of the block's dirty triangles, put in a list first.
+        const int share = skip ? (x.T + (int)gridDim.x - 1) / (int)gridDim.x : 0;
+        const int s0 = min(x.T, (int)blockIdx.x * share), s1 = min(x.T, s0 + share);
+        int base = s0;
+        do {
+          int items = 3 * x.T, it = tid, stride = nth;
+          if (skip) {
+            __syncthreads();   // (the list of the chunk before has been worked off)
+            if (threadIdx.x == 0) s_nd = 0;
+            __syncthreads();
+            const int e1 = min(s1, base + BD_DT_LIST);
+            for (int t = base + (int)threadIdx.x; t < e1; t += blockDim.x)
+              if (!clean(d.tv[t])) s_list[atomicAdd(&s_nd, 1)] = t;
+            __syncthreads();
+            items = 3 * s_nd;
+            it = threadIdx.x;
+            stride = blockDim.x;
+            base += BD_DT_LIST;
           }
-          int fl = tstamp(v.w) == gen8 ? BD_TRI_DIRTY : 0;
-          if (mvd[0] | mvd[1] | mvd[2]) {
-            const int o = flat ? orient_pre(x, isd[0] && isd[1] && isd[2], W[0], W[1], W[2], v.x, v.y, v.z)
-                               : orient_s(x, v.x, tshx<PER>(v.w, 0), tshy<PER>(v.w, 0), v.y, tshx<PER>(v.w, 1),
-                                          tshy<PER>(v.w, 1), v.z, tshx<PER>(v.w, 2), tshy<PER>(v.w, 2));
-            fl = BD_TRI_DIRTY | (o <= 0 ? BD_TRI_INVERTED : 0);
-            if (o <= 0) d.tinv[t] = 1;
-          }
-          const bool inverted = (fl & BD_TRI_INVERTED) != 0;
-          inv += inverted ? 1 : 0;
-          bool owner = false;   // t registered a flip candidate
-          if (inverted && d.rep_stats) {
-            const int rr = tri_rep(d, x.np, v);
-            if (rr >= 0) atomicAdd((unsigned long long *)&d.rep_stats[3 * rr + 2], 1ull);
-          }
-          for (int k = 0; k < 3; ++k) {
-            const int cc = 3 * t + k;
-            const int o = vk(nn, k);
-            // each interior edge once: from its smaller corner, or from this side
-            // when the neighbour is not visited by this pass
-            if (o < 0 || (o <= cc && (full || cmark[o / 3] == gen))) continue;
-            const int ku = (k + 1) % 3, kw = (k + 2) % 3;
-            const int u = vv[ku], w = vv[kw];
-            const bool disks = isd[ku] && isd[kw];
-            const bool mv = (mvd[ku] | mvd[kw]) != 0;
+          for (; it < items; it += stride) {
+            const int t = skip ? s_list[it / 3] : it / 3, k = it % 3, cc = 3 * t + k;
+            const int4 v = d.tv[t];
+            const int o = ((const int *)&d.tn[t])[k];
+            // corners in order: the edge faces ia and runs from ib to ic
+            const int ia = vk(v, k), ib = vk(v, (k + 1) % 3), ic = vk(v, (k + 2) % 3);
+            const bool own = o >= 0 && (o > cc || (skip && clean(d.tv[o / 3])));
+            if (k && !own) continue;
+            const float4 Wa = work_of(x, ia), Wb = work_of(x, ib), Wc = work_of(x, ic);
+            uint8_t ma = 0, mb = 0, mc = 0;   // moved; periodic box: bits 1-4 its re-entry
+            if (fresh) {
+              ma = d.moved[ia];
+              mb = d.moved[ib];
+              mc = d.moved[ic];
+              if (PER) {
+                if (ib < x.np) mb |= (uint8_t)(d.wrap[ib] << 1);
+                if (ic < x.np) mc |= (uint8_t)(d.wrap[ic] << 1);
+              }
+            }
+            int4 v1 = make_int4(0, 0, 0, 0);
+            if (own) v1 = d.tv[o / 3];
+            const int q = own ? vk(v1, o % 3) : 0;
+            const bool flat = !PER || (v.w & BD_TRI_SHIFT_BITS) == 0;
+            const bool all_disks = ia < x.np && ib < x.np && ic < x.np;
+            const bool mvd = ((ma | mb | mc) & 1) != 0;
+            const bool due = own && (mvd || tstamp(v.w) == gen8 || tstamp(v1.w) == gen8 || (fresh && d.moved[q]));
+            float4 Wq = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (due) Wq = work_of(x, q);
+            if (k == 0) {
+              ++vis;
+              if (mvd) {
+                const int in = flat ? orient_pre(x, all_disks, Wa, Wb, Wc, ia, ib, ic)
+                                    : orient_s(x, ia, tshx<PER>(v.w, 0), tshy<PER>(v.w, 0), ib, tshx<PER>(v.w, 1),
+                                               tshy<PER>(v.w, 1), ic, tshx<PER>(v.w, 2), tshy<PER>(v.w, 2));
+                if (in <= 0) {
+                  // (the marks and the scan of a pass that finds one are void)
+                  d.tinv[t] = 1;
+                  ++inv;
+                  if (d.rep_stats) {
+                    const int rr = tri_rep(d, x.np, v);
+                    if (rr >= 0) atomicAdd((unsigned long long *)&d.rep_stats[3 * rr + 2], 1ull);
+                  }
+                }
+              }
+              if (!own) continue;
+            }
+            const int u = ib, w = ic;
+            const bool disks = u < x.np && w < x.np;
             // image shift of w relative to u in this triangle (periodic box; 0 with walls)
-            const int rsx = tshx<PER>(v.w, (k + 2) % 3) - tshx<PER>(v.w, (k + 1) % 3);
-            const int rsy = tshy<PER>(v.w, (k + 2) % 3) - tshy<PER>(v.w, (k + 1) % 3);
-            long long LQ = 0;
-            if (rsx | rsy) LQ = rep_LQ(x, u);
+            const int ku = (k + 1) % 3, kw = (k + 2) % 3;
+            const int rsx = tshx<PER>(v.w, kw) - tshx<PER>(v.w, ku);
+            const int rsy = tshy<PER>(v.w, kw) - tshy<PER>(v.w, ku);
             const bool plain = (rsx | rsy) == 0;   // the edge carries no image shift
-            // r1 = r_w - r_u from the FP32 pairs, or for a shifted edge from the grid
+            long long LQ = plain ? 0 : rep_LQ(x, u);
+            // r1 = r_w - r_u from the FP32 pairs, or for a shifted edge from the grid (one rounding)
             float r1x, r1y;
             if (plain) {
-              r1x = fdiff(W[kw].x, W[kw].z, W[ku].x, W[ku].z);
-              r1y = fdiff(W[kw].y, W[kw].w, W[ku].y, W[ku].w);
+              r1x = fdiff(Wc.x, Wc.z, Wb.x, Wb.z);
+              r1y = fdiff(Wc.y, Wc.w, Wb.y, Wb.w);
             } else {
               const Lift U = lift(x, u, 0, 0, LQ), V = lift(x, w, rsx, rsy, LQ);
               r1x = lift_diff(x, V.x, U.x);
               r1y = lift_diff(x, V.y, U.y);
             }
-            if (disks && mv) {
-              // Sec. 4.3 first criterion: r0 . r1 < 0.  An edge whose ends did
-              // not re-enter is screened in FP32 from r1 and the moves, as with
-              // walls; otherwise, and near zero, exact on the grid (the edge's
-              // shift before the move is the present one less the re-entries
-              // of its end points)
-              int dec = 0;   // 1 reversed, -1 not, 0 undecided
-              if ((wr[ku] | wr[kw]) == 0) {
-                const float2 mu = mvd[ku] ? d.dmove[u] : make_float2(0.f, 0.f);
-                const float2 mw = mvd[kw] ? d.dmove[w] : make_float2(0.f, 0.f);
-                const float r0x = __fsub_rn(r1x, __fsub_rn(mw.x, mu.x)), r0y = __fsub_rn(r1y, __fsub_rn(mw.y, mu.y));
-                const float dot = __fadd_rn(__fmul_rn(r0x, r1x), __fmul_rn(r0y, r1y));
-                const float S = __fadd_rn(__fadd_rn(__fadd_rn(__fmul_rn(r0x, r0x), __fmul_rn(r0y, r0y)),
-                                                    __fadd_rn(__fmul_rn(r1x, r1x), __fmul_rn(r1y, r1y))),
-                                          __fadd_rn(__fadd_rn(__fmul_rn(mu.x, mu.x), __fmul_rn(mu.y, mu.y)),
-                                                    __fadd_rn(__fmul_rn(mw.x, mw.x), __fmul_rn(mw.y, mw.y))));
-                const float bound = 4e-6f * S;
-                dec = dot > bound ? -1 : (-dot > bound ? 1 : 0);
-                if (dec == 0 && plain) count_exact(x);
-              }
-              int ox = rsx, oy = rsy;
-              if (dec == 0) {
-                ox -= wrapx(wr[kw]) - wrapx(wr[ku]);
-                oy -= wrapy(wr[kw]) - wrapy(wr[ku]);
-                if ((ox | oy) && LQ == 0) LQ = rep_LQ(x, u);
-              }
-              if (dec == 1 || (dec == 0 && reversed_exact(x, u, w, ox, oy, rsx, rsy, LQ))) {
-                ++rej;
-                atomicExch(&ctl->st_fail_item, cc);
-              }
-            }
-            if (inverted) continue;   // marks and scan wait for the repair
-            const int4 v1 = d.tv[o / 3];
-            const int q = vk(v1, o % 3);
-            // the edge is tested when a triangle on either side is dirty or one
-            // of its four points moved
-            const bool d1 = (fl & BD_TRI_DIRTY) || tstamp(v1.w) == gen8 || (mvd[ku] | mvd[kw]) ||
-                            (fresh && d.moved[q]);
-            if (d1) {
-              int sqx, sqy;
-              opp_shift<PER>(v.w, k, v1.w, o % 3, sqx, sqy);
-              const int ic = (flat && (sqx | sqy) == 0)
-                                 ? incircle_pre(x, isd[0] && isd[1] && isd[2] && q < x.np, W[0], W[1], W[2],
-                                                work_of(x, q), v.x, v.y, v.z, q)
-                                 : incircle_s<PER>(x, v, q, sqx, sqy);
-              if (ic > 0) {
-                claim6(x, claims(x, epoch), t, k, nn, o, claim_key(epoch, cc));
-                ++cand;
-                if (!owner) {   // t joins the candidate owners once (candidates are rare)
-                  owner = true;
-                  push_owner(x, epoch, t);
-                }
-              }
-            }
-            if (disks && scan) {
-              // FP32 screen: a pair whose FP32 squared distance exceeds
-              // sigma^2 (1 + 1e-5) is farther than sigma (FP32 error ~3e-7)
-              if (__fadd_rn(__fmul_rn(r1x, r1x), __fmul_rn(r1y, r1y)) > x.sig2f) continue;
-              double2 v;
-              double del;
-              if (edge_overlap(x, u, w, rsx, rsy, LQ, v, del)) {
-                disp_add(x, u, -v.x, -v.y);
-                disp_add(x, w, v.x, v.y);
-                if (use_lists) push_tri(nlist, nmark, ncount, ngen, t);   // checked again in the next pass
-                const int k_ov = atomicAdd(pcnt(C_OVERLAP), 1);
-                if (logging) {
-                  if (log_head + k_ov < c.log_pairs_cap) d.log_pairs[log_head + k_ov] = make_int2(u, w);
-                  else atomicExch(&ctl->log_overflow, 1);
-                }
-                mx = fmax(mx, del);
-              }
-            }
-          }
-        }
-        else
-        for (int it = tid; it < dom_n; it += nth) {
-          // walls: the three corners' FP32 pairs and moved flags are loaded once
-          // and serve the orientation, the reversal and in-circle filters and the
-          // overlap screen of all three edges
-          const int t = full ? it : dom[it];
-          const int4 v = d.tv[t];
-          const int4 nn = d.tn[t];
-          const int vv[3] = {v.x, v.y, v.z};
-          const bool isd[3] = {v.x < x.np, v.y < x.np, v.z < x.np};
-          float4 W[3];
-          uint8_t mvd[3];
-  #pragma unroll
-          for (int k = 0; k < 3; ++k) {
-            W[k] = work_of(x, vv[k]);
-            mvd[k] = fresh ? d.moved[vv[k]] : (uint8_t)0;
-          }
-          int fl = tstamp(v.w) == gen8 ? BD_TRI_DIRTY : 0;
-          if (mvd[0] | mvd[1] | mvd[2]) {
-            const int o = orient_pre(x, isd[0] && isd[1] && isd[2], W[0], W[1], W[2], v.x, v.y, v.z);
-            fl = BD_TRI_DIRTY | (o <= 0 ? BD_TRI_INVERTED : 0);
-            if (o <= 0) d.tinv[t] = 1;
-          }
-          const bool inverted = (fl & BD_TRI_INVERTED) != 0;
-          inv += inverted ? 1 : 0;
-          bool owner = false;   // t registered a flip candidate
-          if (inverted && d.rep_stats) {
-            const int rr = tri_rep(d, x.np, v);
-            if (rr >= 0) atomicAdd((unsigned long long *)&d.rep_stats[3 * rr + 2], 1ull);
-          }
-  #pragma unroll
-          for (int k = 0; k < 3; ++k) {
-            const int cc = 3 * t + k;
-            const int o = vk(nn, k);
-            // each interior edge once: from its smaller corner, or from this side
-            // when the neighbour is not visited by this pass
-            if (o < 0 || (o <= cc && (full || cmark[o / 3] == gen))) continue;
-            const int ku = (k + 1) % 3, kw = (k + 2) % 3;
-            const int u = vv[ku], w = vv[kw];
-            const bool disks = isd[ku] && isd[kw];
-            // r1 = r_w - r_u from the FP32 pairs (one rounding)
-            const float r1x = fdiff(W[kw].x, W[kw].z, W[ku].x, W[ku].z);
-            const float r1y = fdiff(W[kw].y, W[kw].w, W[ku].y, W[ku].w);
-            if (disks && (mvd[ku] | mvd[kw])) {
+            if (disks && ((mb | mc) & 1)) {
               // Sec. 4.3 first criterion r0 . r1 < 0; r0 = r1 - (move of w - move
-              // of u), screened in FP32, exact on the grid near zero
-              bool rev;
-              {
-                const float2 mu = mvd[ku] ? d.dmove[u] : make_float2(0.f, 0.f);
-                const float2 mw = mvd[kw] ? d.dmove[w] : make_float2(0.f, 0.f);
+              // of u), screened in FP32 unless an end re-entered, exact on the
+              // grid there and near zero (the edge's shift before the move is
+              // the present one less the re-entries of its end points)
+              int dec = 0;   // 1 reversed, -1 not, 0 undecided
+              if (!PER || ((mb | mc) >> 1) == 0) {
+                const float2 mu = (mb & 1) ? d.dmove[u] : make_float2(0.f, 0.f);
+                const float2 mw = (mc & 1) ? d.dmove[w] : make_float2(0.f, 0.f);
                 const float r0x = __fsub_rn(r1x, __fsub_rn(mw.x, mu.x)), r0y = __fsub_rn(r1y, __fsub_rn(mw.y, mu.y));
                 // every rounding above is relative (one FP32 rounding of a grid
                 // value or of a sum): the computed dot is within ~8 2^-24 S of
@@ -1021,48 +934,41 @@ __device__ __forceinline__ void triangulation_body(const BdDev &d, const BdConst
                                           __fadd_rn(__fadd_rn(__fmul_rn(mu.x, mu.x), __fmul_rn(mu.y, mu.y)),
                                                     __fadd_rn(__fmul_rn(mw.x, mw.x), __fmul_rn(mw.y, mw.y))));
                 const float bound = 4e-6f * S;
-                if (dot > bound) {
-                  rev = false;
-                } else if (-dot > bound) {
-                  rev = true;
-                } else {
-                  count_exact(x);
-                  rev = reversed_exact(x, u, w, 0, 0, 0, 0, 0);
-                }
+                dec = dot > bound ? -1 : (-dot > bound ? 1 : 0);
+                if (dec == 0 && plain) count_exact(x);
               }
-              if (rev) {
+              if (dec == 0) {
+                int ox = rsx, oy = rsy;
+                if (PER) {
+                  ox -= wrapx((uint8_t)(mc >> 1)) - wrapx((uint8_t)(mb >> 1));
+                  oy -= wrapy((uint8_t)(mc >> 1)) - wrapy((uint8_t)(mb >> 1));
+                  if ((ox | oy) && LQ == 0) LQ = rep_LQ(x, u);
+                }
+                dec = reversed_grid(kp == 0 ? d.pos0 : d.prev, d.pos, x.g, u, w, mb & 1, mc & 1, ox, oy, rsx, rsy, LQ) ? 1 : -1;
+              }
+              if (dec == 1) {
                 ++rej;
                 atomicExch(&ctl->st_fail_item, cc);
               }
             }
-            if (inverted) continue;   // marks and scan wait for the repair
-            const int4 v1 = d.tv[o / 3];
-            const int q = vk(v1, o % 3);
-            // the edge is tested when a triangle on either side is dirty or one
-            // of its four points moved
-            const bool d1 = (fl & BD_TRI_DIRTY) || tstamp(v1.w) == gen8 || (mvd[ku] | mvd[kw]) ||
-                            (fresh && d.moved[q]);
-            if (d1) {
-              const bool filt = isd[0] && isd[1] && isd[2] && q < x.np;
-              if (incircle_pre(x, filt, W[0], W[1], W[2], work_of(x, q), v.x, v.y, v.z, q) > 0) {
-                claim6(x, claims(x, epoch), t, k, nn, o, claim_key(epoch, cc));
+            // the edge's in-circle test is due when a triangle on either side is
+            // dirty or one of its four points moved
+            if (due) {
+              int sqx, sqy;
+              opp_shift<PER>(v.w, k, v1.w, o % 3, sqx, sqy);
+              const int in = (flat && (sqx | sqy) == 0)
+                                 ? incircle_pre(x, all_disks && q < x.np, Wa, Wb, Wc, Wq, ia, ib, ic, q)
+                                 : incircle_s<PER>(x, v, q, sqx, sqy);
+              if (in > 0) {
                 ++cand;
-                if (!owner) {   // t joins the candidate owners once (candidates are rare)
-                  owner = true;
-                  push_owner(x, epoch, t);
-                }
+                register_edge(x, claims(x, epoch), epoch, min(cc, o), max(cc, o));   // by its smaller corner
               }
             }
-            if (disks && scan) {
-              // FP32 screen: a pair whose FP32 squared distance exceeds
-              // sigma^2 (1 + 1e-5) is farther than sigma (FP32 error ~3e-7)
-              if (__fadd_rn(__fmul_rn(r1x, r1x), __fmul_rn(r1y, r1y)) > x.sig2f) continue;
-              double2 v;
-              double del;
-              if (edge_overlap(x, u, w, 0, 0, 0, v, del)) {
-                disp_add(x, u, -v.x, -v.y);
-                disp_add(x, w, v.x, v.y);
-                if (use_lists) push_tri(nlist, nmark, ncount, ngen, t);   // checked again in the next pass
+            // FP32 screen: a pair whose FP32 squared distance exceeds
+            // sigma^2 (1 + 1e-5) is farther than sigma (FP32 error ~3e-7)
+            if (disks && scan && !(__fadd_rn(__fmul_rn(r1x, r1x), __fmul_rn(r1y, r1y)) > x.sig2f)) {
+              const double del = overlap_push(d, c, u, w, rsx, rsy, LQ, 1);
+              if (del > 0.0) {
                 const int k_ov = atomicAdd(pcnt(C_OVERLAP), 1);
                 if (logging) {
                   if (log_head + k_ov < c.log_pairs_cap) d.log_pairs[log_head + k_ov] = make_int2(u, w);
@@ -1072,17 +978,19 @@ __device__ __forceinline__ void triangulation_body(const BdDev &d, const BdConst
               }
             }
           }
-        }
+        } while (skip && base < s1);
         {
-          int *const to[3] = {pcnt(C_INV), pcnt(C_REJECT), pcnt(C_CAND)};
-          const int v[3] = {inv, rej, cand};
-          block_add(to, v);
+          int *const to[4] = {pcnt(C_INV), pcnt(C_REJECT), pcnt(C_CAND), pcnt(C_VISIT)};
+          const int n[4] = {inv, rej, cand, vis};
+          block_add(to, n);
         }
-        (void)nov;
         if (mx > 0.0) atomicMax(&ctl->st_max_overlap_bits, (unsigned long long)__double_as_longlong(mx));
       }
       if (!sync()) { leave(); return; }
-      if (lead) stage_tick(ctl, full ? STAGE_P : STAGE_PL, t_mark);
+      if (lead) {
+        stage_tick(ctl, sweep_all || c.tri_all ? STAGE_P : STAGE_PL, t_mark);
+        tri_visits += bc[BC_CNT + C_VISIT];
+      }
       const int n_inv = bc[BC_CNT + C_INV];
       const int n_rej = bc[BC_CNT + C_REJECT];
       n_ov = bc[BC_CNT + C_OVERLAP];
@@ -1136,7 +1044,7 @@ __device__ __forceinline__ void triangulation_body(const BdDev &d, const BdConst
                   const int cm = min(3 * t + k, o);
                   const int tt = cm / 3, kk = cm % 3;
                   const int4 ncm = d.tn[tt];
-                  claim6(x, claims(x, epoch), tt, kk, ncm, vk(ncm, kk), claim_key(epoch, cm));
+                  claim6(d.tn, claims(x, epoch), tt, kk, ncm, vk(ncm, kk), claim_key(epoch, cm));
                   ++ncand;
                 }
               }
@@ -1177,7 +1085,7 @@ __device__ __forceinline__ void triangulation_body(const BdDev &d, const BdConst
         }
         if (status) break;
         fresh = false;
-        full = true;   // the repaired region's marks and scan were skipped: check everything
+        sweep_all = true;   // the repaired region's marks and scan were skipped: check everything
         need_p = scan = true;
         ++kp;
         continue;
@@ -1197,11 +1105,10 @@ __device__ __forceinline__ void triangulation_body(const BdDev &d, const BdConst
       phase_start();
       {
         const bool voided = !fuse && n_ov;   // unfused: the marking pass's scan is void
-        if (voided || fresh)
-          for (int i = tid; i < x.np; i += nth) {
-            if (voided) d.disp[i] = make_double2(0.0, 0.0);
-            if (fresh) d.moved[i] = 0;
-          }
+        if (voided)
+          for (int i = tid; i < x.np; i += nth) d.disp[i] = make_double2(0.0, 0.0);
+        if (fresh)
+          for (int i = tid; i < x.np / 4; i += nth) ((unsigned *)d.moved)[i] = 0u;   // np is a multiple of 512
         int nf = 0, nlose = 0, adj = 0;
         double fmx = 0.0;
         // the triangles that registered a candidate for this round (in the
@@ -1225,43 +1132,37 @@ __device__ __forceinline__ void triangulation_body(const BdDev &d, const BdConst
         // one SM would queue on its load/store unit)
         for (int it = blockIdx.x + threadIdx.x * gridDim.x; it < ncl; it += nth) {
           const int t = cl[it];
-          const unsigned long long key = cb[t];
-          bool flipped = false;
-          if ((key >> 32) == epoch) {
+          int t1 = -1;   // the triangle t was flipped with
+          if (fuse) {
+            const FusedOut fo = fused_flip<PER>(x, t, epoch, cb, nb);
+            t1 = fo.t1;
+            adj += fo.adj;
+            fmx = fmax(fmx, fo.mx);
+          } else {
+            const unsigned long long key = cb[t];
             const int cm = key_corner(key);
-            if (cm / 3 == t) {
+            if ((key >> 32) == epoch && cm / 3 == t) {
               const int4 N0 = d.tn[t];
-              const int k0 = cm % 3;
-              const int o = vk(N0, k0);
-              if (owns6(x, cb, t, k0, N0, o, key)) {
-                if (fuse) {
-                  const FusedOut fo = fused_flip<PER>(x, cm, o, nb, epoch + 1);
-                  adj += fo.adj;
-                  fmx = fmax(fmx, fo.mx);
-                } else {
-                  flip_owned<PER>(x, cm, o, ngen8);
-                }
-                if (!fuse && use_lists) {
-                  push_tri(nlist, nmark, ncount, ngen, t);
-                  push_tri(nlist, nmark, ncount, ngen, o / 3);
-                }
-                flipped = true;
-                ++nf;
-                if (d.rep_stats) {
-                  // the four points of a flipped edge include a disk (ghost
-                  // points never move, so an edge among them stays legal); one
-                  // of the two new triangles may hold only ghost points
-                  int rr = tri_rep(d, x.np, d.tv[t]);
-                  if (rr < 0) rr = tri_rep(d, x.np, d.tv[o / 3]);
-                  if (rr >= 0) atomicAdd((unsigned long long *)&d.rep_stats[3 * rr + 1], 1ull);
-                }
+              const int o = vk(N0, cm % 3);
+              if (owns6(x, cb, t, cm % 3, N0, o, key)) {
+                t1 = o / 3;
+                flip_owned<PER>(x, cm, o, ngen8);
               }
             }
           }
-          if (!flipped) {
+          if (t1 >= 0) {
+            ++nf;
+            if (d.rep_stats) {
+              // the four points of a flipped edge include a disk (ghost
+              // points never move, so an edge among them stays legal); one
+              // of the two new triangles may hold only ghost points
+              int rr = tri_rep(d, x.np, d.tv[t]);
+              if (rr < 0) rr = tri_rep(d, x.np, d.tv[t1]);
+              if (rr >= 0) atomicAdd((unsigned long long *)&d.rep_stats[3 * rr + 1], 1ull);
+            }
+          } else {
             ++nlose;
             stamp_tri(x, t, ngen8);
-            if (use_lists) push_tri(nlist, nmark, ncount, ngen, t);
           }
         }
         {
@@ -1278,16 +1179,15 @@ __device__ __forceinline__ void triangulation_body(const BdDev &d, const BdConst
       st_flips += bc[BC_CNT + C_FLIPS];
       st_rounds += 1;
       fresh = false;
-      full = !use_lists;
       if (!fuse) {
-        need_p = scan = true;   // the next pass marks and scans afresh
+        need_p = scan = sweep_all = true;   // the next pass marks and scans afresh
         ++kp;
         continue;
       }
       ov_now += bc[BC_CNT + C_OVADJ];
       if (bc[BC_CNT + C_LOSE] > 0) {
         need_p = true;          // a pass marks the losers' edges again
-        scan = false;
+        scan = sweep_all = false;
         ++kp;
         continue;
       }
@@ -1336,25 +1236,45 @@ __device__ __forceinline__ void triangulation_body(const BdDev &d, const BdConst
     // ---------------- A: apply (capped at sigma/4) ----------------
     phase_start();
     {
+      // Only the marked disks have a sum: the others cost their mark and their
+      // cleared flag, 2 bytes a disk (with every disk's position, sum and
+      // previous position, some 50 bytes, the pass took 59 us at 2^20 disks for a
+      // few thousand that move).  Four marks are loaded ahead of their use; a
+      // marked disk has a thread to itself, since its chain of loads sets the
+      // length of the pass (four neighbouring disks per thread doubled it).
       int nwrap = 0;
-      for (int i = tid; i < x.np; i += nth) {
-        if (d.ext_id[i] < 0) continue;
-        const double2 p = d.pos[i];
-        d.prev[i] = p;
-        const double2 dd = disp_get(x, i);
-        if (PER) d.wrap[i] = 0;
-        if (dd.x != 0.0 || dd.y != 0.0) {
-          // the first disk of a replica moved by this pass counts the pass
-          const int rr = d.rep_of[i];
-          const unsigned long long stamp = epoch;   // distinct per pass (grows across launches), never 0
-          if (d.rep_stats && atomicExch(&d.rep_mark[rr], stamp) != stamp)
-            atomicAdd((unsigned long long *)&d.rep_stats[3 * rr], 1ull);
+      for (int i0 = tid; i0 < x.np; i0 += 4 * nth) {
+       unsigned marks = 0u;
+#pragma unroll
+       for (int u = 0; u < 4; ++u)
+         if (i0 + u * nth < x.np && d.hit[i0 + u * nth]) marks |= 1u << u;
+#pragma unroll 1
+       for (int u = 0; u < 4; ++u) {
+        const int i = i0 + u * nth;
+        if (i >= x.np) break;
+        if (!(marks >> u & 1u)) {
+          d.moved[i] = 0;
+          if (PER) d.wrap[i] = 0;
+          if (log_pidx >= 0) d.log_pflags[(size_t)log_pidx * x.np + i] = 0;
+          continue;
         }
+        d.hit[i] = 0;
+        if (PER) d.wrap[i] = 0;
+        const double2 p = d.pos[i];
+        const double2 dd = disp_get(x, i);
         if (dd.x == 0.0 && dd.y == 0.0) {
           d.moved[i] = 0;
           if (log_pidx >= 0) d.log_pflags[(size_t)log_pidx * x.np + i] = 0;
           continue;
         }
+        if (d.rep_stats) {
+          // the first disk of a replica moved by this pass counts the pass
+          const int rr = d.rep_of[i];
+          const unsigned long long stamp = epoch;   // distinct per pass (grows across launches), never 0
+          if (atomicExch(&d.rep_mark[rr], stamp) != stamp)
+            atomicAdd((unsigned long long *)&d.rep_stats[3 * rr], 1ull);
+        }
+        d.prev[i] = p;
         const double mag = sqrt(__dadd_rn(__dmul_rn(dd.x, dd.x), __dmul_rn(dd.y, dd.y)));
         // Sec. 4.4: sigma/4, half the disk's radius (its own for polydisperse disks)
         const double cap = d.rad ? 0.5 * d.rad[i] : 0.25 * sigma;
@@ -1386,26 +1306,15 @@ __device__ __forceinline__ void triangulation_body(const BdDev &d, const BdConst
         }
         d.disp[i] = make_double2(0.0, 0.0);
         d.moved[i] = 1;
-        // the next pass visits the star of the moved disk (walked across the
-        // edges (i, p) of its triangles, from the corner vt[i])
-        const int c0 = d.vt[i];
-        int cw = c0;
-        for (int guard = 0; use_lists && guard < 256; ++guard) {
-          const int tw = cw / 3;
-          push_tri(nlist, nmark, ncount, ngen, tw);
-          const int o = ((const int *)&d.tn[tw])[(cw % 3 + 2) % 3];
-          if (o < 0) break;
-          cw = 3 * (o / 3) + (o % 3 + 2) % 3;
-          if (cw == c0) break;
-        }
+       }
       }
       if (PER) block_add(&ctl->n_wrapped, nwrap);
     }
     if (!sync()) { leave(); return; }
     if (lead) stage_tick(ctl, STAGE_A, t_mark);
     fresh = true;
-    full = !use_lists;
     need_p = scan = true;
+    sweep_all = false;   // an edge whose ends both stayed put does not overlap
     ++kp;
   }
 
@@ -1431,7 +1340,7 @@ __device__ __forceinline__ void triangulation_body(const BdDev &d, const BdConst
     }
     if (lead) atomicCAS(&ctl->status, 0, status);
   } else {
-    for (int i = tid; i < x.np; i += nth) d.moved[i] = 0;
+    for (int i = tid; i < x.np / 4; i += nth) ((unsigned *)d.moved)[i] = 0u;
   }
   if (lead) {
     if (logging && !status) {
@@ -1459,11 +1368,13 @@ __device__ __forceinline__ void triangulation_body(const BdDev &d, const BdConst
 }
 
 template <bool PER>
-__global__ void __launch_bounds__(BD_DT_THREADS, 3) k_triangulation(BdDev d, BdConst c, int mode, int log_step) {
+__global__ void __launch_bounds__(BD_DT_THREADS, 3) k_triangulation(const __grid_constant__ BdDev d, const __grid_constant__ BdConst c, int mode,
+                                                                     int log_step) {
   triangulation_body<PER, false>(d, c, mode, log_step);
 }
 template <bool PER>
-__global__ void __launch_bounds__(BD_DTC_THREADS, 1) k_triangulation_cl(BdDev d, BdConst c, int mode, int log_step) {
+__global__ void __launch_bounds__(BD_DTC_THREADS, 1) k_triangulation_cl(const __grid_constant__ BdDev d, const __grid_constant__ BdConst c, int mode,
+                                                                     int log_step) {
   triangulation_body<PER, true>(d, c, mode, log_step);
 }
 
@@ -1503,12 +1414,11 @@ __global__ void k_restore_step(BdDev d, BdConst c) {
         unjournal(d, t);
         d.jmark[t] = 0u;
       }
-      // the abandoned launch did not publish the claim epochs and list
-      // generations it used (the next launch starts from the same ones):
-      // clear its claims (0 matches no epoch) and list marks (0 matches no
-      // generation after the first launch)
-      d.claim[t] = 0ull;
-      for (int l = 0; l < 3; ++l) d.act_mark[(size_t)l * c.nt + t] = 0u;
+      // the abandoned launch did not publish the claim epochs it used (the next
+      // launch starts from the same ones): clear its claims and owner marks (0
+      // matches no epoch)
+      d.claim[t] = d.claim[(size_t)c.nt + t] = 0ull;
+      d.clmark[t] = 0u;
     }
   }
 }
@@ -1522,15 +1432,15 @@ cudaError_t bd_launch_restore_step(const BdDev &d, const BdConst &c, cudaStream_
   return cudaGetLastError();
 }
 
-int bd_dt_grid_for(int work_items, int *grid, int *block) {
+int bd_dt_grid_for(long long work_items, int *grid, int *block) {
   // all co-resident blocks (the phases are latency-bound chains of dependent
   // loads and integer predicates, so more threads in flight help), but no
   // more than about one work item per thread
   int g = 0, b = 0;
   if (bd_dt_grid(&g, &b) != 0) return -1;
-  int want = (work_items + b - 1) / b;
+  long long want = (work_items + b - 1) / b;
   if (want < 1) want = 1;
-  *grid = want < g ? want : g;
+  *grid = want < g ? (int)want : g;
   *block = b;
   return 0;
 }
