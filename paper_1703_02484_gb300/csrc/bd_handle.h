@@ -31,6 +31,7 @@ struct bd_handle {
   std::vector<BdRep> h_rep;
   int n = 0, np = 0, np_i = 0, nt = 0, ng = 0;
   std::vector<int> ext_of_int;    // internal slot -> concatenated external index (-1 = empty)
+  std::vector<int> tri_orig;      // triangle slot -> its place in the order built (and handed out)
   std::vector<int> int_of_ext;    // concatenated external index -> internal slot
   std::vector<double> host_pos;   // (np + ng) * 2 mirror used for uploads
   int dt_grid = 0, dt_block = 0;
