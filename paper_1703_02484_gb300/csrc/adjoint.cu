@@ -48,7 +48,7 @@ __global__ void k_rp_em(BdDev d, BdConst c, long long step, int k_local, double2
   const int e = d.ext_id[i];
   if (e < 0) return;
   const BdRep &R = d.rep[d.rep_of[i]];
-  const double2 F = bdem::force_sum(d, c, R, i);
+  const double2 F = bdem::force_sum(d, c, R, i, d.fpart[i]);
   const double2 p = d.pos[i];
   const float th = d.theta[i];
   if (sx) {

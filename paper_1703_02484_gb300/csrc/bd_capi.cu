@@ -54,6 +54,11 @@ void rep_set_alpha(BdRep &B, const double *alpha, int n_species) {
     }
 }
 
+void rep_set_v0(BdRep &B, double v0) {
+  B.v0 = v0;
+  B.v0f = (float)v0;
+}
+
 }  // namespace bdcapi
 
 using namespace bdcapi;
@@ -849,7 +854,10 @@ int build_handle(const std::vector<Spec> &specs, void *stream, bd_handle **out) 
     B.dt = p.dt;
     B.amp = p.literal_noise ? sqrt(p.D * p.dt) : sqrt(2.0 * p.D * p.dt);
     B.amp_r = sqrt(2.0 * p.Dr * p.dt);
-    B.v0 = p.v0;
+    B.dtf = (float)B.dt;
+    B.ampf = (float)B.amp;
+    B.amp_rf = (float)B.amp_r;
+    rep_set_v0(B, p.v0);
     B.eps = p.eps;
     B.kappa = p.kappa;
     B.r_cut = p.r_cut;
@@ -1766,7 +1774,7 @@ int bd_set_state(bd_handle *h, const double *xy, const float *theta) {
   // in place.
   cudaStream_t st = h->stream;
   const BdDev &d = h->d;
-  // k_state_check also snapshots pos, prev and theta and clears the moved
+  // k_state_check also snapshots pos and theta and clears the moved
   // flags; k_state_in also writes the FP32 copy of what it stores
   cudaError_t e = reset_stats(h);
   if (e == cudaSuccess) e = cudaMemcpyAsync(d.xfer_xy, xy, (size_t)h->n * sizeof(double2), cudaMemcpyHostToDevice, st);

@@ -117,6 +117,7 @@ struct BdRep {
   float Lf, hLf, invLf;
   long long LQ;
   double dt, amp, amp_r, v0;
+  float dtf, ampf, amp_rf, v0f;   // the same rounded to FP32 (the FP32 step)
   double eps, kappa, r_cut, skin, rl2, cell_size;
   float rc2f, epsf, kapf;         // r_cut^2, eps, kappa rounded to FP32
   int vl_shift;                   // Verlet trigger: displacements in steps of 2^vl_shift of the grid,
@@ -134,6 +135,7 @@ struct BdRep {
 
 struct BdDev {
   // disks (internal order, np slots), then the ghost points of every replica
+  // pos0: positions before the last move; prev: before the last correction pass (disks it moved)
   double2 *pos, *prev, *pos0;
   float4 *work;            // (x_hi, y_hi, x_lo, y_lo) FP32 pair of each coordinate (disks and ghosts)
   float *theta, *theta0;

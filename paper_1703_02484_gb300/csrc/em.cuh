@@ -27,11 +27,11 @@ __device__ __forceinline__ float4 split(double2 p) {
   return make_float4(xh, yh, __double2float_rn(p.x - (double)xh), __double2float_rn(p.y - (double)yh));
 }
 
-// sum of the partial-force slots of disk i (a single slot is read as is)
-__device__ __forceinline__ double2 force_sum(const BdDev &d, const BdConst &c, const BdRep &R, int i) {
+// sum of the partial-force slots of disk i (a single slot is read as is); f is
+// slot 0's value
+__device__ __forceinline__ double2 force_sum(const BdDev &d, const BdConst &c, const BdRep &R, int i, double2 f) {
   const int ns = R.law == BD_LAW_LONG ? R.nchunk : (R.law == BD_LAW_SHORT ? 1 : 0);
   if (ns == 0) return make_double2(0.0, 0.0);
-  double2 f = d.fpart[i];
   for (int k = 1; k < ns; ++k) {
     const double2 g = d.fpart[(size_t)k * c.np + i];
     f.x += g.x;
@@ -46,8 +46,30 @@ __device__ __forceinline__ double2 force_sum(const BdDev &d, const BdConst &c, c
 // pattern).  The conversions used here run on the conversion pipe, whereas FP64
 // arithmetic issues at 1/64 of the FP32 rate on this part.
 
-// a float as a double, by its bits: conversions between FP32 and FP64 run on the
-// FP64 pipe (two lanes per SM)
+// 64-bit conversions between integers and floats, and those between FP32 and
+// FP64, run on the FP64 pipe (two lanes per SM); the forms below do the cheap
+// cases with integer operations.
+
+// an integer-valued float as an integer (what __float2ll_rn gives)
+__device__ __forceinline__ long long int_of(float v) {
+  const unsigned u = __float_as_uint(v);
+  const int e = (int)(u >> 23 & 255u);
+  if (e > 150 + 38) return __float2ll_rn(v);   // 2^62 and beyond, infinities, NaN
+  const long long m = (long long)((u & 0x7FFFFFu) | 0x800000u);
+  const long long a = e >= 150 ? m << (e - 150) : (e < 127 ? 0ll : m >> (150 - e));
+  return (int)u < 0 ? -a : a;
+}
+
+// the float nearest a double that is itself a float (zero, or FP32's normal
+// range with 29 trailing zero bits) or any other double
+__device__ __forceinline__ float f32_of(double d) {
+  const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+  const unsigned e = hi >> 20 & 2047u;
+  if ((lo & 0x1FFFFFFFu) != 0u || e - 897u > 253u) return (float)d;
+  return __uint_as_float((hi & 0x80000000u) | (((hi & 0x7FFFFFFFu) - (896u << 20)) << 3) | (lo >> 29));
+}
+
+// a float as a double
 __device__ __forceinline__ double f64_of(float f) {
   const unsigned u = __float_as_uint(f);
   if ((u >> 23 & 255u) - 1u > 253u) return (double)f;   // zero, subnormal, infinity, NaN
@@ -70,8 +92,9 @@ __device__ __forceinline__ float grid_to_float(long long X, int s) {
 // rounded to FP32
 __device__ __forceinline__ float2 grid_split(long long X, int s) {
   const float h = __ll2float_rn(X);          // integer valued
-  const long long r = X - __float2ll_rn(h);  // exact
-  return make_float2(X == 0 ? 0.f : __int_as_float(__float_as_int(h) - (s << 23)), grid_to_float(r, s));
+  const int r = (int)(X - int_of(h));        // exact, below 2^27 for |X| < 2^51
+  const float q = __int_as_float((127 - s) << 23);   // 2^-s
+  return make_float2(h * q, (float)r * q);   // exact scalings
 }
 
 // periodic re-entry in grid units (Sec. 2.1): X, Y brought into [0, LQ).
@@ -138,12 +161,13 @@ __device__ __forceinline__ double3 normals_f64(const bdrng::U4 &r) {
 // *thn = new angle
 __device__ __forceinline__ void em_move_grid(const BdConst &c, const BdRep &R, uint32_t id,
                                              long long step, double2 p, float th, double2 F,
-                                             double v0, float *thn, uint32_t node, long long *X,
-                                             long long *Y) {
+                                             float *thn, uint32_t node, long long *X,
+                                             long long *Y, float2 *move) {
   bdrng::U4 r = bdrng::draw(id, (int64_t)step, R.seed, R.replica, piece_tag(node));
   const int depth = piece_depth(node);
   // length of this move and its noise amplitudes: dt / 2^depth, amp / 2^(depth/2)
-  float dt = (float)R.dt, amp = (float)R.amp, amp_r = (float)R.amp_r;
+  // (rounded to FP32 on the host: a conversion costs a thread as much as 32 FP32 operations)
+  float dt = R.dtf, amp = R.ampf, amp_r = R.amp_rf;
   if (depth) {
     const double sc = sqrt(ldexp(1.0, -depth));
     dt = (float)ldexp(R.dt, -depth);
@@ -154,14 +178,17 @@ __device__ __forceinline__ void em_move_grid(const BdConst &c, const BdRep &R, u
   const float z0 = z.x, z1 = z.y, z2 = z.z;
   float st, ct;
   sincosf(th, &st, &ct);
-  const float v0f = (float)v0;
-  float dxf = dt * ((float)F.x + v0f * ct) + amp * z0;
-  float dyf = dt * ((float)F.y + v0f * st) + amp * z1;
+  const float v0f = R.v0f;
+  float dxf = dt * (f32_of(F.x) + v0f * ct) + amp * z0;
+  float dyf = dt * (f32_of(F.y) + v0f * st) + amp * z1;
   *thn = th + amp_r * z2;
   const bdpred::Grid g{c.q, c.inv_q, c.qshift};
   const float to_grid = __int_as_float((127 + c.qshift) << 23);   // 2^s, exact scaling
-  *X = bdpred::to_int(p.x, g) + __float2ll_rn(dxf * to_grid);
-  *Y = bdpred::to_int(p.y, g) + __float2ll_rn(dyf * to_grid);
+  const float mx = rintf(dxf * to_grid), my = rintf(dyf * to_grid);
+  *X = bdpred::to_int(p.x, g) + int_of(mx);
+  *Y = bdpred::to_int(p.y, g) + int_of(my);
+  const float q = __int_as_float((127 - c.qshift) << 23);
+  *move = make_float2(mx * q, my * q);   // the move in grid steps, exact
 }
 
 // position after the move of piece `node` of step `step` (grid-rounded, before
@@ -171,7 +198,8 @@ __device__ __forceinline__ double2 em_move(const BdConst &c, const BdRep &R, uin
                                            double v0, float *thn, uint32_t node = 1u) {
   if (c.precision == 0) {
     long long X, Y;
-    em_move_grid(c, R, id, step, p, th, F, v0, thn, node, &X, &Y);
+    float2 move;
+    em_move_grid(c, R, id, step, p, th, F, thn, node, &X, &Y, &move);
     return make_double2(grid_to_double(X, c.qshift), grid_to_double(Y, c.qshift));
   }
   bdrng::U4 r = bdrng::draw(id, (int64_t)step, R.seed, R.replica, piece_tag(node));
@@ -226,6 +254,51 @@ __device__ __forceinline__ double2 reflect_as(const BdRep &R, double2 y, int f) 
   if (f & 4) y.y = 2.0 * R.wall_lo - y.y;
   if (f & 8) y.y = 2.0 * R.wall_hi - y.y;
   return y;
+}
+
+// The move of disk i (index e within its replica) from p, th under force F, as
+// the time step makes it: the new position, its FP32 copies and the move, the
+// direction, the moved flag, and what an undo needs.
+__device__ __forceinline__ void move_disk(const BdDev &d, const BdConst &c, const BdRep &R, int i, int e, long long step,
+                                          int log_step, int node, double2 p, float th, double2 F) {
+  d.pos0[i] = p;
+  d.theta0[i] = th;
+  float thn;
+  int flags = 0;
+  const bdpred::Grid g{c.q, c.inv_q, c.qshift};
+  long long X, Y;
+  float2 move;   // X - X0, Y - Y0 rounded to FP32
+  if (c.precision == 0) {
+    // move, reflection and FP32 copy in grid units (no FP64 arithmetic)
+    em_move_grid(c, R, (uint32_t)e, step, p, th, F, &thn, (uint32_t)node, &X, &Y, &move);
+  } else {
+    const double2 y = em_move(c, R, (uint32_t)e, step, p, th, F, R.v0, &thn, (uint32_t)node);
+    X = bdpred::to_int(y.x, g);
+    Y = bdpred::to_int(y.y, g);
+  }
+  const long long X0 = bdpred::to_int(p.x, g), Y0 = bdpred::to_int(p.y, g);
+  if (c.precision != 0) move = make_float2(grid_to_float(X - X0, c.qshift), grid_to_float(Y - Y0, c.qshift));
+  int wr = 0;
+  if (R.periodic) {
+    // the move itself (before re-entry), for the triangulation's reversal screen
+    d.dmove[i] = move;
+    // re-entry at the opposite side (Sec. 2.1); the triangulation kernel
+    // shifts the corners of the disks that re-entered
+    wr = wrap_grid(R.LQ, X, Y);
+    d.wrap[i] = (uint8_t)wr;
+    if (wr && !c.overlap_verlet) atomicAdd(&d.ctl->n_wrapped, 1);
+  } else {
+    const double2 w = walls_of(d, R, i);
+    flags = reflect_grid(bdpred::to_int(w.x, g), bdpred::to_int(w.y, g), X, Y);
+  }
+  d.pos[i] = make_double2(grid_to_double(X, c.qshift), grid_to_double(Y, c.qshift));
+  if (!R.periodic)
+    d.dmove[i] = flags ? make_float2(grid_to_float(X - X0, c.qshift), grid_to_float(Y - Y0, c.qshift)) : move;
+  const float2 sx = grid_split(X, c.qshift), sy = grid_split(Y, c.qshift);
+  d.work[i] = make_float4(sx.x, sy.x, sx.y, sy.y);
+  d.theta[i] = thn;
+  d.moved[i] = 1;
+  if (log_step >= 0 && d.log_refl) d.log_refl[(size_t)log_step * c.np + i] = (uint8_t)flags;
 }
 
 }  // namespace bdem

@@ -531,55 +531,27 @@ __global__ void k_force_sum(BdDev d, BdConst c, double2 *out) {
   out[i] = make_double2(fx, fy);
 }
 
-// step < 0: the index of the step is the device counter (graph replays)
+// step < 0: the index of the step is the device counter (graph replays).
+// At small sizes the kernel is its chain of dependent loads (status, step, slot,
+// replica, force, position one behind the other): they are issued together
+// before any is looked at.  At large sizes it is its memory traffic, about 110
+// bytes a disk (the position before the move is kept once, in pos0).
 __global__ void k_integrate(BdDev d, BdConst c, long long step, int log_step, int node) {
-  if (ctl_failed(d.ctl)) return;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= c.np) return;
-  if (i == 0) d.ctl->in_move = 1;
-  if (step < 0) step = *(volatile const long long *)&d.ctl->step_dev;
+  const int bad = ctl_failed(d.ctl);
+  const long long step_dev = *(volatile const long long *)&d.ctl->step_dev;
   const int e = d.ext_id[i];
-  if (e < 0) return;
-  const BdRep &R = d.rep[d.rep_of[i]];
-  const double2 F = bdem::force_sum(d, c, R, i);
+  const int r = c.R == 1 ? 0 : d.rep_of[i];
   const double2 p = d.pos[i];
-  d.pos0[i] = p;
-  d.prev[i] = p;
   const float th = d.theta[i];
-  d.theta0[i] = th;
-  float thn;
-  int flags = 0;
-  const bdpred::Grid g{c.q, c.inv_q, c.qshift};
-  long long X, Y;
-  if (c.precision == 0) {
-    // move, reflection and FP32 copy in grid units (no FP64 arithmetic)
-    bdem::em_move_grid(c, R, (uint32_t)e, step, p, th, F, R.v0, &thn, (uint32_t)node, &X, &Y);
-  } else {
-    const double2 y = bdem::em_move(c, R, (uint32_t)e, step, p, th, F, R.v0, &thn, (uint32_t)node);
-    X = bdpred::to_int(y.x, g);
-    Y = bdpred::to_int(y.y, g);
-  }
-  const long long X0 = bdpred::to_int(p.x, g), Y0 = bdpred::to_int(p.y, g);
-  if (R.periodic) {
-    // the move itself (before re-entry), for the triangulation's reversal screen
-    d.dmove[i] = make_float2(bdem::grid_to_float(X - X0, c.qshift), bdem::grid_to_float(Y - Y0, c.qshift));
-    // re-entry at the opposite side (Sec. 2.1); the triangulation kernel
-    // shifts the corners of the disks that re-entered
-    const int wr = bdem::wrap_grid(R.LQ, X, Y);
-    d.wrap[i] = (uint8_t)wr;
-    if (wr && !c.overlap_verlet) atomicAdd(&d.ctl->n_wrapped, 1);
-  } else {
-    const double2 w = bdem::walls_of(d, R, i);
-    flags = bdem::reflect_grid(bdpred::to_int(w.x, g), bdpred::to_int(w.y, g), X, Y);
-  }
-  d.pos[i] = make_double2(bdem::grid_to_double(X, c.qshift), bdem::grid_to_double(Y, c.qshift));
-  if (!R.periodic)
-    d.dmove[i] = make_float2(bdem::grid_to_float(X - X0, c.qshift), bdem::grid_to_float(Y - Y0, c.qshift));
-  const float2 sx = bdem::grid_split(X, c.qshift), sy = bdem::grid_split(Y, c.qshift);
-  d.work[i] = make_float4(sx.x, sy.x, sx.y, sy.y);
-  d.theta[i] = thn;
-  d.moved[i] = 1;
-  if (log_step >= 0 && d.log_refl) d.log_refl[(size_t)log_step * c.np + i] = (uint8_t)flags;
+  const double2 F0 = d.fpart[i];
+  if (bad) return;
+  if (i == 0) d.ctl->in_move = 1;
+  if (step < 0) step = step_dev;
+  if (e < 0) return;
+  const BdRep &R = d.rep[r];
+  bdem::move_disk(d, c, R, i, e, step, log_step, node, p, th, bdem::force_sum(d, c, R, i, F0));
 }
 
 // all pieces of a halved step completed: the step counts as one time step

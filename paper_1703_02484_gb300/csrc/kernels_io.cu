@@ -38,7 +38,6 @@ __global__ void k_state_check(BdDev d, BdConst c) {
   if (i >= c.np) return;
   const double2 o = d.pos[i];
   d.pos0[i] = o;
-  d.prev[i] = o;
   d.theta0[i] = d.theta[i];
   d.moved[i] = 0;
   const int e = d.ext_glob[i];

@@ -337,7 +337,7 @@ int bd_set_force_params(bd_handle *h, const double *alpha, double v0) {
     }
     if (isfinite(v0)) {
       p.v0 = v0;
-      B.v0 = v0;
+      bdcapi::rep_set_v0(B, v0);
     }
   }
   if (h->ro) h->ro->recorded = false;
@@ -568,7 +568,7 @@ int bd_rollout_replay(bd_handle *h, const double *alpha, double v0, double *loss
   const BdRep saved = h->h_rep[0];
   BdRep &B = h->h_rep[0];
   if (alpha) bdcapi::rep_set_alpha(B, alpha, h->reps[0].p.n_species);
-  if (isfinite(v0)) B.v0 = v0;
+  if (isfinite(v0)) bdcapi::rep_set_v0(B, v0);
   e = upload_rep(h);
   const BdDev dr = replay_dev(h, r);
   if (e == cudaSuccess) e = load_checkpoint(h, r, dr, 0);
