@@ -1306,19 +1306,23 @@ cudaError_t capture_step_graph(bd_handle *h) {
   e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return e;
   cudaError_t el = cudaSuccess;
-  if (h->c.any_long) {
-    if (tm) el = cudaEventRecordWithFlags(h->graph_ev[0], cs, cudaEventRecordExternal);
+  if (tm) {
+    // the force's launches between the events, the move in a launch of its own
+    el = cudaEventRecordWithFlags(h->graph_ev[0], cs, cudaEventRecordExternal);
     if (el == cudaSuccess) el = bd_launch_force_long(h->d, h->c, cs);
-    if (el == cudaSuccess && tm) el = cudaEventRecordWithFlags(h->graph_ev[1], cs, cudaEventRecordExternal);
+    if (el == cudaSuccess) el = cudaEventRecordWithFlags(h->graph_ev[1], cs, cudaEventRecordExternal);
     launches += bd_force_launches(h->c);
+    if (el == cudaSuccess && h->c.any_short) {
+      el = bd_launch_force_short(h->d, h->c, cs);
+      launches += bd_short_launches();
+    }
+    if (el == cudaSuccess) el = bd_launch_integrate(h->d, h->c, -1, -1, cs);
+    ++launches;
+  } else {
+    el = bd_launch_force_move(h->d, h->c, -1, -1, cs, 1, &launches);
   }
-  if (el == cudaSuccess && h->c.any_short) {
-    el = bd_launch_force_short(h->d, h->c, cs);
-    launches += bd_short_launches();
-  }
-  if (el == cudaSuccess) el = bd_launch_integrate(h->d, h->c, -1, -1, cs);
   if (el == cudaSuccess) el = launch_correction(h, cs);
-  launches += 2;
+  ++launches;
   cudaGraph_t g = nullptr;
   e = cudaStreamEndCapture(cs, &g);
   if (el != cudaSuccess || e != cudaSuccess) {
@@ -1458,19 +1462,12 @@ cudaError_t halving_snapshot(bd_handle *h, bool save) {
 cudaError_t launch_piece(bd_handle *h, int node, int64_t *launches) {
   cudaStream_t st = h->stream;
   cudaError_t e = cudaSuccess;
-  if (h->c.any_long) {
-    e = bd_launch_force_long(h->d, h->c, st);
-    *launches += bd_force_launches(h->c);
-  }
-  if (e == cudaSuccess && h->c.any_short) {
-    e = bd_launch_force_short(h->d, h->c, st);
-    *launches += bd_short_launches();
-  }
-  if (e == cudaSuccess) e = bd_launch_integrate(h->d, h->c, h->step, -1, st, node);
+  int n = 1;
+  e = bd_launch_force_move(h->d, h->c, h->step, -1, st, node, &n);
   if (e == cudaSuccess)
     e = h->c.overlap_verlet ? bd_launch_overlap_verlet(h->d, h->c, st, h->vc_grid, h->vc_block, 0)
                             : bd_launch_dt(h->d, h->c, 2, st, h->dt_grid, h->dt_block);
-  *launches += 2;
+  *launches += n;
   return e;
 }
 

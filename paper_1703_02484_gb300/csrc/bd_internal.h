@@ -280,6 +280,12 @@ int bd_short_launches();
 int bd_vl_grid_for(int np, int *grid);
 cudaError_t bd_launch_force_sum(const BdDev &d, const BdConst &c, double2 *out, cudaStream_t s);
 cudaError_t bd_launch_force_f64s(const BdDev &d, const BdConst &c, cudaStream_t s);
+// forces and the move of a step (or piece), in as few launches as they take; *launches grows by them
+#define BD_MOVE_FUSED 8192   // slots up to which the move runs in the force's reduction
+cudaError_t bd_launch_force_move(const BdDev &d, const BdConst &c, int64_t step, int log_step, cudaStream_t s, int node,
+                                 int *launches);
+cudaError_t bd_launch_force_sym_move(const BdDev &d, const BdConst &c, int variant, int64_t step, int log_step,
+                                     cudaStream_t s, int node);
 cudaError_t bd_launch_force_sym(const BdDev &d, const BdConst &c, int variant, cudaStream_t s);
 // advance = 0: a piece of a halved step (the step counter does not advance);
 // advance = -1: positions set from outside, a pair closer than sigma rejects them

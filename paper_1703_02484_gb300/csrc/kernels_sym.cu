@@ -579,8 +579,14 @@ __global__ void __launch_bounds__(NW * 32, MINB) k_force_long_sym_mb(BdDev d, Bd
 // shares' sums are added in a fixed order.  Sums are float-float (TwoSum into
 // a (hi, lo) FP32 pair, about 48 bits): FP64 adds run at 1/64 of the FP32 rate
 // on this part and would bound the kernel.
-template <int ND, int NS>
-__global__ void __launch_bounds__(ND * NS) k_force_sym_reduce(BdDev d, BdConst c) {
+// MOVE: the disks' move (k_integrate's) in the same kernel by the first share's
+// threads, whose loads are issued before the sums: a step of a few thousand
+// disks spends as long on a launch and its first loads as on the work.
+// Four partials in flight against two: 2884 -> 2871 us for 20 steps of 16384
+// disks, 2009 -> 2004 for four of 350000 in 64 boxes.
+template <int ND, int NS, bool MOVE>
+__global__ void __launch_bounds__(ND * NS) k_force_sym_reduce(BdDev d, BdConst c, long long step, int log_step,
+                                                              int node) {
   __shared__ float4 part[NS][ND];
   if (ctl_failed(d.ctl)) return;
   const int g = threadIdx.x / ND, dl = threadIdx.x % ND;
@@ -588,9 +594,32 @@ __global__ void __launch_bounds__(ND * NS) k_force_sym_reduce(BdDev d, BdConst c
   const int P = i / BD_SB, t = i / BD_SG;            // the same for the whole warp
   const float2 *ib = d.ipart + (i - P * BD_SB);
   const float2 *jb = d.jpart + (i - t * BD_SG);
+  int e = -1;
+  double2 p = make_double2(0.0, 0.0);
+  float th = 0.f;
+  long long step_dev = 0;
+  if (MOVE && g == 0) {
+    e = d.ext_id[i];
+    p = d.pos[i];
+    th = d.theta[i];
+    step_dev = *(volatile const long long *)&d.ctl->step_dev;
+  }
   float xh[2] = {0.f, 0.f}, xl[2] = {0.f, 0.f}, yh[2] = {0.f, 0.f}, yl[2] = {0.f, 0.f};
   auto run = [&](const int *idx, int k0, int k1, const float2 *b, int stride) {
     int k = k0 + g;
+    for (; k + 3 * NS < k1; k += 4 * NS) {   // four partials in flight
+      const int i0 = __ldg(idx + k), i1 = __ldg(idx + k + NS), i2 = __ldg(idx + k + 2 * NS), i3 = __ldg(idx + k + 3 * NS);
+      const float2 v0 = b[(size_t)i0 * stride], v1 = b[(size_t)i1 * stride];
+      const float2 v2 = b[(size_t)i2 * stride], v3 = b[(size_t)i3 * stride];
+      two_sum(xh[0], xl[0], v0.x);
+      two_sum(yh[0], yl[0], v0.y);
+      two_sum(xh[1], xl[1], v1.x);
+      two_sum(yh[1], yl[1], v1.y);
+      two_sum(xh[0], xl[0], v2.x);
+      two_sum(yh[0], yl[0], v2.y);
+      two_sum(xh[1], xl[1], v3.x);
+      two_sum(yh[1], yl[1], v3.y);
+    }
     for (; k + NS < k1; k += 2 * NS) {
       const float2 v0 = b[(size_t)__ldg(idx + k) * stride];
       const float2 v1 = b[(size_t)__ldg(idx + k + NS) * stride];
@@ -613,7 +642,13 @@ __global__ void __launch_bounds__(ND * NS) k_force_sym_reduce(BdDev d, BdConst c
   __syncthreads();
   if (g != 0) return;
   const int r = d.rep_of[i];
-  if (r < 0 || d.rep[r].law != BD_LAW_LONG) return;
+  if (MOVE && i == 0) d.ctl->in_move = 1;
+  if (r < 0) return;
+  const BdRep &R = d.rep[r];
+  if (R.law != BD_LAW_LONG) {   // no force law
+    if (MOVE) bdem::move_disk(d, c, R, i, e, step < 0 ? step_dev : step, log_step, node, p, th, make_double2(0.0, 0.0));
+    return;
+  }
   float sx = 0.f, ex = 0.f, sy = 0.f, ey = 0.f;
 #pragma unroll
   for (int m = 0; m < NS; ++m) {
@@ -623,7 +658,9 @@ __global__ void __launch_bounds__(ND * NS) k_force_sym_reduce(BdDev d, BdConst c
     ex = __fadd_rn(ex, q.y);
     ey = __fadd_rn(ey, q.w);
   }
-  d.fpart[i] = make_double2((double)sx + (double)ex, (double)sy + (double)ey);
+  const double2 F = make_double2((double)sx + (double)ex, (double)sy + (double)ey);
+  d.fpart[i] = F;
+  if (MOVE) bdem::move_disk(d, c, R, i, e, step < 0 ? step_dev : step, log_step, node, p, th, F);
 }
 
 int bd_force_launches(const BdConst &c) { return (c.precision == 0 ? c.force_variant >= 2 : c.f64_sym) ? 2 : 1; }
@@ -645,8 +682,7 @@ int bd_force_sym_blocks_per_sm(int variant, int periodic) {
 }
 
 // variant 2: 4 warps x 4 disks per lane; variant 3: 2 warps x 8 disks per lane
-cudaError_t bd_launch_force_sym(const BdDev &d, const BdConst &c, int variant, cudaStream_t s) {
-  if (c.n_sitems == 0) return cudaSuccess;
+static void launch_sweep(const BdDev &d, const BdConst &c, int variant, cudaStream_t s) {
   // periodic boxes (any replica) take the form with minimum images
   if (c.any_periodic) {
     // measured at N = 1e5 (periodic), step times with pair forms chosen per
@@ -671,7 +707,19 @@ cudaError_t bd_launch_force_sym(const BdDev &d, const BdConst &c, int variant, c
       // lane (+2.7 %)
       k_force_long_sym_mb<2, 4, 1, false, 2, false, 16, 1, 2><<<c.n_sitems, 64, 0, s>>>(d, c);
   }
-  if (c.np < BD_RED_SMALL) k_force_sym_reduce<32, 16><<<c.np / 32, 512, 0, s>>>(d, c);
-  else k_force_sym_reduce<64, 4><<<c.np / 64, 256, 0, s>>>(d, c);
+}
+
+cudaError_t bd_launch_force_sym(const BdDev &d, const BdConst &c, int variant, cudaStream_t s) {
+  if (c.n_sitems == 0) return cudaSuccess;
+  launch_sweep(d, c, variant, s);
+  if (c.np < BD_RED_SMALL) k_force_sym_reduce<32, 16, false><<<c.np / 32, 512, 0, s>>>(d, c, 0, 0, 0);
+  else k_force_sym_reduce<64, 4, false><<<c.np / 64, 256, 0, s>>>(d, c, 0, 0, 0);
+  return cudaGetLastError();
+}
+
+cudaError_t bd_launch_force_sym_move(const BdDev &d, const BdConst &c, int variant, int64_t step, int log_step,
+                                     cudaStream_t s, int node) {
+  launch_sweep(d, c, variant, s);
+  k_force_sym_reduce<32, 16, true><<<c.np / 32, 512, 0, s>>>(d, c, (long long)step, log_step, node);
   return cudaGetLastError();
 }

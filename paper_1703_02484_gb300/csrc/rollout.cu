@@ -421,10 +421,10 @@ int bd_rollout(bd_handle *h, int32_t nsteps, int32_t ckpt_every, int32_t loss_ki
       attach_log(h, r);
       e = bdcapi::reset_stats(h);
       for (int t = t0; t < t1 && e == cudaSuccess; ++t) {
-        e = bd_launch_force_long(h->d, h->c, s);
-        if (e == cudaSuccess) e = bd_launch_integrate(h->d, h->c, r->step0 + t, t, s);
+        int n = 1;
+        e = bd_launch_force_move(h->d, h->c, r->step0 + t, t, s, 1, &n);
         if (e == cudaSuccess) e = bd_launch_dt(h->d, h->c, 0, s, h->dt_grid, h->dt_block, t);
-        launches += 2 + bd_force_launches(h->c);
+        launches += n;
       }
       if (e != cudaSuccess) break;
       int rc = bdcapi::read_ctl(h);
