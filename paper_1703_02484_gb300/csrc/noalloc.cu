@@ -231,15 +231,26 @@ extern "C" int bd_forces_noalloc(int32_t n, const double *xy, const uint8_t *spe
   NaArgs g;
   g.n = n;
   int iblocks = (n + BD_NA_THREADS * BD_NA_IPT - 1) / (BD_NA_THREADS * BD_NA_IPT);
-  // j chunks so that the grid fills the eight blocks an SM holds (once: a
-  // second, partly filled wave would idle SMs), at least 64 disks j each, and
-  // as many as the scratch holds partial forces for
-  int nchunk = 8 * sms / iblocks;
+  // j chunks: at most as many as fill the eight blocks an SM holds (once: a
+  // second, partly filled wave would idle SMs) and as the scratch holds partial
+  // forces for, at least 64 disks j each; among these the count that leaves the
+  // fullest SM the least work, blocks per SM times the chunk (30011 disks: 18
+  // chunks, seven blocks on every SM, instead of 19, eight on some)
+  int most = 8 * sms / iblocks;
   const int room = (int)(BD_NOALLOC_BYTES / 16 / (size_t)n);
-  nchunk = nchunk > room ? room : nchunk;
-  nchunk = nchunk > BD_NOALLOC_MAX_CHUNKS ? BD_NOALLOC_MAX_CHUNKS : nchunk;
-  nchunk = nchunk > (n + 63) / 64 ? (n + 63) / 64 : nchunk;
-  nchunk = nchunk < 1 ? 1 : nchunk;
+  most = most > room ? room : most;
+  most = most > BD_NOALLOC_MAX_CHUNKS ? BD_NOALLOC_MAX_CHUNKS : most;
+  most = most > (n + 63) / 64 ? (n + 63) / 64 : most;
+  most = most < 1 ? 1 : most;
+  int nchunk = most;
+  long long best = -1;
+  for (int k = most; k >= 1 && 2 * k >= most; --k) {
+    const long long load = (long long)((iblocks * k + sms - 1) / sms) * ((n + k - 1) / k);
+    if (best < 0 || load < best) {
+      best = load;
+      nchunk = k;
+    }
+  }
   g.nchunk = nchunk;
   g.xy = (const double2 *)xy;
   g.sp = species;
