@@ -984,7 +984,6 @@ int build_handle(const std::vector<Spec> &specs, void *stream, bd_handle **out) 
     BD_TRY(dalloc(h, &d.iorigin, (size_t)std::max(1, iblock)));
     BD_TRY(dalloc(h, &d.tile_species, std::max<size_t>(1, tile_sp.size())));
     BD_TRY(dalloc(h, &d.ctl, 1));
-    BD_TRY(dalloc(h, &h->d_fsum, (size_t)np));
     BD_TRY(cudaMallocHost((void **)&h->h_ctl, sizeof(BdCtl)));
     // partial-force slots: enough for the finest chunking tried (at most 64).
     // The FP64 sweep (one disk per thread) cuts j ranges finer than tiles:
@@ -1920,24 +1919,22 @@ int bd_set_wait_limit(bd_handle *h, double seconds, int32_t hold_barrier) {
 int bd_compute_forces(bd_handle *h, double *F) {
   if (!h || !F) return BD_ERR_ARG;
   cudaStream_t st = h->stream;
-  const int n = h->n, np = h->np;
   cudaError_t e = cudaSuccess;
   if (h->c.any_long) e = bd_launch_force_long(h->d, h->c, st);
   if (e == cudaSuccess && h->c.any_short) e = bd_launch_force_short(h->d, h->c, st);
-  if (e == cudaSuccess) e = bd_launch_force_sum(h->d, h->c, h->d_fsum, st);
-  std::vector<double2> f(np);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(f.data(), h->d_fsum, np * sizeof(double2), cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return cuda_fail(e);
-  int rc = read_ctl(h);
-  if (rc) return rc;
-  if (h->h_ctl->status) return finish_status(h, h->h_ctl->status);
-  for (int i = 0; i < n; ++i) {
-    double2 v = f[h->int_of_ext[i]];
-    F[2 * i] = v.x;
-    F[2 * i + 1] = v.y;
+  if (h->c.any_short) {
+    // only the Verlet lists' rebuild can fail
+    const int rc = read_ctl(h);
+    if (rc) return rc;
+    if (h->h_ctl->status) return finish_status(h, h->h_ctl->status);
   }
-  return BD_OK;
+  // put into the caller's order on the device, one copy into the caller's array
+  e = bd_launch_force_out(h->d, h->c, h->d.xfer_xy, st);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(F, h->d.xfer_xy, (size_t)h->n * sizeof(double2), cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  return e == cudaSuccess ? BD_OK : cuda_fail(e);
 }
 
 int bd_get_neighbors(bd_handle *h, int32_t max_per, int32_t *counts, int32_t *idx) {

@@ -37,7 +37,6 @@ struct bd_handle {
   int dt_grid = 0, dt_block = 0;
   int vc_grid = 0, vc_block = 0;   // Verlet-list overlap correction launch
   int64_t step = 0;
-  double2 *d_fsum = nullptr;
   BdCtl *h_ctl = nullptr;          // pinned
   std::vector<void *> dev_allocs;
   bool timing = false;

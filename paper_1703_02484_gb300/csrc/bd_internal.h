@@ -278,7 +278,8 @@ cudaError_t bd_launch_periodic_wraps(const BdDev &d, const BdConst &c, cudaStrea
 cudaError_t bd_launch_force_short(const BdDev &d, const BdConst &c, cudaStream_t s);
 int bd_short_launches();
 int bd_vl_grid_for(int np, int *grid);
-cudaError_t bd_launch_force_sum(const BdDev &d, const BdConst &c, double2 *out, cudaStream_t s);
+// the forces of the last evaluation, caller's order (n entries)
+cudaError_t bd_launch_force_out(const BdDev &d, const BdConst &c, double2 *out, cudaStream_t s);
 cudaError_t bd_launch_force_f64s(const BdDev &d, const BdConst &c, cudaStream_t s);
 // forces and the move of a step (or piece), in as few launches as they take; *launches grows by them
 #define BD_MOVE_FUSED 8192   // slots up to which the move runs in the force's reduction

@@ -512,23 +512,13 @@ __global__ void __launch_bounds__(128) k_force_long_f64(BdDev d, BdConst c) {
   if (live && jc < R.nchunk) d.fpart[(size_t)jc * c.np + i] = make_double2(fx, fy);
 }
 
-__global__ void k_force_sum(BdDev d, BdConst c, double2 *out) {
+// the partial forces' sums in the caller's order
+__global__ void k_force_out(BdDev d, BdConst c, double2 *out) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= c.np) return;
-  const int r = d.rep_of[i];
-  if (r < 0) {
-    out[i] = make_double2(0.0, 0.0);
-    return;
-  }
-  const BdRep &R = d.rep[r];
-  const int ns = R.law == BD_LAW_LONG ? R.nchunk : (R.law == BD_LAW_SHORT ? 1 : 0);
-  double fx = 0.0, fy = 0.0;
-  for (int k = 0; k < ns; ++k) {
-    double2 f = d.fpart[(size_t)k * c.np + i];
-    fx += f.x;
-    fy += f.y;
-  }
-  out[i] = make_double2(fx, fy);
+  const int e = d.ext_glob[i];
+  if (e < 0) return;
+  out[e] = bdem::force_sum(d, c, d.rep[d.rep_of[i]], i, d.fpart[i]);
 }
 
 // step < 0: the index of the step is the device counter (graph replays).
@@ -669,7 +659,7 @@ cudaError_t bd_launch_work_copy(const BdDev &d, const BdConst &c, cudaStream_t s
   return cudaGetLastError();
 }
 
-cudaError_t bd_launch_force_sum(const BdDev &d, const BdConst &c, double2 *out, cudaStream_t s) {
-  k_force_sum<<<(c.np + 255) / 256, 256, 0, s>>>(d, c, out);
+cudaError_t bd_launch_force_out(const BdDev &d, const BdConst &c, double2 *out, cudaStream_t s) {
+  k_force_out<<<(c.np + 255) / 256, 256, 0, s>>>(d, c, out);
   return cudaGetLastError();
 }
