@@ -1192,12 +1192,10 @@ int read_ctl(bd_handle *h) {
 }
 
 cudaError_t reset_stats(bd_handle *h) {
-  // zero everything after the barrier words, the status and the epoch
+  // the status, the phase counters and the statistics, which lie together
   char *base = (char *)h->d.ctl;
-  size_t off = offsetof(BdCtl, cnt);
-  cudaError_t e = cudaMemsetAsync(base + off, 0, offsetof(BdCtl, log_npass) - off, h->stream);
-  if (e != cudaSuccess) return e;
-  return cudaMemsetAsync(&h->d.ctl->status, 0, sizeof(int), h->stream);
+  const size_t off = offsetof(BdCtl, status);
+  return cudaMemsetAsync(base + off, 0, offsetof(BdCtl, log_npass) - off, h->stream);
 }
 
 void add_stage_times(bd_handle *h) {

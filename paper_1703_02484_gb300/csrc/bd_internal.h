@@ -51,10 +51,12 @@
 struct BdCtl {
   unsigned int bar_count;          // on a 128-byte line of its own: the blocks at a barrier arrive at it
   unsigned int pad0[31];           // and poll it
-  int status;
   unsigned int exit_count;         // blocks that have left the triangulation kernel
-  unsigned int pad1[30];
+  unsigned int pad1[31];
   unsigned long long epoch;        // flip-round counter, grows across launches
+  // from here to log_npass: cleared by every call (reset_stats)
+  int status;
+  int pad2;
   int cnt[4][8];                   // per-phase counters, rotated every barrier
   // statistics accumulated over a bd_step call
   long long st_corr_iters;
