@@ -69,7 +69,7 @@ __device__ __forceinline__ void stage_tick(BdCtl *ctl, int stage, unsigned long 
 
 }  // namespace
 
-__global__ void __launch_bounds__(BD_VC_THREADS) k_overlap_verlet(BdDev d, BdConst c, int advance) {
+__global__ void __launch_bounds__(BD_VC_THREADS, 4) k_overlap_verlet(BdDev d, BdConst c, int advance) {
   BdCtl *ctl = d.ctl;
   if (ld_status(&ctl->status) != 0) {
     block_exit(ctl);
@@ -84,7 +84,7 @@ __global__ void __launch_bounds__(BD_VC_THREADS) k_overlap_verlet(BdDev d, BdCon
   const int nth = gridDim.x * blockDim.x;
   const bool lead = (blockIdx.x == 0 && threadIdx.x == 0);
   const double sigma = c.sigma;
-  const float sig2f = (float)(sigma * sigma * (1.0 + 1e-5));
+  const float sig2f = c.sig2f;
   int status = 0, corr_iter = 0;
   // launch counter (this kernel's use of the epoch word): stamps of the
   // per-replica pass counts
@@ -127,8 +127,7 @@ __global__ void __launch_bounds__(BD_VC_THREADS) k_overlap_verlet(BdDev d, BdCon
         }
         const float4 wi = d.work[i];
         const int m = d.vl_cnt[i];
-        double sx = 0.0, sy = 0.0;
-        uint8_t hit = 0;
+        unsigned long long close = 0ull;   // entries that may overlap (a list holds at most 64)
         // four entries at a time: their positions (and moved flags) are loaded
         // together, and the next four indices while they are tested
         int jn[4];
@@ -151,23 +150,30 @@ __global__ void __launch_bounds__(BD_VC_THREADS) k_overlap_verlet(BdDev d, BdCon
           for (int u = 0; u < 4; ++u) {
             if (t0 + u >= m) break;
             if (!mv[u]) continue;   // neither end moved since the last pass
-            const int j = jj[u];
             const float fx = fdiff_p(wv[u].x, wv[u].z, wi.x, wi.z, R), fy = fdiff_p(wv[u].y, wv[u].w, wi.y, wi.w, R);
-            if (__fadd_rn(__fmul_rn(fx, fx), __fmul_rn(fy, fy)) > sig2f) continue;
-            const double2 pj = d.pos[j];
-            // the exact difference (grid units), its minimum image in a periodic box
-            const double dx = bdem::grid_to_double(imin_image(bdpred::to_int(pj.x, g) - bdpred::to_int(pi.x, g), R), c.qshift);
-            const double dy = bdem::grid_to_double(imin_image(bdpred::to_int(pj.y, g) - bdpred::to_int(pi.y, g), R), c.qshift);
-            const double r = sqrt(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)));
-            const double sg = d.rad ? d.rad[i] + d.rad[j] : sigma;   // polydisperse: a_i + a_j
-            if (r < sg) {
-              const double del = sg - r;
-              sx -= del * (dx / r);
-              sy -= del * (dy / r);
-              hit = 1;
-              if (j > i) ++nov;      // each pair counted once
-              mx = fmax(mx, del);
-            }
+            if (!(__fadd_rn(__fmul_rn(fx, fx), __fmul_rn(fy, fy)) > sig2f)) close |= 1ull << (t0 + u);
+          }
+        }
+        // the few pairs that pass the screen, decided in FP64
+        double sx = 0.0, sy = 0.0;
+        uint8_t hit = 0;
+        while (close) {
+          const int t = __ffsll((long long)close) - 1;
+          close &= close - 1ull;
+          const int j = d.vl_idx[(size_t)t * c.np + i];
+          const double2 pj = d.pos[j];
+          // the exact difference (grid units), its minimum image in a periodic box
+          const double dx = bdem::grid_to_double(imin_image(bdpred::to_int(pj.x, g) - bdpred::to_int(pi.x, g), R), c.qshift);
+          const double dy = bdem::grid_to_double(imin_image(bdpred::to_int(pj.y, g) - bdpred::to_int(pi.y, g), R), c.qshift);
+          const double r = sqrt(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)));
+          const double sg = d.rad ? d.rad[i] + d.rad[j] : sigma;   // polydisperse: a_i + a_j
+          if (r < sg) {
+            const double del = sg - r;
+            sx -= del * (dx / r);
+            sy -= del * (dy / r);
+            hit = 1;
+            if (j > i) ++nov;      // each pair counted once
+            mx = fmax(mx, del);
           }
         }
         d.disp[i] = make_double2(sx, sy);
