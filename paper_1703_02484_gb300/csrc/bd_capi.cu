@@ -1170,6 +1170,7 @@ int build_handle(const std::vector<Spec> &specs, void *stream, bd_handle **out) 
       bd_free(h);
       return BD_ERR_CUDA;
     }
+    c.tri_queue = bd_dt_queue_for(nt, h->dt_grid, h->dt_block);
   }
 #undef BD_TRY
   *out = h;

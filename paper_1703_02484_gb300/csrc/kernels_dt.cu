@@ -673,7 +673,6 @@ __device__ __forceinline__ int tri_rep(const BdDev &d, int np, const int4 &v) {
   return c < 0 ? -1 : d.rep_of[c];
 }
 
-
 }  // namespace
 
 // One time step's triangulation work (mode 0), the repair of the
@@ -698,12 +697,13 @@ __device__ __forceinline__ int tri_rep(const BdDev &d, int np, const int4 &v) {
 // Three resident blocks per SM (at most 80 registers): the passes are
 // latency-bound chains of dependent loads, and the spills this costs sit in
 // the exact-predicate fallbacks (measured: 3 blocks 20 % faster than 2 on
-// 2^20 disks; 4 blocks (64 registers) 1.5 % faster on 2^20 disks but 16 %
-// slower in the check passes at 1e5; 5 blocks slower on both).
+// 2^20 disks; 4 blocks (64 registers) the same there, 337 us per step, and 1 to
+// 3 % of a step slower at 16384 to 350000 disks).
 //
 // CL: the launch is one thread-block cluster (a small system): hardware
 // barriers, the phase words in the first block's shared memory, 128 registers.
-template <bool PER, bool CL>
+// QUEUE: the check pass of a triangulation of many triangles per thread.
+template <bool PER, bool CL, bool QUEUE>
 __device__ __forceinline__ void triangulation_body(const BdDev &d, const BdConst &c, int mode, int log_step) {
   Ctx x = {d, c, {c.q, c.inv_q, c.qshift}, c.nt, c.np, c.sig2f, 0u, d.ctl->cl_n};
   BdCtl *ctl = d.ctl;
@@ -822,10 +822,26 @@ __device__ __forceinline__ void triangulation_body(const BdDev &d, const BdConst
         int inv = 0, rej = 0, cand = 0, vis = 0;
         double mx = 0.0;
         const bool skip = !sweep_all && !c.tri_all;
-        __shared__ int s_list[BD_DT_LIST], s_nd;
+        __shared__ int s_list[BD_DT_LIST], s_nd, s_queue[QUEUE ? BD_DT_THREADS / 32 : 1][QUEUE ? 128 : 1];
         auto clean = [&](const int4 &v) -> bool {
           if (tstamp(v.w) == gen8) return false;
           return !(fresh && (d.moved[v.x] | d.moved[v.y] | d.moved[v.z]));
+        };
+        // orientation of triangle t after a move of one of its corners
+        auto turned = [&](int t, const int4 &v, const float4 &Wa, const float4 &Wb, const float4 &Wc) {
+          const int in = !PER || (v.w & BD_TRI_SHIFT_BITS) == 0
+                             ? orient_pre(x, v.x < x.np && v.y < x.np && v.z < x.np, Wa, Wb, Wc, v.x, v.y, v.z)
+                             : orient_s(x, v.x, tshx<PER>(v.w, 0), tshy<PER>(v.w, 0), v.y, tshx<PER>(v.w, 1),
+                                        tshy<PER>(v.w, 1), v.z, tshx<PER>(v.w, 2), tshy<PER>(v.w, 2));
+          if (in <= 0) {
+            // (the marks and the scan of a pass that finds one are void)
+            d.tinv[t] = 1;
+            ++inv;
+            if (d.rep_stats) {
+              const int rr = tri_rep(d, x.np, v);
+              if (rr >= 0) atomicAdd((unsigned long long *)&d.rep_stats[3 * rr + 2], 1ull);
+            }
+          }
         };
         // One corner of a triangle per item, testing the edge that faces it (and
         // for the first corner the triangle's orientation): the chain of loads and
@@ -833,11 +849,18 @@ __device__ __forceinline__ void triangulation_body(const BdDev &d, const BdConst
         // largest systems, is a third of a whole triangle's.
         // The first pass takes the corners of all triangles in turn; a later pass
         // those of the block's dirty triangles, put in a list first.
+        // QUEUE, for triangulations of many triangles per thread, whose passes are
+        // bound by instructions, spends no lanes on the half of the corners whose
+        // edge is the other side's to test: a lane takes a triangle, tests its
+        // orientation and puts the corners it has to test into its warp's queue,
+        // and the warp takes corners from there 32 at a time.
+        const int lane = threadIdx.x & 31;
+        int *const queue = s_queue[QUEUE ? threadIdx.x >> 5 : 0];
         const int share = skip ? (x.T + (int)gridDim.x - 1) / (int)gridDim.x : 0;
         const int s0 = min(x.T, (int)blockIdx.x * share), s1 = min(x.T, s0 + share);
         int base = s0;
         do {
-          int items = 3 * x.T, it = tid, stride = nth;
+          int items = x.T, it = tid, stride = nth;   // triangles, this thread's first item, the step to its next
           if (skip) {
             __syncthreads();   // (the list of the chunk before has been worked off)
             if (threadIdx.x == 0) s_nd = 0;
@@ -846,18 +869,57 @@ __device__ __forceinline__ void triangulation_body(const BdDev &d, const BdConst
             for (int t = base + (int)threadIdx.x; t < e1; t += blockDim.x)
               if (!clean(d.tv[t])) s_list[atomicAdd(&s_nd, 1)] = t;
             __syncthreads();
-            items = 3 * s_nd;
+            items = s_nd;
             it = threadIdx.x;
             stride = blockDim.x;
             base += BD_DT_LIST;
           }
-          for (; it < items; it += stride) {
-            const int t = skip ? s_list[it / 3] : it / 3, k = it % 3, cc = 3 * t + k;
+          // triangles a warp puts into its queue at a time: fewer than 32 if that keeps all warps busy
+          const int cw = min(32, (items + (stride >> 5) - 1) / (stride >> 5));
+          int w0 = (it >> 5) * cw, queued = 0;
+          for (;;) {
+            int cc;
+            if (!QUEUE) {
+              if (it >= 3 * items) break;
+              cc = skip ? 3 * s_list[it / 3] + it % 3 : it;
+              it += stride;
+            } else {
+              while (queued < 32 && w0 < items) {
+                unsigned own3 = 0u;
+                int t = w0 + lane;
+                if (lane < cw && t < items) {
+                  if (skip) t = s_list[t];
+                  const int4 v = d.tv[t], nn = d.tn[t];
+                  const int on[3] = {nn.x, nn.y, nn.z};
+#pragma unroll
+                  for (int k = 0; k < 3; ++k)
+                    if (on[k] >= 0 && (on[k] > 3 * t + k || (skip && clean(d.tv[on[k] / 3])))) own3 |= 1u << k;
+                  ++vis;
+                  if (fresh && ((d.moved[v.x] | d.moved[v.y] | d.moved[v.z]) & 1))
+                    turned(t, v, work_of(x, v.x), work_of(x, v.y), work_of(x, v.z));
+                }
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                  const unsigned m = __ballot_sync(0xffffffffu, own3 >> k & 1u);
+                  if (own3 >> k & 1u) queue[queued + __popc(m & ((1u << lane) - 1u))] = 3 * t + k;
+                  queued += __popc(m);
+                }
+                w0 += (stride >> 5) * cw;
+                __syncwarp();
+              }
+              if (queued == 0) break;
+              const int take = min(32, queued);
+              queued -= take;
+              cc = lane < take ? queue[queued + lane] : -1;
+              __syncwarp();   // (read before the next corners are put in)
+              if (cc < 0) break;   // (the last of this warp's corners: fewer than 32, none left to fetch)
+            }
+            const int t = cc / 3, k = cc % 3;
             const int4 v = d.tv[t];
             const int o = ((const int *)&d.tn[t])[k];
             // corners in order: the edge faces ia and runs from ib to ic
             const int ia = vk(v, k), ib = vk(v, (k + 1) % 3), ic = vk(v, (k + 2) % 3);
-            const bool own = o >= 0 && (o > cc || (skip && clean(d.tv[o / 3])));
+            const bool own = QUEUE || (o >= 0 && (o > cc || (skip && clean(d.tv[o / 3]))));
             if (k && !own) continue;
             const float4 Wa = work_of(x, ia), Wb = work_of(x, ib), Wc = work_of(x, ic);
             uint8_t ma = 0, mb = 0, mc = 0;   // moved; periodic box: bits 1-4 its re-entry
@@ -879,22 +941,9 @@ __device__ __forceinline__ void triangulation_body(const BdDev &d, const BdConst
             const bool due = own && (mvd || tstamp(v.w) == gen8 || tstamp(v1.w) == gen8 || (fresh && d.moved[q]));
             float4 Wq = make_float4(0.f, 0.f, 0.f, 0.f);
             if (due) Wq = work_of(x, q);
-            if (k == 0) {
+            if (!QUEUE && k == 0) {
               ++vis;
-              if (mvd) {
-                const int in = flat ? orient_pre(x, all_disks, Wa, Wb, Wc, ia, ib, ic)
-                                    : orient_s(x, ia, tshx<PER>(v.w, 0), tshy<PER>(v.w, 0), ib, tshx<PER>(v.w, 1),
-                                               tshy<PER>(v.w, 1), ic, tshx<PER>(v.w, 2), tshy<PER>(v.w, 2));
-                if (in <= 0) {
-                  // (the marks and the scan of a pass that finds one are void)
-                  d.tinv[t] = 1;
-                  ++inv;
-                  if (d.rep_stats) {
-                    const int rr = tri_rep(d, x.np, v);
-                    if (rr >= 0) atomicAdd((unsigned long long *)&d.rep_stats[3 * rr + 2], 1ull);
-                  }
-                }
-              }
+              if (mvd) turned(t, v, Wa, Wb, Wc);
               if (!own) continue;
             }
             const int u = ib, w = ic;
@@ -1244,69 +1293,69 @@ __device__ __forceinline__ void triangulation_body(const BdDev &d, const BdConst
       // length of the pass (four neighbouring disks per thread doubled it).
       int nwrap = 0;
       for (int i0 = tid; i0 < x.np; i0 += 4 * nth) {
-       unsigned marks = 0u;
+        unsigned marks = 0u;
 #pragma unroll
-       for (int u = 0; u < 4; ++u)
-         if (i0 + u * nth < x.np && d.hit[i0 + u * nth]) marks |= 1u << u;
+        for (int u = 0; u < 4; ++u)
+          if (i0 + u * nth < x.np && d.hit[i0 + u * nth]) marks |= 1u << u;
 #pragma unroll 1
-       for (int u = 0; u < 4; ++u) {
-        const int i = i0 + u * nth;
-        if (i >= x.np) break;
-        if (!(marks >> u & 1u)) {
-          d.moved[i] = 0;
+        for (int u = 0; u < 4; ++u) {
+          const int i = i0 + u * nth;
+          if (i >= x.np) break;
+          if (!(marks >> u & 1u)) {
+            d.moved[i] = 0;
+            if (PER) d.wrap[i] = 0;
+            if (log_pidx >= 0) d.log_pflags[(size_t)log_pidx * x.np + i] = 0;
+            continue;
+          }
+          d.hit[i] = 0;
           if (PER) d.wrap[i] = 0;
-          if (log_pidx >= 0) d.log_pflags[(size_t)log_pidx * x.np + i] = 0;
-          continue;
+          const double2 p = d.pos[i];
+          const double2 dd = disp_get(x, i);
+          if (dd.x == 0.0 && dd.y == 0.0) {
+            d.moved[i] = 0;
+            if (log_pidx >= 0) d.log_pflags[(size_t)log_pidx * x.np + i] = 0;
+            continue;
+          }
+          if (d.rep_stats) {
+            // the first disk of a replica moved by this pass counts the pass
+            const int rr = d.rep_of[i];
+            const unsigned long long stamp = epoch;   // distinct per pass (grows across launches), never 0
+            if (atomicExch(&d.rep_mark[rr], stamp) != stamp)
+              atomicAdd((unsigned long long *)&d.rep_stats[3 * rr], 1ull);
+          }
+          d.prev[i] = p;
+          const double mag = sqrt(__dadd_rn(__dmul_rn(dd.x, dd.x), __dmul_rn(dd.y, dd.y)));
+          // Sec. 4.4: sigma/4, half the disk's radius (its own for polydisperse disks)
+          const double cap = d.rad ? 0.5 * d.rad[i] : 0.25 * sigma;
+          const bool capped = mag > cap;
+          const double sc = capped ? cap / mag : 1.0;
+          const double2 y = make_double2(snap(__dadd_rn(p.x, __dmul_rn(dd.x, sc)), x.g),
+                                         snap(__dadd_rn(p.y, __dmul_rn(dd.y, sc)), x.g));
+          int rfl = 0;
+          const BdRep &R = d.rep[d.rep_of[i]];
+          double2 np2;
+          if (PER && R.periodic) {
+            // Algorithm 2 "applying the periodic boundary conditions": re-entry
+            long long X = bdpred::to_int(y.x, x.g), Y = bdpred::to_int(y.y, x.g);
+            d.dmove[i] = make_float2(bdem::grid_to_float(X - bdpred::to_int(p.x, x.g), x.g.s),
+                                     bdem::grid_to_float(Y - bdpred::to_int(p.y, x.g), x.g.s));
+            const int wr = bdem::wrap_grid(R.LQ, X, Y);
+            d.wrap[i] = (uint8_t)wr;
+            if (wr) ++nwrap;
+            np2 = make_double2(bdem::grid_to_double(X, x.g.s), bdem::grid_to_double(Y, x.g.s));
+          } else {
+            np2 = bdem::reflect_w(bdem::walls_of(d, R, i), y, &rfl);
+          }
+          if (log_pidx >= 0) d.log_pflags[(size_t)log_pidx * x.np + i] = (uint8_t)(rfl | (capped ? 16 : 0));
+          d.pos[i] = np2;
+          d.work[i] = split_pos(np2);
+          if (!(PER && R.periodic)) {
+            d.dmove[i] = make_float2(bdem::grid_to_float(bdpred::to_int(np2.x, x.g) - bdpred::to_int(p.x, x.g), x.g.s),
+                                     bdem::grid_to_float(bdpred::to_int(np2.y, x.g) - bdpred::to_int(p.y, x.g), x.g.s));
+          }
+          d.disp[i] = make_double2(0.0, 0.0);
+          d.moved[i] = 1;
         }
-        d.hit[i] = 0;
-        if (PER) d.wrap[i] = 0;
-        const double2 p = d.pos[i];
-        const double2 dd = disp_get(x, i);
-        if (dd.x == 0.0 && dd.y == 0.0) {
-          d.moved[i] = 0;
-          if (log_pidx >= 0) d.log_pflags[(size_t)log_pidx * x.np + i] = 0;
-          continue;
-        }
-        if (d.rep_stats) {
-          // the first disk of a replica moved by this pass counts the pass
-          const int rr = d.rep_of[i];
-          const unsigned long long stamp = epoch;   // distinct per pass (grows across launches), never 0
-          if (atomicExch(&d.rep_mark[rr], stamp) != stamp)
-            atomicAdd((unsigned long long *)&d.rep_stats[3 * rr], 1ull);
-        }
-        d.prev[i] = p;
-        const double mag = sqrt(__dadd_rn(__dmul_rn(dd.x, dd.x), __dmul_rn(dd.y, dd.y)));
-        // Sec. 4.4: sigma/4, half the disk's radius (its own for polydisperse disks)
-        const double cap = d.rad ? 0.5 * d.rad[i] : 0.25 * sigma;
-        const bool capped = mag > cap;
-        const double sc = capped ? cap / mag : 1.0;
-        const double2 y = make_double2(snap(__dadd_rn(p.x, __dmul_rn(dd.x, sc)), x.g),
-                                       snap(__dadd_rn(p.y, __dmul_rn(dd.y, sc)), x.g));
-        int rfl = 0;
-        const BdRep &R = d.rep[d.rep_of[i]];
-        double2 np2;
-        if (PER && R.periodic) {
-          // Algorithm 2 "applying the periodic boundary conditions": re-entry
-          long long X = bdpred::to_int(y.x, x.g), Y = bdpred::to_int(y.y, x.g);
-          d.dmove[i] = make_float2(bdem::grid_to_float(X - bdpred::to_int(p.x, x.g), x.g.s),
-                                   bdem::grid_to_float(Y - bdpred::to_int(p.y, x.g), x.g.s));
-          const int wr = bdem::wrap_grid(R.LQ, X, Y);
-          d.wrap[i] = (uint8_t)wr;
-          if (wr) ++nwrap;
-          np2 = make_double2(bdem::grid_to_double(X, x.g.s), bdem::grid_to_double(Y, x.g.s));
-        } else {
-          np2 = bdem::reflect_w(bdem::walls_of(d, R, i), y, &rfl);
-        }
-        if (log_pidx >= 0) d.log_pflags[(size_t)log_pidx * x.np + i] = (uint8_t)(rfl | (capped ? 16 : 0));
-        d.pos[i] = np2;
-        d.work[i] = split_pos(np2);
-        if (!(PER && R.periodic)) {
-          d.dmove[i] = make_float2(bdem::grid_to_float(bdpred::to_int(np2.x, x.g) - bdpred::to_int(p.x, x.g), x.g.s),
-                                   bdem::grid_to_float(bdpred::to_int(np2.y, x.g) - bdpred::to_int(p.y, x.g), x.g.s));
-        }
-        d.disp[i] = make_double2(0.0, 0.0);
-        d.moved[i] = 1;
-       }
       }
       if (PER) block_add(&ctl->n_wrapped, nwrap);
     }
@@ -1367,15 +1416,15 @@ __device__ __forceinline__ void triangulation_body(const BdDev &d, const BdConst
   leave();
 }
 
-template <bool PER>
-__global__ void __launch_bounds__(BD_DT_THREADS, 3) k_triangulation(const __grid_constant__ BdDev d, const __grid_constant__ BdConst c, int mode,
-                                                                     int log_step) {
-  triangulation_body<PER, false>(d, c, mode, log_step);
+template <bool PER, bool QUEUE>
+__global__ void __launch_bounds__(BD_DT_THREADS, 3)
+    k_triangulation(const __grid_constant__ BdDev d, const __grid_constant__ BdConst c, int mode, int log_step) {
+  triangulation_body<PER, false, QUEUE>(d, c, mode, log_step);
 }
 template <bool PER>
-__global__ void __launch_bounds__(BD_DTC_THREADS, 1) k_triangulation_cl(const __grid_constant__ BdDev d, const __grid_constant__ BdConst c, int mode,
-                                                                     int log_step) {
-  triangulation_body<PER, true>(d, c, mode, log_step);
+__global__ void __launch_bounds__(BD_DTC_THREADS, 1)
+    k_triangulation_cl(const __grid_constant__ BdDev d, const __grid_constant__ BdConst c, int mode, int log_step) {
+  triangulation_body<PER, true, false>(d, c, mode, log_step);
 }
 
 // Undo a step whose persistent kernel left at a timed-out barrier (the
@@ -1449,9 +1498,13 @@ int bd_dt_grid(int *grid, int *block) {
   int dev = 0, sms = 0, per = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return -1;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return -1;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_triangulation<false>, BD_DT_THREADS, 0) !=
-      cudaSuccess)
-    return -1;
+  const void *fns[4] = {(const void *)k_triangulation<false, false>, (const void *)k_triangulation<true, false>,
+                        (const void *)k_triangulation<false, true>, (const void *)k_triangulation<true, true>};
+  for (int i = 0; i < 4; ++i) {
+    int n = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fns[i], BD_DT_THREADS, 0) != cudaSuccess) return -1;
+    per = i == 0 || n < per ? n : per;
+  }
   if (per < 1) return -1;
   *grid = sms * per;
   *block = BD_DT_THREADS;
@@ -1460,7 +1513,10 @@ int bd_dt_grid(int *grid, int *block) {
 
 // One cluster serves triangulations of up to BD_DTC_TRIS triangles: its barriers
 // cost a fraction of the grid's, its threads (8192 in sixteen blocks) are fewer.
-#define BD_DTC_TRIS 16384
+// Cluster against grid, us per step: 139 -> 117 with walls at 777 disks coupled
+// to a fluid (1985 triangles), 75 -> 67 at 1024 disks (2.6e3), but 172 -> 180 in
+// a rollout of 4096 disks with its gradient (8.6e3).
+#define BD_DTC_TRIS 4096
 int bd_dt_cluster_for(int nt) {
   const char *env = getenv("BD_TRI_CLUSTER");   // 0: never, n: up to n triangles
   const int most = env ? atoi(env) : BD_DTC_TRIS;
@@ -1488,6 +1544,16 @@ int bd_dt_cluster_for(int nt) {
   return 0;
 }
 
+// Check passes through the warps' queues from more than BD_DT_QUEUE triangles per
+// thread on: first check pass of 2^20 disks (18 per thread) 121 -> 84 us, of 64
+// boxes of 350000 disks in all (6) 46 -> 39 us with as much lost in the passes after
+// it, of 16384 disks (a third) 10.0 -> 10.3 us.
+#define BD_DT_QUEUE 8
+int bd_dt_queue_for(int nt, int grid, int block) {
+  const char *env = getenv("BD_TRI_QUEUE");   // triangles per thread
+  return nt > (long long)(env ? atoi(env) : BD_DT_QUEUE) * grid * block;
+}
+
 cudaError_t bd_launch_dt(const BdDev &d, const BdConst &c, int mode, cudaStream_t s, int grid,
                          int block, int log_step) {
   // the barrier words and phase counters were reset by the previous
@@ -1510,6 +1576,8 @@ cudaError_t bd_launch_dt(const BdDev &d, const BdConst &c, int mode, cudaStream_
     return cudaLaunchKernelExC(
         &cfg, c.any_periodic ? (const void *)k_triangulation_cl<true> : (const void *)k_triangulation_cl<false>, args);
   }
-  const void *fn = c.any_periodic ? (const void *)k_triangulation<true> : (const void *)k_triangulation<false>;
+  const void *fn = c.any_periodic
+                       ? c.tri_queue ? (const void *)k_triangulation<true, true> : (const void *)k_triangulation<true, false>
+                       : c.tri_queue ? (const void *)k_triangulation<false, true> : (const void *)k_triangulation<false, false>;
   return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(block), args, 0, s);
 }
