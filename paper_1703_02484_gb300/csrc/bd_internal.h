@@ -285,9 +285,15 @@ int bd_vl_grid_for(int np, int *grid);
 cudaError_t bd_launch_force_out(const BdDev &d, const BdConst &c, double2 *out, cudaStream_t s);
 cudaError_t bd_launch_force_f64s(const BdDev &d, const BdConst &c, cudaStream_t s);
 // forces and the move of a step (or piece), in as few launches as they take; *launches grows by them
-#define BD_MOVE_FUSED 8192   // slots up to which the move runs in the force's reduction
+// Slots up to which the move runs in the FP32 force's reduction: as many as its
+// blocks serve in one wave (152 SMs x 4 blocks x 32 disks).  Step of 16384 disks
+// 137.2 -> 135.5 us, of a 4096-disk rollout with its gradient 173.3 -> 171.9; at
+// 30720 slots in a periodic box 353.3 apart, 355.6 together.
+#define BD_MOVE_FUSED 19456
 cudaError_t bd_launch_force_move(const BdDev &d, const BdConst &c, int64_t step, int log_step, cudaStream_t s, int node,
                                  int *launches);
+cudaError_t bd_launch_force_f64s_move(const BdDev &d, const BdConst &c, int64_t step, int log_step, cudaStream_t s,
+                                      int node);
 cudaError_t bd_launch_force_sym_move(const BdDev &d, const BdConst &c, int variant, int64_t step, int log_step,
                                      cudaStream_t s, int node);
 cudaError_t bd_launch_force_sym(const BdDev &d, const BdConst &c, int variant, cudaStream_t s);

@@ -144,26 +144,55 @@ __device__ __forceinline__ float3 normals_f32(const bdrng::U4 &r) {
                      fminf(3.0f, fmaxf(-3.0f, rb * c2)));
 }
 
-__device__ __forceinline__ double3 normals_f64(const bdrng::U4 &r) {
+__device__ __forceinline__ double2 normal_pair(uint32_t a, uint32_t b) {
   const double sc = 2.3283064365386962890625e-10;
-  double u0 = ((double)r.x + 0.5) * sc, u1 = ((double)r.y + 0.5) * sc;
-  double u2 = ((double)r.z + 0.5) * sc, u3 = ((double)r.w + 0.5) * sc;
-  double ra = sqrt(-2.0 * log(u0)), rb = sqrt(-2.0 * log(u2));
-  double s1, c1, s2, c2;
+  const double u0 = ((double)a + 0.5) * sc, u1 = ((double)b + 0.5) * sc;
+  const double ra = sqrt(-2.0 * log(u0));
+  double s1, c1;
   sincospi(2.0 * u1, &s1, &c1);
-  sincospi(2.0 * u3, &s2, &c2);
-  return make_double3(fmin(3.0, fmax(-3.0, ra * c1)), fmin(3.0, fmax(-3.0, ra * s1)),
-                      fmin(3.0, fmax(-3.0, rb * c2)));
+  return make_double2(fmin(3.0, fmax(-3.0, ra * c1)), fmin(3.0, fmax(-3.0, ra * s1)));
 }
 
-// FP32 move of piece `node` of step `step` in grid units (before
-// reflection): X = x/q + rint(dx/q) with the increment dx formed in FP32;
-// *thn = new angle
-__device__ __forceinline__ void em_move_grid(const BdConst &c, const BdRep &R, uint32_t id,
-                                             long long step, double2 p, float th, double2 F,
-                                             float *thn, uint32_t node, long long *X,
+__device__ __forceinline__ double3 normals_f64(const bdrng::U4 &r) {
+  const double2 a = normal_pair(r.x, r.y), b = normal_pair(r.z, r.w);
+  return make_double3(a.x, a.y, b.x);
+}
+
+// what a move takes from its disk's random numbers and direction alone
+template <class T>
+struct Draw {
+  T z0, z1, z2, st, ct;   // the three normals; sin and cos of the direction
+};
+
+__device__ __forceinline__ bdrng::U4 words_of(const BdRep &R, uint32_t id, long long step, uint32_t node) {
+  return bdrng::draw(id, (int64_t)step, R.seed, R.replica, piece_tag(node));
+}
+
+__device__ __forceinline__ Draw<float> draw_f32(const BdRep &R, uint32_t id, long long step, uint32_t node, float th) {
+  const float3 z = normals_f32(words_of(R, id, step, node));
+  Draw<float> w;
+  w.z0 = z.x;
+  w.z1 = z.y;
+  w.z2 = z.z;
+  sincosf(th, &w.st, &w.ct);
+  return w;
+}
+
+__device__ __forceinline__ Draw<double> draw_f64(const BdRep &R, uint32_t id, long long step, uint32_t node, float th) {
+  const double3 z = normals_f64(words_of(R, id, step, node));
+  Draw<double> w;
+  w.z0 = z.x;
+  w.z1 = z.y;
+  w.z2 = z.z;
+  sincos((double)th, &w.st, &w.ct);
+  return w;
+}
+
+// FP32 move of piece `node` in grid units (before reflection): X = x/q +
+// rint(dx/q) with the increment dx formed in FP32; *thn = new angle
+__device__ __forceinline__ void em_move_grid(const BdConst &c, const BdRep &R, double2 p, float th, double2 F,
+                                             const Draw<float> &w, float *thn, uint32_t node, long long *X,
                                              long long *Y, float2 *move) {
-  bdrng::U4 r = bdrng::draw(id, (int64_t)step, R.seed, R.replica, piece_tag(node));
   const int depth = piece_depth(node);
   // length of this move and its noise amplitudes: dt / 2^depth, amp / 2^(depth/2)
   // (rounded to FP32 on the host: a conversion costs a thread as much as 32 FP32 operations)
@@ -174,14 +203,10 @@ __device__ __forceinline__ void em_move_grid(const BdConst &c, const BdRep &R, u
     amp = (float)(R.amp * sc);
     amp_r = (float)(R.amp_r * sc);
   }
-  const float3 z = normals_f32(r);
-  const float z0 = z.x, z1 = z.y, z2 = z.z;
-  float st, ct;
-  sincosf(th, &st, &ct);
   const float v0f = R.v0f;
-  float dxf = dt * (f32_of(F.x) + v0f * ct) + amp * z0;
-  float dyf = dt * (f32_of(F.y) + v0f * st) + amp * z1;
-  *thn = th + amp_r * z2;
+  float dxf = dt * (f32_of(F.x) + v0f * w.ct) + amp * w.z0;
+  float dyf = dt * (f32_of(F.y) + v0f * w.st) + amp * w.z1;
+  *thn = th + amp_r * w.z2;
   const bdpred::Grid g{c.q, c.inv_q, c.qshift};
   const float to_grid = __int_as_float((127 + c.qshift) << 23);   // 2^s, exact scaling
   const float mx = rintf(dxf * to_grid), my = rintf(dyf * to_grid);
@@ -189,6 +214,20 @@ __device__ __forceinline__ void em_move_grid(const BdConst &c, const BdRep &R, u
   *Y = bdpred::to_int(p.y, g) + int_of(my);
   const float q = __int_as_float((127 - c.qshift) << 23);
   *move = make_float2(mx * q, my * q);   // the move in grid steps, exact
+}
+
+// FP64 move of piece `node` (grid-rounded, before reflection); *thn = new angle
+__device__ __forceinline__ double2 em_move_f64(const BdConst &c, const BdRep &R, double2 p, float th, double2 F,
+                                               double v0, const Draw<double> &w, float *thn, uint32_t node) {
+  const int depth = piece_depth(node);
+  // length of this move and its noise amplitudes: dt / 2^depth, amp / 2^(depth/2)
+  const double dt_p = depth ? ldexp(R.dt, -depth) : R.dt;
+  const double amp_scale = depth ? sqrt(ldexp(1.0, -depth)) : 1.0;
+  const double amp_p = R.amp * amp_scale, amp_rp = R.amp_r * amp_scale;
+  const double nx = p.x + dt_p * (F.x + v0 * w.ct) + amp_p * w.z0;
+  const double ny = p.y + dt_p * (F.y + v0 * w.st) + amp_p * w.z1;
+  *thn = (float)((double)th + amp_rp * w.z2);
+  return make_double2(snapd(nx, c.q, c.inv_q), snapd(ny, c.q, c.inv_q));
 }
 
 // position after the move of piece `node` of step `step` (grid-rounded, before
@@ -199,24 +238,10 @@ __device__ __forceinline__ double2 em_move(const BdConst &c, const BdRep &R, uin
   if (c.precision == 0) {
     long long X, Y;
     float2 move;
-    em_move_grid(c, R, id, step, p, th, F, thn, node, &X, &Y, &move);
+    em_move_grid(c, R, p, th, F, draw_f32(R, id, step, node, th), thn, node, &X, &Y, &move);
     return make_double2(grid_to_double(X, c.qshift), grid_to_double(Y, c.qshift));
   }
-  bdrng::U4 r = bdrng::draw(id, (int64_t)step, R.seed, R.replica, piece_tag(node));
-  const int depth = piece_depth(node);
-  // length of this move and its noise amplitudes: dt / 2^depth, amp / 2^(depth/2)
-  const double dt_p = depth ? ldexp(R.dt, -depth) : R.dt;
-  const double amp_scale = depth ? sqrt(ldexp(1.0, -depth)) : 1.0;
-  const double amp_p = R.amp * amp_scale, amp_rp = R.amp_r * amp_scale;
-  // FP64 mode
-  const double3 z = normals_f64(r);
-  const double z0 = z.x, z1 = z.y, z2 = z.z;
-  double st, ct;
-  sincos((double)th, &st, &ct);
-  const double nx = p.x + dt_p * (F.x + v0 * ct) + amp_p * z0;
-  const double ny = p.y + dt_p * (F.y + v0 * st) + amp_p * z1;
-  *thn = (float)((double)th + amp_rp * z2);
-  return make_double2(snapd(nx, c.q, c.inv_q), snapd(ny, c.q, c.inv_q));
+  return em_move_f64(c, R, p, th, F, v0, draw_f64(R, id, step, node, th), thn, node);
 }
 
 // the walls (lo, hi) that disk i's centre stays between: its own for
@@ -258,9 +283,12 @@ __device__ __forceinline__ double2 reflect_as(const BdRep &R, double2 y, int f) 
 
 // The move of disk i (index e within its replica) from p, th under force F, as
 // the time step makes it: the new position, its FP32 copies and the move, the
-// direction, the moved flag, and what an undo needs.
+// direction, the moved flag, and what an undo needs.  T: float for the FP32 step,
+// double for the FP64 step; draw: its draw, if made already.
+template <class T>
 __device__ __forceinline__ void move_disk(const BdDev &d, const BdConst &c, const BdRep &R, int i, int e, long long step,
-                                          int log_step, int node, double2 p, float th, double2 F) {
+                                          int log_step, int node, double2 p, float th, double2 F,
+                                          const Draw<T> *draw = nullptr) {
   d.pos0[i] = p;
   d.theta0[i] = th;
   float thn;
@@ -268,16 +296,17 @@ __device__ __forceinline__ void move_disk(const BdDev &d, const BdConst &c, cons
   const bdpred::Grid g{c.q, c.inv_q, c.qshift};
   long long X, Y;
   float2 move;   // X - X0, Y - Y0 rounded to FP32
-  if (c.precision == 0) {
+  const uint32_t id = (uint32_t)e, nd = (uint32_t)node;
+  if constexpr (sizeof(T) == 4) {
     // move, reflection and FP32 copy in grid units (no FP64 arithmetic)
-    em_move_grid(c, R, (uint32_t)e, step, p, th, F, &thn, (uint32_t)node, &X, &Y, &move);
+    em_move_grid(c, R, p, th, F, draw ? *draw : draw_f32(R, id, step, nd, th), &thn, nd, &X, &Y, &move);
   } else {
-    const double2 y = em_move(c, R, (uint32_t)e, step, p, th, F, R.v0, &thn, (uint32_t)node);
+    const double2 y = em_move_f64(c, R, p, th, F, R.v0, draw ? *draw : draw_f64(R, id, step, nd, th), &thn, nd);
     X = bdpred::to_int(y.x, g);
     Y = bdpred::to_int(y.y, g);
   }
   const long long X0 = bdpred::to_int(p.x, g), Y0 = bdpred::to_int(p.y, g);
-  if (c.precision != 0) move = make_float2(grid_to_float(X - X0, c.qshift), grid_to_float(Y - Y0, c.qshift));
+  if (sizeof(T) == 8) move = make_float2(grid_to_float(X - X0, c.qshift), grid_to_float(Y - Y0, c.qshift));
   int wr = 0;
   if (R.periodic) {
     // the move itself (before re-entry), for the triangulation's reversal screen

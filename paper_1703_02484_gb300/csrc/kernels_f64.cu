@@ -22,7 +22,8 @@
 //    by a second kernel in the order of the host's lists: deterministic.
 // Measured on one GB300 at N = 1024 (one species, walls): the sweep took 36 us
 // one-sided, and with the move's launch in blocks of one warp (32 us before) the
-// whole step fell from 113 to 88 us.
+// whole step fell from 113 to 88 us.  With the move in the reduction and its
+// draws in warps of their own the step fell from 67.5 to 61.9 us.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -120,40 +121,94 @@ __global__ void __launch_bounds__(BD_F64_SB) k_force_long_f64s(BdDev d, BdConst 
 // into partial-force slot 0.  One warp serves the 32 disks of a group in
 // eight shares (every eighth partial), so that the loads of the few disks of a
 // small system are spread over eight warps; the shares are added in order.
-__global__ void __launch_bounds__(256) k_force_f64_reduce(BdDev d, BdConst c) {
+// MOVE: the disks' move (k_integrate's) in the same kernel.  A move is some 200
+// dependent FP64 instructions of 71 cycles each; three warps of their own take
+// the logarithm and circle functions of two normals, those of the third, and the
+// direction's beside the shares that sum, so that the first share's warp has
+// only the sums left to make.
+template <bool MOVE>
+__global__ void __launch_bounds__(MOVE ? 352 : 256) k_force_f64_reduce(BdDev d, BdConst c, long long step, int log_step,
+                                                                      int node) {
   if (ctl_failed(d.ctl)) return;
   __shared__ double2 sh[8][32];
+  __shared__ bdem::Draw<double> draws[MOVE ? 32 : 1];
   const int g = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int i = g * BD_SG + lane, P = i / BD_F64_SB;
+  int e = -1;
+  double2 p = make_double2(0.0, 0.0);
+  float th = 0.f;
+  if (MOVE && (w == 0 || w >= 8)) {
+    e = d.ext_id[i];
+    p = d.pos[i];
+    th = d.theta[i];
+    const long long step_dev = *(volatile const long long *)&d.ctl->step_dev;
+    if (step < 0) step = step_dev;
+  }
+  if (MOVE && w >= 8) {
+    if (e >= 0) {
+      bdem::Draw<double> &o = draws[lane];
+      if (w == 10) {
+        sincos((double)th, &o.st, &o.ct);
+      } else {
+        const bdrng::U4 u = bdem::words_of(d.rep[d.rep_of[i]], (uint32_t)e, step, (uint32_t)node);
+        const double2 z = w == 8 ? bdem::normal_pair(u.x, u.y) : bdem::normal_pair(u.z, u.w);
+        if (w == 8) {
+          o.z0 = z.x;
+          o.z1 = z.y;
+        } else {
+          o.z2 = z.x;
+        }
+      }
+    }
+  }
   double fx = 0.0, fy = 0.0;
-  for (int k = d.red_iptr[P] + w; k < d.red_iptr[P + 1]; k += 8) {
-    const double2 v = d.ipart64[(size_t)d.red_iidx[k] * BD_F64_SB + (i - P * BD_F64_SB)];
-    fx += v.x;
-    fy += v.y;
+  if (w < 8) {
+    for (int k = d.red_iptr[P] + w; k < d.red_iptr[P + 1]; k += 8) {
+      const double2 v = d.ipart64[(size_t)d.red_iidx[k] * BD_F64_SB + (i - P * BD_F64_SB)];
+      fx += v.x;
+      fy += v.y;
+    }
+    for (int k = d.red_jptr[g] + w; k < d.red_jptr[g + 1]; k += 8) {
+      const double2 v = d.jpart64[(size_t)d.red_jidx[k] * BD_SG + lane];
+      fx += v.x;
+      fy += v.y;
+    }
+    sh[w][lane] = make_double2(fx, fy);
   }
-  for (int k = d.red_jptr[g] + w; k < d.red_jptr[g + 1]; k += 8) {
-    const double2 v = d.jpart64[(size_t)d.red_jidx[k] * BD_SG + lane];
-    fx += v.x;
-    fy += v.y;
-  }
-  sh[w][lane] = make_double2(fx, fy);
   __syncthreads();
   if (w) return;
   const int r = d.rep_of[i];
-  if (r < 0 || d.rep[r].law != BD_LAW_LONG) return;
+  if (MOVE && i == 0) d.ctl->in_move = 1;
+  if (r < 0) return;
+  const BdRep &R = d.rep[r];
+  const bool law = R.law == BD_LAW_LONG;
+  if (!MOVE && !law) return;
   fx = fy = 0.0;
 #pragma unroll
   for (int s = 0; s < 8; ++s) {
     fx += sh[s][lane].x;
     fy += sh[s][lane].y;
   }
-  d.fpart[i] = make_double2(fx, fy);
+  if (law) d.fpart[i] = make_double2(fx, fy);
+  else fx = fy = 0.0;
+  if (MOVE) bdem::move_disk<double>(d, c, R, i, e, step, log_step, node, p, th, make_double2(fx, fy), &draws[lane]);
+}
+
+static void launch_sweep(const BdDev &d, const BdConst &c, cudaStream_t s) {
+  if (c.any_periodic) k_force_long_f64s<true><<<c.n_sitems, BD_F64_SB, 0, s>>>(d, c);
+  else k_force_long_f64s<false><<<c.n_sitems, BD_F64_SB, 0, s>>>(d, c);
 }
 
 cudaError_t bd_launch_force_f64s(const BdDev &d, const BdConst &c, cudaStream_t s) {
   if (c.n_sitems == 0) return cudaSuccess;
-  if (c.any_periodic) k_force_long_f64s<true><<<c.n_sitems, BD_F64_SB, 0, s>>>(d, c);
-  else k_force_long_f64s<false><<<c.n_sitems, BD_F64_SB, 0, s>>>(d, c);
-  k_force_f64_reduce<<<c.np / BD_SG, 256, 0, s>>>(d, c);
+  launch_sweep(d, c, s);
+  k_force_f64_reduce<false><<<c.np / BD_SG, 256, 0, s>>>(d, c, 0, 0, 0);
+  return cudaGetLastError();
+}
+
+cudaError_t bd_launch_force_f64s_move(const BdDev &d, const BdConst &c, int64_t step, int log_step, cudaStream_t s,
+                                      int node) {
+  launch_sweep(d, c, s);
+  k_force_f64_reduce<true><<<c.np / BD_SG, 352, 0, s>>>(d, c, (long long)step, log_step, node);
   return cudaGetLastError();
 }

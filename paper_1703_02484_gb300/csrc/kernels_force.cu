@@ -526,6 +526,7 @@ __global__ void k_force_out(BdDev d, BdConst c, double2 *out) {
 // replica, force, position one behind the other): they are issued together
 // before any is looked at.  At large sizes it is its memory traffic, about 110
 // bytes a disk (the position before the move is kept once, in pos0).
+template <class T>
 __global__ void k_integrate(BdDev d, BdConst c, long long step, int log_step, int node) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= c.np) return;
@@ -541,7 +542,7 @@ __global__ void k_integrate(BdDev d, BdConst c, long long step, int log_step, in
   if (step < 0) step = step_dev;
   if (e < 0) return;
   const BdRep &R = d.rep[r];
-  bdem::move_disk(d, c, R, i, e, step, log_step, node, p, th, bdem::force_sum(d, c, R, i, F0));
+  bdem::move_disk<T>(d, c, R, i, e, step, log_step, node, p, th, bdem::force_sum(d, c, R, i, F0));
 }
 
 // all pieces of a halved step completed: the step counts as one time step
@@ -595,23 +596,25 @@ cudaError_t bd_launch_integrate(const BdDev &d, const BdConst &c, int64_t step, 
                                 cudaStream_t s, int node) {
   // the FP64 move is some 300 instructions of the FP64 pipe (two lanes per
   // SM): one warp per block spreads a small system over the SMs
-  const int b = c.precision == 1 ? 32 : 256;
-  k_integrate<<<(c.np + b - 1) / b, b, 0, s>>>(d, c, (long long)step, log_step, node);
+  if (c.precision == 1) k_integrate<double><<<(c.np + 31) / 32, 32, 0, s>>>(d, c, (long long)step, log_step, node);
+  else k_integrate<float><<<(c.np + 255) / 256, 256, 0, s>>>(d, c, (long long)step, log_step, node);
   return cudaGetLastError();
 }
 
 cudaError_t bd_launch_force_move(const BdDev &d, const BdConst &c, int64_t step, int log_step, cudaStream_t s, int node,
                                  int *launches) {
   cudaError_t e = cudaSuccess;
-  // The move in the reduction's kernel for small systems: forward and reverse
-  // step of a 4096-disk rollout 180.5 -> 176.4 us, 777 disks coupled to a fluid
-  // 119.4 -> 118.3, but 136.9 -> 137.3 at 16384 disks and 353.7 -> 358.0 at 30011
-  // in a periodic box, where one share's threads make every move.  (A mix with
-  // disks under the short-range law keeps the move after both forces; a rank
-  // without sweep items has no sums to make.)
-  if (c.np <= BD_MOVE_FUSED && c.any_long && !c.any_short && c.precision == 0 && c.force_variant >= 2 && c.n_sitems > 0) {
-    *launches += bd_force_launches(c);
-    return bd_launch_force_sym_move(d, c, c.force_variant, step, log_step, s, node);
+  // (a mix with disks under the short-range law keeps the move after both
+  // forces; a rank without sweep items has no sums to make)
+  if (c.any_long && !c.any_short && c.n_sitems > 0) {
+    if (c.precision == 0 && c.force_variant >= 2 && c.np <= BD_MOVE_FUSED) {
+      *launches += bd_force_launches(c);
+      return bd_launch_force_sym_move(d, c, c.force_variant, step, log_step, s, node);
+    }
+    if (c.precision == 1 && c.f64_sym) {
+      *launches += bd_force_launches(c);
+      return bd_launch_force_f64s_move(d, c, step, log_step, s, node);
+    }
   }
   if (c.any_long) {
     e = bd_launch_force_long(d, c, s);

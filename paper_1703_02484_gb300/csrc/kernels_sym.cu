@@ -579,15 +579,16 @@ __global__ void __launch_bounds__(NW * 32, MINB) k_force_long_sym_mb(BdDev d, Bd
 // shares' sums are added in a fixed order.  Sums are float-float (TwoSum into
 // a (hi, lo) FP32 pair, about 48 bits): FP64 adds run at 1/64 of the FP32 rate
 // on this part and would bound the kernel.
-// MOVE: the disks' move (k_integrate's) in the same kernel by the first share's
-// threads, whose loads are issued before the sums: a step of a few thousand
-// disks spends as long on a launch and its first loads as on the work.
 // Four partials in flight against two: 2884 -> 2871 us for 20 steps of 16384
 // disks, 2009 -> 2004 for four of 350000 in 64 boxes.
+// MOVE: the disks' move (k_integrate's) in the same kernel, whose launch and
+// first loads cost a small system as much as its work.  A warp of its own draws
+// the noise beside the shares that sum; the first share's then moves the disks.
 template <int ND, int NS, bool MOVE>
-__global__ void __launch_bounds__(ND * NS) k_force_sym_reduce(BdDev d, BdConst c, long long step, int log_step,
-                                                              int node) {
+__global__ void __launch_bounds__(ND * (NS + (MOVE ? 1 : 0))) k_force_sym_reduce(BdDev d, BdConst c, long long step,
+                                                                                 int log_step, int node) {
   __shared__ float4 part[NS][ND];
+  __shared__ bdem::Draw<float> draws[MOVE ? ND : 1];
   if (ctl_failed(d.ctl)) return;
   const int g = threadIdx.x / ND, dl = threadIdx.x % ND;
   const int i = blockIdx.x * ND + dl;               // np is a multiple of 512: i < np
@@ -597,12 +598,12 @@ __global__ void __launch_bounds__(ND * NS) k_force_sym_reduce(BdDev d, BdConst c
   int e = -1;
   double2 p = make_double2(0.0, 0.0);
   float th = 0.f;
-  long long step_dev = 0;
-  if (MOVE && g == 0) {
+  if (MOVE && (g == 0 || g == NS)) {
     e = d.ext_id[i];
     p = d.pos[i];
     th = d.theta[i];
-    step_dev = *(volatile const long long *)&d.ctl->step_dev;
+    const long long step_dev = *(volatile const long long *)&d.ctl->step_dev;
+    if (step < 0) step = step_dev;
   }
   float xh[2] = {0.f, 0.f}, xl[2] = {0.f, 0.f}, yh[2] = {0.f, 0.f}, yl[2] = {0.f, 0.f};
   auto run = [&](const int *idx, int k0, int k1, const float2 *b, int stride) {
@@ -634,11 +635,15 @@ __global__ void __launch_bounds__(ND * NS) k_force_sym_reduce(BdDev d, BdConst c
       two_sum(yh[0], yl[0], v0.y);
     }
   };
-  run(d.red_iidx, d.red_iptr[P], d.red_iptr[P + 1], ib, BD_SB);
-  run(d.red_jidx, d.red_jptr[t], d.red_jptr[t + 1], jb, BD_SG);
-  two_sum(xh[0], xl[0], xh[1]);
-  two_sum(yh[0], yl[0], yh[1]);
-  part[g][dl] = make_float4(xh[0], __fadd_rn(xl[0], xl[1]), yh[0], __fadd_rn(yl[0], yl[1]));
+  if (MOVE && g == NS) {
+    if (e >= 0) draws[dl] = bdem::draw_f32(d.rep[d.rep_of[i]], (uint32_t)e, step, (uint32_t)node, th);
+  } else {
+    run(d.red_iidx, d.red_iptr[P], d.red_iptr[P + 1], ib, BD_SB);
+    run(d.red_jidx, d.red_jptr[t], d.red_jptr[t + 1], jb, BD_SG);
+    two_sum(xh[0], xl[0], xh[1]);
+    two_sum(yh[0], yl[0], yh[1]);
+    part[g][dl] = make_float4(xh[0], __fadd_rn(xl[0], xl[1]), yh[0], __fadd_rn(yl[0], yl[1]));
+  }
   __syncthreads();
   if (g != 0) return;
   const int r = d.rep_of[i];
@@ -646,7 +651,7 @@ __global__ void __launch_bounds__(ND * NS) k_force_sym_reduce(BdDev d, BdConst c
   if (r < 0) return;
   const BdRep &R = d.rep[r];
   if (R.law != BD_LAW_LONG) {   // no force law
-    if (MOVE) bdem::move_disk(d, c, R, i, e, step < 0 ? step_dev : step, log_step, node, p, th, make_double2(0.0, 0.0));
+    if (MOVE) bdem::move_disk<float>(d, c, R, i, e, step, log_step, node, p, th, make_double2(0.0, 0.0), &draws[dl]);
     return;
   }
   float sx = 0.f, ex = 0.f, sy = 0.f, ey = 0.f;
@@ -660,7 +665,7 @@ __global__ void __launch_bounds__(ND * NS) k_force_sym_reduce(BdDev d, BdConst c
   }
   const double2 F = make_double2((double)sx + (double)ex, (double)sy + (double)ey);
   d.fpart[i] = F;
-  if (MOVE) bdem::move_disk(d, c, R, i, e, step < 0 ? step_dev : step, log_step, node, p, th, F);
+  if (MOVE) bdem::move_disk<float>(d, c, R, i, e, step, log_step, node, p, th, F, &draws[dl]);
 }
 
 int bd_force_launches(const BdConst &c) { return (c.precision == 0 ? c.force_variant >= 2 : c.f64_sym) ? 2 : 1; }
@@ -720,6 +725,6 @@ cudaError_t bd_launch_force_sym(const BdDev &d, const BdConst &c, int variant, c
 cudaError_t bd_launch_force_sym_move(const BdDev &d, const BdConst &c, int variant, int64_t step, int log_step,
                                      cudaStream_t s, int node) {
   launch_sweep(d, c, variant, s);
-  k_force_sym_reduce<32, 16, true><<<c.np / 32, 512, 0, s>>>(d, c, (long long)step, log_step, node);
+  k_force_sym_reduce<32, 15, true><<<c.np / 32, 512, 0, s>>>(d, c, (long long)step, log_step, node);
   return cudaGetLastError();
 }
