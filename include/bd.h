@@ -346,7 +346,11 @@ int bd_get_replica(bd_handle *h, int32_t r, double *xy, float *theta, int32_t *t
  * BD_FORCE_TILES fix them (BD_NCHUNK = k: a single system's one-sided
  * sweeps split each row of tiles into k chunks).  BD_TRI_LISTS = 2 makes
  * every check pass of the triangulation test every triangle (by default only
- * the first of a move does; later ones test those near moved disks and flips). */
+ * the first of a move does; later ones test those near moved disks and flips).
+ * BD_TRI_CLUSTER = n runs triangulations of up to n triangles as one
+ * thread-block cluster (0: none), BD_TRI_QUEUE = n queues the edges of a check
+ * pass from more than n triangles per thread on, BD_ADJ_PAIRS = n runs the
+ * rollout's correction passes of up to n pairs as one launch; all read at init. */
 int bd_get_tuning(bd_handle *h, int32_t *tiles_per_item, int32_t *variant, int32_t *n_items);
 
 /* Copy the current state to host memory ("Ensure P updated to current

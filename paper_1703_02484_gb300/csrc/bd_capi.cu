@@ -819,6 +819,10 @@ int build_handle(const std::vector<Spec> &specs, void *stream, bd_handle **out) 
   {
     const char *tl = getenv("BD_TRI_LISTS");
     c.tri_all = tl && atoi(tl) == 2 ? 1 : 0;
+    // each block of a one-launch pass reads all its pairs: sixteen rounds for
+    // 1024 of them, about what the launches cost that it saves
+    const char *ap = getenv("BD_ADJ_PAIRS");
+    c.adj_pairs = ap ? atoi(ap) : 1024;
     const char *tf = getenv("BD_TRI_FUSE");
     c.tri_fuse = tf ? (atoi(tf) != 0 ? 1 : 0) : 1;
   }

@@ -88,15 +88,18 @@ void fill_stats(bd_handle *h, int status, int64_t halvings);   // h->last_stats 
 // adjoint kernels (adjoint.cu)
 // sx, sth / z, zd (null = none): where a replayed move / pass keeps the state it starts from
 cudaError_t bd_adj_rp_em(const BdDev &d, const BdConst &c, long long step, int k_local, double2 *sx, float *sth,
-                         cudaStream_t s);
+                         double2 *z, cudaStream_t s);
 cudaError_t bd_adj_rp_pass(const BdDev &d, const BdConst &c, int pass, int pb, int pe, double2 *z, double2 *zd,
-                           cudaStream_t s);
+                           double2 *zn, cudaStream_t s);
 cudaError_t bd_adj_vjp_pass(const BdDev &d, const BdConst &c, int pass, int pb, int pe, const double2 *z,
                             const double2 *zd, double2 *lam, double2 *mud, cudaStream_t s);
+cudaError_t bd_adj_vjp_pass1(const BdDev &d, const BdConst &c, int pass, int pb, int pe, const double2 *z,
+                             const double2 *zd, const double2 *lin, double2 *lout, int k_local, const double2 *x,
+                             float4 *vx, float2 *vm, cudaStream_t s);
 int bd_adj_force_chunks(const BdConst &c, int *jchunk);
 cudaError_t bd_adj_vjp_em(const BdDev &d, const BdConst &c, int k_local, const double2 *x, const float *th,
                           double2 *lam, float4 *vx, float2 *vm, double2 *jpart, double *gpart, double *grad,
-                          cudaStream_t s);
+                          bool ready, cudaStream_t s);
 cudaError_t bd_adj_msd(const BdDev &d, const BdConst &c, const double2 *x0, double *acc, double target,
                        double dscale, double2 *lam, double *loss, cudaStream_t s);
 // pair-distance histogram of the disk slots' positions x (n disks) into h[32]

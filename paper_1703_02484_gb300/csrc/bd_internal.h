@@ -242,6 +242,7 @@ struct BdConst {
   int tri_fuse;            // 1: a Lawson round tests the outer edges of its flips and keeps the
                            // overlap sums (no check pass between rounds); 0: a check pass after
                            // every round (environment variable BD_TRI_FUSE at init)
+  int adj_pairs;           // rollout: passes of up to so many pairs run as one launch (BD_ADJ_PAIRS at init)
   int tri_queue;           // 1: its check passes run through the warps' queues (many triangles per thread)
   int tri_cluster;         // > 0: the triangulation kernel runs as one cluster of so many blocks
   int vl_grid;             // blocks of the Verlet-list rebuild launch

@@ -245,14 +245,16 @@ cudaError_t replay(bd_handle *h, BdRollout *r, const BdDev &dr, int t0, int t1, 
   const int pb0 = r->step_pass[t0];
   cudaError_t e = cudaSuccess;
   for (int t = t0; t < t1 && e == cudaSuccess; ++t) {
+    const int p0 = r->step_pass[t], p1 = r->step_pass[t + 1];
+    // where the positions before pass p are kept (null: there is no such pass in this step)
+    auto z_of = [&](int p) { return store && p < p1 ? r->seg_z + (size_t)(p - pb0) * np : nullptr; };
     e = bd_launch_force_long(dr, h->c, s);
     if (e == cudaSuccess)
       e = bd_adj_rp_em(dr, h->c, (long long)(r->step0 + t), t, store ? r->seg_x + (size_t)(t - t0) * np : nullptr,
-                       store ? r->seg_th + (size_t)(t - t0) * np : nullptr, s);
-    for (int p = r->step_pass[t]; p < r->step_pass[t + 1] && e == cudaSuccess; ++p)
-      e = bd_adj_rp_pass(dr, h->c, p, r->pass_begin[p], r->pass_begin[p + 1],
-                         store ? r->seg_z + (size_t)(p - pb0) * np : nullptr,
-                         store ? r->seg_zd + (size_t)(p - pb0) * np : nullptr, s);
+                       store ? r->seg_th + (size_t)(t - t0) * np : nullptr, z_of(p0), s);
+    for (int p = p0; p < p1 && e == cudaSuccess; ++p)
+      e = bd_adj_rp_pass(dr, h->c, p, r->pass_begin[p], r->pass_begin[p + 1], z_of(p),
+                         store ? r->seg_zd + (size_t)(p - pb0) * np : nullptr, z_of(p + 1), s);
   }
   return e;
 }
@@ -524,21 +526,32 @@ int bd_rollout_vjp(bd_handle *h, double *grad) {
   int64_t launches = 0;
   e = cudaMemsetAsync(r->acc + 8, 0, 5 * sizeof(double), s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(r->lam, r->lam_T, np * sizeof(double2), cudaMemcpyDeviceToDevice, s);
+  double2 *lam = r->lam, *other = r->mud;   // lambda; scratch, which it changes places with in a one-launch pass
   for (int g = r->nseg - 1; g >= 0 && e == cudaSuccess; --g) {
     const int t0 = g * r->every, t1 = std::min(r->nsteps, t0 + r->every);
     const int pb0 = r->step_pass[t0];
     e = load_checkpoint(h, r, dr, g);
     if (e == cudaSuccess) e = replay(h, r, dr, t0, t1, true);
     for (int t = t1 - 1; t >= t0 && e == cudaSuccess; --t) {
+      const double2 *const x = r->seg_x + (size_t)(t - t0) * np;
+      bool ready = false;   // the step's first pass has prepared the force adjoint
       for (int p = r->step_pass[t + 1] - 1; p >= r->step_pass[t] && e == cudaSuccess; --p) {
-        e = bd_adj_vjp_pass(dr, h->c, p, r->pass_begin[p], r->pass_begin[p + 1], r->seg_z + (size_t)(p - pb0) * np,
-                            r->seg_zd + (size_t)(p - pb0) * np, r->lam, r->mud, s);
-        launches += 2;
+        const int pb = r->pass_begin[p], pe = r->pass_begin[p + 1];
+        const double2 *const z = r->seg_z + (size_t)(p - pb0) * np, *const zd = r->seg_zd + (size_t)(p - pb0) * np;
+        if (pe - pb <= h->c.adj_pairs) {
+          ready = p == r->step_pass[t];
+          e = bd_adj_vjp_pass1(dr, h->c, p, pb, pe, z, zd, lam, other, t, ready ? x : nullptr, r->vx, r->vm, s);
+          std::swap(lam, other);
+          launches += 1;
+        } else {
+          e = bd_adj_vjp_pass(dr, h->c, p, pb, pe, z, zd, lam, other, s);
+          launches += 2;
+        }
       }
       if (e == cudaSuccess)
-        e = bd_adj_vjp_em(dr, h->c, t, r->seg_x + (size_t)(t - t0) * np, r->seg_th + (size_t)(t - t0) * np,
-                          r->lam, r->vx, r->vm, r->jpart, r->gpart, r->acc + 8, s);
-      launches += 3;
+        e = bd_adj_vjp_em(dr, h->c, t, x, r->seg_th + (size_t)(t - t0) * np, lam, r->vx, r->vm, r->jpart, r->gpart,
+                          r->acc + 8, ready, s);
+      launches += ready ? 2 : 3;
     }
   }
   double gh[5] = {0, 0, 0, 0, 0};

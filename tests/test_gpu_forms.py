@@ -172,3 +172,21 @@ def test_move_in_the_reduction(monkeypatch, n, variant, tiles, periodic, precisi
     assert np.array_equal(a["theta"], b["theta"])
     fused.close()
     apart.close()
+
+
+@pytest.mark.parametrize("n", [257, 1601])
+def test_rollout_passes_in_one_launch(monkeypatch, n):
+    # the reverse pass (and its replay) with every correction pass as one launch
+    # against two; they share all terms but the order of the additions to a disk,
+    # whose last bits may round its FP32 multiplier (2^-24) in a later step
+    p, xy, sp, th = crowded(monkeypatch, n, 7, False)
+    out = []
+    for pairs in ("1024", "-1"):
+        monkeypatch.setenv("BD_ADJ_PAIRS", pairs)
+        s = bd.System(p, xy, sp, th, stream=stream())
+        loss, st = s.rollout(9, ckpt_every=4)
+        assert st["corr_iters"] > 0
+        out.append((loss, s.rollout_vjp()))
+        s.close()
+    assert out[0][0] == out[1][0]
+    assert float(np.max(np.abs(out[0][1] - out[1][1]))) <= 1e-6 * float(np.max(np.abs(out[1][1])))
