@@ -682,7 +682,7 @@ def main():
             # FP64 issues at 1/64 of the FP32 rate on this part
             p64 = peak_tflops / 64.0
             a64 = FLOPS_PER_PAIR * pairs / avg_force_s / 1e12
-            line["roofline"] = {"bound": "fp64", "kernel": "k_force_long_f64", "achieved": a64, "peak": p64,
+            line["roofline"] = {"bound": "fp64", "kernel": "k_force_long_f64s + k_force_f64_reduce", "achieved": a64, "peak": p64,
                                 "unit": "TFLOP/s", "frac": a64 / p64, "traffic": None,
                                 "avg_launch_ms": avg_force_s * 1e3,
                                 "peak_note": "FP32 peak / 64 (the part's FP64 issue rate)"}

@@ -149,7 +149,7 @@ struct BdDev {
   float *xfer_th;          //   directions,
   uint8_t *xfer_sp;        //   species
   uint8_t *moved;
-  float2 *dmove;           // position less prev, FP32 (disks with the moved flag; the reversal filter)
+  float2 *dmove;           // the last move, FP32 (disks with the moved flag; the reversal filter)
   long long *rep_stats;    // [R][3] per-replica counters of a bd_batch_step call: correction passes that
                            // moved the replica, Lawson flips, inverted triangles
   unsigned long long *rep_mark;   // [R] the last correction pass counted for each replica (a stamp
