@@ -597,7 +597,7 @@ cudaError_t bd_launch_integrate(const BdDev &d, const BdConst &c, int64_t step, 
   // the FP64 move is some 300 instructions of the FP64 pipe (two lanes per
   // SM): one warp per block spreads a small system over the SMs
   if (c.precision == 1) k_integrate<double><<<(c.np + 31) / 32, 32, 0, s>>>(d, c, (long long)step, log_step, node);
-  else k_integrate<float><<<(c.np + 255) / 256, 256, 0, s>>>(d, c, (long long)step, log_step, node);
+  else k_integrate<float><<<(c.np + 127) / 128, 128, 0, s>>>(d, c, (long long)step, log_step, node);
   return cudaGetLastError();
 }
 

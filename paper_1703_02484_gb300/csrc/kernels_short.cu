@@ -28,6 +28,8 @@
 #include "gridsync.cuh"
 
 
+#define BD_VF_THREADS 128   // threads per block of the force over the lists
+
 namespace {
 
 // float-float arithmetic (value = hi + lo, |lo| <= ulp(hi)/2), about 48
@@ -329,27 +331,34 @@ __device__ __forceinline__ void pair_diff(const BdDev &d, const BdConst &c, cons
 // some 150 instructions for the two or three contacts of a disk.  In one pass a
 // warp ran the core for nearly every list position, since at each one some lane
 // of the 32 had a contact there.  The sums take the same terms in the same
-// order.  Four resident blocks of 256 per SM (64 registers, without spills now): the
-// gathers want the warps, and the polydisperse branch must not cost the
+// order.  32 warps per SM (64 registers, without spills now) in blocks of 128, whose
+// last ones end sooner than those of 256; with that and a disk's own loads issued
+// together (slot, replica, list length and the first four entries waited for one
+// another) a step of 2^20 disks fell from 335.6 to 327 us, of 200003 from 112.1 to
+// 111.0.  The gathers want the warps, and the polydisperse branch must not cost the
 // equal-disk case its occupancy.  The law's constants come rounded from the
 // host and the result is widened by its bits: formed here, their dozen FP64
 // products and conversions a disk kept the FP64 pipe (two lanes per SM) busy for
 // 59 % of the kernel's time.
-__global__ void __launch_bounds__(256, 4) k_force_verlet(BdDev d, BdConst c) {
-  if (failed(d.ctl)) return;
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(BD_VF_THREADS, 1024 / BD_VF_THREADS) k_force_verlet(BdDev d, BdConst c) {
+  const int i = blockIdx.x * BD_VF_THREADS + threadIdx.x;
+  if (i >= c.np) return;
+  // every load of a disk's own data is issued before any is looked at
+  const bool bad = failed(d.ctl);
+  const int e = d.ext_id[i], r = c.R == 1 ? 0 : d.rep_of[i], m = d.vl_cnt[i];
+  const float4 wi = d.work[i];
+  int jn[4];   // (the first rows of the lists, whatever their length)
+#pragma unroll
+  for (int u = 0; u < 4; ++u) jn[u] = d.vl_idx[(size_t)u * c.np + i];
+  if (bad) return;
   if (i == 0) {
     if (need(d.ctl)) {
       d.ctl->vl_need = 0;
       d.ctl->st_verlet_rebuilds += 1;
     }
   }
-  if (i >= c.np) return;
-  const BdRep *Rp = short_rep(d, i);
-  if (!Rp || d.ext_id[i] < 0) return;
-  const BdRep &R = *Rp;
-  const float4 wi = d.work[i];
-  const int m = d.vl_cnt[i];
+  if (e < 0 || d.rep[r].law != BD_LAW_SHORT) return;
+  const BdRep &R = d.rep[r];
   const float rc2 = R.rc2f;
   const float eps = R.epsf, kap = R.kapf;
   // the law's length scale s: 2a, or a_i + a_j for polydisperse disks (then
@@ -363,9 +372,8 @@ __global__ void __launch_bounds__(256, 4) k_force_verlet(BdDev d, BdConst c) {
   // four list entries at a time: their position gathers are issued before
   // any of them is used, and the next four indices are loaded while these
   // are evaluated
-  int jn[4];
 #pragma unroll
-  for (int u = 0; u < 4; ++u) jn[u] = u < m ? d.vl_idx[(size_t)u * c.np + i] : i;
+  for (int u = 0; u < 4; ++u) jn[u] = u < m ? jn[u] : i;
   for (int t0 = 0; t0 < m; t0 += 4) {
     int jj[4];
     float4 wv[4];
@@ -468,7 +476,7 @@ cudaError_t bd_launch_force_short(const BdDev &d, const BdConst &c, cudaStream_t
   void *args[] = {&dd, &cc};
   cudaError_t e = cudaLaunchCooperativeKernel((const void *)k_vl_rebuild, dim3(c.vl_grid), dim3(BD_VL_THREADS), args, 0, s);
   if (e != cudaSuccess) return e;
-  k_force_verlet<<<gn, 256, 0, s>>>(d, c);
+  k_force_verlet<<<(c.np + BD_VF_THREADS - 1) / BD_VF_THREADS, BD_VF_THREADS, 0, s>>>(d, c);
   return cudaGetLastError();
 }
 
