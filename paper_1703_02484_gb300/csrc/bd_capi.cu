@@ -933,8 +933,11 @@ int build_handle(const std::vector<Spec> &specs, void *stream, bd_handle **out) 
       BD_TRY(cudaMemsetAsync(d.rep_mark, 0, (size_t)R * sizeof(unsigned long long), h->stream));
     }
     if (c.any_periodic) {
-      BD_TRY(dalloc(h, &d.wrap, (size_t)np));
-      BD_TRY(cudaMemsetAsync(d.wrap, 0, (size_t)np, h->stream));
+      // (with the ghost points' bytes, which stay 0: the shift pass reads the
+      // re-entries of every triangle's corners, and in a batch that mixes walls
+      // and periodic boxes some of those are ghost points)
+      BD_TRY(dalloc(h, &d.wrap, nv));
+      BD_TRY(cudaMemsetAsync(d.wrap, 0, nv, h->stream));
     }
     BD_TRY(dalloc(h, &d.disp, (size_t)np));
     BD_TRY(dalloc(h, &d.hit, (size_t)np));
