@@ -760,10 +760,12 @@ __device__ __forceinline__ void triangulation_body(const BdDev &d, const BdConst
   int log_pidx = -1;
   // Check passes.  The first pass of a move (and the pass after an inversion
   // repair) tests every triangle; a later pass only the dirty ones: those with a
-  // corner that the last correction moved, and those stamped with the pass's
+  // corner that the last correction pushed, and those stamped with the pass's
   // generation byte (flips, flip candidates left unresolved).  Every other edge
   // kept its end points and its place in the triangulation since it was last
-  // checked, so its earlier verdicts (legal, not overlapping) stand.  A clean
+  // checked and was not overlapping then (both ends of an overlapping edge
+  // count as pushed, even when their pushes cancel and they stay), so its
+  // earlier verdicts (legal, not overlapping) stand.  A clean
   // triangle costs its corner table and three flags.  (Lists of the triangles
   // to visit, kept by the flips and by walks round the moved disks, measured
   // slower at every size: 513 against 492 us per step in a batch of 350000 disks,
@@ -1311,8 +1313,13 @@ __device__ __forceinline__ void triangulation_body(const BdDev &d, const BdConst
           if (PER) d.wrap[i] = 0;
           const double2 p = d.pos[i];
           const double2 dd = disp_get(x, i);
+          d.prev[i] = p;
           if (dd.x == 0.0 && dd.y == 0.0) {
-            d.moved[i] = 0;
+            // Its pushes cancel: it stays where it is, overlapping.  Flagged as
+            // moved, its edges are looked at again by the next pass, which
+            // would otherwise pass over an edge both of whose ends stay.
+            d.dmove[i] = make_float2(0.f, 0.f);
+            d.moved[i] = 1;
             if (log_pidx >= 0) d.log_pflags[(size_t)log_pidx * x.np + i] = 0;
             continue;
           }
@@ -1323,7 +1330,6 @@ __device__ __forceinline__ void triangulation_body(const BdDev &d, const BdConst
             if (atomicExch(&d.rep_mark[rr], stamp) != stamp)
               atomicAdd((unsigned long long *)&d.rep_stats[3 * rr], 1ull);
           }
-          d.prev[i] = p;
           const double mag = sqrt(__dadd_rn(__dmul_rn(dd.x, dd.x), __dmul_rn(dd.y, dd.y)));
           // Sec. 4.4: sigma/4, half the disk's radius (its own for polydisperse disks)
           const double cap = d.rad ? 0.5 * d.rad[i] : 0.25 * sigma;
@@ -1363,7 +1369,7 @@ __device__ __forceinline__ void triangulation_body(const BdDev &d, const BdConst
     if (lead) stage_tick(ctl, STAGE_A, t_mark);
     fresh = true;
     need_p = scan = true;
-    sweep_all = false;   // an edge whose ends both stayed put does not overlap
+    sweep_all = false;   // an edge neither of whose ends had a push did not overlap and still does not
     ++kp;
   }
 

@@ -54,3 +54,82 @@ def test_walled_boxes_take_no_image_shifts(monkeypatch, cluster):
             assert not b.tri_shifts(r).any()
     assert entered > 0
     b.close()
+
+
+# ---------------------------------------------------------------- pushes that cancel
+
+FORMS = [{"BD_TRI_CLUSTER": "0"}, {"BD_TRI_CLUSTER": "0", "BD_TRI_LISTS": "2"},
+         {"BD_TRI_CLUSTER": "0", "BD_TRI_QUEUE": "0"}, {"BD_TRI_CLUSTER": "1000000"},
+         {"BD_TRI_CLUSTER": "1000000", "BD_TRI_LISTS": "2"}]
+FORM_IDS = ["grid", "grid-all", "queue", "cluster", "cluster-all"]
+
+
+def system_moving_to(target, dy, L, periodic, precision, **kw):
+    # a handle whose next step ends at `target` before any correction: no force,
+    # no noise, every disk driven up or down by about dy.  The move does not
+    # depend on the positions, so it is read off a step of the same disks on a
+    # wide jittered lattice; all coordinates are multiples of 2^-5, so nothing rounds
+    n = len(target)
+    theta = np.where(np.arange(n) % 2 == 0, 0.5 * math.pi, -0.5 * math.pi).astype(np.float32)
+
+    def make(xy, side, **kw):
+        p = bd.make_params(n, L=side, D=0.0, v0=dy / 0.125, dt=0.125, precision=precision,
+                           boundary=bd.BOUNDARY_PERIODIC if periodic else bd.BOUNDARY_WALLS, **kw)
+        return bd.System(p, xy, theta=theta, stream=stream())
+
+    m = math.ceil(math.sqrt(n))
+    wide = np.array([(4.0 * (k % m) + 3.0, 4.0 * (k // m) + 3.0) for k in range(n)])
+    wide += np.random.default_rng(1).integers(-16, 17, wide.shape) / 32.0
+    s = make(wide, max(L, 4.0 * m + 4.0))
+    q0, _ = s.geometry()
+    s.step(1)
+    move = s.state()["xy"] - wide
+    s.close()
+    s = make(target - move, L, **kw)
+    q1, _ = s.geometry()
+    assert q1 <= q0      # the move is on the finer grid too
+    start = s.state()["xy"]
+    assert np.array_equal(start + move, target)
+    return s, start
+
+
+@pytest.mark.parametrize("env", FORMS, ids=FORM_IDS)
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("periodic", [False, True])
+def test_overlap_between_disks_whose_pushes_cancel(monkeypatch, periodic, precision, env):
+    # four disks in a row, each overlapping the next by 1/16: the inner two
+    # are pushed equally from both sides, so the first pass moves the outer
+    # two only and leaves the inner pair as it was
+    from oracle import overlap
+    for k, v in env.items():
+        monkeypatch.setenv(k, v)
+    L = 30.0
+    target = np.array([(10.0 + 1.9375 * k, 15.0) for k in range(4)]
+                      + [(5.0 + 4 * k, y) for y in (4.0, 26.0) for k in range(6)]
+                      + [(x, y) for x in (7.0, 12.90625, 19.0) for y in (11.0, 19.0)])
+    s, _ = system_moving_to(target, 0.3, L, periodic, precision)
+    st = s.step(1)
+    ref = (overlap.correct_periodic if periodic else overlap.correct)(target, L, 1.0)
+    assert ref[2] == 4 and not ref[4]
+    out = s.state()["xy"]
+    s.close()
+    assert st["steps_done"] == 1 and st["corr_iters"] == 4
+    assert float(np.max(np.abs(out - ref[0]))) <= 1e-9
+    d = out[:4, None] - out[None, :4]
+    assert float(np.min(np.hypot(d[..., 0], d[..., 1]) + 9.0 * np.eye(4))) >= 2.0 * (1 - 1e-12)
+
+
+@pytest.mark.parametrize("env", FORMS, ids=FORM_IDS)
+def test_closed_row_of_overlapping_disks_does_not_converge(monkeypatch, env):
+    # a row round the periodic box, each disk pushed equally from both sides:
+    # no pass moves any, and the step is undone with an error
+    for k, v in env.items():
+        monkeypatch.setenv(k, v)
+    L = 30.0
+    target = np.array([(0.9375 + 1.875 * k, 15.0) for k in range(16)]
+                      + [(1.5 + 3.0 * k, y) for y in (4.0, 10.0, 20.0, 26.0) for k in range(10)])
+    s, start = system_moving_to(target, 0.35, L, True, 0, max_corr_iters=20)
+    st, code = s.step(1, raise_on_error=False)
+    assert code == -5 and st["fail_phase"] == 5 and st["steps_done"] == 0
+    assert np.array_equal(s.state()["xy"], start)
+    s.close()
