@@ -57,6 +57,13 @@ __device__ __forceinline__ u64 mul2(u64 a, u64 b) {
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
+// the rounded sums of two packed pairs, and their rounding errors
+__device__ __forceinline__ u64 two_sum2(u64 a, u64 b, u64 &err) {
+  const u64 s = add2(a, b);
+  const u64 bp = sub2(s, a);
+  err = add2(sub2(a, sub2(s, bp)), sub2(b, bp));
+  return s;
+}
 
 // x^(-3/2) for finite x > 0, in six FP64 instructions (FP64 issues at 1/64 of
 // the FP32 rate on this part).  x = m 2^(2k), m in [1, 4); y = rsqrt(m) 2^-k to

@@ -576,9 +576,9 @@ __global__ void __launch_bounds__(NW * 32, MINB) k_force_long_sym_mb(BdDev d, Bd
 // Bound by the partials' reads.  ND disks per block, NS shares: thread share g
 // takes every NS-th partial (entries g, g + NS, ...) of the ND disks, so the
 // loads stay coalesced and NS times as many warps hide their latency; the
-// shares' sums are added in a fixed order.  Sums are float-float (TwoSum into
-// a (hi, lo) FP32 pair, about 48 bits): FP64 adds run at 1/64 of the FP32 rate
-// on this part and would bound the kernel.
+// shares' sums are added in a fixed order.  A share's sum is float-float (TwoSum
+// into a (hi, lo) FP32 pair, about 48 bits): FP64 adds run at 1/64 of the FP32
+// rate on this part and would bound the kernel.
 // Four partials in flight against two: 2884 -> 2871 us for 20 steps of 16384
 // disks, 2009 -> 2004 for four of 350000 in 64 boxes.
 // MOVE: the disks' move (k_integrate's) in the same kernel, whose launch and
@@ -587,7 +587,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) k_force_long_sym_mb(BdDev d, Bd
 template <int ND, int NS, bool MOVE>
 __global__ void __launch_bounds__(ND * (NS + (MOVE ? 1 : 0))) k_force_sym_reduce(BdDev d, BdConst c, long long step,
                                                                                  int log_step, int node) {
-  __shared__ float4 part[NS][ND];
+  __shared__ float4 part[NS][ND];   // each share's sum: (x, y) and their low parts
   __shared__ bdem::Draw<float> draws[MOVE ? ND : 1];
   if (ctl_failed(d.ctl)) return;
   const int g = threadIdx.x / ND, dl = threadIdx.x % ND;
@@ -642,7 +642,7 @@ __global__ void __launch_bounds__(ND * (NS + (MOVE ? 1 : 0))) k_force_sym_reduce
     run(d.red_jidx, d.red_jptr[t], d.red_jptr[t + 1], jb, BD_SG);
     two_sum(xh[0], xl[0], xh[1]);
     two_sum(yh[0], yl[0], yh[1]);
-    part[g][dl] = make_float4(xh[0], __fadd_rn(xl[0], xl[1]), yh[0], __fadd_rn(yl[0], yl[1]));
+    part[g][dl] = make_float4(xh[0], yh[0], __fadd_rn(xl[0], xl[1]), __fadd_rn(yl[0], yl[1]));
   }
   __syncthreads();
   if (g != 0) return;
@@ -654,16 +654,28 @@ __global__ void __launch_bounds__(ND * (NS + (MOVE ? 1 : 0))) k_force_sym_reduce
     if (MOVE) bdem::move_disk<float>(d, c, R, i, e, step, log_step, node, p, th, make_double2(0.0, 0.0), &draws[dl]);
     return;
   }
-  float sx = 0.f, ex = 0.f, sy = 0.f, ey = 0.f;
+  // The shares in three FP32 words (about 72 bits), x and y packed: what an
+  // addition to the first loses goes into the second, and what that loses into the
+  // third, so that the sum is rounded once, to FP64, as fine as one of FP64
+  // additions.  (Those and their conversions would keep this warp's FP64 pipe,
+  // two lanes per SM, for sixteen cycles each, eight times per share; unpacked,
+  // the three words cost a 4096-disk rollout with its gradient 2 us per step.)
+  u64 s0 = 0ull, s1 = 0ull, s2 = 0ull;
 #pragma unroll
   for (int m = 0; m < NS; ++m) {
     const float4 q = part[m][dl];
-    two_sum(sx, ex, q.x);
-    two_sum(sy, ey, q.z);
-    ex = __fadd_rn(ex, q.y);
-    ey = __fadd_rn(ey, q.w);
+    u64 lost, rest;
+    s0 = two_sum2(s0, pk2(q.x, q.y), lost);
+    s1 = two_sum2(s1, lost, rest);
+    s2 = add2(s2, rest);
+    s1 = two_sum2(s1, pk2(q.z, q.w), rest);
+    s2 = add2(s2, rest);
   }
-  const double2 F = make_double2((double)sx + (double)ex, (double)sy + (double)ey);
+  float x0, x1, x2, y0, y1, y2;
+  up2(s0, x0, y0);
+  up2(s1, x1, y1);
+  up2(s2, x2, y2);
+  const double2 F = make_double2((double)x0 + ((double)x1 + (double)x2), (double)y0 + ((double)y1 + (double)y2));
   d.fpart[i] = F;
   if (MOVE) bdem::move_disk<float>(d, c, R, i, e, step, log_step, node, p, th, F, &draws[dl]);
 }
