@@ -1364,8 +1364,9 @@ bool step_graph_ready(bd_handle *h) {
 }
 
 // Queue nsteps whole steps (one graph replay each, or plain launches when
-// every force launch is timed), wait for them, read the control block and fold
-// the force timings in.  A failed step makes the later ones no-ops.
+// every force launch is timed or graphs are off), wait for them, read the
+// control block and fold the force timings in.  A failed step makes the later
+// ones no-ops.
 int queue_steps(bd_handle *h, int32_t nsteps, int64_t *launches_out) {
   cudaStream_t st = h->stream;
   cudaError_t e = cudaSuccess;
@@ -1390,27 +1391,29 @@ int queue_steps(bd_handle *h, int32_t nsteps, int64_t *launches_out) {
     launches = (int64_t)nsteps * h->graph_launches;
   }
   for (int s = 0; s < (use_graph ? 0 : nsteps); ++s) {
-    if (long_range) {
-      bool tm = h->timing;
-      if (tm) cudaEventRecord(h->ev_pool[2 * s], st);
+    int n = 1;
+    if (h->timing && long_range) {
+      // the force's launches between the events, the move in a launch of its own
+      cudaEventRecord(h->ev_pool[2 * s], st);
       e = bd_launch_force_long(h->d, h->c, st);
       if (e != cudaSuccess) return cuda_fail(e);
-      if (tm) {
-        cudaEventRecord(h->ev_pool[2 * s + 1], st);
-        ++timed;
+      cudaEventRecord(h->ev_pool[2 * s + 1], st);
+      ++timed;
+      n += bd_force_launches(h->c);
+      if (h->c.any_short) {
+        e = bd_launch_force_short(h->d, h->c, st);
+        if (e != cudaSuccess) return cuda_fail(e);
+        n += bd_short_launches();
       }
-      launches += bd_force_launches(h->c);
+      e = bd_launch_integrate(h->d, h->c, h->step + s, -1, st);
+      ++n;
+    } else {
+      e = bd_launch_force_move(h->d, h->c, h->step + s, -1, st, 1, &n);
     }
-    if (h->c.any_short) {
-      e = bd_launch_force_short(h->d, h->c, st);
-      if (e != cudaSuccess) return cuda_fail(e);
-      launches += bd_short_launches();
-    }
-    e = bd_launch_integrate(h->d, h->c, h->step + s, -1, st);
     if (e != cudaSuccess) return cuda_fail(e);
     e = launch_correction(h, st);
     if (e != cudaSuccess) return cuda_fail(e);
-    launches += 2;
+    launches += n;
   }
   *launches_out += launches;
   int rc = read_ctl(h);

@@ -42,9 +42,14 @@
 
 using namespace bdf;
 
-// below this many slots the reduction takes sixteen shares per disk, not four:
-// about the slots whose four shares fill the SMs' threads
+// below this many slots the reduction takes fifteen shares per disk, not four:
+// about the slots whose four shares fill the SMs' threads.  Fifteen whether the
+// move is in it (with the warp that draws, four blocks of 512 threads fill an SM)
+// or not: the shares set the order of the sum, and a step's force is the same
+// bits in a graph, in launches of its own, timed, and in a rollout's replay.
 #define BD_RED_SMALL 65536
+#define BD_RED_SHARES 15
+static_assert(BD_MOVE_FUSED < BD_RED_SMALL, "a fused move and the force apart take the same shares");
 
 namespace {
 
@@ -729,7 +734,8 @@ static void launch_sweep(const BdDev &d, const BdConst &c, int variant, cudaStre
 cudaError_t bd_launch_force_sym(const BdDev &d, const BdConst &c, int variant, cudaStream_t s) {
   if (c.n_sitems == 0) return cudaSuccess;
   launch_sweep(d, c, variant, s);
-  if (c.np < BD_RED_SMALL) k_force_sym_reduce<32, 16, false><<<c.np / 32, 512, 0, s>>>(d, c, 0, 0, 0);
+  constexpr int NS = BD_RED_SHARES;
+  if (c.np < BD_RED_SMALL) k_force_sym_reduce<32, NS, false><<<c.np / 32, 32 * NS, 0, s>>>(d, c, 0, 0, 0);
   else k_force_sym_reduce<64, 4, false><<<c.np / 64, 256, 0, s>>>(d, c, 0, 0, 0);
   return cudaGetLastError();
 }
@@ -737,6 +743,7 @@ cudaError_t bd_launch_force_sym(const BdDev &d, const BdConst &c, int variant, c
 cudaError_t bd_launch_force_sym_move(const BdDev &d, const BdConst &c, int variant, int64_t step, int log_step,
                                      cudaStream_t s, int node) {
   launch_sweep(d, c, variant, s);
-  k_force_sym_reduce<32, 15, true><<<c.np / 32, 512, 0, s>>>(d, c, (long long)step, log_step, node);
+  constexpr int NS = BD_RED_SHARES;
+  k_force_sym_reduce<32, NS, true><<<c.np / 32, 32 * (NS + 1), 0, s>>>(d, c, (long long)step, log_step, node);
   return cudaGetLastError();
 }

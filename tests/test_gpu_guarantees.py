@@ -133,3 +133,70 @@ def test_closed_row_of_overlapping_disks_does_not_converge(monkeypatch, env):
     assert code == -5 and st["fail_phase"] == 5 and st["steps_done"] == 0
     assert np.array_equal(s.state()["xy"], start)
     s.close()
+
+
+# ---------------------------------------------------------------- one result however a step is launched
+
+def test_step_is_the_same_bits_however_it_is_launched(monkeypatch):
+    # a graph's replay, launches of their own, and the force timed apart from the
+    # move.  16384 disks for 600 steps: about 2e7 force components, enough that
+    # two orders of the partial sums (2^-46 apart, the move reads 2^-24) differ
+    monkeypatch.setenv("BD_FORCE_VARIANT", "3")
+    monkeypatch.setenv("BD_FORCE_TILES", "1")
+    cfg = workloads.CONFIGS["c2"]
+    n = 16384
+    xy, sp, th = workloads.initial_state(cfg, n=n)
+    out = []
+    for form in ("graph", "plain", "timed"):
+        with monkeypatch.context() as m:
+            if form == "plain":
+                m.setenv("BD_NO_GRAPH", "1")
+            s = bd.System(bd.params_from_config(cfg, n=n), xy, sp, th, stream=stream())
+        if form == "timed":
+            s.force_timing(True)
+        for _ in range(6):
+            assert s.step(100)["steps_done"] == 100
+        out.append(s.state())
+        s.close()
+    for o in out[1:]:
+        assert np.array_equal(o["xy"], out[0]["xy"]) and np.array_equal(o["theta"], out[0]["theta"])
+        assert np.array_equal(o["tri"], out[0]["tri"])
+
+
+def test_plain_launches_are_those_of_the_graph(monkeypatch):
+    cfg = workloads.CONFIGS["c2"]
+    monkeypatch.setenv("BD_FORCE_VARIANT", "2")
+    monkeypatch.setenv("BD_FORCE_TILES", "1")
+    xy, sp, th = workloads.initial_state(cfg, n=3000)
+    counts = []
+    for off in (False, True):
+        if off:
+            monkeypatch.setenv("BD_NO_GRAPH", "1")
+        s = bd.System(bd.params_from_config(cfg, n=3000), xy, sp, th, stream=stream())
+        s.step(3)
+        counts.append(s.last_launch_count())
+        s.close()
+    assert counts[0] == counts[1]
+
+
+def test_fp32_rollout_replay_follows_the_recorded_run(monkeypatch):
+    # without contacts (a wide lattice) the replay is the recorded moves from the
+    # same forces, bit for bit; 16384 disks for 600 steps as above
+    monkeypatch.setenv("BD_FORCE_VARIANT", "3")
+    monkeypatch.setenv("BD_FORCE_TILES", "1")
+    cfg = workloads.CONFIGS["c5"]
+    m, h = 128, 8.0
+    n = m * m
+    rng = np.random.default_rng(5)
+    xy = (np.stack(np.meshgrid(np.arange(m), np.arange(m)), -1).reshape(-1, 2) + 0.5) * h + rng.uniform(-1, 1, (n, 2))
+    sp = rng.integers(0, 2, n).astype(np.uint8)
+    th = rng.uniform(0, 2 * math.pi, n).astype(np.float32)
+    p = bd.params_from_config(cfg, n=n)
+    p.box_L = m * h
+    s = bd.System(p, xy, sp, th, stream=stream())
+    loss, st = s.rollout(600, ckpt_every=200)
+    assert st["steps_done"] == 600 and st["corr_iters"] == 0
+    end = s.state(want_tri=False)["xy"]
+    assert s.rollout_replay() == loss
+    assert np.array_equal(s.rollout_positions(1), end)
+    s.close()
