@@ -1215,13 +1215,14 @@ void add_stage_times(bd_handle *h) {
 
 int finish_status(bd_handle *h, int status) {
   // clear the sticky status so the handle keeps working from the last good
-  // state; after a timed-out barrier the kernel left without undoing its
-  // step: undo it (step-start copies, undo journal), and reset the barrier words
+  // state.  After a timed-out barrier the kernel left without undoing its step:
+  // undo it (step-start copies, undo journal), and reset the barrier words.
+  // After a list overflow (the one device status BD_ERR_UNSUPPORTED) the
+  // lists are cut short and the kernels behind the rebuild did not run: have
+  // them built again, and take back positions that bd_set_state had stored.
   cudaStream_t st = h->stream;
-  if (status == BD_ERR_DEVICE_TIMEOUT) {
-    bd_launch_restore_step(h->d, h->c, st);
-    cudaMemsetAsync(h->d.ctl, 0, offsetof(BdCtl, epoch), st);
-  }
+  if (status == BD_ERR_DEVICE_TIMEOUT || status == BD_ERR_UNSUPPORTED) bd_launch_restore_step(h->d, h->c, st);
+  if (status == BD_ERR_DEVICE_TIMEOUT) cudaMemsetAsync(h->d.ctl, 0, offsetof(BdCtl, epoch), st);
   cudaMemsetAsync(&h->d.ctl->cnt[0][0], 0, sizeof(h->d.ctl->cnt), st);
   cudaMemsetAsync(&h->d.ctl->in_move, 0, sizeof(int), st);
   cudaMemsetAsync(&h->d.ctl->status, 0, sizeof(int), st);

@@ -305,8 +305,8 @@ cudaError_t bd_launch_overlap_verlet(const BdDev &d, const BdConst &c, cudaStrea
                                      int advance = 1);
 // a halved step completed: advance the device step counter and the step count
 cudaError_t bd_launch_advance_step(const BdDev &d, cudaStream_t s);
-// after a timed-out grid barrier: make the next step rebuild Verlet lists whose
-// rebuild it cut off and, if positions had moved, undo the step (or the new positions of
+// after a timed-out grid barrier or a list overflow: make the next step rebuild
+// Verlet lists whose rebuild was cut off and, if positions had moved, undo the step (or the new positions of
 // bd_set_state) from the step-start copies and the undo journal, as their own
 // failure path does, and clear the flip claims and list marks the abandoned
 // launch may have left

@@ -1433,8 +1433,9 @@ __global__ void __launch_bounds__(BD_DTC_THREADS, 1)
   triangulation_body<PER, true, false>(d, c, mode, log_step);
 }
 
-// Undo a step whose persistent kernel left at a timed-out barrier (the
-// kernel's own failure path did not run).  The launch journaled every
+// Undo a step whose persistent kernel left at a timed-out barrier, or did not
+// start because the Verlet lists overflowed (the kernel's own failure path did
+// not run).  The launch journaled every
 // triangle before its first change to it, and all its blocks have finished
 // (this kernel runs after it in stream order), so replaying the journal
 // restores the triangulation; positions and directions come from pos0 /
@@ -1443,8 +1444,9 @@ __global__ void __launch_bounds__(BD_DTC_THREADS, 1)
 __global__ void k_restore_step(BdDev d, BdConst c) {
   const int tid = blockIdx.x * blockDim.x + threadIdx.x;
   const int nth = gridDim.x * blockDim.x;
-  // a rebuild of the Verlet lists was cut off (the force that follows it takes
-  // the request back): references parked far away make the next step rebuild
+  // a rebuild of the Verlet lists was cut off or ran out of room (the force that
+  // follows it takes the request back): references parked far away make the
+  // next use of the lists rebuild them
   if (c.any_short && *(volatile const int *)&d.ctl->vl_need)
     for (int i = tid; i < c.np; i += nth) d.vl_ref[i] = make_double2(1e30, 1e30);
   if (!*(volatile const int *)&d.ctl->in_move) return;   // nothing had moved yet

@@ -200,3 +200,56 @@ def test_fp32_rollout_replay_follows_the_recorded_run(monkeypatch):
     assert s.rollout_replay() == loss
     assert np.array_equal(s.rollout_positions(1), end)
     s.close()
+
+
+# ---------------------------------------------------------------- Verlet lists that run out of room
+
+def dense_block(n, h, L):
+    # n disks on a square lattice of spacing h in a corner of the box
+    m = math.ceil(math.sqrt(n))
+    k = np.arange(n)
+    return np.stack([2.0 + h * (k % m), 2.0 + h * (k // m)], 1) + 0.5
+
+
+@pytest.mark.parametrize("verlet", [False, True])
+def test_list_overflow_is_an_error_each_time(verlet):
+    # 400 disks 2.05 apart within reach 10.6: inner disks have some 80
+    # neighbours, a list holds 64
+    L = 90.0
+    p = bd.make_params(400, L=L, law=bd.LAW_SHORT, r_cut=10.0, skin=0.6, D=0.01, dt=1e-4)
+    if verlet:
+        p.overlap_mode = bd.OVERLAP_VERLET
+    s = bd.System(p, dense_block(400, 2.05, L), stream=stream())
+    start = s.state()["xy"]
+    for _ in range(3):
+        st, code = s.step(2, raise_on_error=False)
+        assert code == -10 and st["steps_done"] == 0
+        with pytest.raises(bd.BDError) as e:
+            s.forces()
+        assert e.value.code == -10
+    assert np.array_equal(s.state()["xy"], start)
+    s.close()
+
+
+def test_state_whose_lists_overflow_is_refused_whole():
+    L = 90.0
+    p = bd.make_params(400, L=L, law=bd.LAW_SHORT, r_cut=10.0, skin=0.6, D=0.01, Dr=0.1, v0=1.0, dt=1e-4)
+    p.overlap_mode = bd.OVERLAP_VERLET
+    wide = dense_block(400, 4.0, L)
+    s = bd.System(p, wide, stream=stream())
+    twin = bd.System(p, wide, stream=stream())
+    s.step(3)
+    twin.step(3)
+    before = s.state()
+    with pytest.raises(bd.BDError) as e:
+        s.set_state(dense_block(400, 2.05, L), before["theta"] + np.float32(1.0))
+    assert e.value.code == -10
+    after = s.state()
+    assert np.array_equal(after["xy"], before["xy"]) and np.array_equal(after["theta"], before["theta"])
+    # and the handle goes on as if nothing had been asked (entries beyond the
+    # cut-off, which a later rebuild may drop, add nothing to a force)
+    s.step(3)
+    twin.step(3)
+    assert np.array_equal(s.state()["xy"], twin.state()["xy"])
+    s.close()
+    twin.close()
