@@ -604,9 +604,8 @@ cudaError_t bd_launch_integrate(const BdDev &d, const BdConst &c, int64_t step, 
 cudaError_t bd_launch_force_move(const BdDev &d, const BdConst &c, int64_t step, int log_step, cudaStream_t s, int node,
                                  int *launches) {
   cudaError_t e = cudaSuccess;
-  // (a mix with disks under the short-range law keeps the move after both
-  // forces; a rank without sweep items has no sums to make)
-  if (c.any_long && !c.any_short && c.n_sitems > 0) {
+  // (a mix with disks under the short-range law keeps the move after both forces)
+  if (c.any_long && !c.any_short) {
     if (c.precision == 0 && c.force_variant >= 2 && c.np <= BD_MOVE_FUSED) {
       *launches += bd_force_launches(c);
       return bd_launch_force_sym_move(d, c, c.force_variant, step, log_step, s, node);

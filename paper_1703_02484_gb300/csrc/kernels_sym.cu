@@ -704,7 +704,10 @@ int bd_force_sym_blocks_per_sm(int variant, int periodic) {
 }
 
 // variant 2: 4 warps x 4 disks per lane; variant 3: 2 warps x 8 disks per lane
+// (a rank with none of the work items sweeps nothing; its reduction still writes
+// the sums, all 0, over what fpart held)
 static void launch_sweep(const BdDev &d, const BdConst &c, int variant, cudaStream_t s) {
+  if (c.n_sitems == 0) return;
   // periodic boxes (any replica) take the form with minimum images
   if (c.any_periodic) {
     // measured at N = 1e5 (periodic), step times with pair forms chosen per
@@ -732,7 +735,6 @@ static void launch_sweep(const BdDev &d, const BdConst &c, int variant, cudaStre
 }
 
 cudaError_t bd_launch_force_sym(const BdDev &d, const BdConst &c, int variant, cudaStream_t s) {
-  if (c.n_sitems == 0) return cudaSuccess;
   launch_sweep(d, c, variant, s);
   constexpr int NS = BD_RED_SHARES;
   if (c.np < BD_RED_SMALL) k_force_sym_reduce<32, NS, false><<<c.np / 32, 32 * NS, 0, s>>>(d, c, 0, 0, 0);

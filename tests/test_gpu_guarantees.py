@@ -253,3 +253,45 @@ def test_state_whose_lists_overflow_is_refused_whole():
     assert np.array_equal(s.state()["xy"], twin.state()["xy"])
     s.close()
     twin.close()
+
+
+# ---------------------------------------------------------------- force shards without work items
+
+def test_ranks_without_work_items_add_nothing(monkeypatch):
+    # more ranks than the sweep has work items: a rank without any contributes a
+    # force of 0 at every step, not what its arrays held before
+    monkeypatch.setenv("BD_FORCE_VARIANT", "3")
+    monkeypatch.setenv("BD_FORCE_TILES", "8")
+    cfg = workloads.CONFIGS["c2"]
+    n, world = 1024, 5
+    xy, sp, th = workloads.initial_state(cfg, n=n)
+
+    def make():
+        return bd.System(bd.params_from_config(cfg, n=n), xy, sp, th, stream=stream())
+
+    whole = make()
+    assert whole.tuning()["n_items"] < world
+    ranks = [make() for _ in range(world)]
+    for r, h in enumerate(ranks):
+        h.forces()                       # (the whole force is in every rank's arrays)
+        h.set_force_shard(r, world)
+    F = torch.empty(2 * whole.force_slots(), dtype=torch.float64, device="cuda")
+    tot = torch.empty_like(F)
+    for step in range(3):
+        whole.step_begin(F.data_ptr())
+        ref = F.clone()
+        scale = float(torch.sqrt(torch.mean(ref.view(-1, 2).pow(2).sum(1))))
+        tot.zero_()
+        zero = 0
+        for h in ranks:
+            h.step_begin(F.data_ptr())
+            zero += int(float(F.abs().max()) == 0.0)
+            tot += F
+        assert zero == world - whole.tuning()["n_items"]
+        # (FP32 partial sums, split otherwise: a few roundings of 2^-46 apart)
+        assert float((tot - ref).abs().max()) <= 1e-10 * scale
+        for h in ranks:
+            h.step_end(tot.data_ptr())
+        whole.step_end(tot.data_ptr())
+    for h in ranks + [whole]:
+        h.close()
