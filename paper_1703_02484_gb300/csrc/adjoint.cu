@@ -21,7 +21,8 @@
 //   ((dF/dx)^T mu)_i = sum_j M(r_ij) (A_ij mu_i - A_ji mu_j),  M(r) = I/r^3 - 3 r r^T/r^5,
 // and the parameter gradients dL/dA_ab += dt sum_{i in a} mu_i . sum_{j in b} r_ij/r_ij^3,
 // dL/dv0 += dt sum_i mu_i . e(theta_i).
-// Pair terms are computed in FP32; every accumulation is FP64.
+// The force adjoint's pair terms are FP32, summed in FP32 over at most 128 disks
+// j and in FP64 beyond; everything else is FP64.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -301,17 +302,19 @@ __device__ __forceinline__ double adj_warp_sum(double v) {
 // Bound by the FP32 pipe: 22 lane operations per ordered pair, in packed f32x2
 // instructions for two disks i per thread.  Blocks and tiles of j hold one
 // species each (slots are species-major in whole 512-disk blocks), so both table
-// entries are constants of the tile and A_ji mu_j is formed once per j.  The
-// pair j = i needs no test: A_ij mu_i - A_ji mu_j and r are exactly 0 there.
-// M(r) w = q3 w - 3 q3 (r . w) r / r^2 is summed as its two terms.  Chunks go
-// down to one tile of 128 j so that small systems still have about eight
-// blocks per SM.  One scalar pair at a time in 256 blocks, with FP64 staging and
-// shared FP64 atomics, it took 62 us at 4096 disks; a 40-step rollout with its
-// reverse pass went from 10.8 to 8.0 ms.
+// entries are constants of the tile.  In a tile of the block's own species
+// A_ij = A_ji is taken out of the sum, w = mu_i - mu_j, and the pair j = i needs
+// no test: w and r are exactly 0 there.  Between two species A_ji mu_j is formed
+// once per j.  A tile's sums are FP32, sums beyond a tile FP64 (sixteen FP64
+// instructions a thread and tile, a sixth of the time its FP32 work takes).
+// Chunks go down to one tile of 128 j so that small systems still have about
+// eight blocks per SM.  One scalar pair at a time in 256 blocks, with FP64
+// staging and shared FP64 atomics, it took 62 us at 4096 disks; a 40-step
+// rollout with its reverse pass went from 10.8 to 8.0 ms.
 __global__ void __launch_bounds__(BD_ADJ_T, 6) k_vjp_force(BdDev d, BdConst c, const float4 *vx, const float2 *vm,
                                                            const float *th, const double2 *mu, int jchunk,
                                                            double2 *jpart, double *gpart) {
-  __shared__ ulonglong2 sh[BD_ADJ_T], sl[BD_ADJ_T], sm[BD_ADJ_T];   // ((v, v), (w, w)) of the hi, lo parts, A_ji mu_j
+  __shared__ ulonglong2 sh[BD_ADJ_T], sl[BD_ADJ_T], sm[BD_ADJ_T];   // ((v, v), (w, w)) of the hi, lo parts, -A_ji mu_j
   __shared__ double sg[BD_ADJ_T / 32][3];
   const int tid = threadIdx.x;
   const int ib = blockIdx.x * 2 * BD_ADJ_T;
@@ -321,26 +324,28 @@ __global__ void __launch_bounds__(BD_ADJ_T, 6) k_vjp_force(BdDev d, BdConst c, c
   const float4 p0 = vx[i0], p1 = vx[i1];
   const float2 m0 = vm[i0], m1 = vm[i1];
   const u64 xh = pk2(p0.x, p1.x), yh = pk2(p0.y, p1.y), xl = pk2(p0.z, p1.z), yl = pk2(p0.w, p1.w);
-  // sums beyond a tile as float-float pairs: [i0, i1][x, y]
-  float jh[2][2] = {{0.f, 0.f}, {0.f, 0.f}}, jl[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
-  float gh[2][2][2] = {}, gl[2][2][2] = {};   // [species of j][i0, i1][x, y]
-  const u64 eps2 = pk2(1e-20f, 1e-20f);
+  const u64 mx = pk2(m0.x, m1.x), my = pk2(m0.y, m1.y);
+  double js[2][2] = {{0.0, 0.0}, {0.0, 0.0}};   // [i0, i1][x, y]
+  double gs[2][2][2] = {};                      // [species of j][i0, i1][x, y]
+  const u64 eps2 = pk2(1e-20f, 1e-20f), m3 = pk2(-3.f, -3.f);
   const int jb = blockIdx.y * jchunk, je = min(c.np, jb + jchunk);
   for (int j0 = jb; j0 < je; j0 += BD_ADJ_T) {
     const int sj = d.tile_species[j0 / BD_TJ];
+    const bool same = sj == si;
     const float aij = R.alpha[BD_MAX_SPECIES * si + sj], aji = R.alpha[BD_MAX_SPECIES * sj + si];
     {
       const float4 q = vx[j0 + tid];
       const float2 m = vm[j0 + tid];
-      const float mx = __fmul_rn(aji, m.x), my = __fmul_rn(aji, m.y);
+      const float nx = same ? -m.x : -__fmul_rn(aji, m.x), ny = same ? -m.y : -__fmul_rn(aji, m.y);
       sh[tid] = make_ulonglong2(pk2(q.x, q.x), pk2(q.y, q.y));
       sl[tid] = make_ulonglong2(pk2(q.z, q.z), pk2(q.w, q.w));
-      sm[tid] = make_ulonglong2(pk2(mx, mx), pk2(my, my));
+      sm[tid] = make_ulonglong2(pk2(nx, nx), pk2(ny, ny));
     }
     __syncthreads();
-    const u64 mix = pk2(__fmul_rn(aij, m0.x), __fmul_rn(aij, m1.x));
-    const u64 miy = pk2(__fmul_rn(aij, m0.y), __fmul_rn(aij, m1.y));
-    u64 ax = 0ull, ay = 0ull, bx = 0ull, by = 0ull, tx = 0ull, ty = 0ull;
+    const float ai = same ? 1.f : aij;
+    const double sc = same ? (double)aij : 1.0;
+    const u64 ai2 = pk2(ai, ai);
+    u64 ax = 0ull, ay = 0ull, tx = 0ull, ty = 0ull;
 #pragma unroll 4
     for (int k = 0; k < BD_ADJ_T; ++k) {
       const ulonglong2 qh = sh[k], ql = sl[k], qm = sm[k];
@@ -352,24 +357,21 @@ __global__ void __launch_bounds__(BD_ADJ_T, 6) k_vjp_force(BdDev d, BdConst c, c
       const u64 ir = pk2(rsqrt_apx(ra), rsqrt_apx(rb));
       const u64 ir2 = mul2(ir, ir);
       const u64 q3 = mul2(ir2, ir);
-      const u64 wx = sub2(mix, qm.x), wy = sub2(miy, qm.y);   // w = A_ij mu_i - A_ji mu_j
-      const u64 u = mul2(mul2(fma2(rx, wx, mul2(ry, wy)), ir2), q3);
-      ax = fma2(wx, q3, ax);
-      ay = fma2(wy, q3, ay);
-      bx = fma2(rx, u, bx);
-      by = fma2(ry, u, by);
+      const u64 wx = fma2(ai2, mx, qm.x), wy = fma2(ai2, my, qm.y);   // A_ij mu_i - A_ji mu_j, less the factor sc
+      const u64 u = mul2(mul2(fma2(rx, wx, mul2(ry, wy)), ir2), m3);
+      ax = fma2(fma2(rx, u, wx), q3, ax);   // (w - 3 r (r . w) / r^2) / r^3
+      ay = fma2(fma2(ry, u, wy), q3, ay);
       tx = fma2(rx, q3, tx);   // r_ij / r^3
       ty = fma2(ry, q3, ty);
     }
     float a[2], b[2];
     up2(ax, a[0], a[1]);
-    up2(bx, b[0], b[1]);
+    up2(ay, b[0], b[1]);
 #pragma unroll
-    for (int h = 0; h < 2; ++h) two_sum(jh[h][0], jl[h][0], __fmaf_rn(-3.f, b[h], a[h]));
-    up2(ay, a[0], a[1]);
-    up2(by, b[0], b[1]);
-#pragma unroll
-    for (int h = 0; h < 2; ++h) two_sum(jh[h][1], jl[h][1], __fmaf_rn(-3.f, b[h], a[h]));
+    for (int h = 0; h < 2; ++h) {
+      js[h][0] = __fma_rn(sc, (double)a[h], js[h][0]);
+      js[h][1] = __fma_rn(sc, (double)b[h], js[h][1]);
+    }
     up2(tx, a[0], a[1]);
     up2(ty, b[0], b[1]);
 #pragma unroll
@@ -377,8 +379,8 @@ __global__ void __launch_bounds__(BD_ADJ_T, 6) k_vjp_force(BdDev d, BdConst c, c
       if ((sj ? 1 : 0) == s)
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-          two_sum(gh[s][h][0], gl[s][h][0], a[h]);
-          two_sum(gh[s][h][1], gl[s][h][1], b[h]);
+          gs[s][h][0] += (double)a[h];
+          gs[s][h][1] += (double)b[h];
         }
     __syncthreads();
   }
@@ -386,13 +388,11 @@ __global__ void __launch_bounds__(BD_ADJ_T, 6) k_vjp_force(BdDev d, BdConst c, c
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     const int i = h ? i1 : i0;
-    jpart[(size_t)blockIdx.y * c.np + i] =
-        make_double2((double)jh[h][0] + (double)jl[h][0], (double)jh[h][1] + (double)jl[h][1]);
+    jpart[(size_t)blockIdx.y * c.np + i] = make_double2(js[h][0], js[h][1]);
     if (d.ext_id[i] < 0) continue;
     const double2 m = mu[i];
 #pragma unroll
-    for (int s = 0; s < 2; ++s)
-      g[s] += m.x * ((double)gh[s][h][0] + (double)gl[s][h][0]) + m.y * ((double)gh[s][h][1] + (double)gl[s][h][1]);
+    for (int s = 0; s < 2; ++s) g[s] += m.x * gs[s][h][0] + m.y * gs[s][h][1];
     if (blockIdx.y == 0) {
       float st, ct;
       sincosf(th[i], &st, &ct);
