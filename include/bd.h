@@ -336,7 +336,7 @@ int bd_get_replica(bd_handle *h, int32_t r, double *xy, float *theta, int32_t *t
                    int32_t *n, double *L);
 
 /* The all-pairs sweep's tuning: j tiles (256 disks each; a part of one counts
- * as one) per work item, the
+ * as one: bd_get_force_groups tells it exactly) per work item, the
  * kernel variant (0 scalar FP32 one-sided, 1 packed f32x2 one-sided, 2 and 3
  * symmetric packed f32x2 -- each unordered pair once -- with 4 warps x 4 or
  * 2 warps x 8 disks per lane) and the number of work items.  Periodic boxes
@@ -344,7 +344,9 @@ int bd_get_replica(bd_handle *h, int32_t r, double *xy, float *theta, int32_t *t
  * bd_init picks the FP32 variant and chunk size by timing the candidates on
  * the device; the environment variables BD_FORCE_VARIANT (0-3) and
  * BD_FORCE_TILES fix them (BD_NCHUNK = k: a single system's one-sided
- * sweeps split each row of tiles into k chunks).  BD_TRI_LISTS = 2 makes
+ * sweeps split each row of tiles into k chunks; BD_FORCE_GROUPS = g: the
+ * symmetric variants' items take g groups of 32 disks, whatever
+ * BD_FORCE_TILES says).  BD_TRI_LISTS = 2 makes
  * every check pass of the triangulation test every triangle (by default only
  * the first of a move does; later ones test those near moved disks and flips).
  * BD_TRI_CLUSTER = n runs triangulations of up to n triangles as one
@@ -352,6 +354,11 @@ int bd_get_replica(bd_handle *h, int32_t r, double *xy, float *theta, int32_t *t
  * pass from more than n triangles per thread on, BD_ADJ_PAIRS = n runs the
  * rollout's correction passes of up to n pairs as one launch; all read at init. */
 int bd_get_tuning(bd_handle *h, int32_t *tiles_per_item, int32_t *variant, int32_t *n_items);
+
+/* Groups of 32 disks j per work item of the symmetric sweeps (0 with a one-sided
+ * one): BD_FORCE_VARIANT and BD_FORCE_GROUPS set to a handle's values make the
+ * same work items again, and with them the same sums.  Errors: BD_ERR_ARG. */
+int bd_get_force_groups(bd_handle *h, int32_t *groups_per_item);
 
 /* Copy the current state to host memory ("Ensure P updated to current
  * time", Algorithm 1).  Any pointer may be NULL to skip that output.  With

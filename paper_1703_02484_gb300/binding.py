@@ -90,6 +90,7 @@ SIGNATURES = [
                                       ctypes.POINTER(ctypes.c_int32), ctypes.POINTER(ctypes.c_double)]),
     ("bd_get_tuning", ctypes.c_int, [_P, ctypes.POINTER(ctypes.c_int32), ctypes.POINTER(ctypes.c_int32),
                                      ctypes.POINTER(ctypes.c_int32)]),
+    ("bd_get_force_groups", ctypes.c_int, [_P, ctypes.POINTER(ctypes.c_int32)]),
     ("bd_set_force_params", ctypes.c_int, [_P, _P, ctypes.c_double]),
     ("bd_set_step", ctypes.c_int, [_P, ctypes.c_int64]),
     ("bd_rollout", ctypes.c_int, [_P, ctypes.c_int32, ctypes.c_int32, ctypes.c_int32, ctypes.c_double,
@@ -369,7 +370,9 @@ class System:
         a, b, c = ctypes.c_int32(), ctypes.c_int32(), ctypes.c_int32()
         _check(load().bd_get_tuning(self.h, ctypes.byref(a), ctypes.byref(b), ctypes.byref(c)),
                "bd_get_tuning")
-        return dict(tiles_per_item=a.value, variant=b.value, n_items=c.value)
+        g = ctypes.c_int32()
+        _check(load().bd_get_force_groups(self.h, ctypes.byref(g)), "bd_get_force_groups")
+        return dict(tiles_per_item=a.value, variant=b.value, n_items=c.value, groups_per_item=g.value)
 
     def neighbors(self, max_per=64):
         n = self.n

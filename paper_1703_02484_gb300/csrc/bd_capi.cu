@@ -1138,7 +1138,7 @@ int build_handle(const std::vector<Spec> &specs, void *stream, bd_handle **out) 
     }
     BD_TRY(cudaStreamSynchronize(st));
     // force work items: the FP64 sweep fills whole waves; the FP32 sweep is
-    // chosen by timing (or fixed by BD_FORCE_VARIANT / BD_FORCE_TILES)
+    // chosen by timing (or fixed by BD_FORCE_VARIANT and BD_FORCE_TILES or BD_FORCE_GROUPS)
     {
       BD_TRY(bd_launch_work_copy(d, c, st));
       // the ghost points' FP32 pairs (they never move)
@@ -1161,8 +1161,11 @@ int build_handle(const std::vector<Spec> &specs, void *stream, bd_handle **out) 
       } else if (fv) {
         int v = std::min(3, std::max(0, atoi(fv)));
         if (c.any_periodic && v == 1) v = 0;   // the packed one-sided sweep has no periodic form
-        const int t = ft && atoi(ft) > 0 ? atoi(ft) : (v >= 2 ? 8 : (R == 1 ? single_system_tiles(h) : 16));
-        BD_TRY(use_variant(h, v, v >= 2 ? t * (BD_TJ / BD_SG) : t));
+        const int most = 1 << 24;   // (beyond any row of tiles; counts groups without overflow)
+        const int t = ft && atoi(ft) > 0 ? std::min(most, atoi(ft)) : (v >= 2 ? 8 : (R == 1 ? single_system_tiles(h) : 16));
+        const char *fg = getenv("BD_FORCE_GROUPS");
+        if (v >= 2 && fg && atoi(fg) > 0) BD_TRY(use_variant(h, v, std::min(most, atoi(fg))));
+        else BD_TRY(use_variant(h, v, v >= 2 ? t * (BD_TJ / BD_SG) : t));
       } else if (nmax * nmax > 180000000000LL) {
         // a launch takes more than ~50 ms: no timing at init
         BD_TRY(use_variant(h, 2, 128));
@@ -1984,6 +1987,12 @@ int bd_get_tuning(bd_handle *h, int32_t *tiles_per_item, int32_t *variant, int32
   if (tiles_per_item) *tiles_per_item = sym ? (h->tune_chunk + per - 1) / per : h->tune_chunk;
   if (variant) *variant = h->c.force_variant;
   if (n_items) *n_items = sym ? h->c.n_sitems : h->c.n_items;
+  return BD_OK;
+}
+
+int bd_get_force_groups(bd_handle *h, int32_t *groups_per_item) {
+  if (!h || !groups_per_item) return BD_ERR_ARG;
+  *groups_per_item = h->c.force_variant >= 2 || h->c.f64_sym ? h->tune_chunk : 0;
   return BD_OK;
 }
 

@@ -295,3 +295,47 @@ def test_ranks_without_work_items_add_nothing(monkeypatch):
         whole.step_end(tot.data_ptr())
     for h in ranks + [whole]:
         h.close()
+
+
+# ---------------------------------------------------------------- a tuning read back
+
+@pytest.mark.parametrize("groups", [2, 4, 8, 24])
+@pytest.mark.parametrize("variant", [2, 3])
+def test_tuning_read_back_makes_the_same_sweep(monkeypatch, variant, groups):
+    cfg = workloads.CONFIGS["c2"]
+    n = 3001
+    xy, sp, th = workloads.initial_state(cfg, n=n)
+    monkeypatch.setenv("BD_FORCE_VARIANT", str(variant))
+    monkeypatch.setenv("BD_FORCE_GROUPS", str(groups))
+    a = bd.System(bd.params_from_config(cfg, n=n), xy, sp, th, stream=stream())
+    t = a.tuning()
+    assert t["variant"] == variant and t["groups_per_item"] == groups
+    assert t["tiles_per_item"] == (groups + 7) // 8
+    F = a.forces()
+    a.close()
+    monkeypatch.setenv("BD_FORCE_VARIANT", str(t["variant"]))
+    monkeypatch.setenv("BD_FORCE_TILES", str(t["tiles_per_item"]))
+    monkeypatch.setenv("BD_FORCE_GROUPS", str(t["groups_per_item"]))
+    b = bd.System(bd.params_from_config(cfg, n=n), xy, sp, th, stream=stream())
+    assert b.tuning() == t and np.array_equal(b.forces(), F)
+    b.close()
+
+
+def test_autotuned_sweep_can_be_asked_for_again(monkeypatch):
+    for k in ("BD_FORCE_VARIANT", "BD_FORCE_TILES", "BD_FORCE_GROUPS", "BD_NCHUNK"):
+        monkeypatch.delenv(k, raising=False)
+    cfg = workloads.CONFIGS["c2"]
+    for n in (777, 4096, 16384):
+        xy, sp, th = workloads.initial_state(cfg, n=n)
+        a = bd.System(bd.params_from_config(cfg, n=n), xy, sp, th, stream=stream())
+        t, F = a.tuning(), a.forces()
+        a.close()
+        with monkeypatch.context() as m:
+            m.setenv("BD_FORCE_VARIANT", str(t["variant"]))
+            if t["variant"] >= 2:
+                m.setenv("BD_FORCE_GROUPS", str(t["groups_per_item"]))
+            else:
+                m.setenv("BD_FORCE_TILES", str(t["tiles_per_item"]))
+            b = bd.System(bd.params_from_config(cfg, n=n), xy, sp, th, stream=stream())
+        assert b.tuning() == t and np.array_equal(b.forces(), F)
+        b.close()
