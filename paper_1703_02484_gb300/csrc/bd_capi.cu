@@ -986,7 +986,6 @@ int build_handle(const std::vector<Spec> &specs, void *stream, bd_handle **out) 
     BD_TRY(dalloc(h, &d.clmark, (size_t)nt));
     BD_TRY(cudaMemsetAsync(d.clmark, 0, (size_t)nt * sizeof(unsigned), h->stream));
     BD_TRY(cudaMemsetAsync(d.tinv, 0, (size_t)nt, h->stream));
-    BD_TRY(dalloc(h, &d.vt, nv));
     BD_TRY(dalloc(h, &d.iperm, (size_t)std::max(1, h->np_i)));
     BD_TRY(dalloc(h, &d.iorigin, (size_t)std::max(1, iblock)));
     BD_TRY(dalloc(h, &d.tile_species, std::max<size_t>(1, tile_sp.size())));
@@ -1037,7 +1036,6 @@ int build_handle(const std::vector<Spec> &specs, void *stream, bd_handle **out) 
       BD_TRY(dalloc(h, &h->hs_theta, (size_t)np));
       BD_TRY(dalloc(h, &h->hs_tv, (size_t)nt));
       BD_TRY(dalloc(h, &h->hs_tn, (size_t)nt));
-      BD_TRY(dalloc(h, &h->hs_vt, nv));
     }
 
     cudaStream_t st = h->stream;
@@ -1105,16 +1103,6 @@ int build_handle(const std::vector<Spec> &specs, void *stream, bd_handle **out) 
     BD_TRY(cudaMemsetAsync(d.disp, 0, np * sizeof(double2), st));
     BD_TRY(cudaMemcpyAsync(d.tv, tv_all.data(), nt * sizeof(int4), cudaMemcpyHostToDevice, st));
     BD_TRY(cudaMemcpyAsync(d.tn, tn_all.data(), nt * sizeof(int4), cudaMemcpyHostToDevice, st));
-    {
-      // one corner per vertex (the star walks of the triangulation kernel start there)
-      std::vector<int> vt(nv, -1);
-      for (int t = 0; t < nt; ++t) {
-        vt[tv_all[t].x] = 3 * t;
-        vt[tv_all[t].y] = 3 * t + 1;
-        vt[tv_all[t].z] = 3 * t + 2;
-      }
-      BD_TRY(cudaMemcpy(d.vt, vt.data(), nv * sizeof(int), cudaMemcpyHostToDevice));
-    }
     BD_TRY(cudaMemsetAsync(d.claim, 0, 2 * nt * sizeof(unsigned long long), st));
     if (!iperm.empty())
       BD_TRY(cudaMemcpyAsync(d.iperm, iperm.data(), iperm.size() * sizeof(int), cudaMemcpyHostToDevice, st));
@@ -1457,9 +1445,6 @@ cudaError_t halving_snapshot(bd_handle *h, bool save) {
     e = cudaMemcpyAsync(save ? h->hs_tv : h->d.tv, save ? h->d.tv : h->hs_tv, nt * sizeof(int4), k, st);
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(save ? h->hs_tn : h->d.tn, save ? h->d.tn : h->hs_tn, nt * sizeof(int4), k, st);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(save ? h->hs_vt : h->d.vt, save ? h->d.vt : h->hs_vt,
-                          ((size_t)h->np + h->ng) * sizeof(int), k, st);
   }
   if (e == cudaSuccess && !save) {
     e = cudaMemcpyAsync(h->d.prev, h->d.pos, np * sizeof(double2), k, st);

@@ -35,9 +35,6 @@
 // threads (and i disks) per block of the all-pairs force adjoint
 #define BD_ADJ_T 128
 
-// a check pass's verdict bits for the triangle it visits (held in registers)
-#define BD_TRI_INVERTED 1
-#define BD_TRI_DIRTY 2
 // tv[t].w bits 24-31: the low byte of the generation of the check pass that
 // must test the triangle's edges (set by flips and by flip candidates left
 // unresolved; a stale byte that happens to match only adds tests)
@@ -173,7 +170,6 @@ struct BdDev {
   // 2 x nt flip claims: the round of epoch e claims in half e % 2 (so a round
   // can claim for the next while its own claims are read)
   unsigned long long *claim;
-  int *vt;                 // per vertex: one corner holding it (kept by the flips)
   // tinv = 1 while a triangle is inverted (set by a check pass, cleared by
   // the triangle's flip); clist = 3 x nt: the triangles that registered a flip
   // candidate for the round of epoch e sit in list e % 3 (BdCtl::cl_n)

@@ -398,15 +398,12 @@ __device__ __forceinline__ void journal(const Ctx &x, int t, const int4 &V, cons
   x.d.jtv[t] = V;
   x.d.jtn[t] = N;
 }
-// undo of a journaled triangle t: its corners and neighbours as they were, a
-// corner for each of its vertices, and its neighbours' back-pointers
+// undo of a journaled triangle t: its corners and neighbours as they were, and
+// its neighbours' back-pointers
 __device__ __forceinline__ void unjournal(const BdDev &d, int t) {
   const int4 vs = d.jtv[t], ns = d.jtn[t];
   d.tv[t] = vs;
   d.tn[t] = ns;
-  d.vt[vs.x] = 3 * t;
-  d.vt[vs.y] = 3 * t + 1;
-  d.vt[vs.z] = 3 * t + 2;
   const int nk[3] = {ns.x, ns.y, ns.z};
   for (int k = 0; k < 3; ++k)
     if (nk[k] >= 0) ((int *)&d.tn[nk[k] / 3])[nk[k] % 3] = 3 * t + k;
@@ -470,11 +467,7 @@ __device__ void flip_owned(const Ctx &x, int c0, int o0, uint8_t stamp) {
   x.d.tn[t1] = N1;
   x.d.tinv[t0] = 0;
   x.d.tinv[t1] = 0;
-  // the four vertices' corners moved: t0 = (b, d, a), t1 = (c, a, d)
-  x.d.vt[b] = 3 * t0 + k0;
-  x.d.vt[dd] = 3 * t0 + (k0 + 1) % 3;
-  x.d.vt[a] = 3 * t0 + (k0 + 2) % 3;
-  x.d.vt[c] = 3 * t1 + k1;
+  // t0 = (b, d, a), t1 = (c, a, d)
   if (n_ab >= 0) ((int *)&x.d.tn[n_ab / 3])[n_ab % 3] = 3 * t0 + (k0 + 1) % 3;
   if (n_bd >= 0) ((int *)&x.d.tn[n_bd / 3])[n_bd % 3] = 3 * t0 + (k0 + 2) % 3;
   if (n_dc >= 0) ((int *)&x.d.tn[n_dc / 3])[n_dc % 3] = 3 * t1 + (k1 + 1) % 3;
@@ -635,10 +628,6 @@ __device__ __forceinline__ FusedOut fused_flip(const Ctx &x, int t0, unsigned lo
   d.tn[t1] = N1;
   d.tinv[t0] = 0;
   d.tinv[t1] = 0;
-  d.vt[b] = 3 * t0 + k0;
-  d.vt[dd] = 3 * t0 + (k0 + 1) % 3;
-  d.vt[a] = 3 * t0 + (k0 + 2) % 3;
-  d.vt[c] = 3 * t1 + k1;
   if (n_ab >= 0) ((int *)&d.tn[n_ab / 3])[n_ab % 3] = 3 * t0 + (k0 + 1) % 3;
   if (n_bd >= 0) ((int *)&d.tn[n_bd / 3])[n_bd % 3] = 3 * t0 + (k0 + 2) % 3;
   if (n_dc >= 0) ((int *)&d.tn[n_dc / 3])[n_dc % 3] = 3 * t1 + (k1 + 1) % 3;
@@ -1387,8 +1376,7 @@ __device__ __forceinline__ void triangulation_body(const BdDev &d, const BdConst
       d.disp[i] = make_double2(0.0, 0.0);
       d.moved[i] = 0;
     }
-    // the journaled triangles as they were; a corner for each of their
-    // vertices (flips re-point only the vertices of the triangles they change)
+    // the journaled triangles as they were
     for (int t = tid; t < x.T; t += nth) {
       d.tinv[t] = 0;
       if (d.jmark[t] == x.jstamp) unjournal(d, t);
@@ -1461,9 +1449,8 @@ __global__ void k_restore_step(BdDev d, BdConst c) {
     d.moved[i] = 0;
   }
   if (!c.overlap_verlet) {
-    // the journaled triangles as they were, a corner for each of their
-    // vertices; their marks cleared (the abandoned launch did not publish its
-    // epoch, so the next launch takes the same stamp)
+    // the journaled triangles as they were; their marks cleared (the abandoned
+    // launch did not publish its epoch, so the next launch takes the same stamp)
     const unsigned jstamp = ((unsigned)d.ctl->epoch << 1) | 1u;
     for (int t = tid; t < c.nt; t += nth) {
       d.tinv[t] = 0;

@@ -100,9 +100,6 @@ __device__ __forceinline__ float4 swarp_box(float4 bx) {
   return bx;
 }
 __device__ __forceinline__ float4 sempty_box() { return make_float4(3e38f, -3e38f, 3e38f, -3e38f); }
-__device__ __forceinline__ float4 smerge_box(float4 a, float4 b) {
-  return make_float4(fminf(a.x, b.x), fmaxf(a.y, b.y), fminf(a.z, b.z), fmaxf(a.w, b.w));
-}
 
 // minimum image of a packed pair of coordinate differences in (-3L/2, 3L/2):
 // t = rint(dx / L) by the 1.5 2^23 rounding constant, dx - t L exact (Sterbenz)
@@ -136,13 +133,15 @@ __device__ __forceinline__ float4 ld_local4(const float4 *p) {
 
 }  // namespace
 
-// NW warps per block, NP packed i pairs (2 NP disks) per lane, NJ disks j
-// carried per lane, COMB: fold the packed halves of a j accumulator before
-// passing it (2 shuffles instead of 4), UR: unrolled ring steps.
-// NW * 32 * 2 * NP = BD_SB.  Shapes built: (4 warps, 4 disks per lane) and
-// (2 warps, 8 disks per lane), one j per lane, halves passed unfolded; the
-// second halves the ring's shuffles and register moves per pair.  (Two j per
-// lane, folded halves and deeper unrolling measured within 3 % of these.)
+// NW warps per block, NP packed i pairs (2 NP disks) per lane, one disk j
+// carried per lane; NW * 32 * 2 * NP = BD_SB.  Shapes built: (4 warps, 4 disks per
+// lane) and (2 warps, 8 disks per lane); the second halves the ring's shuffles
+// and register moves per pair.  (Two j per lane, the packed halves of a j
+// accumulator folded before it is passed, and deeper unrolling measured within
+// 3 % of these.)  A tile of j is copied raw with cp.async (no registers held
+// across the tile's arithmetic) and each j re-centred as it is read (walls),
+// or, PER, the tile is re-centred in place once it has landed.  The i side's sum
+// over an item's tiles is float-float.
 //
 // PER (periodic boxes, Sec. 2.1): every coordinate is re-centred on the block
 // origin as its minimum image, as an FP32 (hi, lo) pair (rel_raw); each warp
@@ -152,25 +151,16 @@ __device__ __forceinline__ float4 ld_local4(const float4 *p) {
 // one spanning the box) tell which pair form every pair of the two may take
 // (pair_mode): hi parts alone; per-pair minimum image on one axis or both;
 // the exact vector for boxes closer than 20.
-// STAGE: 0 stage the next j tile through registers (re-centred on the way to
-// shared memory); 1 copy it raw with cp.async (no registers held across the
-// tile's arithmetic) and re-centre each j as it is read (walls), or, PER,
-// re-centre the tile in place once it has landed.  PER takes STAGE 1.
-// ACC: the i side's sum over an item's tiles, 2 in (hi, lo) float-float, 1 in
-// FP32 (half the registers).
-template <int NW, int NP, int NJ, bool COMB, int UR, bool PER, int STAGE = 0, int ACC = 2>
+template <int NW, int NP, bool PER>
 __device__ __forceinline__ void force_long_sym_body(const BdDev &d, const BdConst &c) {
-  static_assert(!PER || STAGE == 1, "the periodic form re-centres tiles in shared memory");
   if (ctl_failed(d.ctl)) return;
   constexpr int T = NW * 32;         // threads
   constexpr int NQ = 2 * NP;         // disks i per thread
   constexpr int NS = BD_TJ / T;      // j disks each thread stages per tile
   constexpr int NG = BD_TJ / BD_SG;  // groups of 32 disks j per tile
-  static_assert(NJ == 1, "a ring carries one group of 32 disks j");
   static_assert(BD_SB == T * NQ, "a block is BD_SB disks");
-  __shared__ float2 sjp[2][STAGE ? 1 : BD_TJ];   // j positions, re-centred
-  __shared__ __align__(16) float4 sraw[2][STAGE ? BD_TJ : 1];   // STAGE 1: j as stored (x_hi, y_hi, x_lo, y_lo);
-                                                                // PER: re-centred in place (hi, lo)
+  __shared__ __align__(16) float4 sraw[2][BD_TJ];   // j as stored (x_hi, y_hi, x_lo, y_lo);
+                                                    // PER: re-centred in place (hi, lo)
   __shared__ float2 shw[NW][BD_TJ];  // per-warp j-side sums of the current tile
   __shared__ float4 sgbox[2][PER ? NG : 1];   // PER: per-group boxes of the staged tile
   __shared__ int sgpad[2][PER ? NG : 1];      //      and whether the group holds inert slots
@@ -201,7 +191,7 @@ __device__ __forceinline__ void force_long_sym_body(const BdDev &d, const BdCons
   auto islot = [&](int q) -> int { return PER ? warp * (BD_SB / NW) + q * 32 + lane : q * T + tid; };
   u64 xi2[NP], yi2[NP], ax2[NP], ay2[NP];
   float4 ilo[PER ? NP : 1];          // PER: lo parts of the disks i (x0, y0, x1, y1), local memory
-  float fxh[NQ], fxl[ACC == 2 ? NQ : 1], fyh[NQ], fyl[ACC == 2 ? NQ : 1];
+  float fxh[NQ], fxl[NQ], fyh[NQ], fyl[NQ];
   float4 ibox = sempty_box();
   bool ipad = false;
 #pragma unroll
@@ -229,74 +219,60 @@ __device__ __forceinline__ void force_long_sym_body(const BdDev &d, const BdCons
   const u64 invL2 = pk2(Lf > 0.f ? 1.0f / Lf : 0.f, Lf > 0.f ? 1.0f / Lf : 0.f);
   const u64 nL2 = pk2(-Lf, -Lf), M2 = pk2(12582912.0f, 12582912.0f);
 #pragma unroll
-  for (int q = 0; q < NQ; ++q) {
-    fxh[q] = fyh[q] = 0.f;
-    if (ACC == 2) fxl[q] = fyl[q] = 0.f;
-  }
+  for (int q = 0; q < NQ; ++q) fxh[q] = fyh[q] = fxl[q] = fyl[q] = 0.f;
   const float e0 = 1e-20f * (float)(c.a * c.a);   // makes the self pair exactly 0
   const u64 eps2 = pk2(e0, e0);
   const int t_begin = item.y / NG, t_end = (item.z + NG - 1) / NG;   // tiles staged
   // j sums: group G of the item at slot item.w + G - max(item.y, gsym)
   float2 *const jout = d.jpart + ((ptrdiff_t)item.w - max(item.y, gsym)) * BD_SG;
-  float4 st[STAGE ? 1 : NS];
   int buf = 0;
   auto fetch = [&](int tile) {
-    if constexpr (STAGE == 1) {
-      // asynchronous 16-byte copies straight into shared memory
+    // asynchronous 16-byte copies straight into shared memory
 #pragma unroll
-      for (int m = 0; m < NS; ++m) {
-        const unsigned dst = (unsigned)__cvta_generic_to_shared(&sraw[buf ^ 1][m * T + tid]);
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst),
-                     "l"(d.work + (size_t)tile * BD_TJ + m * T + tid)
-                     : "memory");
-      }
-      asm volatile("cp.async.commit_group;" ::: "memory");
-    } else {
-#pragma unroll
-      for (int m = 0; m < NS; ++m) st[m] = rel(tile * BD_TJ + m * T + tid);
+    for (int m = 0; m < NS; ++m) {
+      const unsigned dst = (unsigned)__cvta_generic_to_shared(&sraw[buf ^ 1][m * T + tid]);
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst),
+                   "l"(d.work + (size_t)tile * BD_TJ + m * T + tid)
+                   : "memory");
     }
+    asm volatile("cp.async.commit_group;" ::: "memory");
   };
   auto store = [&](int b) {
-    if constexpr (STAGE == 1) {
-      asm volatile("cp.async.wait_group 0;" ::: "memory");
-      if constexpr (PER) {
-        // each thread re-centres the slots it copied (its own copies are
-        // visible to it after the wait), in place; the warp's 32 slots of
-        // stage m are group m NW + warp, whose box is taken about its first
-        // live disk (minimum images about it), then shifted back
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    if constexpr (PER) {
+      // each thread re-centres the slots it copied (its own copies are
+      // visible to it after the wait), in place; the warp's 32 slots of
+      // stage m are group m NW + warp, whose box is taken about its first
+      // live disk (minimum images about it), then shifted back
 #pragma unroll
-        for (int m = 0; m < NS; ++m) {
-          const float4 v = rel_raw(sraw[b][m * T + tid], org, Lf, hLf);
-          sraw[b][m * T + tid] = v;
-          const bool live = v.x < 1.0e17f;
-          const unsigned bal = __ballot_sync(0xffffffffu, live);
-          float4 bx = sempty_box();
-          if (bal) {
-            const int src = __ffs(bal) - 1;
-            const float rx = __shfl_sync(0xffffffffu, v.x, src), ry = __shfl_sync(0xffffffffu, v.y, src);
-            if (live) {
-              float dx = __fsub_rn(v.x, rx), dy = __fsub_rn(v.y, ry);
-              if (per) {
-                dx = dx > hLf ? __fsub_rn(dx, Lf) : (dx < -hLf ? __fadd_rn(dx, Lf) : dx);
-                dy = dy > hLf ? __fsub_rn(dy, Lf) : (dy < -hLf ? __fadd_rn(dy, Lf) : dy);
-              }
-              bx = make_float4(dx, dx, dy, dy);
+      for (int m = 0; m < NS; ++m) {
+        const float4 v = rel_raw(sraw[b][m * T + tid], org, Lf, hLf);
+        sraw[b][m * T + tid] = v;
+        const bool live = v.x < 1.0e17f;
+        const unsigned bal = __ballot_sync(0xffffffffu, live);
+        float4 bx = sempty_box();
+        if (bal) {
+          const int src = __ffs(bal) - 1;
+          const float rx = __shfl_sync(0xffffffffu, v.x, src), ry = __shfl_sync(0xffffffffu, v.y, src);
+          if (live) {
+            float dx = __fsub_rn(v.x, rx), dy = __fsub_rn(v.y, ry);
+            if (per) {
+              dx = dx > hLf ? __fsub_rn(dx, Lf) : (dx < -hLf ? __fadd_rn(dx, Lf) : dx);
+              dy = dy > hLf ? __fsub_rn(dy, Lf) : (dy < -hLf ? __fadd_rn(dy, Lf) : dy);
             }
-            bx = swarp_box(bx);
-            bx = make_float4(__fadd_rn(rx, bx.x), __fadd_rn(rx, bx.y), __fadd_rn(ry, bx.z), __fadd_rn(ry, bx.w));
+            bx = make_float4(dx, dx, dy, dy);
           }
-          if (lane == 0) {
-            sgbox[b][m * NW + warp] = bx;
-            sgpad[b][m * NW + warp] = bal != 0xffffffffu ? 1 : 0;
-          }
+          bx = swarp_box(bx);
+          bx = make_float4(__fadd_rn(rx, bx.x), __fadd_rn(rx, bx.y), __fadd_rn(ry, bx.z), __fadd_rn(ry, bx.w));
+        }
+        if (lane == 0) {
+          sgbox[b][m * NW + warp] = bx;
+          sgpad[b][m * NW + warp] = bal != 0xffffffffu ? 1 : 0;
         }
       }
-    } else {
-#pragma unroll
-      for (int m = 0; m < NS; ++m) sjp[b][m * T + tid] = make_float2(st[m].x, st[m].y);
     }
   };
-  buf = STAGE ? 1 : 0;   // STAGE 1: fetch fills sraw[buf ^ 1]
+  buf = 1;   // fetch fills sraw[buf ^ 1]
   if (t_begin < t_end) {
     fetch(t_begin);
     store(0);
@@ -305,9 +281,8 @@ __device__ __forceinline__ void force_long_sym_body(const BdDev &d, const BdCons
   __syncthreads();
   // the j disk in slot jj of the current staging buffer, re-centred
   auto jpos = [&](int jj) -> float2 {
-    if constexpr (STAGE == 1 && PER) return make_float2(sraw[buf][jj].x, sraw[buf][jj].y);
-    else if constexpr (STAGE == 1) return recentre(sraw[buf][jj], org);
-    else return sjp[buf][jj];
+    if constexpr (PER) return make_float2(sraw[buf][jj].x, sraw[buf][jj].y);
+    else return recentre(sraw[buf][jj], org);
   };
   // PER: its lo parts
   auto jlo = [&](int jj) -> float2 { return make_float2(sraw[buf][jj].z, sraw[buf][jj].w); };
@@ -337,22 +312,17 @@ __device__ __forceinline__ void force_long_sym_body(const BdDev &d, const BdCons
   };
   using AXX = std::integral_constant<int, 0>;
   using AXY = std::integral_constant<int, 1>;
-  // PER: the pair form of this warp's disks i with the j groups g0 .. g0 +
-  // ng - 1 of the current tile.  Pair components range over [j_min - i_max,
+  // PER: the pair form of this warp's disks i with the j group g0 of the current tile.  Pair components range over [j_min - i_max,
   // j_max - i_min]; a plain difference is the minimum image when that range
   // and the j coordinates themselves lie inside (-L/2, L/2) (then each j is
   // stored as the image its box describes), with a margin of 2^-16 L/2 for
   // the rounding of the boxes.  Near: the range comes within 20 of 0 or L.
-  auto pair_mode = [&](int g0, int ng) -> int {
+  auto pair_mode = [&](int g0) -> int {
     if constexpr (!PER) return 0;
     const float4 ib = sibox[warp];
     if (ib.x > ib.y) return 0;                 // the warp's disks i are all inert
-    float4 jb = sempty_box();
-    int pad = sipad[warp];
-    for (int u = 0; u < ng; ++u) {
-      jb = smerge_box(jb, sgbox[buf][g0 + u]);
-      pad |= sgpad[buf][g0 + u];
-    }
+    const float4 jb = sgbox[buf][g0];
+    const int pad = sipad[warp] | sgpad[buf][g0];
     if (jb.x > jb.y) return 0;                 // inert disks j only: their pairs vanish
     const float lox = __fsub_rn(jb.x, ib.y), hix = __fsub_rn(jb.y, ib.x);
     const float loy = __fsub_rn(jb.z, ib.w), hiy = __fsub_rn(jb.w, ib.z);
@@ -429,90 +399,69 @@ __device__ __forceinline__ void force_long_sym_body(const BdDev &d, const BdCons
     }
   };
   auto ring_group = [&](auto MODE, int g) {
-    // a later tile's group g: every pair once, both sides; each lane carries NJ disks j
+    // a later tile's group g: every pair once, both sides; each lane carries one disk j
     constexpr bool LO = decltype(MODE)::value == 1 || decltype(MODE)::value == 4;
-    float jx[NJ], jy[NJ], jxl[NJ], jyl[NJ];
-    u64 hx2[NJ], hy2[NJ];
-#pragma unroll
-    for (int m = 0; m < NJ; ++m) {
-      const float2 p = jpos((g * NJ + m) * 32 + lane);
-      jx[m] = p.x;
-      jy[m] = p.y;
-      jxl[m] = jyl[m] = 0.f;
-      if constexpr (LO) {
-        const float2 pl = jlo((g * NJ + m) * 32 + lane);
-        jxl[m] = pl.x;
-        jyl[m] = pl.y;
-      }
-      hx2[m] = hy2[m] = 0ull;
+    const float2 p = jpos(g * 32 + lane);
+    float jx = p.x, jy = p.y, jxl = 0.f, jyl = 0.f;
+    if constexpr (LO) {
+      const float2 pl = jlo(g * 32 + lane);
+      jxl = pl.x;
+      jyl = pl.y;
     }
-#pragma unroll UR
+    u64 hx2 = 0ull, hy2 = 0ull;
+    float h0, h1, h2, h3;
+#pragma unroll 2
     for (int rot = 0; rot < 32; ++rot) {
       const int src = (lane + 1) & 31;
-#pragma unroll
-      for (int m = 0; m < NJ; ++m) {
-        const u64 jx2 = pk2(jx[m], jx[m]), jy2 = pk2(jy[m], jy[m]);
-        const u64 jxl2 = LO ? pk2(jxl[m], jxl[m]) : 0ull, jyl2 = LO ? pk2(jyl[m], jyl[m]) : 0ull;
-        // the next j position does not depend on this step's arithmetic
-        const float njx = __shfl_sync(0xffffffffu, jx[m], src);
-        const float njy = __shfl_sync(0xffffffffu, jy[m], src);
-        float njxl = 0.f, njyl = 0.f;
-        if constexpr (LO) {
-          njxl = __shfl_sync(0xffffffffu, jxl[m], src);
-          njyl = __shfl_sync(0xffffffffu, jyl[m], src);
-        }
-#pragma unroll
-        for (int k = 0; k < NP; ++k) {
-          u64 ixl2 = 0ull, iyl2 = 0ull;
-          if constexpr (LO) {
-            const float4 il = ld_local4(&ilo[k]);
-            ixl2 = pk2(il.x, il.z);
-            iyl2 = pk2(il.y, il.w);
-          }
-          const u64 dx = diff(MODE, AXX(), jx2, xi2[k], jxl2, ixl2);
-          const u64 dy = diff(MODE, AXY(), jy2, yi2[k], jyl2, iyl2);
-          u64 r2 = fma2(dx, dx, eps2);
-          r2 = fma2(dy, dy, r2);
-          float ra, rb;
-          up2(r2, ra, rb);
-          const u64 sv = pk2(rsqrt_apx(ra), rsqrt_apx(rb));
-          const u64 s3 = mul2(mul2(sv, sv), sv);
-          ax2[k] = fma2(dx, s3, ax2[k]);
-          ay2[k] = fma2(dy, s3, ay2[k]);
-          hx2[m] = fma2(dx, s3, hx2[m]);
-          hy2[m] = fma2(dy, s3, hy2[m]);
-        }
-        // pass the j accumulator one lane down the ring, after its disk
-        float h0, h1, h2, h3;
-        up2(hx2[m], h0, h1);
-        up2(hy2[m], h2, h3);
-        if (COMB) {
-          h0 = __shfl_sync(0xffffffffu, __fadd_rn(h0, h1), src);
-          h2 = __shfl_sync(0xffffffffu, __fadd_rn(h2, h3), src);
-          hx2[m] = pk2(h0, 0.f);
-          hy2[m] = pk2(h2, 0.f);
-        } else {
-          h0 = __shfl_sync(0xffffffffu, h0, src);
-          h1 = __shfl_sync(0xffffffffu, h1, src);
-          h2 = __shfl_sync(0xffffffffu, h2, src);
-          h3 = __shfl_sync(0xffffffffu, h3, src);
-          hx2[m] = pk2(h0, h1);
-          hy2[m] = pk2(h2, h3);
-        }
-        jx[m] = njx;
-        jy[m] = njy;
-        jxl[m] = njxl;
-        jyl[m] = njyl;
+      const u64 jx2 = pk2(jx, jx), jy2 = pk2(jy, jy);
+      const u64 jxl2 = LO ? pk2(jxl, jxl) : 0ull, jyl2 = LO ? pk2(jyl, jyl) : 0ull;
+      // the next j position does not depend on this step's arithmetic
+      const float njx = __shfl_sync(0xffffffffu, jx, src);
+      const float njy = __shfl_sync(0xffffffffu, jy, src);
+      float njxl = 0.f, njyl = 0.f;
+      if constexpr (LO) {
+        njxl = __shfl_sync(0xffffffffu, jxl, src);
+        njyl = __shfl_sync(0xffffffffu, jyl, src);
       }
+#pragma unroll
+      for (int k = 0; k < NP; ++k) {
+        u64 ixl2 = 0ull, iyl2 = 0ull;
+        if constexpr (LO) {
+          const float4 il = ld_local4(&ilo[k]);
+          ixl2 = pk2(il.x, il.z);
+          iyl2 = pk2(il.y, il.w);
+        }
+        const u64 dx = diff(MODE, AXX(), jx2, xi2[k], jxl2, ixl2);
+        const u64 dy = diff(MODE, AXY(), jy2, yi2[k], jyl2, iyl2);
+        u64 r2 = fma2(dx, dx, eps2);
+        r2 = fma2(dy, dy, r2);
+        float ra, rb;
+        up2(r2, ra, rb);
+        const u64 sv = pk2(rsqrt_apx(ra), rsqrt_apx(rb));
+        const u64 s3 = mul2(mul2(sv, sv), sv);
+        ax2[k] = fma2(dx, s3, ax2[k]);
+        ay2[k] = fma2(dy, s3, ay2[k]);
+        hx2 = fma2(dx, s3, hx2);
+        hy2 = fma2(dy, s3, hy2);
+      }
+      // pass the j accumulator one lane down the ring, after its disk
+      up2(hx2, h0, h1);
+      up2(hy2, h2, h3);
+      h0 = __shfl_sync(0xffffffffu, h0, src);
+      h1 = __shfl_sync(0xffffffffu, h1, src);
+      h2 = __shfl_sync(0xffffffffu, h2, src);
+      h3 = __shfl_sync(0xffffffffu, h3, src);
+      hx2 = pk2(h0, h1);
+      hy2 = pk2(h2, h3);
+      jx = njx;
+      jy = njy;
+      jxl = njxl;
+      jyl = njyl;
     }
     // after 32 passes every j is back in its own lane
-#pragma unroll
-    for (int m = 0; m < NJ; ++m) {
-      float h0, h1, h2, h3;
-      up2(hx2[m], h0, h1);
-      up2(hy2[m], h2, h3);
-      shw[warp][(g * NJ + m) * 32 + lane] = make_float2(__fadd_rn(h0, h1), __fadd_rn(h2, h3));
-    }
+    up2(hx2, h0, h1);
+    up2(hy2, h2, h3);
+    shw[warp][g * 32 + lane] = make_float2(__fadd_rn(h0, h1), __fadd_rn(h2, h3));
   };
   for (int t = t_begin; t < t_end; ++t) {
     if (t + 1 < t_end) fetch(t + 1);
@@ -520,10 +469,10 @@ __device__ __forceinline__ void force_long_sym_body(const BdDev &d, const BdCons
     const int ga = max(item.y - t * NG, 0), gz = min(item.z - t * NG, NG);   // the item's groups of the tile
     if (t * NG < gsym) {
       for (int g = ga; g < gz; ++g)
-        dispatch(pair_mode(g, 1), [&](auto M) { own_group(M, g); });
+        dispatch(pair_mode(g), [&](auto M) { own_group(M, g); });
     } else {
       for (int g = ga; g < gz; ++g)
-        dispatch(pair_mode(g, 1), [&](auto M) { ring_group(M, g); });
+        dispatch(pair_mode(g), [&](auto M) { ring_group(M, g); });
       __syncthreads();
       // j side of this tile: F_j += A[s_j][s_i] sum_i (r_j - r_i)/r^3
       const float alj = R.alpha[BD_MAX_SPECIES * b + a];
@@ -545,17 +494,10 @@ __device__ __forceinline__ void force_long_sym_body(const BdDev &d, const BdCons
       float ax0, ax1, ay0, ay1;
       up2(ax2[k], ax0, ax1);
       up2(ay2[k], ay0, ay1);
-      if constexpr (ACC == 2) {
-        two_sum(fxh[2 * k], fxl[2 * k], -ali * ax0);
-        two_sum(fyh[2 * k], fyl[2 * k], -ali * ay0);
-        two_sum(fxh[2 * k + 1], fxl[2 * k + 1], -ali * ax1);
-        two_sum(fyh[2 * k + 1], fyl[2 * k + 1], -ali * ay1);
-      } else {
-        fxh[2 * k] = __fmaf_rn(-ali, ax0, fxh[2 * k]);
-        fyh[2 * k] = __fmaf_rn(-ali, ay0, fyh[2 * k]);
-        fxh[2 * k + 1] = __fmaf_rn(-ali, ax1, fxh[2 * k + 1]);
-        fyh[2 * k + 1] = __fmaf_rn(-ali, ay1, fyh[2 * k + 1]);
-      }
+      two_sum(fxh[2 * k], fxl[2 * k], -ali * ax0);
+      two_sum(fyh[2 * k], fyl[2 * k], -ali * ay0);
+      two_sum(fxh[2 * k + 1], fxl[2 * k + 1], -ali * ax1);
+      two_sum(fyh[2 * k + 1], fyl[2 * k + 1], -ali * ay1);
       ax2[k] = ay2[k] = 0ull;
     }
     if (t + 1 < t_end) store(buf ^ 1);
@@ -564,16 +506,13 @@ __device__ __forceinline__ void force_long_sym_body(const BdDev &d, const BdCons
   }
   float2 *ip = d.ipart + (size_t)item_id * BD_SB;
 #pragma unroll
-  for (int q = 0; q < NQ; ++q) {
-    if constexpr (ACC == 2) ip[islot(q)] = make_float2(__fadd_rn(fxh[q], fxl[q]), __fadd_rn(fyh[q], fyl[q]));
-    else ip[islot(q)] = make_float2(fxh[q], fyh[q]);
-  }
+  for (int q = 0; q < NQ; ++q) ip[islot(q)] = make_float2(__fadd_rn(fxh[q], fxl[q]), __fadd_rn(fyh[q], fyl[q]));
 }
 
 // with a register budget for MINB resident blocks per SM
-template <int NW, int NP, int NJ, bool COMB, int UR, bool PER, int MINB, int STAGE, int ACC>
+template <int NW, int NP, bool PER, int MINB>
 __global__ void __launch_bounds__(NW * 32, MINB) k_force_long_sym_mb(BdDev d, BdConst c) {
-  force_long_sym_body<NW, NP, NJ, COMB, UR, PER, STAGE, ACC>(d, c);
+  force_long_sym_body<NW, NP, PER>(d, c);
 }
 
 // F_i = sum of its block's i partials + sum of its group's j partials, in the
@@ -692,14 +631,14 @@ int bd_force_sym_blocks_per_sm(int variant, int periodic) {
   cudaError_t e;
   if (periodic)
     e = variant == 2 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                           &per, k_force_long_sym_mb<4, 2, 1, false, 2, true, 8, 1, 2>, 128, 0)
+                           &per, k_force_long_sym_mb<4, 2, true, 8>, 128, 0)
                      : cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                           &per, k_force_long_sym_mb<2, 4, 1, false, 2, true, 12, 1, 2>, 64, 0);
+                           &per, k_force_long_sym_mb<2, 4, true, 12>, 64, 0);
   else
     e = variant == 2 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                           &per, k_force_long_sym_mb<4, 2, 1, false, 2, false, 8, 1, 2>, 128, 0)
+                           &per, k_force_long_sym_mb<4, 2, false, 8>, 128, 0)
                      : cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                           &per, k_force_long_sym_mb<2, 4, 1, false, 2, false, 16, 1, 2>, 64, 0);
+                           &per, k_force_long_sym_mb<2, 4, false, 16>, 64, 0);
   return e == cudaSuccess ? per : 0;
 }
 
@@ -716,12 +655,12 @@ static void launch_sweep(const BdDev &d, const BdConst &c, int variant, cudaStre
     // 2.86 ms before, with one form per (block, tile) and the tiles staged
     // through registers
     if (variant == 2)
-      k_force_long_sym_mb<4, 2, 1, false, 2, true, 8, 1, 2><<<c.n_sitems, 128, 0, s>>>(d, c);
+      k_force_long_sym_mb<4, 2, true, 8><<<c.n_sitems, 128, 0, s>>>(d, c);
     else
-      k_force_long_sym_mb<2, 4, 1, false, 2, true, 12, 1, 2><<<c.n_sitems, 64, 0, s>>>(d, c);
+      k_force_long_sym_mb<2, 4, true, 12><<<c.n_sitems, 64, 0, s>>>(d, c);
   } else {
     if (variant == 2)
-      k_force_long_sym_mb<4, 2, 1, false, 2, false, 8, 1, 2><<<c.n_sitems, 128, 0, s>>>(d, c);
+      k_force_long_sym_mb<4, 2, false, 8><<<c.n_sitems, 128, 0, s>>>(d, c);
     else
       // 16 resident blocks (32 warps) per SM in 64 registers, j tiles staged by
       // cp.async: measured 1.776 -> 1.668 ms at N = 1e5 against the
@@ -730,7 +669,7 @@ static void launch_sweep(const BdDev &d, const BdConst &c, int variant, cudaStre
       // unrolled 1 or 4 steps deep (+1.7 %, +1.1 %), two j disks per lane
       // (+1.9 %), folded j accumulators (+3.5 %), one warp of 16 disks per
       // lane (+2.7 %)
-      k_force_long_sym_mb<2, 4, 1, false, 2, false, 16, 1, 2><<<c.n_sitems, 64, 0, s>>>(d, c);
+      k_force_long_sym_mb<2, 4, false, 16><<<c.n_sitems, 64, 0, s>>>(d, c);
   }
 }
 
