@@ -233,17 +233,21 @@ int bd_noise_sample(uint64_t seed, int32_t replica, int32_t n, const uint32_t *c
 int bd_set_loop_caps(bd_handle *h, int32_t max_corr_iters, int32_t max_flip_rounds);
 
 /* Time limit of the device-side waits of h's persistent kernels (the grid
- * barriers of the triangulation kernel and of the Verlet-list correction):
+ * barriers of the triangulation kernel, the Verlet-list rebuild and the
+ * Verlet-list correction; triangulations of up to 4096 triangles run as one
+ * thread-block cluster, whose hardware barrier takes no limit):
  * a barrier that waits longer sets BD_ERR_DEVICE_TIMEOUT, every block leaves
  * its kernel, and the call that launched it undoes the step (or the new
  * positions of bd_set_state) from its step-start copies and returns
  * BD_ERR_DEVICE_TIMEOUT, the handle usable.  Default 2 s.
  *   seconds       1e-3 .. 60.
- *   hold_barrier  0 for normal use.  k > 0 makes the k-th grid barrier of every
- *                 later launch of those kernels wait for one block more than
- *                 the launch has, so that it runs out: a way to test the
- *                 timeout path that faults nothing (each block gives up after
- *                 `seconds`).  Set it back to 0 to step normally.
+ *   hold_barrier  0 for normal use.  k > 0 makes the k-th barrier of every
+ *                 later launch of the triangulation kernel and the Verlet-list
+ *                 correction run out (a grid waits for one block more than the
+ *                 launch has, a cluster waits out the limit behind its
+ *                 barrier): a way to test the timeout path that faults nothing
+ *                 (each block gives up after `seconds`).  Set it back to 0 to
+ *                 step normally.
  * Errors: BD_ERR_ARG, BD_ERR_CUDA. */
 int bd_set_wait_limit(bd_handle *h, double seconds, int32_t hold_barrier);
 

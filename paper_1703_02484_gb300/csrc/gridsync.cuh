@@ -1,9 +1,12 @@
 // Grid-wide barrier and block-level helpers of the persistent kernels
 // (triangulation maintenance, Verlet-list overlap correction).  The kernels
-// are launched cooperatively (every block resident), and every wait is
-// bounded: a barrier that waits longer than its limit (BD_BARRIER_TIMEOUT_NS,
+// are launched cooperatively (every block resident), and every wait of a grid
+// is bounded: a barrier that waits longer than its limit (BD_BARRIER_TIMEOUT_NS,
 // or the limit the host set in the control block) sets BD_ERR_DEVICE_TIMEOUT
-// and every block leaves.
+// and every block leaves.  A small system's triangulation runs in one
+// thread-block cluster and waits at the hardware's cluster barrier, which takes
+// no limit: the blocks of a cluster are resident together and take every branch
+// on the same words, so each of them arrives.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -46,6 +49,9 @@ enum { BC_CNT = 0, BC_CL = 8, BC_N = 11 };
 // the same word: each adds 1, the first block what brings the sum of all to
 // 2^31, so the last arrival flips the top bit and is itself the release; the
 // word needs no reset between barriers (the launch's last block clears it).
+// (The flipped bit is the scheme of cooperative groups' grid barrier, public in
+// the CUDA toolkit's cooperative_groups/details/sync.h; the limit, the hold and
+// the words read behind it are this kernel's.)
 // Measured at 8 to 456 blocks: 1.5 us, against 2.5 with a separate word that the
 // last block to arrive publishes and 3 with a count it also resets.
 template <bool HOLD = true>
