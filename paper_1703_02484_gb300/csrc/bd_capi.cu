@@ -370,6 +370,16 @@ cudaError_t use_variant(bd_handle *h, int variant, int chunk) {
   h->c.force_variant = variant;
   h->tune_chunk = chunk;
   if (variant >= 2 || h->c.f64_sym) {
+    // the j partials alone must fit the device: asked before the plan is made,
+    // whose host lists take a word per j partial group (and count them in ints)
+    const long long jgroups = sym_units(h, h->c.f64_sym ? BD_F64_SB : BD_SB);
+    const size_t jbytes = (size_t)jgroups * BD_SG * (h->c.f64_sym ? sizeof(double2) : sizeof(float2));
+    if (jbytes >> 32) {
+      size_t mem_free = 0, mem_total = 0;
+      const cudaError_t em = cudaMemGetInfo(&mem_free, &mem_total);
+      if (em != cudaSuccess) return em;
+      if (jbytes > mem_total || jgroups > 0x7FFFFFFFll) return cudaErrorMemoryAllocation;
+    }
     SymPlan S;
     make_sym(h, chunk, variant, S);
     return upload_sym(h, S);
